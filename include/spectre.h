@@ -49,12 +49,12 @@ typedef enum { SPECTRE_F32 = 0, SPECTRE_BF16 = 1, SPECTRE_F16 = 2 } spectre_dtyp
 
 typedef struct spectre_ctx spectre_ctx;   /* opaque: device properties, launch limits */
 
-/* Creates a context for CUDA device `device`.  Besides host memory it owns six small device
+/* Creates a context for CUDA device `device`.  Besides host memory it owns seven small device
  * tables (the 64-point and 49-point DFT matrices of the tensor-core mixers, 32 KiB each; the
  * twiddles between two 64-point stages and a quarter-wave twiddle table, 16 KiB each; the twiddles
  * of the four-step splits n = 4096 R, 63 KiB; the DFT matrices of the tensor-core radix-32 ... 2
- * kernels, 320 KiB) and one pinned status word, all released by spectre_destroy.  No other
- * call allocates. */
+ * kernels, 320 KiB; the twiddles of the register-resident fp32 transforms, 52 KiB)
+ * and one pinned status word, all released by spectre_destroy.  No other call allocates. */
 int spectre_create(spectre_ctx** out, int device);
 int spectre_destroy(spectre_ctx* ctx);
 /* The tensor-core mixers record two kinds of trouble in a status word instead of failing on
@@ -203,8 +203,9 @@ typedef struct {
  *   v, y     activations of identical shape and dtype; y may alias v where the
  *            transform is one kernel (the workspace query returns 0, and the
  *            bf16 / fp16 tensor-core paths n_fft = 196 with D = 64 and
- *            n_fft = 8192); on a multi-pass path a call whose v and y overlap
- *            anywhere between their first and last byte is refused with
+ *            n_fft = 8192; the fp32 path at n_fft = 4096 and 8192 is one, slower,
+ *            kernel too when y overlaps v or no workspace is given); on a multi-pass
+ *            path a call whose v and y overlap anywhere between their first and last byte is refused with
  *            SPECTRE_ERR_INVALID_ARG
  *   g        [B, H, K, 2] float32, K = n_fft/2 + 1; one gain per bin per head,
  *            applied to all D columns; Im of the DC / Nyquist gains is ignored

@@ -11,8 +11,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libspectre.so")
 OBJ = os.path.join(PKG, "build")
-SOURCES = ["api.cu", "mixer.cu", "mixer_tc.cu", "mixer_tc8k.cu", "mixer_tc4k.cu", "gate.cu", "cache.cu", "wavelet.cu",
-           "backward.cu", "project.cu"]
+SOURCES = ["reg_grad.cu", "reg_mix.cu", "reg_inverse.cu", "reg_forward.cu", "api.cu", "mixer.cu", "mixer_tc.cu", "mixer_tc8k.cu",
+           "mixer_tc4k.cu", "gate.cu", "cache.cu", "wavelet.cu", "backward.cu", "project.cu"]
 FLAGS = ["-std=c++17", "-O3", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
          "-Xcompiler", "-fPIC", "-shared"]
 

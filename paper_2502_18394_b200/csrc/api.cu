@@ -2,6 +2,7 @@
 #include <cstdio>
 #include <new>
 
+#include "reg_fft.h"
 #include "tc_common.cuh"
 
 namespace spectre {
@@ -99,6 +100,7 @@ extern "C" int spectre_create(spectre_ctx** out, int device) {
   c->tw64x64 = nullptr;
   c->tw_staged = nullptr;
   c->dft32 = nullptr;
+  c->tw_reg = nullptr;
   c->status_host = nullptr;
   c->status_dev = nullptr;
   cudaError_t e2 = cudaSetDevice(device);
@@ -108,6 +110,7 @@ extern "C" int spectre_create(spectre_ctx** out, int device) {
   if (e2 == cudaSuccess) e2 = cudaMalloc(&c->tw64x64, 2048 * sizeof(float2));
   if (e2 == cudaSuccess) e2 = cudaMalloc(&c->tw_staged, 63 * 128 * sizeof(float2));
   if (e2 == cudaSuccess) e2 = cudaMalloc(&c->dft32, 5 * 4 * 16384);
+  if (e2 == cudaSuccess) e2 = cudaMalloc(&c->tw_reg, reg_table_bytes());
   if (e2 == cudaSuccess) e2 = cudaHostAlloc(reinterpret_cast<void**>(&c->status_host), sizeof(int), cudaHostAllocMapped);
   if (e2 == cudaSuccess) {
     *c->status_host = 0;
@@ -120,6 +123,7 @@ extern "C" int spectre_create(spectre_ctx** out, int device) {
     if (rc == SPECTRE_OK) rc = build_tw64x64(reinterpret_cast<float2*>(c->tw64x64), 0);
     if (rc == SPECTRE_OK) rc = build_tw_staged(reinterpret_cast<float2*>(c->tw_staged), 0);
     if (rc == SPECTRE_OK) rc = build_dft32(c->dft32, 0);
+    if (rc == SPECTRE_OK) rc = reg_build_tables(c->tw_reg, 0);
     if (rc == SPECTRE_OK) e2 = cudaStreamSynchronize(0);
     else e2 = cudaErrorUnknown;
   }
@@ -139,6 +143,7 @@ extern "C" int spectre_destroy(spectre_ctx* ctx) {
     if (ctx->tw64x64) cudaFree(ctx->tw64x64);
     if (ctx->tw_staged) cudaFree(ctx->tw_staged);
     if (ctx->dft32) cudaFree(ctx->dft32);
+    if (ctx->tw_reg) cudaFree(ctx->tw_reg);
     if (ctx->status_host) cudaFreeHost(ctx->status_host);
   }
   delete ctx;

@@ -7,13 +7,13 @@
 // column pairs that uses  conj(A^V) A^G + conj(B^V) B^G = ( conj(Z^V_k) Z^G_k + Z^V_{n-k} conj(Z^G_{n-k}) ) / 2.
 // Beyond one CTA's 2048 rows the passes leave the spectra of the N1 decimated sequences and the reduction
 // runs the last radix-N1 step itself.
-#include "common.cuh"
+#include "reg_fft.h"
 
 namespace spectre {
 
 // from mixer.cu
 int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, int n, int slab0, int cnt,
-                      float2* ws, int* N1_out, int* M_out, void* ring, int* ring_done);
+                      float2* ws, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done);
 bool transform_supported(const spectre_ctx* ctx, int n);
 size_t transform_slab_bytes(int n, int D);
 
@@ -23,6 +23,25 @@ __global__ void __launch_bounds__(256) conj_gate_kernel(const float2* __restrict
     float2 v = g[i];
     gc[i] = make_float2(v.x, -v.y);
   }
+}
+
+// dg from the partial sums S_k = sum over the pairs of conj(Z^V_k) Z^G_k of all n bins, which the transform kernels
+// leave per group of pairs: dg_k = (w_k / 2n) (S_k + conj(S_{n-k})).
+__global__ void __launch_bounds__(256) gate_grad_sum_kernel(const float2* __restrict__ sums, float2* __restrict__ dg, int n, int K,
+                                                            int parts, int slab0, int nslab) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (size_t)nslab * K) return;
+  const int k = (int)(i % K), slab_local = (int)(i / K), km = k == 0 ? 0 : n - k;
+  const float2* s = sums + (size_t)slab_local * parts * n;
+  float2 acc = make_float2(0.f, 0.f);
+#pragma unroll 4
+  for (int p = 0; p < parts; ++p) {
+    const float2 a = __ldg(s + (size_t)p * n + k), b = __ldg(s + (size_t)p * n + km);
+    acc.x += a.x + b.x;
+    acc.y += a.y - b.y;
+  }
+  const float w = ((k == 0 || 2 * k == n) ? 0.5f : 1.0f) / (float)n;
+  dg[(size_t)(slab0 + slab_local) * K + k] = cscale(acc, w);
 }
 
 // One warp per (slab, bin): lanes over the column pairs, both workspaces hold the spectrum itself,
@@ -170,6 +189,32 @@ static size_t spectrum_group(int n, int D, int nslab) {
   return g;
 }
 
+// Lengths one CTA transforms: dg, and dv with it, from one kernel over both tensors.
+static size_t grad_slab_bytes(int n, int D) { return (size_t)reg_parts(n, D) * n * sizeof(float2); }
+static int backward_reg(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const spectre_act* dy, const float* g,
+                        const spectre_act* dv, float* dg, int n, void* ws, size_t ws_bytes) {
+  const int nslab = v->B * v->H, K = n / 2 + 1, parts = reg_parts(n, v->D);
+  RegParams p = {};
+  p.n = n; p.K = K; p.H = v->H; p.D = v->D; p.L = v->L; p.N1 = 1;
+  p.scale = 1.0f / (float)n;
+  p.g = reinterpret_cast<const float2*>(g);
+  p.src = v->ptr; p.s_sb = v->stride_b; p.s_sl = v->stride_l; p.s_sh = v->stride_h;
+  p.src2 = dy->ptr; p.s2_sb = dy->stride_b; p.s2_sl = dy->stride_l; p.s2_sh = dy->stride_h;
+  if (dv) { p.dst = dv->ptr; p.d_sb = dv->stride_b; p.d_sl = dv->stride_l; p.d_sh = dv->stride_h; }
+  p.sums = reinterpret_cast<float2*>(ws);
+  size_t group = ws_bytes / grad_slab_bytes(n, v->D);
+  if (group > (size_t)nslab) group = (size_t)nslab;
+  for (int s0 = 0; s0 < nslab; s0 += (int)group) {
+    const int cnt = nslab - s0 < (int)group ? nslab - s0 : (int)group;
+    p.slab0 = s0;
+    int rc = reg_grad(ctx, st, p, n, cnt, v->dtype);
+    if (rc != SPECTRE_OK) return rc;
+    gate_grad_sum_kernel<<<(unsigned)(((size_t)cnt * K + 255) / 256), 256, 0, st>>>(p.sums, reinterpret_cast<float2*>(dg), n, K, parts, s0, cnt);
+    SPECTRE_LAUNCH_OK("gate_grad_sum_kernel");
+  }
+  return SPECTRE_OK;
+}
+
 }  // namespace spectre
 
 using namespace spectre;
@@ -215,6 +260,9 @@ extern "C" int spectre_mixer_backward(spectre_ctx* ctx, void* stream, const spec
   SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   unsigned char* base = reinterpret_cast<unsigned char*>(workspace);
+  auto pitch_ok = [](const spectre_act* a) { return !a || (a->stride_l >= 0 && a->stride_l <= (1 << 18)); };   // 32-bit row offsets
+  if (dg && reg_supported(n_fft) && pitch_ok(v) && pitch_ok(dy) && pitch_ok(dv))
+    return backward_reg(ctx, st, v, dy, g, dv, dg, n_fft, base + gc_bytes + mix_bytes, workspace_bytes - gc_bytes - mix_bytes);
   if (dv) {
     float2* gc = reinterpret_cast<float2*>(base);
     const size_t total = (size_t)nslab * K;
@@ -233,9 +281,9 @@ extern "C" int spectre_mixer_backward(spectre_ctx* ctx, void* stream, const spec
       const int cnt = nslab - s0 < (int)group ? nslab - s0 : (int)group;
       int N1 = 1, M = n_fft;
       int no_ring = 0;
-      rc = forward_decimated(ctx, st, v, n_fft, s0, cnt, wsV, &N1, &M, nullptr, &no_ring);
+      rc = forward_decimated(ctx, st, v, n_fft, s0, cnt, wsV, &N1, &M, 16, nullptr, &no_ring);
       if (rc != SPECTRE_OK) return rc;
-      rc = forward_decimated(ctx, st, dy, n_fft, s0, cnt, wsG, &N1, &M, nullptr, &no_ring);
+      rc = forward_decimated(ctx, st, dy, n_fft, s0, cnt, wsG, &N1, &M, 16, nullptr, &no_ring);
       if (rc != SPECTRE_OK) return rc;
       float2* dgc = reinterpret_cast<float2*>(dg);
       switch (N1) {

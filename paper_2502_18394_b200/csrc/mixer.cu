@@ -11,14 +11,20 @@
 // the inverse is the mirrored decimation-in-time network, so no reordering pass
 // exists.  A tile is 8 complex pairs (16 real columns) of one (batch, head).
 //
-//   onchip kernel   whole transform of a tile in shared memory; optionally a
-//                   cluster of C CTAs splits the sequence and exchanges one
-//                   radix-C stage through distributed shared memory.
+//   register-resident kernels (reg_fft.h) for the lengths of a CTA: powers of two
+//                   64 ... 2048 and some squares; n = 4096 ... 32768 as N1 1024 with
+//                   a strided pass on either side.
+//   onchip kernel   every other length: whole transform of a tile in shared memory; a
+//                   cluster of C CTAs splits the sequence and exchanges one radix-C
+//                   stage through distributed shared memory (n = 4096, 8192 in place
+//                   or without a workspace, and the inner transform beyond 32768).
 //   strided kernels the outer factor N1 of a four-step transform n = N1 * M for
 //                   n beyond the on-chip range, with the twiddles fused.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "fft_reg.cuh"
+#include "reg_fft.h"
 
 namespace cg = cooperative_groups;
 
@@ -83,8 +89,6 @@ struct OnchipParams {
                          // 2: inverse only, from the gated half spectra in `spec`
   int src_ws, dst_ws;
   int decim;             // src_ws = 0 only: element j of sequence k1 is token N1 j + k1 (decimated input)
-  int direct;            // C = 1, 2048 rows, 512 threads: the tile is fetched in one round of 16-byte loads
-  void* ring;            // direct only: dense [B][n][H][D] copy of the (zero-padded) input written while loading, or NULL
   const float2* twq;     // (cos, sin)(2 pi r / 8192), r = 0..2048 (quarter wave): source of the twiddles of the fixed plan
   float scale;           // 1/n, folded into the gate
 };
@@ -350,80 +354,6 @@ __device__ __forceinline__ void cross_stage(const OnchipParams& p, const TileCoo
   }
 }
 
-// 16 bytes of a row as float4 groups of 4 columns: one group for fp32, two for the 16-bit types
-template <typename T> struct RowPiece;
-template <> struct RowPiece<float> {
-  static constexpr int kGroups = 1;
-  static __device__ __forceinline__ float4 group(const uint4& r, int) {
-    return make_float4(__uint_as_float(r.x), __uint_as_float(r.y), __uint_as_float(r.z), __uint_as_float(r.w));
-  }
-};
-template <> struct RowPiece<bf16> {
-  static constexpr int kGroups = 2;
-  static __device__ __forceinline__ float4 group(const uint4& r, int g) {
-    const unsigned lo = g ? r.z : r.x, hi = g ? r.w : r.y;
-    return make_float4(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u), __uint_as_float(hi << 16),
-                       __uint_as_float(hi & 0xffff0000u));
-  }
-};
-template <> struct RowPiece<f16> {
-  static constexpr int kGroups = 2;
-  static __device__ __forceinline__ float4 group(const uint4& r, int g) {
-    const unsigned lo = g ? r.z : r.x, hi = g ? r.w : r.y;
-    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&lo));
-    const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&hi));
-    return make_float4(a.x, a.y, b.x, b.y);
-  }
-};
-
-// Input of a single-CTA transform of 2048 rows, 512 threads: the tile's 16 columns of a row are 4 / G
-// 16-byte pieces, exactly kPieces per thread, fetched in one round with all loads in flight: fetch() issues
-// them (first thing in the kernel, so their latency runs under the set-up), place() converts them into the
-// shared-memory tile, ring() stores the raw pieces into a dense copy of the input, if one is wanted.
-template <typename T>
-struct TileRows {
-  static constexpr int G = RowPiece<T>::kGroups;
-  static constexpr int kPieces = 16 / G;
-  static constexpr int kPerRow = 4 / G;              // pieces of a row that belong to the tile
-  uint4 v[kPieces];
-
-  static __device__ __forceinline__ int token(const OnchipParams& p, const TileCoord& tc, int i) {
-    const int j = i / kPerRow;
-    return p.decim ? j * p.N1 + tc.k1 : j;
-  }
-  __device__ __forceinline__ void fetch(const OnchipParams& p, const TileCoord& tc) {
-    const T* src = reinterpret_cast<const T*>(p.src) + tc.b * p.s_sb + tc.h * p.s_sh + tc.tile * 16;
-#pragma unroll
-    for (int u = 0; u < kPieces; ++u) {
-      const int i = threadIdx.x + u * blockDim.x;
-      const int t = token(p, tc, i), col = 4 * G * (i % kPerRow);
-      v[u] = make_uint4(0u, 0u, 0u, 0u);
-      if (i < p.Mloc * kPerRow && t < p.L && tc.tile * 16 + col < p.D)
-        v[u] = __ldcs(reinterpret_cast<const uint4*>(src + (int64_t)t * p.s_sl + col));
-    }
-  }
-  __device__ __forceinline__ void place(const OnchipParams& p, float4* sm) const {
-#pragma unroll
-    for (int u = 0; u < kPieces; ++u) {
-      const int i = threadIdx.x + u * blockDim.x;
-      if (i < p.Mloc * kPerRow) {
-#pragma unroll
-        for (int g = 0; g < G; ++g) sm[(size_t)(i / kPerRow) * 4 + (i % kPerRow) * G + g] = RowPiece<T>::group(v[u], g);
-      }
-    }
-  }
-  __device__ __forceinline__ void ring(const OnchipParams& p, const TileCoord& tc) const {
-    T* dst = reinterpret_cast<T*>(p.ring) + ((size_t)tc.b * p.n * p.H + tc.h) * p.D + tc.tile * 16;
-#pragma unroll
-    for (int u = 0; u < kPieces; ++u) {
-      const int i = threadIdx.x + u * blockDim.x;
-      const int col = 4 * G * (i % kPerRow);
-      if (i < p.Mloc * kPerRow && tc.tile * 16 + col < p.D)
-        __stcs(reinterpret_cast<uint4*>(dst + (size_t)token(p, tc, i) * p.H * p.D + col), v[u]);
-    }
-  }
-};
-
 template <typename T, int C, bool FIX>
 __global__ void __launch_bounds__(512, 1) onchip_kernel(const OnchipParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -432,9 +362,6 @@ __global__ void __launch_bounds__(512, 1) onchip_kernel(const OnchipParams p) {
   float2* tw = reinterpret_cast<float2*>(smem_raw + (size_t)Mloc * 64);    // [Mloc] exp(-j 2 pi i / Mloc)
   float2* tw128 = tw + Mloc;                                               // FIX: [16][8] W_128^{m q}, the second stage's factors
   const TileCoord tc = tile_coord(p);
-  const bool direct = C == 1 && p.direct && p.mode != 2;
-  TileRows<T> rows;
-  if (direct) rows.fetch(p, tc);
 
   if (FIX) {
     // W_2048^i = exp(-j(quadrant pi/2 + 2 pi 4 (i % 512) / 8192)) from the quarter-wave table: one load serves
@@ -458,11 +385,7 @@ __global__ void __launch_bounds__(512, 1) onchip_kernel(const OnchipParams p) {
     if (FIX) S = 8;
     else for (int s = 0; s + 1 < p.nstage; ++s) S /= p.radix[s];   // where the forward stages would have left off
   } else {
-    if (direct) {
-      rows.place(p, sm);
-      if (p.ring) rows.ring(p, tc);
-      __syncthreads();
-    } else if (C == 1) {
+    if (C == 1) {
       // four elements per thread and round, their loads issued together
       for (int i0 = threadIdx.x; i0 < Mloc * 4; i0 += 4 * blockDim.x) {
         float4 v[4];
@@ -537,67 +460,76 @@ struct StridedParams {
   int H, D, L, n, M, slab0, nslab;
 };
 
+// A thread takes PP column pairs of one n2: two up to N1 = 16, one at 32, whose 32 points fill the registers.
 template <typename T, int N1, bool INV>
 __global__ void __launch_bounds__(256) strided_kernel(const StridedParams p) {
-  const int npg = p.D / 4;
+  constexpr int PP = N1 <= 16 ? 2 : 1;
+  const int npg = p.D / (2 * PP);
   const size_t total = (size_t)p.nslab * p.M * npg;
   size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= total) return;
-  int pg = (int)(idx % npg);
+  const int pg = (int)(idx % npg);
   size_t r = idx / npg;
-  int n2 = (int)(r % p.M);
-  int slab_local = (int)(r / p.M);
-  int slab = p.slab0 + slab_local;
-  int b = slab / p.H, h = slab - b * p.H;
-  const int col = pg * 4;
+  const int n2 = (int)(r % p.M);
+  const int slab_local = (int)(r / p.M);
+  const int slab = p.slab0 + slab_local;
+  const int b = slab / p.H, h = slab - b * p.H;
+  const int col = pg * 2 * PP;
+  float2* ws = p.ws + ((size_t)slab_local * N1 * p.M + n2) * (p.D / 2) + col / 2;
+  const size_t wstep = (size_t)p.M * (p.D / 2);
 
-  float2 w1 = twiddle_fwd((unsigned)n2, (unsigned)p.n);
   float2 wq[N1];
   wq[0] = make_float2(1.f, 0.f);
 #pragma unroll
-  for (int q = 1; q < N1; ++q) wq[q] = (q == 1) ? w1 : cmul(wq[q / 2], wq[q - q / 2]);
+  for (int q = 1; q < N1; ++q) wq[q] = (q == 1) ? twiddle_fwd((unsigned)n2, (unsigned)p.n) : cmul(wq[q / 2], wq[q - q / 2]);
 
-  float2 xa[N1], xb[N1];
+  float2 x[PP][N1];
   if (!INV) {
-    const T* src = reinterpret_cast<const T*>(p.src) + b * p.s_sb + h * p.s_sh + col;
+    const T* src = reinterpret_cast<const T*>(p.src) + b * p.s_sb + (int64_t)n2 * p.s_sl + h * p.s_sh + col;
+    typename ColumnGroup<T, PP>::raw v[N1];
 #pragma unroll
     for (int n1 = 0; n1 < N1; ++n1) {
-      int t = n1 * p.M + n2;
-      float4 v = (t < p.L) ? io<T>::load4(src + (int64_t)t * p.s_sl) : make_float4(0.f, 0.f, 0.f, 0.f);
-      xa[n1] = make_float2(v.x, v.y);
-      xb[n1] = make_float2(v.z, v.w);
+      v[n1] = ColumnGroup<T, PP>::zero();
+      if (n1 * p.M + n2 < p.L) v[n1] = ColumnGroup<T, PP>::load(src + (int64_t)n1 * p.M * p.s_sl);
+    }
+#pragma unroll
+    for (int n1 = 0; n1 < N1; ++n1) {
+      float2 t[PP];
+      ColumnGroup<T, PP>::cvt(v[n1], t);
+#pragma unroll
+      for (int i = 0; i < PP; ++i) x[i][n1] = t[i];
     }
   } else {
 #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1) {
-      size_t row = ((size_t)slab_local * N1 + k1) * p.M + n2;
-      float4 v = *reinterpret_cast<const float4*>(p.ws + row * (p.D / 2) + col / 2);
-      xa[k1] = make_float2(v.x, v.y);
-      xb[k1] = make_float2(v.z, v.w);
-      if (k1 > 0) {
-        xa[k1] = cmulc(xa[k1], wq[k1]);
-        xb[k1] = cmulc(xb[k1], wq[k1]);
-      }
+      float2 t[PP];
+      ColumnGroup<float, PP>::cvt(ColumnGroup<float, PP>::load(reinterpret_cast<const float*>(ws + k1 * wstep)), t);
+#pragma unroll
+      for (int i = 0; i < PP; ++i) x[i][k1] = t[i];
     }
+#pragma unroll
+    for (int k1 = 1; k1 < N1; ++k1)
+#pragma unroll
+      for (int i = 0; i < PP; ++i) x[i][k1] = cmulc(x[i][k1], wq[k1]);
   }
-  Dft<N1, INV>::run(xa);
-  Dft<N1, INV>::run(xb);
+#pragma unroll
+  for (int i = 0; i < PP; ++i) RegDft<N1, INV>::run(x[i]);
   if (!INV) {
 #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1) {
-      if (k1 > 0) {
-        xa[k1] = cmul(xa[k1], wq[k1]);
-        xb[k1] = cmul(xb[k1], wq[k1]);
-      }
-      size_t row = ((size_t)slab_local * N1 + k1) * p.M + n2;
-      *reinterpret_cast<float4*>(p.ws + row * (p.D / 2) + col / 2) = make_float4(xa[k1].x, xa[k1].y, xb[k1].x, xb[k1].y);
+      float2 t[PP];
+#pragma unroll
+      for (int i = 0; i < PP; ++i) t[i] = k1 > 0 ? cmul(x[i][k1], wq[k1]) : x[i][k1];
+      ColumnGroup<float, PP>::store(reinterpret_cast<float*>(ws + k1 * wstep), t);
     }
   } else {
-    T* dst = reinterpret_cast<T*>(p.dst) + b * p.d_sb + h * p.d_sh + col;
+    T* dst = reinterpret_cast<T*>(p.dst) + b * p.d_sb + (int64_t)n2 * p.d_sl + h * p.d_sh + col;
 #pragma unroll
     for (int n1 = 0; n1 < N1; ++n1) {
-      int t = n1 * p.M + n2;
-      if (t < p.L) io<T>::store4(dst + (int64_t)t * p.d_sl, make_float4(xa[n1].x, xa[n1].y, xb[n1].x, xb[n1].y));
+      float2 t[PP];
+#pragma unroll
+      for (int i = 0; i < PP; ++i) t[i] = x[i][n1];
+      if (n1 * p.M + n2 < p.L) ColumnGroup<T, PP>::store(dst + (int64_t)n1 * p.M * p.d_sl, t);
     }
   }
 }
@@ -661,31 +593,26 @@ static int launch_onchip_cf(const OnchipParams& p, const TransformPlan& pl, int 
   return SPECTRE_OK;
 }
 
-template <typename T, int C>
-static int launch_onchip_c(const OnchipParams& p, const TransformPlan& pl, int nslab, cudaStream_t st) {
-  const bool fix = pl.Mloc == kFixMloc && pl.nstage == 3 && pl.radix[0] == 16 && pl.radix[1] == 16 && pl.radix[2] == 8;
-  return fix ? launch_onchip_cf<T, C, true>(p, pl, nslab, st) : launch_onchip_cf<T, C, false>(p, pl, nslab, st);
-}
-
 template <typename T>
 static int launch_onchip(const OnchipParams& p, const TransformPlan& pl, int nslab, cudaStream_t st) {
   switch (pl.C) {
-    case 1: return launch_onchip_c<T, 1>(p, pl, nslab, st);
-    case 2: return launch_onchip_c<T, 2>(p, pl, nslab, st);
-    case 4: return launch_onchip_c<T, 4>(p, pl, nslab, st);
+    case 1: return launch_onchip_cf<T, 1, false>(p, pl, nslab, st);
+    case 2: return launch_onchip_cf<T, 2, true>(p, pl, nslab, st);     // clusters hold 2048 rows per CTA: 16 x 16 x 8
+    case 4: return launch_onchip_cf<T, 4, true>(p, pl, nslab, st);
     default: return fail(SPECTRE_ERR_UNSUPPORTED, "cluster size not supported");
   }
 }
 
 template <typename T, bool INV>
 static int launch_strided(const StridedParams& p, int N1, cudaStream_t st) {
-  size_t total = (size_t)p.nslab * p.M * (p.D / 4);
+  size_t total = (size_t)p.nslab * p.M * (N1 <= 16 ? p.D / 4 : p.D / 2);
   unsigned blocks = (unsigned)((total + 255) / 256);
   switch (N1) {
     case 2: strided_kernel<T, 2, INV><<<blocks, 256, 0, st>>>(p); break;
     case 4: strided_kernel<T, 4, INV><<<blocks, 256, 0, st>>>(p); break;
     case 8: strided_kernel<T, 8, INV><<<blocks, 256, 0, st>>>(p); break;
     case 16: strided_kernel<T, 16, INV><<<blocks, 256, 0, st>>>(p); break;
+    case 32: strided_kernel<T, 32, INV><<<blocks, 256, 0, st>>>(p); break;
     default: return fail(SPECTRE_ERR_UNSUPPORTED, "outer factor not supported");
   }
   SPECTRE_LAUNCH_OK("strided_kernel");
@@ -716,10 +643,62 @@ static int preferred_group(const spectre_ctx* ctx, int n, int D, int nslab_total
   return g;
 }
 
+// ---- register-resident transforms (reg_fft.h) ----
+// One CTA's length as it is; 4096 ... 32768 as n = N1 1024 with a strided pass over a complex workspace on either side
+// (two 1024-point CTAs per SM overlap; a 2048-point one fills the SM alone and is a third slower per point).
+constexpr int kRegM = kRegWsM;
+static bool reg_multi(int n) { return is_pow2(n) && n >= 4 * kRegM && n <= 32 * kRegM; }
+// Rows are addressed by 32-bit offsets from a uniform base: at most 2048 rows of at most 2^18 elements pitch.
+static bool reg_strides_ok(const spectre_act* a) { return a->stride_l >= 0 && a->stride_l <= (1 << 18); }
+static RegParams reg_params(int n, int H, int D, int L) {
+  RegParams p = {};
+  p.n = n; p.K = n / 2 + 1; p.H = H; p.D = D; p.L = L; p.N1 = 1;
+  p.scale = 1.0f / (float)n;
+  return p;
+}
+static void reg_source(RegParams& p, const spectre_act* a) { p.src = a->ptr; p.s_sb = a->stride_b; p.s_sl = a->stride_l; p.s_sh = a->stride_h; }
+static void reg_dest(RegParams& p, const spectre_act* a) { p.dst = a->ptr; p.d_sb = a->stride_b; p.d_sl = a->stride_l; p.d_sh = a->stride_h; }
+static StridedParams strided_params(const spectre_act* a, bool out, int n, int M, float2* ws, int slab0, int cnt) {
+  StridedParams sp = {};
+  sp.ws = ws; sp.H = a->H; sp.D = a->D; sp.L = a->L; sp.n = n; sp.M = M; sp.slab0 = slab0; sp.nslab = cnt;
+  if (out) { sp.dst = a->ptr; sp.d_sb = a->stride_b; sp.d_sl = a->stride_l; sp.d_sh = a->stride_h; }
+  else { sp.src = a->ptr; sp.s_sb = a->stride_b; sp.s_sl = a->stride_l; sp.s_sh = a->stride_h; }
+  return sp;
+}
+
+// y = R^{-1}(diag(g) R(v)) through the workspace, in groups of slabs that stay in L2
+template <typename T>
+static int reg_mixer_multi(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, const spectre_act* y, int n,
+                           void* ws, size_t ws_bytes) {
+  const int nslab = v->B * v->H;
+  RegParams p = reg_params(n, v->H, v->D, v->L);
+  p.N1 = n / kRegM; p.ws = reinterpret_cast<float2*>(ws); p.g = reinterpret_cast<const float2*>(g);
+  int group = (int)(ws_bytes / slab_ws_bytes(n, v->D));
+  const int pref = preferred_group(ctx, n, v->D, nslab);
+  if (group > pref) group = pref;
+  for (int s0 = 0; s0 < nslab; s0 += group) {
+    const int cnt = nslab - s0 < group ? nslab - s0 : group;
+    int rc = launch_strided<T, false>(strided_params(v, false, n, kRegM, p.ws, s0, cnt), p.N1, st);
+    p.slab0 = s0;
+    if (rc == SPECTRE_OK) rc = reg_mix(ctx, st, p, kRegM, cnt, true, v->dtype);
+    if (rc == SPECTRE_OK) rc = launch_strided<T, true>(strided_params(y, true, n, kRegM, p.ws, s0, cnt), p.N1, st);
+    if (rc != SPECTRE_OK) return rc;
+  }
+  return SPECTRE_OK;
+}
+
 template <typename T>
 static int mixer_typed(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g,
-                       const spectre_act* y, const TransformPlan& pl, void* ws, size_t ws_bytes) {
+                       const spectre_act* y, const TransformPlan& pl, bool multi, void* ws, size_t ws_bytes) {
   const int nslab = v->B * v->H;
+  if (multi) return reg_mixer_multi<T>(ctx, st, v, g, y, pl.n, ws, ws_bytes);
+  if (reg_supported(pl.n) && reg_strides_ok(v) && reg_strides_ok(y)) {
+    RegParams r = reg_params(pl.n, v->H, v->D, v->L);
+    reg_source(r, v);
+    reg_dest(r, y);
+    r.g = reinterpret_cast<const float2*>(g);
+    return reg_mix(ctx, st, r, pl.n, nslab, false, v->dtype);
+  }
   OnchipParams p = {};
   fill_common(ctx, p, pl, v->H, v->D, v->L);
   p.src = v->ptr; p.dst = y->ptr;
@@ -759,31 +738,29 @@ static int mixer_typed(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
 // Forward transforms of the decimated sequences (used by the cache prefill and the gate gradient): with n = N1 M and token
 // t = N1 n2 + n1, ws[slab_local][n1][k2][D/2] = sum_n2 z[N1 n2 + n1] W_M^{n2 k2}, read straight from the
 // activations.  The radix-N1 step over n1 (bin k2 + M k1 = sum_n1 W_N1^{n1 k1} W_n^{n1 k2} ws[n1][k2]) is
-// left to the caller, which can fuse it with what follows.  N1 = 1: the spectrum itself.  With `ring`
+// left to the caller, which can fuse it with what follows (N1 <= N1_max, at least 16).  N1 = 1: the spectrum itself.  With `ring`
 // (dense [B][n][H][D], the activations' dtype) the pass also writes the zero-padded input there when its
 // load path can; *ring_done tells the caller whether it did.
 int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, int n, int slab0, int cnt,
-                      float2* ws, int* N1_out, int* M_out, void* ring, int* ring_done) {
+                      float2* ws, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done) {
+  if ((reg_supported(n) || reg_multi(n)) && reg_strides_ok(v)) {
+    RegParams r = reg_params(n, v->H, v->D, v->L);
+    reg_source(r, v);
+    const int M = n <= 2048 ? n : (n / 1024 <= N1_max ? 1024 : 2048);
+    r.N1 = n / M; r.decim = r.N1 > 1; r.ws = ws; r.slab0 = slab0; r.ring = ring;
+    *N1_out = r.N1; *M_out = M; *ring_done = ring != nullptr;
+    return reg_forward(ctx, st, r, M, cnt, v->dtype);
+  }
   TransformPlan pl;
   if (!make_plan(ctx, n, &pl)) return fail(SPECTRE_ERR_UNSUPPORTED, "transform length not supported");
-  // Up to 16 sequences of kLocalMax tokens: single-CTA transforms, no exchange between CTAs.
-  const bool direct = n > kLocalMax && n <= 16 * kLocalMax && v->D % 8 == 0;
-  if (direct) {
-    TransformPlan one;
-    if (!make_plan(ctx, kLocalMax, &one)) return fail(SPECTRE_ERR_UNSUPPORTED, "transform length not supported");
-    pl = one;
-    pl.n = n;
-    pl.N1 = n / kLocalMax;
-  }
   *N1_out = pl.N1; *M_out = pl.M;
   OnchipParams p = {};
   fill_common(ctx, p, pl, v->H, v->D, v->L);
   p.src = v->ptr;
   p.s_sb = v->stride_b; p.s_sl = v->stride_l; p.s_sh = v->stride_h;
   p.ws = ws; p.mode = 1; p.dst_ws = 1; p.slab0 = slab0;
-  p.src_ws = 0; p.decim = pl.N1 > 1; p.direct = direct;
-  p.ring = direct ? ring : nullptr;
-  *ring_done = direct && ring != nullptr;
+  p.src_ws = 0; p.decim = pl.N1 > 1;
+  *ring_done = 0;
   SPECTRE_IO_DISPATCH(v->dtype, return launch_onchip<T>(p, pl, cnt, st));
 }
 
@@ -793,6 +770,27 @@ template <typename T>
 static int inverse_typed(const spectre_ctx* ctx, cudaStream_t st, const float2* spec, const float* g, const spectre_act* y,
                          const TransformPlan& pl, void* ws, size_t ws_bytes) {
   const int nslab = y->B * y->H;
+  if (reg_supported(pl.n) && reg_strides_ok(y)) {
+    RegParams r = reg_params(pl.n, y->H, y->D, y->L);
+    reg_dest(r, y);
+    r.g = reinterpret_cast<const float2*>(g); r.spec = spec;
+    return reg_inverse(ctx, st, r, pl.n, nslab, false, y->dtype);
+  }
+  if (reg_multi(pl.n) && ws_bytes >= slab_ws_bytes(pl.n, y->D) && ws && !(reinterpret_cast<uintptr_t>(ws) & 15)) {
+    RegParams r = reg_params(pl.n, y->H, y->D, y->L);
+    r.N1 = pl.n / kRegM; r.ws = reinterpret_cast<float2*>(ws); r.g = reinterpret_cast<const float2*>(g); r.spec = spec;
+    int group = (int)(ws_bytes / slab_ws_bytes(pl.n, y->D));
+    const int pref = preferred_group(ctx, pl.n, y->D, nslab);
+    if (group > pref) group = pref;
+    for (int s0 = 0; s0 < nslab; s0 += group) {
+      const int cnt = nslab - s0 < group ? nslab - s0 : group;
+      r.slab0 = s0;
+      int rc = reg_inverse(ctx, st, r, kRegM, cnt, true, y->dtype);
+      if (rc == SPECTRE_OK) rc = launch_strided<T, true>(strided_params(y, true, pl.n, kRegM, r.ws, s0, cnt), r.N1, st);
+      if (rc != SPECTRE_OK) return rc;
+    }
+    return SPECTRE_OK;
+  }
   OnchipParams p = {};
   fill_common(ctx, p, pl, y->H, y->D, y->L);
   p.dst = y->ptr;
@@ -830,7 +828,7 @@ static int inverse_typed(const spectre_ctx* ctx, cudaStream_t st, const float2* 
 size_t inverse_workspace_bytes(const spectre_ctx* ctx, int n, int D, int nslab) {
   TransformPlan pl;
   if (!make_plan(ctx, n, &pl)) return 0;
-  size_t a = pl.N1 == 1 ? 0 : (size_t)preferred_group(ctx, n, D, nslab) * slab_ws_bytes(n, D);
+  size_t a = pl.N1 == 1 && !reg_multi(n) ? 0 : (size_t)preferred_group(ctx, n, D, nslab) * slab_ws_bytes(n, D);
   if (ctx->dft64 && tc4k_supported(n, D) && D <= 64 && forced_path() != kPathAlu) {
     const size_t b = tc4k_readout_workspace_bytes(n, D, nslab);
     if (b > a) a = b;
@@ -867,7 +865,6 @@ using namespace spectre;
 
 extern "C" size_t spectre_mixer_workspace_bytes(const spectre_ctx* ctx, int32_t B, int32_t L, int32_t H, int32_t D,
                                                 int32_t n_fft, int32_t dtype) {
-  (void)L;
   TransformPlan pl;
   if (!ctx || B < 1 || H < 1 || D < 8 || !make_plan(ctx, n_fft, &pl)) return 0;
   const int force = forced_path();
@@ -876,7 +873,9 @@ extern "C" size_t spectre_mixer_workspace_bytes(const spectre_ctx* ctx, int32_t 
     return tc4k_workspace_bytes(ctx, n_fft, D, B * H);
   if ((dtype == SPECTRE_BF16 || dtype == SPECTRE_F16) && n_fft == 196 && D == 64 && ctx->dft49 && force != kPathAlu)
     return tc196_level_gate_bytes(B, H);                     // level gates of a fused refinement
-  if (pl.N1 == 1) return 0;
+  // the single-kernel path of n = 8192 takes whole 64-row blocks and needs no workspace
+  if ((dtype == SPECTRE_BF16 || dtype == SPECTRE_F16) && ctx->dft64 && n_fft == 8192 && L % 64 == 0 && force != kPathAlu) return 0;
+  if (pl.N1 == 1 && !reg_multi(n_fft)) return 0;
   return (size_t)preferred_group(ctx, n_fft, D, B * H) * slab_ws_bytes(n_fft, D);
 }
 
@@ -899,14 +898,17 @@ extern "C" int spectre_mixer_forward(spectre_ctx* ctx, void* stream, const spect
   const bool ws_ok = workspace && !(reinterpret_cast<uintptr_t>(workspace) & 15);
   const bool tc196 = tc_ok && n_fft == 196 && v->D == 64 && ctx->dft49 != nullptr;
   const bool fused = tc_ok && n_fft == 8192 && force != kPathStaged && tc8192_supported(v, y);
-  const bool staged = !fused && tc_ok && force != kPathFused && tc4k_supported(n_fft, v->D) && ws_ok &&
+  // n = 8192 that the fused kernel cannot take (no whole 64-row blocks) stays on the fp32 kernels unless forced
+  const bool staged = !fused && tc_ok && force != kPathFused && (n_fft != 8192 || force == kPathStaged) &&
+                      tc4k_supported(n_fft, v->D) && ws_ok &&
                       workspace_bytes >= tc4k_min_workspace(n_fft, v->D);
   if (!staged && !fused && pl.N1 > 1) {
     if (!ws_ok) return fail(SPECTRE_ERR_WORKSPACE, "workspace is NULL or not 16-byte aligned");
     if (workspace_bytes < slab_ws_bytes(n_fft, v->D))
       return fail(SPECTRE_ERR_WORKSPACE, "mixer workspace smaller than one (batch, head) slab");
   }
-  if (staged || pl.N1 > 1) {
+  bool overlap = false;
+  {
     // any overlap of the two views' byte extents counts, not only equal base pointers
     auto extent = [](const spectre_act* a, const char** lo, const char** hi) {
       const int64_t es = io_elem_bytes(a->dtype);
@@ -917,7 +919,8 @@ extern "C" int spectre_mixer_forward(spectre_ctx* ctx, void* stream, const spect
     const char *vl, *vh, *yl, *yh;
     extent(v, &vl, &vh);
     extent(y, &yl, &yh);
-    if (vl < yh && yl < vh) return fail(SPECTRE_ERR_INVALID_ARG, "y may not overlap v on the multi-pass path");
+    overlap = vl < yh && yl < vh;
+    if (overlap && (staged || pl.N1 > 1)) return fail(SPECTRE_ERR_INVALID_ARG, "y may not overlap v on the multi-pass path");
   }
   if (wrm) {
     if (wrm->levels < 1 || wrm->levels > 10 || (v->L % (1 << wrm->levels)) != 0)
@@ -940,7 +943,9 @@ extern "C" int spectre_mixer_forward(spectre_ctx* ctx, void* stream, const spect
     if (wrm && !fuse_wrm) return spectre_wavelet_refine(ctx, stream, y, y, wrm);
     return SPECTRE_OK;
   }
-  SPECTRE_IO_DISPATCH(v->dtype, rc = mixer_typed<T>(ctx, st, v, g, y, pl, workspace, workspace_bytes));
+  // n = 4096 and 8192 in place or without a workspace: one kernel, a cluster of CTAs per tile
+  const bool multi = reg_multi(n_fft) && !overlap && ws_ok && workspace_bytes >= slab_ws_bytes(n_fft, v->D);
+  SPECTRE_IO_DISPATCH(v->dtype, rc = mixer_typed<T>(ctx, st, v, g, y, pl, multi, workspace, workspace_bytes));
   if (rc != SPECTRE_OK) return rc;
   if (wrm) return spectre_wavelet_refine(ctx, stream, y, y, wrm);
   return SPECTRE_OK;

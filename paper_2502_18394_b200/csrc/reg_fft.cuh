@@ -1,0 +1,511 @@
+// Transforms of up to 2048 points per CTA with the points in registers (fp32): decompositions, parameters and
+// the kernel.  Instantiated per activation type in reg_*.cu, launched through the functions of reg_fft.h.
+//
+// A thread holds 32 points of one column pair (see mixer.cu for the pair packing).  A 1024-point transform is a 32-point
+// DFT in registers, one exchange through shared memory and a second 32-point DFT; the spectrum is then still in
+// registers, where the gate is applied, and the inverse runs the same steps backwards, so that a point crosses shared
+// memory twice in all and global rows move straight from and to registers.  Bound by instruction issue (about 2700 per
+// thread and tile, half of them floating point); two CTAs per SM overlap one another's loads and barriers.
+// Measured, mixer call at B = 16, H = 12, D = 64, bf16, n = 1024: 86 us on the shared-memory kernel (eleven passes over the
+// tile, run-time radices) -> 30 us = 1.7 TB/s of its rows; its backward 287 us (four transforms and a reduction) -> 57 us;
+// n = 2048 86 -> 43 us at the same size.
+#pragma once
+#include "fft_reg.cuh"
+#include "reg_fft.h"
+
+namespace spectre {
+
+// Twiddle loads.  Volatile, so that the forward transform's factors are not kept in registers (and spilled) for the
+// inverse's use of the same ones.
+__device__ __forceinline__ float4 tw_load4(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float2 tw_load2(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+
+// Keeps the work in front of this point in front of it: without it the compiler interleaves the end of the forward
+// transform with the start of the inverse one and runs out of registers.
+template <int E> __device__ __forceinline__ void settle(float2 (&x)[E]) {
+#pragma unroll
+  for (int i = 0; i < E; ++i) asm volatile("" : "+f"(x[i].x), "+f"(x[i].y));
+}
+
+enum RegMode { kRegMix = 0, kRegForward = 1, kRegInverse = 2, kRegGrad = 3 };
+
+// n = R1 R2 in two steps (R1 a multiple of R2): j = j1 R2 + j2, k = k1 + R1 k2.  Thread (pair p, m): the R1-point DFT
+// over j1 at j2 = m, then R1 / R2 DFTs of R2 points at k1 = m + R2 u.  Rows of the exchange buffer (k1, j2) lie
+// R2 + 1 apart per k1: an odd pitch keeps the side whose lanes differ in k1 free of bank conflicts.
+template <int R1, int R2, int C_>
+struct TwoStep {
+  static constexpr int C = C_, M = R1 * R2, E = R1, S = R2, U = R1 / R2;
+  static constexpr int kActive = S * C, kThreads = (kActive + 31) / 32 * 32;
+  static constexpr int kExch = R1 * (R2 + 1) * C;                   // elements of the exchange buffer
+  static constexpr int kGate = M;
+  static constexpr int kParts = 1, kRed = C, kRedShift = 0;         // pairs side by side in a warp after the transform
+  int p, m;
+  __device__ __forceinline__ explicit TwoStep(int tid) : p(tid % C), m(tid / C) {}
+  __device__ __forceinline__ int pair_in() const { return p; }
+  __device__ __forceinline__ int pair_out() const { return p; }
+  __device__ __forceinline__ int part() const { return 0; }
+  __device__ __forceinline__ int bin(int i) const { return m + S * (i / R2) + R1 * (i % R2); }
+  static __device__ __forceinline__ int gate_slot(int k) { return k; }
+
+  template <bool HALF>
+  __device__ __forceinline__ void forward(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act) const {
+    RegDft<R1, false>::run(x);
+#pragma unroll
+    for (int a = 0; a < R1 / 2; ++a) {
+      const float4 w = tw_load4(tw + a * R1 + m);
+      if (a > 0) x[2 * a] = cmul(x[2 * a], make_float2(w.x, w.y));
+      x[2 * a + 1] = cmul(x[2 * a + 1], make_float2(w.z, w.w));
+    }
+    exchange<HALF, true>(x, buf, act);
+#pragma unroll
+    for (int u = 0; u < U; ++u) sub<false>(x, u);
+  }
+  template <bool HALF>
+  __device__ __forceinline__ void inverse(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act) const {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      sub<true>(x, u);
+#pragma unroll
+      for (int a = 0; a < R2 / 2; ++a) {
+        const float4 w = tw_load4(tw + a * R1 + m + S * u);
+        if (a > 0) x[u * R2 + 2 * a] = cmulc(x[u * R2 + 2 * a], make_float2(w.x, w.y));
+        x[u * R2 + 2 * a + 1] = cmulc(x[u * R2 + 2 * a + 1], make_float2(w.z, w.w));
+      }
+    }
+    exchange<HALF, false>(x, buf, act);
+    RegDft<R1, true>::run(x);
+  }
+
+ private:
+  template <bool INV>
+  __device__ __forceinline__ void sub(float2 (&x)[E], int u) const {
+    float2 y[R2];
+#pragma unroll
+    for (int i = 0; i < R2; ++i) y[i] = x[u * R2 + i];
+    RegDft<R2, INV>::run(y);
+#pragma unroll
+    for (int i = 0; i < R2; ++i) x[u * R2 + i] = y[i];
+  }
+  // element i of the first step's side is (k1 = i, j2 = m), of the second step's (k1 = m + S u, j2 = i % R2)
+  __device__ __forceinline__ int at(bool first, int i) const {
+    return first ? (i * (R2 + 1) + m) * C + p : ((m + S * (i / R2)) * (R2 + 1) + i % R2) * C + p;
+  }
+  // FWD: first step's order -> second step's.  The inverse writes the positions this thread read last, so it needs no
+  // barrier in front.  HALF: real and imaginary parts one after the other through half the space.
+  template <bool HALF, bool FWD>
+  __device__ __forceinline__ void exchange(float2 (&x)[E], void* buf, bool act) const {
+    if constexpr (!HALF) {
+      float2* b = reinterpret_cast<float2*>(buf);
+      if (act) {
+#pragma unroll
+        for (int i = 0; i < E; ++i) b[at(FWD, i)] = x[i];
+      }
+      __syncthreads();
+
+#pragma unroll
+      for (int i = 0; i < E; ++i) x[i] = b[at(!FWD, i)];
+    } else {
+      float* b = reinterpret_cast<float*>(buf);
+      if (act) {
+#pragma unroll
+        for (int i = 0; i < E; ++i) b[at(FWD, i)] = x[i].x;
+      }
+      __syncthreads();
+
+#pragma unroll
+      for (int i = 0; i < E; ++i) x[i].x = b[at(!FWD, i)];
+      __syncthreads();
+
+      if (act) {
+#pragma unroll
+        for (int i = 0; i < E; ++i) b[at(FWD, i)] = x[i].y;
+      }
+      __syncthreads();
+
+#pragma unroll
+      for (int i = 0; i < E; ++i) x[i].y = b[at(!FWD, i)];
+    }
+  }
+};
+
+// n = 2048 = 32 x (8 x 8).  Step one as above with j2 = 8 ja + jb in 0..63.  The 64-point DFT over j2 is two steps of 8
+// points whose exchange stays inside a warp: after the first exchange lane l serves jb (later ka) = l % 8 and pair
+// l / 8 (+ 4 per further warp), the warp index the group of k1, so a __syncwarp is enough.
+//   k = k1 + 32 (ka + 8 kb),  k1 = kg + 8 u for u < 4
+// Row (k1, j2) of the exchange buffer sits at row + row / 8, its C slots permuted by bits of the row (an exclusive or
+// with f(jb) and f(ja)), so that all four access patterns are free of bank conflicts.
+template <int C_>
+struct ThreeStep2048 {
+  static constexpr int C = C_, M = 2048, E = 32, S = 64, PW = C / 4;
+  static constexpr int kActive = S * C, kThreads = kActive;
+  static constexpr int kExch = (2048 + 256) * C;
+  static constexpr int kGate = 2048 + 64;
+  static constexpr int kParts = PW, kRed = 4, kRedShift = 3;
+  int p, m, p2, kg, l8;
+  int o1, ojb, oka, q;                                    // offsets of the three access patterns, slot of row digit 0
+  static __device__ __forceinline__ int f(int digit) { return C == 8 ? digit : 2 * (digit >> 2); }
+  __device__ __forceinline__ explicit ThreeStep2048(int tid) : p(tid % C), m(tid / C) {
+    const int warp = tid >> 5, lane = tid & 31;
+    l8 = lane & 7;
+    p2 = (lane >> 3) + 4 * (warp % PW);
+    kg = warp / PW;
+    o1 = (m + (m >> 3)) * C + (p ^ f(m & 7) ^ f(m >> 3));
+    ojb = (72 * kg + l8) * C;
+    oka = (72 * kg + 9 * l8) * C;
+    q = p2 ^ f(l8);
+  }
+  __device__ __forceinline__ int pair_in() const { return p; }
+  __device__ __forceinline__ int pair_out() const { return p2; }
+  __device__ __forceinline__ int part() const { return p2 >> 2; }
+  __device__ __forceinline__ int bin(int i) const { return kg + 8 * (i >> 3) + 32 * l8 + 256 * (i & 7); }
+  static __device__ __forceinline__ int gate_slot(int k) { return k + (k >> 5); }
+
+  template <bool HALF>
+  __device__ __forceinline__ void forward(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool) const {
+    RegDft<32, false>::run(x);
+#pragma unroll
+    for (int a = 0; a < 16; ++a) {
+      const float4 w = tw_load4(tw + a * 64 + m);
+      if (a > 0) x[2 * a] = cmul(x[2 * a], make_float2(w.x, w.y));
+      x[2 * a + 1] = cmul(x[2 * a + 1], make_float2(w.z, w.w));
+    }
+    move<HALF, 0, 1>(x, buf);
+    const float2* w64 = reinterpret_cast<const float2*>(tw + 16 * 64);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sub<false>(x, u);
+#pragma unroll
+    for (int a = 1; a < 8; ++a) {
+      const float2 w = tw_load2(w64 + 8 * a + l8);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[8 * u + a] = cmul(x[8 * u + a], w);
+    }
+    move<HALF, 1, 2>(x, buf);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sub<false>(x, u);
+  }
+  template <bool HALF>
+  __device__ __forceinline__ void inverse(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool) const {
+    const float2* w64 = reinterpret_cast<const float2*>(tw + 16 * 64);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sub<true>(x, u);
+    move<HALF, 2, 1>(x, buf);
+#pragma unroll
+    for (int a = 1; a < 8; ++a) {
+      const float2 w = tw_load2(w64 + 8 * a + l8);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[8 * u + a] = cmulc(x[8 * u + a], w);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sub<true>(x, u);
+    move<HALF, 1, 0>(x, buf);
+#pragma unroll
+    for (int a = 0; a < 16; ++a) {
+      const float4 w = tw_load4(tw + a * 64 + m);
+      if (a > 0) x[2 * a] = cmulc(x[2 * a], make_float2(w.x, w.y));
+      x[2 * a + 1] = cmulc(x[2 * a + 1], make_float2(w.z, w.w));
+    }
+    RegDft<32, true>::run(x);
+  }
+
+ private:
+  template <bool INV>
+  __device__ __forceinline__ void sub(float2 (&x)[E], int u) const {
+    float2 y[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) y[i] = x[u * 8 + i];
+    RegDft<8, INV>::run(y);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[u * 8 + i] = y[i];
+  }
+  // position of element i: 0 = (k1 = i, j2 = m); 1 = (k1 = kg + 8 u, ja or ka = i % 8, jb = l8); 2 = (k1, ka = l8, jb = i % 8)
+  template <int KIND>
+  __device__ __forceinline__ int at(int i) const {
+    if (KIND == 0) return o1 + i * 72 * C;
+    const int u = i >> 3, a = i & 7;
+    return (KIND == 1 ? ojb + (u * 576 + a * 9) * C : oka + (u * 576 + a) * C) + (q ^ f(a));
+  }
+  // between kinds 0 and 1 across the CTA, between 1 and 2 inside the warp, over positions that only it uses meanwhile
+  template <bool HALF, int FROM, int TO>
+  __device__ __forceinline__ void move(float2 (&x)[E], void* buf) const {
+    auto sync = [] { if (FROM == 0 || TO == 0) __syncthreads(); else __syncwarp(); };
+    if constexpr (!HALF) {
+      float2* b = reinterpret_cast<float2*>(buf);
+#pragma unroll
+      for (int i = 0; i < E; ++i) b[at<FROM>(i)] = x[i];
+      sync();
+#pragma unroll
+      for (int i = 0; i < E; ++i) x[i] = b[at<TO>(i)];
+    } else {
+      float* b = reinterpret_cast<float*>(buf);
+#pragma unroll
+      for (int i = 0; i < E; ++i) b[at<FROM>(i)] = x[i].x;
+      sync();
+#pragma unroll
+      for (int i = 0; i < E; ++i) x[i].x = b[at<TO>(i)];
+      sync();
+#pragma unroll
+      for (int i = 0; i < E; ++i) b[at<FROM>(i)] = x[i].y;
+      sync();
+#pragma unroll
+      for (int i = 0; i < E; ++i) x[i].y = b[at<TO>(i)];
+    }
+  }
+};
+
+// how many of the rows m, m + step, ... lie below `rows` (0 for an idle thread)
+__device__ __forceinline__ int rows_below(int rows, int m, int step, bool live) { return live && rows > m ? (rows - m + step - 1) / step : 0; }
+
+// Rows m, m + S, ... of the CTA's sequence at this thread's column pair, all loads in flight before the first
+// conversion.  Tokens beyond L are the zero padding; `ring`: they also go, as loaded, into the cache's buffer.
+// The base of every row is uniform over the CTA and the thread's part one 32-bit offset, so that a load takes no
+// address arithmetic of its own; whole tiles take no predicates either.
+template <typename T, class P, int MODE>
+__device__ __forceinline__ void reg_load_tokens(float2 (&x)[P::E], const void* src, int64_t sb, int64_t sl, int64_t sh,
+                                                const RegParams& p, int b, int h, int k1, int col, int m, bool live) {
+  typedef typename PairIo<T>::raw raw;
+  const int step = MODE == kRegForward && p.decim ? p.N1 : 1, off = MODE == kRegForward && p.decim ? k1 : 0;
+  const char* base = reinterpret_cast<const char*>(reinterpret_cast<const T*>(src) + b * sb + (int64_t)off * sl + h * sh);
+  const int64_t ds = (int64_t)(P::S * step) * sl * (int64_t)sizeof(T);
+  const uint32_t mine = (uint32_t)((int64_t)m * step * sl + col) * (uint32_t)sizeof(T);
+  const int count = rows_below(p.L, m * step + off, P::S * step, live);
+  raw v[P::E];
+  if (count >= P::E) {
+#pragma unroll
+    for (int i = 0; i < P::E; ++i) v[i] = *reinterpret_cast<const raw*>(base + i * ds + mine);
+  } else {
+#pragma unroll
+    for (int i = 0; i < P::E; ++i) {
+      v[i] = PairIo<T>::zero();
+      if (i < count) v[i] = *reinterpret_cast<const raw*>(base + i * ds + mine);
+    }
+  }
+  if (MODE == kRegForward && p.ring && live) {
+    T* out = reinterpret_cast<T*>(p.ring) + (((size_t)b * p.n + (m * step + off)) * p.H + h) * p.D + col;
+    const size_t dr = (size_t)(P::S * step) * p.H * p.D;
+#pragma unroll
+    for (int i = 0; i < P::E; ++i) __stcs(reinterpret_cast<raw*>(out + i * dr), v[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < P::E; ++i) x[i] = PairIo<T>::cvt(v[i]);
+}
+
+template <class P>
+__device__ __forceinline__ void reg_load_ws(float2 (&x)[P::E], const float2* ws, int half, int m, int pair) {
+  // an idle thread reads row m of pair 0 like the others and stores nothing
+  const char* base = reinterpret_cast<const char*>(ws);
+  const uint32_t mine = (uint32_t)(m * half + pair) * 8u;
+#pragma unroll
+  for (int i = 0; i < P::E; ++i) x[i] = *reinterpret_cast<const float2*>(base + (size_t)(P::S * i) * half * 8 + mine);
+}
+
+// Sum over the RL pairs that sit side by side in the warp (lane bits SHIFT ...) of RL values each; the lane whose pair
+// is s keeps the sum of value s.
+template <int RL, int SHIFT>
+__device__ __forceinline__ float2 reduce_scatter(float2 (&q)[RL], int s) {
+#pragma unroll
+  for (int h = RL / 2; h >= 1; h >>= 1) {
+    const bool up = s & h;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float2 send = up ? q[i] : q[i + h], keep = up ? q[i + h] : q[i];
+      const float rx = __shfl_xor_sync(0xffffffffu, send.x, h << SHIFT), ry = __shfl_xor_sync(0xffffffffu, send.y, h << SHIFT);
+      q[i] = make_float2(keep.x + rx, keep.y + ry);
+    }
+  }
+  return q[0];
+}
+
+// 128 registers a thread for 20 and more points; fewer points leave room for more CTAs
+template <class P> constexpr int reg_min_blocks() {
+  constexpr int r = P::E > 16 ? 512 : 768, b = r / P::kThreads;
+  return b < 1 ? 1 : (b > 16 ? 16 : b);
+}
+template <class P, int MODE> __host__ __device__ constexpr size_t reg_exch_bytes() { return ((size_t)P::kExch * (MODE == kRegGrad ? 4 : 8) + 15) / 16 * 16; }
+template <class P, int MODE> constexpr size_t reg_smem_bytes() {
+  return reg_exch_bytes<P, MODE>() + (MODE == kRegGrad ? (size_t)P::E * P::kThreads * 8 : 0) + (MODE == kRegMix ? (size_t)P::kGate * 8 : 0);
+}
+
+// MODE kRegMix      rows -> forward, gate, inverse -> rows
+//      kRegForward  rows -> spectrum rows in ws
+//      kRegInverse  gated half spectra -> inverse -> rows
+//      kRegGrad     two tensors' rows: the sum over the pairs of conj(Vhat) Ghat for every bin (sums), and the inverse
+//                   transform of conj(gate) Ghat (dst).  Vhat waits in shared memory, one slot per thread and
+//                   element; exchanging real and imaginary parts in turn keeps two CTAs on an SM (one at M = 2048).
+// WS: rows of the complex workspace instead of tokens.
+template <typename T, class P, int MODE, bool WS>
+__global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(const __grid_constant__ RegParams p) {
+  extern __shared__ __align__(16) unsigned char reg_smem[];
+  constexpr int E = P::E;
+  constexpr bool HALF = MODE == kRegGrad;
+  void* buf = reg_smem;
+  float2* extra = reinterpret_cast<float2*>(reg_smem + reg_exch_bytes<P, MODE>());     // gate table, or the parked spectrum
+  const bool act = threadIdx.x < P::kActive;
+  const P pl(act ? (int)threadIdx.x : 0);
+  int u = blockIdx.x;
+  const int tile = u % p.ntile; u /= p.ntile;
+  const int k1 = u % p.N1; u /= p.N1;
+  const int slab_local = u, slab = p.slab0 + u;
+  const int b = slab / p.H, h = slab - b * p.H;
+  const int half = p.D / 2;
+  const int pin = tile * P::C + pl.pair_in(), pout = tile * P::C + pl.pair_out();
+  const bool live = act && pin < half, live_out = act && pout < half;
+  const size_t wrow = ((size_t)slab_local * p.N1 + k1) * P::M;                    // first workspace row of the sequence
+  const float2* g = p.g + (size_t)slab * p.K;
+  // a programmatic dependent of the kernel before it: the set-up overlaps that kernel's end, nothing is read earlier
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  float2 x[E];
+  if constexpr (MODE != kRegInverse) {
+    if constexpr (WS) reg_load_ws<P>(x, p.ws + wrow * half, half, pl.m, live ? pin : 0);
+    else reg_load_tokens<T, P, MODE>(x, p.src, p.s_sb, p.s_sl, p.s_sh, p, b, h, k1, 2 * pin, pl.m, live);
+  }
+  if constexpr (MODE == kRegMix) {
+    for (int i = threadIdx.x; i < P::M; i += P::kThreads) {
+      const int k = k1 + p.N1 * i, kk = 2 * k <= p.n ? k : p.n - k;
+      float2 v = cscale(__ldg(g + kk), p.scale);
+      if (kk != k) v.y = -v.y;
+      if (k == 0 || 2 * k == p.n) v.y = 0.f;
+      extra[P::gate_slot(i)] = v;
+    }
+  }
+  if constexpr (MODE != kRegInverse) pl.template forward<HALF>(x, buf, p.tw, act);
+
+  settle(x);
+  if constexpr (MODE == kRegMix) {                         // the gate table is complete: the exchange had a barrier
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+      x[i] = cmul(x[i], extra[P::gate_slot(pl.bin(i))]);
+      if (i % 4 == 3) asm volatile("" ::: "memory");        // four gates at a time: there are no registers for more
+    }
+  }
+  if constexpr (MODE == kRegForward) {
+    float2* out = p.ws + wrow * half + pout;
+    if (live_out) {
+#pragma unroll
+      for (int i = 0; i < E; ++i) out[(size_t)pl.bin(i) * half] = x[i];
+    }
+    return;
+  }
+  if constexpr (MODE == kRegInverse) {
+    const float2* spec = p.spec + (size_t)slab * p.K * p.D + 2 * pout;
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+      const int k = k1 + p.N1 * pl.bin(i), kk = 2 * k <= p.n ? k : p.n - k;
+      x[i] = make_float2(0.f, 0.f);
+      if (live_out) {
+        const float4 ab = *reinterpret_cast<const float4*>(spec + (size_t)kk * p.D);
+        x[i] = pair_from_half(cscale(__ldg(g + kk), p.scale), ab, k, kk, p.n);
+      }
+    }
+  }
+  if constexpr (MODE == kRegGrad) {
+#pragma unroll
+    for (int i = 0; i < E; ++i) extra[i * P::kThreads + threadIdx.x] = x[i];
+    reg_load_tokens<T, P, MODE>(x, p.src2, p.s2_sb, p.s2_sl, p.s2_sh, p, b, h, k1, 2 * pin, pl.m, live);
+    __syncthreads();
+    pl.template forward<HALF>(x, buf, p.tw, act);
+    if (p.sums) {
+      constexpr int RL = P::kRed;
+      const int s = (threadIdx.x >> P::kRedShift) % RL;
+      float2* out = p.sums + (((size_t)slab_local * p.ntile + tile) * P::kParts + pl.part()) * p.n;
+#pragma unroll
+      for (int i0 = 0; i0 < E; i0 += RL) {
+        float2 q[RL];
+#pragma unroll
+        for (int i = 0; i < RL; ++i)
+          q[i] = i0 + i < E && act ? cmulc(x[(i0 + i) % E], extra[((i0 + i) % E) * P::kThreads + threadIdx.x]) : make_float2(0.f, 0.f);
+        const float2 r = reduce_scatter<RL, P::kRedShift>(q, s);
+        if (act && i0 + s < E) out[pl.bin(i0 + s)] = r;
+      }
+    }
+    if (!p.dst) return;
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+      const int k = pl.bin(i), kk = 2 * k <= p.n ? k : p.n - k;
+      float2 v = cscale(__ldg(g + kk), p.scale);
+      if (kk == k) v.y = -v.y;
+      if (k == 0 || 2 * k == p.n) v.y = 0.f;
+      x[i] = cmul(x[i], v);
+    }
+  }
+
+  settle(x);
+  pl.template inverse<HALF>(x, buf, p.tw, act);
+  if (!live) return;
+  if constexpr (WS) {
+    char* base = reinterpret_cast<char*>(p.ws + wrow * half);
+    const uint32_t mine = (uint32_t)(pl.m * half + pin) * 8u;
+#pragma unroll
+    for (int i = 0; i < E; ++i) *reinterpret_cast<float2*>(base + (size_t)(P::S * i) * half * 8 + mine) = x[i];
+  } else {
+    typedef typename PairIo<T>::raw raw;
+    char* base = reinterpret_cast<char*>(reinterpret_cast<T*>(p.dst) + b * p.d_sb + h * p.d_sh);
+    const int64_t ds = (int64_t)P::S * p.d_sl * (int64_t)sizeof(T);
+    const uint32_t mine = (uint32_t)((int64_t)pl.m * p.d_sl + 2 * pin) * (uint32_t)sizeof(T);
+    const int count = rows_below(p.L, pl.m, P::S, live);
+    if (count >= E) {
+#pragma unroll
+      for (int i = 0; i < E; ++i) *reinterpret_cast<raw*>(base + i * ds + mine) = PairIo<T>::pack(x[i]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < E; ++i)
+        if (i < count) *reinterpret_cast<raw*>(base + i * ds + mine) = PairIo<T>::pack(x[i]);
+    }
+  }
+}
+
+template <typename T, class P, int MODE, bool WS>
+static int reg_launch(RegParams p, int nslab, cudaStream_t st) {
+  auto kern = reg_kernel<T, P, MODE, WS>;
+  constexpr size_t smem = reg_smem_bytes<P, MODE>();
+  if (smem > 48 * 1024) SPECTRE_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  p.ntile = (p.D / 2 + P::C - 1) / P::C;
+  cfg.gridDim = dim3((unsigned)((size_t)nslab * p.N1 * p.ntile));
+  cfg.blockDim = dim3(P::kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, p));
+  return SPECTRE_OK;
+}
+
+// Pairs per CTA: 32-byte pieces of a 16-bit row (a whole sector), 64 bytes of an fp32 or workspace row.  With 4 pairs the
+// same tiles are 20 % slower (batch of 16 x 12 heads, n = 1024: fp32 45 us against 38, workspace rows 35 against 32): a
+// request covers more rows, and each row costs the load/store unit a cycle.
+constexpr int kRegPairs = 8;
+
+template <typename T, int MODE>
+static int reg_launch_tokens(const spectre_ctx* ctx, const RegParams& q, int M, int nslab, cudaStream_t st) {
+  constexpr int C = kRegPairs;
+  RegParams p = q;
+  p.tw = reg_table(ctx, M);
+#define SPECTRE_REG_CASE(R1, R2) case R1 * R2: return reg_launch<T, TwoStep<R1, R2, C>, MODE, false>(p, nslab, st);
+  switch (M) {
+    SPECTRE_REG_TWO_STEP(SPECTRE_REG_CASE)
+    case 2048: return reg_launch<T, ThreeStep2048<C>, MODE, false>(p, nslab, st);
+    default: return fail(SPECTRE_ERR_UNSUPPORTED, "transform length not supported");
+  }
+#undef SPECTRE_REG_CASE
+}
+template <int MODE>
+static int reg_launch_ws(const spectre_ctx* ctx, const RegParams& q, int M, int nslab, cudaStream_t st) {
+  if (M != kRegWsM) return fail(SPECTRE_ERR_UNSUPPORTED, "transform length not supported");
+  RegParams p = q;
+  p.tw = reg_table(ctx, M);
+  return reg_launch<float, TwoStep<32, 32, kRegPairs>, MODE, true>(p, nslab, st);
+}
+
+}  // namespace spectre

@@ -1,0 +1,46 @@
+// Host interface of the register-resident fp32 transforms (reg_fft.cuh).
+#pragma once
+#include "common.cuh"
+
+namespace spectre {
+
+struct RegParams {
+  const void* src;          // tokens [B, L, H, D]
+  const void* src2;         // second tensor of the gradient
+  void* dst;                // tokens out
+  float2* ws;               // complex rows [slab_local][N1][M][D/2]: input and / or output
+  const float2* g;          // gate [B*H][K]
+  const float2* spec;       // half spectra [B*H][K][D] (inverse)
+  float2* sums;             // gradient: partial sums [slab_local][parts][n]; NULL: not wanted
+  void* ring;               // forward: dense [B][n][H][D] copy of the zero-padded input, or NULL
+  const float4* tw;         // twiddles of the plan
+  int64_t s_sb, s_sl, s_sh;
+  int64_t s2_sb, s2_sl, s2_sh;
+  int64_t d_sb, d_sl, d_sh;
+  int H, D, L, n, K;
+  int N1;                   // outer factor of n = N1 M; a CTA's sequence is k1 of N1
+  int decim;                // forward, from tokens: element j of sequence k1 is token N1 j + k1
+  int slab0, ntile;
+  float scale;              // 1/n, folded into the gate
+};
+
+// Lengths M that one CTA transforms: powers of two 64 ... 2048 and the squares of 14, 20, 24, 28 (patch grids).
+#define SPECTRE_REG_TWO_STEP(X) X(8, 8) X(16, 8) X(16, 16) X(32, 16) X(32, 32) X(14, 14) X(20, 20) X(24, 24) X(28, 28)
+bool reg_supported(int M);
+constexpr int kRegWsM = 1024;    // the length whose rows may also come from the complex workspace
+// partial sums per (batch, head) and bin that the gradient leaves, one per group of pairs summed inside a warp
+int reg_parts(int M, int D);
+
+// One launch over nslab slabs (p.tw and p.ntile are filled in); `ws`: rows of the complex workspace (M = kRegWsM)
+// instead of tokens of type dtype.
+int reg_mix(const spectre_ctx* ctx, cudaStream_t st, RegParams p, int M, int nslab, bool ws, int dtype);
+int reg_forward(const spectre_ctx* ctx, cudaStream_t st, RegParams p, int M, int nslab, int dtype);
+int reg_inverse(const spectre_ctx* ctx, cudaStream_t st, RegParams p, int M, int nslab, bool ws, int dtype);
+int reg_grad(const spectre_ctx* ctx, cudaStream_t st, RegParams p, int M, int nslab, int dtype);
+
+// Twiddle tables of all plans: built once per context.
+size_t reg_table_bytes();
+int reg_build_tables(void* tab, cudaStream_t st);
+const float4* reg_table(const spectre_ctx* ctx, int M);
+
+}  // namespace spectre

@@ -48,6 +48,27 @@ def test_mixer_f32_four_step(ctx, n):
     assert run_mixer(ctx, w) < TOL["f32"]
 
 
+@pytest.mark.parametrize("dt,n,L,D", [("f32", 64, 1, 8), ("bf16", 128, 127, 24), ("f16", 256, 129, 40), ("bf16", 400, 400, 64),
+                                      ("f32", 576, 290, 16), ("f16", 784, 784, 24), ("bf16", 512, 511, 8), ("f32", 1024, 1000, 24),
+                                      ("bf16", 2048, 1025, 40), ("f32", 4096, 2049, 24), ("f16", 8192, 5003, 40), ("f32", 16384, 9001, 8),
+                                      ("f32", 32768, 20011, 24)])
+def test_register_transforms(ctx, dt, n, L, D):
+    # partial column tiles, idle threads, rows cut anywhere; the workspace route and, at 4096 / 8192, in place without one
+    w = W.Workload("t", B=2, L=L, H=3, D=D, dtype=dt, n_fft=n, seed=n + L)
+    assert run_mixer(ctx, w, n_fft=n) < TOL[dt]
+    if n in (4096, 8192):
+        x, g = W.activations(w), W.random_gate(w)
+        y = x.cuda()
+        S.spectre_mixer_forward(ctx, y, g.cuda(), y=y, n_fft=n, workspace=torch.empty(0, dtype=torch.uint8, device="cuda"))
+        torch.cuda.synchronize()
+        assert_close(W.to_f64(y), O.mixer(W.to_f64(x), gate_to_complex(g), n_fft=n), dt)
+    if n <= 2048:
+        v, dy, g = W.activations(w, stream=1), W.activations(w, stream=2), W.random_gate(w)
+        dv, dg = S.spectre_mixer_backward(ctx, v.cuda(), dy.cuda(), g.cuda(), n_fft=n)
+        rv, rg = O.mixer_backward(W.to_f64(v), W.to_f64(dy), gate_to_complex(g), n_fft=n)
+        assert slab_err(W.to_f64(dv), rv) < TOL[dt] and rel_err(gate_to_complex(dg), rg) < TOL["f32"]
+
+
 @pytest.mark.parametrize("n,D", [(196, 64), (1024, 64), (8192, 64), (65536, 16), (2048, 8), (512, 24), (8192, 40)])
 def test_mixer_bf16(ctx, n, D):
     w = W.Workload("t", B=2, L=n, H=2, D=D, dtype="bf16", seed=7 * n + D)
