@@ -1,10 +1,11 @@
-"""Thin ctypes binding over the C ABI of libspectre.so.
+"""Thin binding over the C ABI of libspectre.so.
 
 Argument marshalling only: every step of the path runs in the CUDA kernels.
-Function names are those of include/spectre.h.  PyTorch appears here for device
-memory (tensors, workspace) and the current stream, nothing else.  If the
-shared library is missing the import of any entry point raises: there is no CPU
-or PyTorch fallback.
+Function names are those of include/spectre.h.  The per-step calls are marshalled
+in native code (csrc/native.cpp, the _native extension), contexts, queries and
+pre-marshalled calls through ctypes.  PyTorch appears here for device memory
+(tensors, workspace) and the current stream, nothing else.  If the shared library
+or the extension is missing every call raises: there is no CPU or PyTorch fallback.
 """
 from __future__ import annotations
 
@@ -130,6 +131,23 @@ def lib():
     return L
 
 
+_ext = None
+
+
+def _native():
+    """The extension module (built in-tree by paper_2502_18394_b200.build); fails loudly if absent."""
+    global _ext
+    if _ext is None:
+        lib()
+        try:
+            from . import _native as ext
+        except ImportError as e:
+            raise RuntimeError("the _native extension cannot be loaded: build it with `python -m paper_2502_18394_b200.build`") from e
+        ext.set_error(SpectreError)
+        _ext = ext
+    return _ext
+
+
 def _check(status: int):
     if status != SPECTRE_OK:
         L = lib()
@@ -168,6 +186,7 @@ class Context:
 
     def __init__(self, device: int = 0):
         self.handle = C.c_void_p()
+        _native()
         _check(lib().spectre_create(C.byref(self.handle), device))
         self.device = device
 
@@ -219,10 +238,6 @@ def _wavelet_struct(w: dict | None, keep: list):
                    None if w.get("skip") is None else w["skip"].data_ptr())
 
 
-def _workspace(nbytes: int, device) -> torch.Tensor | None:
-    return torch.empty(max(nbytes, 16), dtype=torch.uint8, device=device) if nbytes > 0 else None
-
-
 def spectre_gate_workspace_bytes(ctx: Context, B, H, D, n_fft, toeplitz_r=0) -> int:
     return lib().spectre_gate_workspace_bytes(ctx.handle, B, H, D, n_fft, toeplitz_r)
 
@@ -232,23 +247,8 @@ def spectre_gate(ctx: Context, params: dict, n_fft: int, q: torch.Tensor | None 
                  shift_all: int = 0, g_out: torch.Tensor | None = None, qbar_out: torch.Tensor | None = None,
                  workspace: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """g[B,H,K,2] = gate(...) (Sec. 3.2 step 3).  Allocates g_out / workspace with torch when not given."""
-    ref = q if q is not None else sum_q
-    if q is not None:
-        B, _, H, D = q.shape
-    else:
-        B, H, D = sum_q.shape
-    K = n_fft // 2 + 1
-    keep: list = []
-    gp = _gate_struct(params, keep)
-    if g_out is None:
-        g_out = torch.empty((B, H, K, 2), dtype=torch.float32, device=ref.device)
-    if workspace is None:
-        workspace = _workspace(spectre_gate_workspace_bytes(ctx, B, H, D, n_fft, gp.toeplitz_r), ref.device)
-    a = act(q) if q is not None else None
-    _check(lib().spectre_gate(ctx.handle, _stream(stream), None if a is None else C.byref(a), _ptr(sum_q), B, H, D,
-                              float(inv_count), C.byref(gp), n_fft, _ptr(shift), int(shift_all), _ptr(g_out),
-                              _ptr(qbar_out), _ptr(workspace), 0 if workspace is None else workspace.numel()))
-    return g_out
+    return _ext.gate(ctx.handle.value, params, n_fft, q, sum_q, inv_count, shift, shift_all, g_out, qbar_out, workspace, stream,
+                     False)
 
 
 def spectre_gate_static_max_bytes() -> int:
@@ -262,17 +262,7 @@ def spectre_gate_static(ctx: Context, params: dict, n_fft: int, g_out: torch.Ten
     """spectre_gate with the scratch inside the library: for callers that may not allocate device
     memory where the gate runs.  Nothing is allocated here either, so the output tensor g_out
     [B,H,K,2] is a required argument.  Calls on one device share the scratch: do not overlap them."""
-    if q is not None:
-        B, _, H, D = q.shape
-    else:
-        B, H, D = sum_q.shape
-    keep: list = []
-    gp = _gate_struct(params, keep)
-    a = act(q) if q is not None else None
-    _check(lib().spectre_gate_static(ctx.handle, _stream(stream), None if a is None else C.byref(a), _ptr(sum_q),
-                                     B, H, D, float(inv_count), C.byref(gp), n_fft, _ptr(shift), int(shift_all),
-                                     _ptr(g_out), _ptr(qbar_out)))
-    return g_out
+    return _ext.gate(ctx.handle.value, params, n_fft, q, sum_q, inv_count, shift, shift_all, g_out, qbar_out, None, stream, True)
 
 
 def spectre_mixer_workspace_bytes(ctx: Context, B, L, H, D, n_fft, dtype_code) -> int:
@@ -283,31 +273,13 @@ def spectre_mixer_forward(ctx: Context, v: torch.Tensor, g: torch.Tensor, y: tor
                           n_fft: int | None = None, wrm: dict | None = None,
                           workspace: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """Y = irfft(g * rfft(V)) per head (Sec. 3.2 steps 2, 4)."""
-    B, L, H, D = v.shape
-    n = L if n_fft is None else n_fft
-    if y is None:
-        y = torch.empty_like(v)
-    if workspace is None:
-        workspace = _workspace(spectre_mixer_workspace_bytes(ctx, B, L, H, D, n, _dtype_code(v)), v.device)
-    keep: list = []
-    w = _wavelet_struct(wrm, keep)
-    av, ay = act(v), act(y)
-    _check(lib().spectre_mixer_forward(ctx.handle, _stream(stream), C.byref(av), _ptr(g), C.byref(ay), n,
-                                       None if w is None else C.byref(w), _ptr(workspace),
-                                       0 if workspace is None else workspace.numel()))
-    return y
+    return _ext.mixer_forward(ctx.handle.value, v, g, y, n_fft, wrm, workspace, stream)
 
 
 def spectre_wavelet_refine(ctx: Context, y_in: torch.Tensor, wrm: dict, y_out: torch.Tensor | None = None,
                            stream=None) -> torch.Tensor:
     """Y_out = Y_in + W^-1(s * W Y_in) (Sec. 3.5)."""
-    if y_out is None:
-        y_out = torch.empty_like(y_in)
-    keep: list = []
-    w = _wavelet_struct(wrm, keep)
-    ai, ao = act(y_in), act(y_out)
-    _check(lib().spectre_wavelet_refine(ctx.handle, _stream(stream), C.byref(ai), C.byref(ao), C.byref(w)))
-    return y_out
+    return _ext.wavelet_refine(ctx.handle.value, y_in, wrm, y_out, stream)
 
 
 class PrefixCache:
@@ -333,21 +305,13 @@ def spectre_prefill_workspace_bytes(ctx: Context, B, H, D, N_max) -> int:
 def spectre_prefix_cache_prefill(ctx: Context, cache: PrefixCache, q: torch.Tensor, v: torch.Tensor,
                                  workspace: torch.Tensor | None = None, stream=None) -> None:
     """PreFill of Alg. 1."""
-    if workspace is None:
-        workspace = _workspace(spectre_prefill_workspace_bytes(ctx, cache.B, cache.H, cache.D, cache.N_max), v.device)
-    cs = cache.struct()
-    aq, av = act(q), act(v)
-    _check(lib().spectre_prefix_cache_prefill(ctx.handle, _stream(stream), C.byref(cs), C.byref(aq), C.byref(av),
-                                              _ptr(workspace), 0 if workspace is None else workspace.numel()))
+    _ext.prefill(ctx.handle.value, cache, q, v, workspace, stream)
 
 
 def spectre_prefix_cache_append(ctx: Context, cache: PrefixCache, q_t: torch.Tensor, v_t: torch.Tensor, t: int,
                                 stream=None) -> None:
     """DecodeStep of Alg. 1, steps (a)-(b)."""
-    if not (q_t.is_contiguous() and v_t.is_contiguous()):
-        raise ValueError("q_t and v_t must be contiguous [B, H, D]")
-    cs = cache.struct()
-    _check(lib().spectre_prefix_cache_append(ctx.handle, _stream(stream), C.byref(cs), _ptr(q_t), _ptr(v_t), int(t)))
+    _ext.append(ctx.handle.value, cache, q_t, v_t, t, stream)
 
 
 def spectre_decode_workspace_bytes(ctx: Context, B, H, D, N_max, nrows, toeplitz_r=0) -> int:
@@ -359,26 +323,7 @@ def spectre_prefix_cache_decode_step(ctx: Context, cache: PrefixCache, q_t: torc
                                      g_out: torch.Tensor | None = None, workspace: torch.Tensor | None = None,
                                      stream=None):
     """Whole DecodeStep of Alg. 1 with the listed read-out rows.  Returns (y_rows [B,len(rows),H,D], g [B,H,K,2])."""
-    if not (q_t.is_contiguous() and v_t.is_contiguous()):
-        raise ValueError("q_t and v_t must be contiguous [B, H, D]")
-    rows = [int(r) for r in rows]
-    keep: list = []
-    gp = _gate_struct(params, keep)
-    K = cache.N_max // 2 + 1
-    if y_rows is None:
-        y_rows = torch.empty((cache.B, len(rows), cache.H, cache.D), dtype=v_t.dtype, device=v_t.device)
-    if g_out is None:
-        g_out = torch.empty((cache.B, cache.H, K, 2), dtype=torch.float32, device=v_t.device)
-    if workspace is None:
-        workspace = _workspace(spectre_decode_workspace_bytes(ctx, cache.B, cache.H, cache.D, cache.N_max,
-                                                              max(1, min(len(rows), DECODE_MAX_ROWS)), gp.toeplitz_r),
-                               v_t.device)
-    cs = cache.struct()
-    arr = (C.c_int32 * max(1, len(rows)))(*rows)
-    _check(lib().spectre_prefix_cache_decode_step(ctx.handle, _stream(stream), C.byref(cs), _ptr(q_t), _ptr(v_t), int(t),
-                                                  C.byref(gp), arr, len(rows), _ptr(y_rows), _ptr(g_out),
-                                                  _ptr(workspace), 0 if workspace is None else workspace.numel()))
-    return y_rows, g_out
+    return _ext.decode_step(ctx.handle.value, cache, q_t, v_t, t, params, rows, y_rows, g_out, workspace, stream)
 
 
 def spectre_project_workspace_bytes(ctx: Context, H, D) -> int:
@@ -389,20 +334,7 @@ def spectre_project_qv(ctx: Context, x: torch.Tensor, Wq: torch.Tensor, Wv: torc
                        v: torch.Tensor | None = None, sum_q: torch.Tensor | None = None, need_sum: bool = True,
                        workspace: torch.Tensor | None = None, stream=None):
     """Q = X Wq, V = X Wv per head (Eq. 2) and sum_q = sum over the sequence of Q.  Returns (q, v, sum_q)."""
-    B, L, H, D = x.shape
-    if Wq.dtype != Wv.dtype or not (Wq.is_contiguous() and Wv.is_contiguous()):
-        raise ValueError("Wq and Wv must be contiguous and of one dtype")
-    q = torch.empty_like(x) if q is None else q
-    v = torch.empty_like(x) if v is None else v
-    if sum_q is None and need_sum:
-        sum_q = torch.empty((B, H, D), dtype=torch.float32, device=x.device)
-    if workspace is None:
-        workspace = _workspace(spectre_project_workspace_bytes(ctx, H, D), x.device)
-    ax, aq, av = act(x), act(q), act(v)
-    _check(lib().spectre_project_qv(ctx.handle, _stream(stream), C.byref(ax), _ptr(Wq), _ptr(Wv), _dtype_code(Wq),
-                                    C.byref(aq), C.byref(av), _ptr(sum_q), _ptr(workspace),
-                                    0 if workspace is None else workspace.numel()))
-    return q, v, sum_q
+    return _ext.project_qv(ctx.handle.value, x, Wq, Wv, q, v, sum_q, need_sum, workspace, stream)
 
 
 def spectre_mixer_backward_workspace_bytes(ctx: Context, B, L, H, D, n_fft, dtype_code) -> int:
@@ -413,18 +345,7 @@ def spectre_mixer_backward(ctx: Context, v: torch.Tensor, dy: torch.Tensor, g: t
                            need_dv: bool = True, need_dg: bool = True, workspace: torch.Tensor | None = None,
                            stream=None):
     """Gradients of <dy, mixer(v, g)>: (dv like v or None, dg [B,H,K,2] float32 or None)."""
-    B, L, H, D = v.shape
-    n = L if n_fft is None else n_fft
-    dv = torch.empty_like(v) if need_dv else None
-    dg = torch.empty((B, H, n // 2 + 1, 2), dtype=torch.float32, device=v.device) if need_dg else None
-    if workspace is None:
-        workspace = _workspace(spectre_mixer_backward_workspace_bytes(ctx, B, L, H, D, n, _dtype_code(v)), v.device)
-    av, ady = act(v), act(dy)
-    adv = act(dv) if need_dv else None
-    _check(lib().spectre_mixer_backward(ctx.handle, _stream(stream), C.byref(av), C.byref(ady), _ptr(g),
-                                        None if adv is None else C.byref(adv), _ptr(dg), n, _ptr(workspace),
-                                        0 if workspace is None else workspace.numel()))
-    return dv, dg
+    return _ext.mixer_backward(ctx.handle.value, v, dy, g, n_fft, need_dv, need_dg, workspace, stream)
 
 
 def spectre_readout_workspace_bytes(ctx: Context, B, H, D, N_max) -> int:
@@ -434,15 +355,7 @@ def spectre_readout_workspace_bytes(ctx: Context, B, H, D, N_max) -> int:
 def spectre_prefix_cache_readout(ctx: Context, cache: PrefixCache, g: torch.Tensor, y: torch.Tensor | None = None,
                                  workspace: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """Whole-window read-out irfft(g * prefix_fft) (Sec. 3.3.2 step e) -> [B, N_max, H, D]."""
-    if y is None:
-        y = torch.empty((cache.B, cache.N_max, cache.H, cache.D), dtype=cache.V_buf.dtype, device=g.device)
-    if workspace is None:
-        workspace = _workspace(spectre_readout_workspace_bytes(ctx, cache.B, cache.H, cache.D, cache.N_max), g.device)
-    cs = cache.struct()
-    ay = act(y)
-    _check(lib().spectre_prefix_cache_readout(ctx.handle, _stream(stream), C.byref(cs), _ptr(g), C.byref(ay),
-                                              _ptr(workspace), 0 if workspace is None else workspace.numel()))
-    return y
+    return _ext.readout(ctx.handle.value, cache, g, y, workspace, stream)
 
 
 # ---- pre-marshalled calls ---------------------------------------------------------------

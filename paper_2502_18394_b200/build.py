@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Builds, in-tree, the CUDA library with nvcc for sm_100a and the CPython extension that marshals its arguments with g++
+(no JIT cache)."""
 from __future__ import annotations
 
 import os
@@ -10,6 +11,8 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libspectre.so")
+NATIVE = os.path.join(PKG, "_native.so")
+NATIVE_SRC = os.path.join(CSRC, "native.cpp")
 OBJ = os.path.join(PKG, "build")
 SOURCES = ["reg_grad.cu", "reg_mix.cu", "reg_inverse.cu", "reg_forward.cu", "api.cu", "mixer.cu", "mixer_tc.cu", "mixer_tc8k.cu",
            "mixer_tc4k.cu", "gate.cu", "cache.cu", "wavelet.cu", "backward.cu", "project.cu"]
@@ -48,7 +51,39 @@ def _compile(src: str, obj: str, verbose: bool) -> str:
     return res.stderr
 
 
+def native_is_stale() -> bool:
+    if not os.path.exists(NATIVE):
+        return True
+    return os.path.getmtime(NATIVE) < max(os.path.getmtime(f) for f in (NATIVE_SRC, os.path.join(ROOT, "include", "spectre.h")))
+
+
+def build_native(force: bool = False) -> str:
+    """The extension links against torch's libraries (loaded with torch itself) and, by $ORIGIN, against libspectre.so."""
+    if not force and not native_is_stale():
+        return NATIVE
+    import sysconfig
+
+    import torch
+    t = os.path.dirname(torch.__file__)
+    cmd = ["g++", "-std=c++17", "-O2", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-I", os.path.join(t, "include"),
+           "-I", os.path.join(t, "include", "torch", "csrc", "api", "include"), "-I", "/usr/local/cuda/include",
+           "-I", sysconfig.get_paths()["include"], "-o", NATIVE, NATIVE_SRC, "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch",
+           "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda", "-L", PKG, "-l:libspectre.so", "-Wl,-rpath,$ORIGIN"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed on " + NATIVE_SRC + ":\n" + res.stdout + res.stderr)
+    return NATIVE
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    """The library, then the extension over it."""
+    lib = build_library(force, verbose)
+    build_native(force)
+    return lib
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
     """One object per source file (compiled side by side, only the stale ones), then one link."""
     if not force and not is_stale():
         return LIB
