@@ -202,8 +202,8 @@ typedef struct {
  * [B, L, H, D], which is the concatenation of step 4.
  *   v, y     activations of identical shape and dtype; y may alias v where the
  *            transform is one kernel (the workspace query returns 0, and the
- *            bf16 / fp16 tensor-core paths n_fft = 196 with D = 64 and
- *            n_fft = 8192; the fp32 path at n_fft = 4096 and 8192 is one, slower,
+ *            bf16 / fp16 tensor-core paths n_fft = 196 with D = 64,
+ *            n_fft = 4096 and n_fft = 8192; the fp32 path at n_fft = 4096 and 8192 is one, slower,
  *            kernel too when y overlaps v or no workspace is given); on a multi-pass
  *            path a call whose v and y overlap anywhere between their first and last byte is refused with
  *            SPECTRE_ERR_INVALID_ARG

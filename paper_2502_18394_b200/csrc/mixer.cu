@@ -36,6 +36,8 @@ namespace spectre {
 int launch_mixer_tc8192(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g,
                         const spectre_act* y);   // mixer_tc.cu
 bool tc8192_supported(const spectre_act* v, const spectre_act* y);                     // mixer_tc8k.cu
+bool tc4096_supported(const spectre_act* v, const spectre_act* y);                     // mixer_tc4096.cu
+int launch_mixer_tc4096(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, const spectre_act* y);
 int launch_mixer_tc196(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g,
                        const spectre_act* y, const spectre_wavelet* wrm, float* level_gate_scratch);
 bool tc196_fuses_wavelet(const spectre_wavelet* w);
@@ -53,7 +55,7 @@ int launch_mixer_tc4k(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
 
 // Path choice for bf16 transforms.  SPECTRE_FORCE_PATH = alu | fused | staged overrides it (tests):
 //   alu     fp32 butterflies only
-//   fused   the single-kernel tensor-core mixer (n = 8192 only)
+//   fused   the single-kernel tensor-core mixers (n = 4096 and 8192 only)
 //   staged  transpose-in / tensor-core units / transpose-out (n = 4096 ... 131072, needs workspace)
 enum { kPathAuto = 0, kPathAlu = 1, kPathFused = 2, kPathStaged = 3 };
 static int forced_path() {
@@ -869,12 +871,14 @@ extern "C" size_t spectre_mixer_workspace_bytes(const spectre_ctx* ctx, int32_t 
   if (!ctx || B < 1 || H < 1 || D < 8 || !make_plan(ctx, n_fft, &pl)) return 0;
   const int force = forced_path();
   if ((dtype == SPECTRE_BF16 || dtype == SPECTRE_F16) && ctx->dft64 && tc4k_supported(n_fft, D) && force != kPathAlu && force != kPathFused &&
-      (n_fft != 8192 || force == kPathStaged))               // n = 8192 defaults to the single-kernel path
+      ((n_fft != 8192 && (n_fft != 4096 || L < 64)) || force == kPathStaged))   // those default to a single kernel
     return tc4k_workspace_bytes(ctx, n_fft, D, B * H);
   if ((dtype == SPECTRE_BF16 || dtype == SPECTRE_F16) && n_fft == 196 && D == 64 && ctx->dft49 && force != kPathAlu)
     return tc196_level_gate_bytes(B, H);                     // level gates of a fused refinement
-  // the single-kernel path of n = 8192 takes whole 64-row blocks and needs no workspace
-  if ((dtype == SPECTRE_BF16 || dtype == SPECTRE_F16) && ctx->dft64 && n_fft == 8192 && L % 64 == 0 && force != kPathAlu) return 0;
+  // the single-kernel paths need no workspace; n = 8192 takes whole 64-row blocks, n = 4096 any L with one such block
+  if ((dtype == SPECTRE_BF16 || dtype == SPECTRE_F16) && ctx->dft64 && force != kPathAlu &&
+      ((n_fft == 8192 && L % 64 == 0) || (n_fft == 4096 && L >= 64)))
+    return 0;
   if (pl.N1 == 1 && !reg_multi(n_fft)) return 0;
   return (size_t)preferred_group(ctx, n_fft, D, B * H) * slab_ws_bytes(n_fft, D);
 }
@@ -897,7 +901,7 @@ extern "C" int spectre_mixer_forward(spectre_ctx* ctx, void* stream, const spect
   const bool tc_ok = (v->dtype == SPECTRE_BF16 || v->dtype == SPECTRE_F16) && ctx->dft64 != nullptr && force != kPathAlu;
   const bool ws_ok = workspace && !(reinterpret_cast<uintptr_t>(workspace) & 15);
   const bool tc196 = tc_ok && n_fft == 196 && v->D == 64 && ctx->dft49 != nullptr;
-  const bool fused = tc_ok && n_fft == 8192 && force != kPathStaged && tc8192_supported(v, y);
+  const bool fused = tc_ok && force != kPathStaged && ((n_fft == 8192 && tc8192_supported(v, y)) || (n_fft == 4096 && tc4096_supported(v, y)));
   // n = 8192 that the fused kernel cannot take (no whole 64-row blocks) stays on the fp32 kernels unless forced
   const bool staged = !fused && tc_ok && force != kPathFused && (n_fft != 8192 || force == kPathStaged) &&
                       tc4k_supported(n_fft, v->D) && ws_ok &&
@@ -938,7 +942,7 @@ extern "C" int spectre_mixer_forward(spectre_ctx* ctx, void* stream, const spect
                                                workspace_bytes >= tc196_level_gate_bytes(v->B, v->H)));
     rc = tc196 ? launch_mixer_tc196(ctx, st, v, g, y, fuse_wrm ? wrm : nullptr, reinterpret_cast<float*>(workspace))
                : (staged ? launch_mixer_tc4k(ctx, st, v, g, y, n_fft, workspace, workspace_bytes)
-                         : launch_mixer_tc8192(ctx, st, v, g, y));
+                         : (n_fft == 4096 ? launch_mixer_tc4096(ctx, st, v, g, y) : launch_mixer_tc8192(ctx, st, v, g, y)));
     if (rc != SPECTRE_OK) return rc;
     if (wrm && !fuse_wrm) return spectre_wavelet_refine(ctx, stream, y, y, wrm);
     return SPECTRE_OK;

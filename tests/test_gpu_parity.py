@@ -148,6 +148,22 @@ def test_mixer_bf16_tensor_core_zero_pad_and_strides(ctx):
     assert float(y[:, :, :2].abs().max()) == 0.0
 
 
+@pytest.mark.parametrize("dt,L,D", [("bf16", 4096, 64), ("f16", 4095, 24), ("bf16", 64, 8), ("f16", 127, 64), ("bf16", 2050, 40)])
+def test_mixer_4096_single_kernel(ctx, dt, L, D, monkeypatch):
+    # whole and partial 64-row blocks through the tensor maps, strided head views, against the oracle and the staged path
+    w = W.Workload("t", B=2, L=L, H=3, D=D, dtype=dt, n_fft=4096, seed=L + D)
+    assert run_mixer(ctx, w, n_fft=4096) < TOL[dt]
+    x, g = W.activations(w), W.random_gate(w)
+    wide = torch.full((2, L + 3, 3, D), 7.0, dtype=x.dtype, device="cuda")
+    y = S.spectre_mixer_forward(ctx, x.cuda(), g.cuda(), y=wide[:, :L], n_fft=4096)
+    monkeypatch.setenv("SPECTRE_FORCE_PATH", "staged")
+    ys = S.spectre_mixer_forward(ctx, x.cuda(), g.cuda(), n_fft=4096)
+    torch.cuda.synchronize()
+    ctx.poll_status()
+    assert slab_err(W.to_f64(y), W.to_f64(ys)) < TOL[dt]
+    assert bool((wide[:, L:] == 7.0).all())                       # nothing beyond row L is written
+
+
 @pytest.mark.parametrize("L", [64, 4160, 8128])
 def test_mixer_bf16_8192_short_sequences_through_the_tensor_maps(ctx, L):
     # whole 64-row blocks shorter than n: rows beyond L read as zero and are not written;
