@@ -4,6 +4,7 @@
 //   gate_out_kernel    LayerNorm + hidden layer (per CTA, short transforms) and the output layer as a
 //                      stream over W2, 1-8 batch entries per pass; with the Toeplitz update off it also applies modReLU and
 //                      the positional phase
+//   gate_mma_kernel    the same on the tensor cores, several batch entries with bf16 weights
 //   gate_post_kernel Toeplitz update, modReLU, phase (only when r > 0)
 #include "tc_common.cuh"
 
@@ -195,6 +196,11 @@ int pool_sum_ring(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* q,
   return pool_launch(ctx, st, q, sums, 1, &used, ring, N);
 }
 
+__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
 // ---- MLP ---------------------------------------------------------------------
 template <typename WT> __device__ __forceinline__ float wload(const WT* p);
 template <> __device__ __forceinline__ float wload<float>(const float* p) { return __ldg(p); }
@@ -348,17 +354,19 @@ __device__ __forceinline__ void stage_weights(const void* src, void* dst, int by
   }
 }
 
-// modReLU: max(|z| + b, 0) z / |z|   (0 at z = 0)
+// modReLU: max(|z| + b, 0) z / |z| = max(1 + b / |z|, 0) z   (0 at z = 0)
 __device__ __forceinline__ float2 modrelu(float2 gk, float bias) {
-  const float mag = sqrtf(fmaf(gk.x, gk.x, gk.y * gk.y));
-  const float sc = mag > 0.f ? fmaxf(mag + bias, 0.f) / mag : 0.f;
+  const float m2 = fmaf(gk.x, gk.x, gk.y * gk.y);
+  const float sc = m2 > 0.f ? fmaxf(fmaf(bias, rsqrtf(m2), 1.0f), 0.f) : 0.f;
   return cscale(gk, sc);
 }
 // positional phase exp(+j 2 pi k p / n), angle reduced in integers
 // pm = shift mod n in [0, n)
 __device__ __forceinline__ float2 phase_reduced(int k, int n, unsigned pm) {
   if (pm == 0u) return make_float2(1.f, 0.f);
-  const unsigned kp = (unsigned)(((unsigned long long)k * (unsigned long long)pm) % (unsigned)n);
+  // a power of two: the product's low bits are the remainder, and wrap-around does not touch them
+  const unsigned kp = (n & (n - 1)) == 0 ? ((unsigned)k * pm) & (unsigned)(n - 1)
+                                         : (unsigned)(((unsigned long long)k * (unsigned long long)pm) % (unsigned)n);
   const float2 w = twiddle_fwd(kp, (unsigned)n);  // exp(-j ...)
   return make_float2(w.x, -w.y);
 }
@@ -595,6 +603,170 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
   }
 }
 
+// ---- output layer for several batch entries on the tensor cores ----
+// o[b][col] = sum_j u[b][j] W2[j][col] for up to NB entries of one head is a [NB x hidden] x [hidden x 2K] contraction.
+// With one bin per thread it took 15 instructions per weight word of 8 entries and 71 us at B = 8, H = 32, n = 32768, where
+// W2 and the gate take 27.  Here: mma.m16n8k16 with the bf16 weights as they are and the fp32 activations split into three
+// bf16 parts (hi + mid + lo, 24 bits), fp32 accumulation.  The 16 rows of A are, NB = 8: hi of the entries over mid, and
+// lo over zeros in a second product; NB = 4: hi, mid, lo, zeros in one.
+// A weight word is one (re, im) pair and W2 rows start on 4-byte boundaries only (2K values of 2 bytes, K odd), so a lane
+// loads the words of its bin in rows 2q, 2q + 1, 2q + 8, 2q + 9 of every 16 (q = lane % 4), and two byte permutations make them
+// the B fragments of the real and of the imaginary columns.  A warp walks a contiguous range of chunks of 16 bins (the second
+// half of a line is still in L1 then), the next chunk's 32 words per lane in flight under the products of the current one.
+// 71 -> 45 us; B = 2: 43 -> 37.  Bringing the words in by 4-byte asynchronous copies (61 us) or by a bulk copy per row and
+// block (88 us: its producer and the barriers around it) was slower.
+template <int NB> struct MmaRows { static constexpr int kSets = NB == 8 ? 2 : 1; };
+
+__device__ __forceinline__ void split3(float x, float (&p)[3]) {
+  p[0] = __bfloat162float(__float2bfloat16_rn(x));
+  p[1] = __bfloat162float(__float2bfloat16_rn(x - p[0]));
+  p[2] = x - p[0] - p[1];
+}
+// part of row `row` of A in set `set`: which entry, which part (3: zero)
+template <int NB> __device__ __forceinline__ int mma_row_part(int set, int row) {
+  if (NB == 8) return set == 0 ? (row >> 3) : (row < 8 ? 2 : 3);
+  return row >> 2;
+}
+
+struct GateChunk {
+  unsigned w[2][16];      // [group of 8 bins][row slot s]: row 16 (s / 4) + 8 (s / 2 % 2) + 2 q + s % 2
+  float2 b2;              // of bin lane % 16
+  float mb;
+};
+// A chunk's first bin: the last chunk ends at bin K - 1, so that none needs predicates (the bins it shares with the one
+// before it get the same values twice).
+__device__ __forceinline__ int gate_chunk_bin(int chunk, int K) { return min(16 * chunk, K - 16); }
+// src: W2 of the head at row 2 q, bin i8
+__device__ __forceinline__ void gate_fetch_chunk(GateChunk& x, const unsigned* __restrict__ src, const float2* __restrict__ b2,
+                                                 const float* __restrict__ mb, int K, int chunk, int lane) {
+  const int k0 = gate_chunk_bin(chunk, K);
+  const unsigned* r = src + k0;
+  const size_t far = 7 * (size_t)K;
+#pragma unroll
+  for (int s = 0; s < 16; ++s) {
+    x.w[0][s] = __ldg(r);
+    x.w[1][s] = __ldg(r + 8);
+    r += (s & 1) ? far : (size_t)K;
+  }
+  x.b2 = __ldg(b2 + k0 + (lane & 15));
+  x.mb = mb ? __ldg(mb + k0 + (lane & 15)) : 0.f;
+}
+// out: g_out of the lane's entry (i8) at bin 2 q; pm: the positional phase (per lane where entries differ)
+template <int NB, bool SHIFTS>
+__device__ __forceinline__ void gate_use_chunk(const GateChunk& x, const uint32_t (&A)[4][MmaRows<NB>::kSets][4], float2* __restrict__ out,
+                                               int n, int k0, bool write, bool relu, unsigned pm, int q, int lane) {
+  // the phase of bin k0 + lane % 16, handed round below (per-entry shifts: evaluated where they are used)
+  float2 ph = make_float2(1.f, 0.f);
+  if (!SHIFTS && pm) ph = phase_reduced(k0 + (lane & 15), n, pm);
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+      const unsigned a = x.w[g][4 * ks], b = x.w[g][4 * ks + 1], c = x.w[g][4 * ks + 2], d = x.w[g][4 * ks + 3];
+      const uint32_t r0 = __byte_perm(a, b, 0x5410), r1 = __byte_perm(c, d, 0x5410);
+      const uint32_t m0 = __byte_perm(a, b, 0x7632), m1 = __byte_perm(c, d, 0x7632);
+#pragma unroll
+      for (int set = 0; set < MmaRows<NB>::kSets; ++set) {
+        mma_16816(re, A[ks][set], r0, r1);
+        mma_16816(im, A[ks][set], m0, m1);
+      }
+    }
+    // C fragment: rows i8 and i8 + 8 (the entry's parts), columns = bins 8 g + 2 q + {0, 1}
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      float2 o = make_float2(re[c] + re[2 + c], im[c] + im[2 + c]);
+      if (NB == 4) {                               // hi and lo here, mid 4 rows (16 lanes) further on
+        o.x += __shfl_down_sync(0xffffffffu, re[c], 16);
+        o.y += __shfl_down_sync(0xffffffffu, im[c], 16);
+      }
+      const int src = 8 * g + 2 * q + c;
+      o.x += __shfl_sync(0xffffffffu, x.b2.x, src);
+      o.y += __shfl_sync(0xffffffffu, x.b2.y, src);
+      if (relu) o = modrelu(o, __shfl_sync(0xffffffffu, x.mb, src));
+      if (SHIFTS) o = cmul(o, phase_reduced(k0 + src, n, pm));
+      else if (pm) o = cmul(o, make_float2(__shfl_sync(0xffffffffu, ph.x, src), __shfl_sync(0xffffffffu, ph.y, src)));
+      if (write) out[k0 + 8 * g + c] = o;
+    }
+  }
+}
+
+// SHIFTS: the entries' phases differ.  Every CTA computes the hidden layer of its head and entries itself, under the first
+// chunks' loads: a kernel in front of this one for it takes longer than all of them (49 us in all against 45).
+template <int NB, bool SHIFTS>
+__global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p) {
+  extern __shared__ __align__(16) float u[];       // [hidden][NB], then q_bar [NB][D], then W1
+  asm volatile("griddepcontrol.launch_dependents;");
+  constexpr int kSets = MmaRows<NB>::kSets;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane & 3, i8 = lane >> 2, nw = blockDim.x >> 5;
+  const int nbg = (p.B + NB - 1) / NB;
+  const int h = blockIdx.y / nbg, b0 = (blockIdx.y - h * nbg) * NB, nb = min(NB, p.B - b0);
+  const unsigned* src = reinterpret_cast<const unsigned*>(reinterpret_cast<const bf16*>(p.W2) + h * p.hs_w2) + (size_t)(2 * q) * p.K + i8;
+  const float2* b2 = reinterpret_cast<const float2*>(p.b2 + h * p.hs_b2);
+  const float* mb = !p.post && p.modrelu_bias ? p.modrelu_bias + h * p.hs_mb : nullptr;
+  bf16* w1s = reinterpret_cast<bf16*>(u + ((NB * (p.hidden + p.D) + 3) & ~3));
+  if (p.stage_w1) stage_weights(reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, w1s, p.D * p.hidden * 2);
+  // a CTA's chunks are contiguous, its warps take neighbouring ones
+  const int nchunk = (p.K + 15) / 16, per = (nchunk + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int c0 = blockIdx.x * per + warp, c1 = min(nchunk, (int)(blockIdx.x + 1) * per);
+  GateChunk x, y;
+  gate_fetch_chunk(x, src, b2, mb, p.K, min(c0, nchunk - 1), lane);
+  // everything above reads only weights; the sums / hidden activations come from the kernel before
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  float* qbar = u + NB * p.hidden;
+  const float* sums = p.sums + ((size_t)b0 * p.H + h) * p.D;
+  const float *gamma = p.gamma + h * p.hs_ln, *beta = p.beta + h * p.hs_ln, *b1 = p.b1 + h * p.hs_b1;
+  if (p.stage_w1)
+    descriptor_and_hidden<bf16, NB, true>(sums, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, gamma, beta,
+                                          p.eps, w1s, b1, qbar, u, NB);
+  else
+    descriptor_and_hidden<bf16, NB, false>(sums, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, gamma, beta,
+                                           p.eps, reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, b1, qbar, u, NB);
+  if (p.qbar_out && blockIdx.x == 0)
+    for (int e = threadIdx.x; e < nb * p.D; e += blockDim.x) {
+      const int bb = e / p.D, c = e - bb * p.D;
+      p.qbar_out[((size_t)(b0 + bb) * p.H + h) * p.D + c] = qbar[e];
+    }
+  // A fragments: rows i8 and i8 + 8, columns 2q, 2q + 1 and + 8 of every 16 hidden units
+  uint32_t A[4][kSets][4];
+#pragma unroll
+  for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int j = 16 * ks + 8 * c + 2 * q;
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const int row = i8 + 8 * r, e = row % NB;
+        float x0[3] = {0.f, 0.f, 0.f}, x1[3] = {0.f, 0.f, 0.f};
+        if (e < nb) {
+          split3(u[j * NB + e], x0);
+          split3(u[(j + 1) * NB + e], x1);
+        }
+#pragma unroll
+        for (int set = 0; set < kSets; ++set) {
+          const int part = mma_row_part<NB>(set, row);
+          const float a = part == 0 ? x0[0] : (part == 1 ? x0[1] : (part == 2 ? x0[2] : 0.f));
+          const float b = part == 0 ? x1[0] : (part == 1 ? x1[1] : (part == 2 ? x1[2] : 0.f));
+          A[ks][set][2 * c + r] = pack_bf2(a, b);
+        }
+      }
+    }
+  const bool write = i8 < nb;
+  float2* out = p.g_out + ((size_t)(b0 + (write ? i8 : 0)) * p.H + h) * p.K + 2 * q;
+  unsigned pm = p.post ? 0u : p.pm_all;
+  if (SHIFTS) {
+    long long s = (p.shift_all + p.shift[b0 + (write ? i8 : 0)]) % p.n;
+    pm = (unsigned)(s < 0 ? s + p.n : s);
+  }
+  for (int c = c0; c < c1; c += 2 * nw) {
+    gate_fetch_chunk(y, src, b2, mb, p.K, min(c + nw, nchunk - 1), lane);
+    gate_use_chunk<NB, SHIFTS>(x, A, out, p.n, gate_chunk_bin(c, p.K), write, mb != nullptr, pm, q, lane);
+    if (c + nw >= c1) break;
+    gate_fetch_chunk(x, src, b2, mb, p.K, min(c + 2 * nw, nchunk - 1), lane);
+    gate_use_chunk<NB, SHIFTS>(y, A, out, p.n, gate_chunk_bin(c + nw, p.K), write, mb != nullptr, pm, q, lane);
+  }
+}
+
 struct GatePostParams {
   const float2* g_raw; float2* g_out;
   const float2* taps; size_t hs_t; int r;
@@ -725,7 +897,11 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   // block sized to the bin count for short transforms (K = 99 does not need 256 threads)
   const int thr_out = K >= 256 ? 256 : ((K + 31) / 32 * 32 < 64 ? 64 : (K + 31) / 32 * 32);
   // batch entries per CTA: the weights of a head are fetched once for all of them
-  const int BB = (gp->hidden > 256 || B < 2) ? 1 : (B < 4 ? 2 : (B < 8 ? 4 : 8));
+  // Tensor cores for bf16 weights and the usual 64 hidden units (the fragments of A fill the registers): 4 or 8 entries (5 ... 7
+  // would need two passes over W2 with 4).  With under 256 bins the 8 warps of its CTAs have no chunk each and the
+  // narrower CTAs below, more of them per SM, are faster (99 bins, 256 entries: 15 us against 16).
+  const bool mma = gp->wdtype == SPECTRE_BF16 && gp->hidden == 64 && K >= 256 && B >= 2;
+  const int BB = mma ? (B <= 4 ? 4 : 8) : (gp->hidden > 256 || B < 2) ? 1 : (B < 4 ? 2 : (B < 8 ? 4 : 8));
   dim3 grid_out((K + thr_out - 1) / thr_out, (unsigned)(H * ((B + BB - 1) / BB)));
   if (grid_out.y > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "H * ceil(B / 8) exceeds 65535");
   const bool wb = gp->wdtype == SPECTRE_BF16;
@@ -744,6 +920,13 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   cfg_out.attrs = pdl; cfg_out.numAttrs = 1;
   cfg_hid = cfg_out;
   cfg_hid.gridDim = dim3(grid_out.y, 1, 1); cfg_hid.blockDim = dim3(256, 1, 1);
+  // the tensor-core kernel: at most the two CTAs per SM that are resident, never a second wave of a few
+  cudaLaunchConfig_t cfg_mma = cfg_out;
+  if (mma) {
+    const int blocks = ((K + 15) / 16 + 7) / 8, fit = 2 * ctx->sm_count / (int)grid_out.y;
+    cfg_mma.gridDim = dim3((unsigned)(fit < 1 ? 1 : (blocks < fit ? blocks : fit)), grid_out.y, 1);
+    cfg_mma.blockDim = dim3(256, 1, 1);
+  }
 #define SPECTRE_GATE_LAUNCH(WT, NB)                                                              \
   do {                                                                                           \
     if (pre) {                                                                                   \
@@ -753,13 +936,21 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
       SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_out, gate_out_kernel<WT, NB, false>, mp));         \
     }                                                                                            \
   } while (0)
-  switch (BB) {
+#define SPECTRE_GATE_MMA(NB)                                                                     \
+  do {                                                                                           \
+    if (mp.shift && !mp.post) SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_mma, gate_mma_kernel<NB, true>, mp)); \
+    else SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_mma, gate_mma_kernel<NB, false>, mp));          \
+  } while (0)
+  if (mma) {
+    if (BB == 8) SPECTRE_GATE_MMA(8); else SPECTRE_GATE_MMA(4);
+  } else switch (BB) {
     case 8: if (wb) SPECTRE_GATE_LAUNCH(bf16, 8); else SPECTRE_GATE_LAUNCH(float, 8); break;
     case 4: if (wb) SPECTRE_GATE_LAUNCH(bf16, 4); else SPECTRE_GATE_LAUNCH(float, 4); break;
     case 2: if (wb) SPECTRE_GATE_LAUNCH(bf16, 2); else SPECTRE_GATE_LAUNCH(float, 2); break;
     default: if (wb) SPECTRE_GATE_LAUNCH(bf16, 1); else SPECTRE_GATE_LAUNCH(float, 1); break;
   }
 #undef SPECTRE_GATE_LAUNCH
+#undef SPECTRE_GATE_MMA
   SPECTRE_LAUNCH_OK("gate_out_kernel");
   if (r > 0) {
     GatePostParams pp = {};

@@ -285,6 +285,20 @@ def test_gate_shapes(ctx, B, L, H, D, hid, dt, wdt, n):
     assert eg < GATE_TOL["16bit"] and eq < GATE_TOL["16bit"]
 
 
+@pytest.mark.parametrize("B,H,n,r,shifts", [(2, 3, 510, 0, False), (4, 2, 4096, 0, True), (5, 2, 1000, 2, False), (8, 1, 32768, 0, False),
+                                             (17, 2, 512, 0, True)])
+def test_gate_batches_on_tensor_cores(ctx, B, H, n, r, shifts):
+    # 4- and 8-entry groups, the last group ragged, the last chunk of bins overlapping the one before, phases per entry
+    w = W.Workload("t", B=B, L=33, H=H, D=64, dtype="bf16", n_fft=n, seed=n + B)
+    p = W.gate_params(w, modrelu_bias_std=0.01, toeplitz_r=r, bias_std=0.1)
+    x = W.activations(w, structured=True)
+    shift = torch.arange(B, dtype=torch.int64) * 7 - 3 if shifts else None
+    g = S.spectre_gate(ctx, to_dev(p), n, q=x.cuda(), shift=shift.cuda() if shifts else None, shift_all=11)
+    ref = O.gate(W.to_f64(x).sum(axis=1), 1.0 / w.L, n, shift=(shift.numpy() if shifts else np.zeros(B, dtype=np.int64)) + 11,
+                 **gate_params_np(p))
+    assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
+
+
 def test_gate_from_running_sum_and_shared_heads(ctx):
     w = W.Workload("t", B=2, L=64, H=4, D=32, dtype="f32", wdtype="f32", n_fft=64, seed=13)
     p = W.gate_params(w)
