@@ -219,11 +219,14 @@ __global__ void __launch_bounds__(256) append_ring_kernel(T* __restrict__ V_buf,
 template <typename T>
 __global__ void __launch_bounds__(256) decode_ring_kernel(T* __restrict__ V_buf, T* __restrict__ Q_buf,
                                                           float* __restrict__ sum_q, float* __restrict__ delta,
-                                                          const T* __restrict__ q_t, const T* __restrict__ v_t, int B,
-                                                          int H, int D, int N, int slot, int evict) {
+                                                          int* __restrict__ done, const T* __restrict__ q_t,
+                                                          const T* __restrict__ v_t, int B, int H, int D, int N, int slot,
+                                                          int evict) {
+  asm volatile("griddepcontrol.launch_dependents;");      // the gate kernel behind streams weights before it needs sum_q
   const int total = B * H * D;
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= total) return;
+  if (idx < B * H) done[idx] = 0;                          // the spectrum pass counts a slab's finished blocks here
   int b = idx / (H * D), hd = idx - b * (H * D);
   size_t o = ((size_t)b * N + slot) * H * D + hd;
   float qn = io<T>::load1(q_t + idx), vn = io<T>::load1(v_t + idx);
@@ -243,33 +246,51 @@ struct DecodeRows { int r[SPECTRE_DECODE_MAX_ROWS]; };
 // consecutive bins of one (batch, head), a warp 32 of them: lane l evaluates bin k0 + l's
 // update twiddle and its NR read-out coefficients once, then the warp walks the 32 bins with
 // every lane holding 2 channels.  Row sums are reduced over the CTA and written as one
-// partial per (slab, bin block); decode_reduce_kernel adds the partials in a fixed order.
-template <int NR>
+// partial per (slab, bin block); the CTA that finishes a slab last adds its partials in a fixed order (a kernel of its
+// own for that took 10 us behind the 650 us pass of 256 x 32k slabs and 2.7 us of a short window's 19).
+// Bound by HBM (16 bytes per bin and channel).  Launched as a programmatic dependent of the gate kernel: the first bins are
+// on their way before the gate is complete (the spectrum itself was written by kernels in front of the ring kernel).
+template <typename T, int NR>
 __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* __restrict__ prefix, const float* __restrict__ delta,
                                                               const float2* __restrict__ g, float* __restrict__ partial,
-                                                              int D, int N, int K, unsigned tm, DecodeRows rows,
-                                                              int nblk) {
+                                                              int* __restrict__ done, T* __restrict__ y, int H, int D, int N, int K,
+                                                              unsigned tm, DecodeRows rows, int nrows, int nblk) {
   __shared__ float red[8][NR][64];
+  __shared__ int last;
   const int slab = blockIdx.x / nblk, blk = blockIdx.x - slab * nblk;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k0 = (blk * 8 + warp) * 32, k = k0 + lane;
+  const int nb = max(0, min(32, K - k0));
+  const int half = D / 2;
+  float* base = prefix + (((size_t)slab * K + k0) * D) * 2;
+  // eight bins per round, their loads issued together (the compiler cannot move a load of this array above the store
+  // before it)
+  float4 v[8];
+  auto fetch = [&](int i0, int c) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c < half && i0 + u < nb) v[u] = *reinterpret_cast<const float4*>(base + ((size_t)(i0 + u) * D + 2 * c) * 2);
+    }
+  };
+  fetch(0, lane);
   float2 my = make_float2(1.f, 0.f);
   float2 coef[NR];
+  const float wk = ((k == 0 || 2 * k == N) ? 1.0f : 2.0f) / (float)N;
 #pragma unroll
   for (int r = 0; r < NR; ++r) coef[r] = make_float2(0.f, 0.f);
   if (k < K) {
     my = twiddle_fwd((unsigned)(((unsigned long long)k * tm) % (unsigned)N), (unsigned)N);
-    const float2 gk = __ldg(g + (size_t)slab * K + k);
-    const float wk = ((k == 0 || 2 * k == N) ? 1.0f : 2.0f) / (float)N;
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const float2 e = twiddle_fwd((unsigned)(((unsigned long long)k * (unsigned)rows.r[r]) % (unsigned)N), (unsigned)N);
-      coef[r] = cscale(cmulc(gk, e), wk);               // g_k exp(+j theta) w_k / N
-    }
+    for (int r = 0; r < NR; ++r)
+      coef[r] = cscale(twiddle_fwd((unsigned)(((unsigned long long)k * (unsigned)rows.r[r]) % (unsigned)N), (unsigned)N), wk);
   }
-  const int nb = max(0, min(32, K - k0));
-  const int half = D / 2;
-  float* base = prefix + (((size_t)slab * K + k0) * D) * 2;
+  asm volatile("griddepcontrol.wait;" ::: "memory");      // delta and g
+  if (k < K) {
+    const float2 gk = g[(size_t)slab * K + k];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) coef[r] = cmulc(gk, coef[r]);   // g_k exp(+j theta) w_k / N
+  }
   for (int c0 = 0; c0 < half; c0 += 32) {               // uniform trip count: every lane takes part in the shuffles
     const int c = c0 + lane;
     const bool live = c < half;
@@ -281,15 +302,8 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* __restrict_
     float acc[NR][2];
 #pragma unroll
     for (int r = 0; r < NR; ++r) acc[r][0] = acc[r][1] = 0.f;
-    // eight bins per round, their loads issued together (the compiler cannot move a load of this array
-    // above the store before it)
     for (int i0 = 0; i0 < nb; i0 += 8) {
-      float4 v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (live && i0 + u < nb) v[u] = *reinterpret_cast<const float4*>(base + ((size_t)(i0 + u) * D + 2 * c) * 2);
-      }
+      if (i0 + c0 > 0) fetch(i0, c);
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int i = min(i0 + u, 31);
@@ -327,25 +341,30 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* __restrict_
     }
     __syncthreads();
   }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) decode_reduce_kernel(const float* __restrict__ partial, T* __restrict__ y, int B, int H,
-                                                            int D, int nblk, int NR, int nrows) {
-  const int total = B * nrows * H * D;
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= total) return;
-  int c = idx % D, h = (idx / D) % H, r = (idx / (D * H)) % nrows, b = idx / (D * H * nrows);
-  const float* p = partial + (((size_t)(b * H + h) * nblk) * NR + r) * D + c;
-  float s = 0.f;
-  for (int blk0 = 0; blk0 < nblk; blk0 += 16) {              // 16 partials in flight; the order of the sum is fixed
-    float v[16];
+  // the slab's last block: partials of all blocks, four threads per output
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(done + slab, 1) == nblk - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int b = slab / H, h = slab - b * H, part = threadIdx.x & 3;
+  for (int o0 = 0; o0 < nrows * D; o0 += 64) {                 // uniform trip count for the shuffles
+    const int o = o0 + (int)(threadIdx.x >> 2), r = o / D, c = o - r * D;
+    const bool in = o < nrows * D;
+    const float* p = partial + ((size_t)slab * nblk * NR + r) * D + c;
+    float s = 0.f;
+    for (int j0 = part; j0 < nblk; j0 += 32) {
+      float t[8];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) v[u] = blk0 + u < nblk ? __ldg(p + (size_t)(blk0 + u) * NR * D) : 0.f;
+      for (int u = 0; u < 8; ++u) t[u] = in && j0 + 4 * u < nblk ? __ldcg(p + (size_t)(j0 + 4 * u) * NR * D) : 0.f;
 #pragma unroll
-    for (int u = 0; u < 16; ++u) s += v[u];
+      for (int u = 0; u < 8; ++u) s += t[u];
+    }
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if (in && part == 0) io<T>::store1(y + (((size_t)b * nrows + r) * H + h) * D + c, s);
   }
-  io<T>::store1(y + idx, s);
 }
 
 static int check_cache(const spectre_cache* c) {
@@ -481,7 +500,7 @@ extern "C" size_t spectre_decode_workspace_bytes(const spectre_ctx* ctx, int32_t
   if (B < 1 || H < 1 || D < 1 || N_max < 2 || nrows < 1 || nrows > SPECTRE_DECODE_MAX_ROWS || toeplitz_r < 0) return 0;
   const int K = N_max / 2 + 1, nblk = (K + 255) / 256;
   return round256((size_t)B * H * D * 4) + round256((size_t)B * H * nblk * decode_nr(nrows) * D * 4) +
-         gate_min_workspace(B, H, D, N_max, toeplitz_r);
+         round256((size_t)B * H * sizeof(int)) + gate_min_workspace(B, H, D, N_max, toeplitz_r);
 }
 
 extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, const spectre_cache* cache, const void* q_t,
@@ -506,20 +525,22 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
     return fail(SPECTRE_ERR_WORKSPACE, "workspace is NULL or not 16-byte aligned");
   const size_t delta_bytes = round256((size_t)B * H * D * 4);
   const size_t part_bytes = round256((size_t)B * H * nblk * NR * D * 4);
+  const size_t done_bytes = round256((size_t)B * H * sizeof(int));
   const size_t gate_bytes = gate_min_workspace(B, H, D, N, params->toeplitz_r < 0 ? 0 : params->toeplitz_r);
-  if (workspace_bytes < delta_bytes + part_bytes + gate_bytes) return fail(SPECTRE_ERR_WORKSPACE, "decode workspace too small");
+  if (workspace_bytes < delta_bytes + part_bytes + done_bytes + gate_bytes) return fail(SPECTRE_ERR_WORKSPACE, "decode workspace too small");
   SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   float* delta = reinterpret_cast<float*>(workspace);
   float* partial = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(workspace) + delta_bytes);
-  void* gate_ws = reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes;
+  int* done = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes);
+  void* gate_ws = reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes + done_bytes;
   const int slot = (int)(t % N);
   const int evict = t >= N ? 1 : 0;
   // (a)-(b) ring buffers, running sum, delta
   const unsigned blocks_r = (unsigned)(((size_t)B * H * D + 255) / 256);
   SPECTRE_IO_DISPATCH(cache->buf_dtype,
                       decode_ring_kernel<T><<<blocks_r, 256, 0, st>>>(reinterpret_cast<T*>(cache->V_buf), reinterpret_cast<T*>(cache->Q_buf),
-                                                                      cache->sum_q, delta, reinterpret_cast<const T*>(q_t),
+                                                                      cache->sum_q, delta, done, reinterpret_cast<const T*>(q_t),
                                                                       reinterpret_cast<const T*>(v_t), B, H, D, N, slot, evict));
   SPECTRE_LAUNCH_OK("decode_ring_kernel");
   // (c)-(d) gate from the running sum with phase p = t
@@ -531,14 +552,20 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   for (int i = 0; i < SPECTRE_DECODE_MAX_ROWS; ++i) dr.r[i] = rows[i < nrows ? i : nrows - 1];
   const unsigned blocks_s = (unsigned)((size_t)B * H * nblk);
   const float2* g2 = reinterpret_cast<const float2*>(g_out);
-  if (NR == 1) decode_spectrum_kernel<1><<<blocks_s, 256, 0, st>>>(cache->prefix_fft, delta, g2, partial, D, N, K, (unsigned)slot, dr, nblk);
-  else if (NR == 2) decode_spectrum_kernel<2><<<blocks_s, 256, 0, st>>>(cache->prefix_fft, delta, g2, partial, D, N, K, (unsigned)slot, dr, nblk);
-  else decode_spectrum_kernel<SPECTRE_DECODE_MAX_ROWS><<<blocks_s, 256, 0, st>>>(cache->prefix_fft, delta, g2, partial, D, N, K, (unsigned)slot, dr, nblk);
-  SPECTRE_LAUNCH_OK("decode_spectrum_kernel");
-  const unsigned blocks_y = (unsigned)(((size_t)B * nrows * H * D + 255) / 256);
-  SPECTRE_IO_DISPATCH(cache->buf_dtype,
-                      decode_reduce_kernel<T><<<blocks_y, 256, 0, st>>>(partial, reinterpret_cast<T*>(y_rows), B, H, D, nblk, NR, nrows));
-  SPECTRE_LAUNCH_OK("decode_reduce_kernel");
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks_s);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  SPECTRE_IO_DISPATCH(cache->buf_dtype, {
+    auto kern = NR == 1 ? decode_spectrum_kernel<T, 1> : (NR == 2 ? decode_spectrum_kernel<T, 2> : decode_spectrum_kernel<T, SPECTRE_DECODE_MAX_ROWS>);
+    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, cache->prefix_fft, static_cast<const float*>(delta), g2, partial, done,
+                                       reinterpret_cast<T*>(y_rows), H, D, N, K, (unsigned)slot, dr, (int)nrows, nblk));
+  });
   return SPECTRE_OK;
 }
 
