@@ -658,7 +658,7 @@ static RegParams reg_params(int n, int H, int D, int L) {
   p.scale = 1.0f / (float)n;
   return p;
 }
-static void reg_source(RegParams& p, const spectre_act* a) { p.src = a->ptr; p.s_sb = a->stride_b; p.s_sl = a->stride_l; p.s_sh = a->stride_h; }
+static void reg_source(RegParams& p, const spectre_act* a) { p.batch = a->B; p.src = a->ptr; p.s_sb = a->stride_b; p.s_sl = a->stride_l; p.s_sh = a->stride_h; }
 static void reg_dest(RegParams& p, const spectre_act* a) { p.dst = a->ptr; p.d_sb = a->stride_b; p.d_sl = a->stride_l; p.d_sh = a->stride_h; }
 static StridedParams strided_params(const spectre_act* a, bool out, int n, int M, float2* ws, int slab0, int cnt) {
   StridedParams sp = {};

@@ -17,7 +17,8 @@ struct RegParams {
   int64_t s_sb, s_sl, s_sh;
   int64_t s2_sb, s2_sl, s2_sh;
   int64_t d_sb, d_sl, d_sh;
-  int H, D, L, n, K;
+  int batch, H, D, L, n, K;
+  int* status;              // host-mapped status word (bounded waits)
   int N1;                   // outer factor of n = N1 M; a CTA's sequence is k1 of N1
   int decim;                // forward, from tokens: element j of sequence k1 is token N1 j + k1
   int slab0, ntile;
