@@ -55,11 +55,10 @@ struct TwoStep {
   __device__ __forceinline__ int bin(int i) const { return m + S * (i / R2) + R1 * (i % R2); }
   static __device__ __forceinline__ int gate_slot(int k) { return k; }
 
-  // before / after: called in front of and behind the exchange's (first) barrier
+  // before: called in front of the exchange's (first) barrier
   struct Nothing { __device__ __forceinline__ void operator()() const {} };
-  template <bool HALF, class Before = Nothing, class After = Nothing>
-  __device__ __forceinline__ void forward(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before = Before(),
-                                          After after = After()) const {
+  template <bool HALF, class Before = Nothing>
+  __device__ __forceinline__ void forward(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before = Before()) const {
     RegDft<R1, false>::run(x);
 #pragma unroll
     for (int a = 0; a < R1 / 2; ++a) {
@@ -67,7 +66,7 @@ struct TwoStep {
       if (a > 0) x[2 * a] = cmul(x[2 * a], make_float2(w.x, w.y));
       x[2 * a + 1] = cmul(x[2 * a + 1], make_float2(w.z, w.w));
     }
-    exchange<HALF, true>(x, buf, act, before, after);
+    exchange<HALF, true>(x, buf, act, before);
 #pragma unroll
     for (int u = 0; u < U; ++u) sub<false>(x, u);
   }
@@ -83,7 +82,7 @@ struct TwoStep {
         x[u * R2 + 2 * a + 1] = cmulc(x[u * R2 + 2 * a + 1], make_float2(w.z, w.w));
       }
     }
-    exchange<HALF, false>(x, buf, act, Nothing(), Nothing());
+    exchange<HALF, false>(x, buf, act, Nothing());
     RegDft<R1, true>::run(x);
   }
 
@@ -103,8 +102,8 @@ struct TwoStep {
   }
   // FWD: first step's order -> second step's.  The inverse writes the positions this thread read last, so it needs no
   // barrier in front.  HALF: real and imaginary parts one after the other through half the space.
-  template <bool HALF, bool FWD, class Before, class After>
-  __device__ __forceinline__ void exchange(float2 (&x)[E], void* buf, bool act, Before before, After after) const {
+  template <bool HALF, bool FWD, class Before>
+  __device__ __forceinline__ void exchange(float2 (&x)[E], void* buf, bool act, Before before) const {
     if constexpr (!HALF) {
       float2* b = reinterpret_cast<float2*>(buf);
       if (act) {
@@ -113,7 +112,6 @@ struct TwoStep {
       }
       before();
       __syncthreads();
-      after();
 
 #pragma unroll
       for (int i = 0; i < E; ++i) x[i] = b[at(!FWD, i)];
@@ -311,6 +309,24 @@ __device__ __forceinline__ void reg_load_ws(float2 (&x)[P::E], const float2* ws,
   for (int i = 0; i < P::E; ++i) x[i] = *reinterpret_cast<const float2*>(base + (size_t)(P::S * i) * half * 8 + mine);
 }
 
+// the rows back, those below L
+template <typename T, class P>
+__device__ __forceinline__ void reg_store_tokens(const float2 (&x)[P::E], const RegParams& p, int b, int h, int col, int m, bool live) {
+  typedef typename PairIo<T>::raw raw;
+  char* base = reinterpret_cast<char*>(reinterpret_cast<T*>(p.dst) + b * p.d_sb + h * p.d_sh);
+  const int64_t ds = (int64_t)P::S * p.d_sl * (int64_t)sizeof(T);
+  const uint32_t mine = (uint32_t)((int64_t)m * p.d_sl + col) * (uint32_t)sizeof(T);
+  const int count = rows_below(p.L, m, P::S, live);
+  if (count >= P::E) {
+#pragma unroll
+    for (int i = 0; i < P::E; ++i) *reinterpret_cast<raw*>(base + i * ds + mine) = PairIo<T>::pack(x[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < P::E; ++i)
+      if (i < count) *reinterpret_cast<raw*>(base + i * ds + mine) = PairIo<T>::pack(x[i]);
+  }
+}
+
 // Sum over the RL pairs that sit side by side in the warp (lane bits SHIFT ...) of RL values each; the lane whose pair
 // is s keeps the sum of value s.
 template <int RL, int SHIFT>
@@ -451,34 +467,22 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
 #pragma unroll
     for (int i = 0; i < E; ++i) *reinterpret_cast<float2*>(base + (size_t)(P::S * i) * half * 8 + mine) = x[i];
   } else {
-    typedef typename PairIo<T>::raw raw;
-    char* base = reinterpret_cast<char*>(reinterpret_cast<T*>(p.dst) + b * p.d_sb + h * p.d_sh);
-    const int64_t ds = (int64_t)P::S * p.d_sl * (int64_t)sizeof(T);
-    const uint32_t mine = (uint32_t)((int64_t)pl.m * p.d_sl + 2 * pin) * (uint32_t)sizeof(T);
-    const int count = rows_below(p.L, pl.m, P::S, live);
-    if (count >= E) {
-#pragma unroll
-      for (int i = 0; i < E; ++i) *reinterpret_cast<raw*>(base + i * ds + mine) = PairIo<T>::pack(x[i]);
-    } else {
-#pragma unroll
-      for (int i = 0; i < E; ++i)
-        if (i < count) *reinterpret_cast<raw*>(base + i * ds + mine) = PairIo<T>::pack(x[i]);
-    }
+    reg_store_tokens<T, P>(x, p, b, h, 2 * pin, pl.m, live);
   }
 }
 
-// The same for 16-bit tokens and more tiles than are resident: persistent CTAs, the next tile's rows on their way by TMA under
-// this one's arithmetic (kRegMix, kRegForward of the two-step plans).  Waiting for its rows at the start of every tile left
-// the issue slots half idle with two CTAs per SM.
-//   map   dims (column, k1 of N1, j, head, batch) of the tokens t = N1 j + k1 with j below L / N1; boxes of 16 columns x
-//         reg_box_rows() rows land as [row][8 pairs], from which the threads of a warp read 128 contiguous bytes.  The
-//         L % N1 rows of the last, partial j are read with plain loads.
+// kRegMix of the two-step plans for 16-bit tokens and more tiles than are resident: persistent CTAs, the next tile's rows on
+// their way by TMA under this one's arithmetic.  Measured at 12.6 M elements: n = 1024 32.0 -> 29.6 us, 784 29.9 -> 26.7,
+// 576 28.6 -> 25.9, 512 23.4 -> 21.2, 256 20.7 -> 19.6.  The forward-only mode lost by it (prefill of 2 x 32 x 32k 513 -> 620 us:
+// rows N1 tokens apart).
+//   map   dims (column, row, head, batch) of the tokens; boxes of 16 columns x reg_box_rows() rows land as [row][8 pairs],
+//         from which the threads of a warp read 128 contiguous bytes; rows and columns beyond the tensor are zeros
 template <class P> __host__ __device__ constexpr int reg_box_rows() { return P::M / ((P::M + 255) / 256); }     // at most 256, dividing M
-template <class P, int MODE> __host__ __device__ constexpr size_t reg_stream_bytes() {            // rows, exchange, gate table, barrier
-  return (size_t)P::M * P::C * 4 + reg_exch_bytes<P, MODE>() + (MODE == kRegMix ? (size_t)P::kGate * 8 : 0) + 16;
+template <class P> __host__ __device__ constexpr size_t reg_stream_bytes() {            // rows, exchange, gate table, barrier
+  return (size_t)P::M * P::C * 4 + reg_exch_bytes<P, kRegMix>() + (size_t)P::kGate * 8 + 16;
 }
 
-template <typename T, class P, int MODE>
+template <typename T, class P>
 __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_stream_kernel(const __grid_constant__ CUtensorMap map,
                                                                                       const __grid_constant__ RegParams p, int ntotal) {
   extern __shared__ __align__(1024) unsigned char reg_stream_smem[];               // all of it dynamic: TMA needs the base 128-byte aligned
@@ -488,112 +492,61 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_stream_k
   static_assert(P::M % kRows == 0 && kRows * 32 % 128 == 0 && P::C == 8, "whole boxes, 128-byte aligned");
   raw* rows = reinterpret_cast<raw*>(reg_stream_smem);                             // [M][8]
   void* buf = reg_stream_smem + kRaw;
-  float2* gs = reinterpret_cast<float2*>(reg_stream_smem + kRaw + reg_exch_bytes<P, MODE>());
-  const uint32_t bar = smem_u32(reg_stream_smem + reg_stream_bytes<P, MODE>() - 16);
+  float2* gs = reinterpret_cast<float2*>(reg_stream_smem + kRaw + reg_exch_bytes<P, kRegMix>());
+  const uint32_t bar = smem_u32(reg_stream_smem + reg_stream_bytes<P>() - 16);
   const bool act = threadIdx.x < P::kActive;
   const P pl(act ? (int)threadIdx.x : 0);
-  const int half = p.D / 2, jfull = p.L / p.N1, jrest = p.L - jfull * p.N1;
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  auto fetch = [&](int u) {                                                        // one thread
-    const int tile = u % p.ntile; u /= p.ntile;
-    const int k1 = u % p.N1, slab = p.slab0 + u / p.N1, b = slab / p.H, h = slab - b * p.H;
+  auto fetch = [&](int w) {                                                        // one thread
+    const int slab = p.slab0 + w / p.ntile, b = slab / p.H;
     mbar_expect_tx(bar, kRaw);
 #pragma unroll 1
-    for (int r = 0; r < P::M; r += kRows) tma_load_5d(smem_u32(rows) + r * 32, &map, 16 * tile, k1, r, h, b, bar);
+    for (int r = 0; r < P::M; r += kRows) tma_load_4d(smem_u32(rows) + r * 32, &map, 16 * (w % p.ntile), r, slab - b * p.H, b, bar);
   };
   if (threadIdx.x == 0) fetch(blockIdx.x);
   uint32_t par = 0;
   bool ok = true;
 #pragma unroll 1
   for (int w = blockIdx.x; w < ntotal; w += gridDim.x, par ^= 1) {
-    int u = w;
-    const int tile = u % p.ntile; u /= p.ntile;
-    const int k1 = u % p.N1; u /= p.N1;
-    const int slab_local = u, slab = p.slab0 + u, b = slab / p.H, h = slab - b * p.H;
-    const int pair = tile * P::C + pl.p;
-    const bool live = act && pair < half;
+    const int slab = p.slab0 + w / p.ntile, b = slab / p.H, h = slab - b * p.H;
+    const int pair = (w % p.ntile) * P::C + pl.p;
     float2 gv[kGv];                                                                // the tile's gates wait in registers for the table
-    if constexpr (MODE == kRegMix) {                                               // N1 = 1
-      const float2* g = p.g + (size_t)slab * p.K;
+    const float2* g = p.g + (size_t)slab * p.K;
 #pragma unroll
-      for (int i = 0; i < kGv; ++i) {
-        const int k = threadIdx.x + i * P::kThreads;
-        gv[i] = k < P::M ? __ldg(g + (2 * k <= P::M ? k : P::M - k)) : make_float2(0.f, 0.f);
-      }
+    for (int i = 0; i < kGv; ++i) {
+      const int k = threadIdx.x + i * P::kThreads;
+      gv[i] = k < P::M ? __ldg(g + (2 * k <= P::M ? k : P::M - k)) : make_float2(0.f, 0.f);
     }
     ok = mbar_wait(bar, par);
     float2 x[E];
-    {
-      raw v[E];
 #pragma unroll
-      for (int i = 0; i < E; ++i) v[i] = rows[(pl.m + P::S * i) * 8 + pl.p];
-      if (MODE == kRegForward && k1 < jrest && live && jfull % P::S == pl.m) {     // row jfull exists for this k1
-        const raw last = *reinterpret_cast<const raw*>(reinterpret_cast<const T*>(p.src) + b * p.s_sb + (int64_t)(jfull * p.N1 + k1) * p.s_sl +
-                                                       h * p.s_sh + 2 * pair);
+    for (int i = 0; i < E; ++i) x[i] = PairIo<T>::cvt(rows[(pl.m + P::S * i) * 8 + pl.p]);
+    if (__syncthreads_or(!ok)) break;
+    if (threadIdx.x == 0 && w + (int)gridDim.x < ntotal) fetch(w + gridDim.x);     // every thread has its rows: the buffer is free
+    pl.template forward<false>(x, buf, p.tw, act, [&] {
 #pragma unroll
-        for (int i = 0; i < E; ++i)
-          if (i == jfull / P::S) v[i] = last;
+      for (int i = 0; i < kGv; ++i) {
+        const int k = threadIdx.x + i * P::kThreads;
+        float2 v = cscale(gv[i], p.scale);
+        if (2 * k > P::M) v.y = -v.y;
+        if (k == 0 || 2 * k == P::M) v.y = 0.f;
+        if (k < P::M) gs[P::gate_slot(k)] = v;
       }
-      if (MODE == kRegForward && p.ring && live) {
-        T* out = reinterpret_cast<T*>(p.ring) + (((size_t)b * p.n + (pl.m * p.N1 + k1)) * p.H + h) * p.D + 2 * pair;
-        const size_t dr = (size_t)(P::S * p.N1) * p.H * p.D;
-#pragma unroll
-        for (int i = 0; i < E; ++i) __stcs(reinterpret_cast<raw*>(out + i * dr), v[i]);
-      }
-#pragma unroll
-      for (int i = 0; i < E; ++i) x[i] = PairIo<T>::cvt(v[i]);
-    }
-    if (__syncthreads_or(!ok)) break;                                              // also: the last tile's exchange has been read
-    pl.template forward<false>(
-        x, buf, p.tw, act,
-        [&] {
-          if constexpr (MODE == kRegMix) {
-#pragma unroll
-            for (int i = 0; i < kGv; ++i) {
-              const int k = threadIdx.x + i * P::kThreads;
-              float2 v = cscale(gv[i], p.scale);
-              if (2 * k > P::M) v.y = -v.y;
-              if (k == 0 || 2 * k == P::M) v.y = 0.f;
-              if (k < P::M) gs[P::gate_slot(k)] = v;
-            }
-          }
-        },
-        [&] {                                                                      // every thread has its rows: the buffer is free
-          if (threadIdx.x == 0 && w + (int)gridDim.x < ntotal) fetch(w + gridDim.x);
-        });
+    });
     settle(x);
-    if constexpr (MODE == kRegMix) {
 #pragma unroll
-      for (int i = 0; i < E; ++i) {
-        x[i] = cmul(x[i], gs[P::gate_slot(pl.bin(i))]);
-        if (i % 4 == 3) asm volatile("" ::: "memory");
-      }
-      settle(x);
-      pl.template inverse<false>(x, buf, p.tw, act);
-      char* base = reinterpret_cast<char*>(reinterpret_cast<T*>(p.dst) + b * p.d_sb + h * p.d_sh);
-      const int64_t ds = (int64_t)P::S * p.d_sl * (int64_t)sizeof(T);
-      const uint32_t mine = (uint32_t)((int64_t)pl.m * p.d_sl + 2 * pair) * (uint32_t)sizeof(T);
-      const int count = rows_below(p.L, pl.m, P::S, live);
-      if (count >= E) {
-#pragma unroll
-        for (int i = 0; i < E; ++i) *reinterpret_cast<raw*>(base + i * ds + mine) = PairIo<T>::pack(x[i]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < E; ++i)
-          if (i < count) *reinterpret_cast<raw*>(base + i * ds + mine) = PairIo<T>::pack(x[i]);
-      }
-    } else {
-      float2* out = p.ws + ((size_t)slab_local * p.N1 + k1) * P::M * half + pair;
-      if (live) {
-#pragma unroll
-        for (int i = 0; i < E; ++i) out[(size_t)pl.bin(i) * half] = x[i];
-      }
+    for (int i = 0; i < E; ++i) {
+      x[i] = cmul(x[i], gs[P::gate_slot(pl.bin(i))]);
+      if (i % 4 == 3) asm volatile("" ::: "memory");
     }
+    settle(x);
+    pl.template inverse<false>(x, buf, p.tw, act);
+    reg_store_tokens<T, P>(x, p, b, h, 2 * pair, pl.m, act && pair < p.D / 2);
   }
   if (!ok) {                                       // do not leave with copies in flight (bounded again)
     report_timeout(p.status);
@@ -621,25 +574,24 @@ static int reg_launch(RegParams p, int nslab, cudaStream_t st) {
   return SPECTRE_OK;
 }
 
-template <typename T, class P, int MODE>
+template <typename T, class P>
 static int reg_launch_stream(RegParams p, int nslab, cudaStream_t st, int sm_count, bool* done) {
-  constexpr size_t smem = reg_stream_bytes<P, MODE>();
+  constexpr size_t smem = reg_stream_bytes<P>();
   constexpr int fit = (int)(233472 / (smem + 1024)), resident = fit < reg_min_blocks<P>() ? fit : reg_min_blocks<P>();
   p.ntile = (p.D / 2 + P::C - 1) / P::C;
-  const long long total = (long long)nslab * p.N1 * p.ntile;
+  const long long total = (long long)nslab * p.ntile;
   *done = false;
-  if (total <= (long long)resident * sm_count || total > 0x7fffffff || p.L < p.N1 || !tensor_map_encoder()) return SPECTRE_OK;
+  if (total <= (long long)resident * sm_count || total > 0x7fffffff || !tensor_map_encoder()) return SPECTRE_OK;
   const cuuint64_t sl = (cuuint64_t)p.s_sl * 2, sh = (cuuint64_t)p.s_sh * 2, sb = (cuuint64_t)p.s_sb * 2;
-  const cuuint64_t dims[5] = {(cuuint64_t)p.D, (cuuint64_t)p.N1, (cuuint64_t)(p.L / p.N1), (cuuint64_t)p.H, (cuuint64_t)p.batch};
-  const cuuint64_t strides[4] = {sl, p.N1 * sl, sh, sb};
-  const cuuint32_t box[5] = {16, 1, (cuuint32_t)reg_box_rows<P>(), 1, 1}, es[5] = {1, 1, 1, 1, 1};
+  const cuuint64_t dims[4] = {(cuuint64_t)p.D, (cuuint64_t)p.L, (cuuint64_t)p.H, (cuuint64_t)p.batch}, strides[3] = {sl, sh, sb};
+  const cuuint32_t box[4] = {16, (cuuint32_t)reg_box_rows<P>(), 1, 1}, es[4] = {1, 1, 1, 1};
   CUtensorMap map;
   const CUresult r = tensor_map_encoder()(
-      &map, std::is_same<T, f16>::value ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(p.src), dims,
+      &map, std::is_same<T, f16>::value ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(p.src), dims,
       strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return SPECTRE_OK;                         // strides that a map cannot describe (a broadcast view)
-  auto kern = reg_stream_kernel<T, P, MODE>;
+  auto kern = reg_stream_kernel<T, P>;
   SPECTRE_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -667,13 +619,12 @@ static int reg_launch_tokens(const spectre_ctx* ctx, const RegParams& q, int M, 
   RegParams p = q;
   p.tw = reg_table(ctx, M);
   p.status = ctx->status_dev;
-  // Rows by TMA ahead of their tile where CTAs have more than one; not for the gradient, whose two tiles leave no room
-  constexpr bool kStream = sizeof(T) == 2 && (MODE == kRegMix || MODE == kRegForward);
+  constexpr bool kStream = sizeof(T) == 2 && MODE == kRegMix;      // rows by TMA ahead of their tile where CTAs have more than one
 #define SPECTRE_REG_CASE(R1, R2)                                                                     \
   case R1 * R2:                                                                                      \
     if constexpr (kStream) {                                                                         \
       bool done = false;                                                                             \
-      const int rc = reg_launch_stream<T, TwoStep<R1, R2, C>, MODE>(p, nslab, st, ctx->sm_count, &done); \
+      const int rc = reg_launch_stream<T, TwoStep<R1, R2, C>>(p, nslab, st, ctx->sm_count, &done); \
       if (rc != SPECTRE_OK || done) return rc;                                                       \
     }                                                                                                \
     return reg_launch<T, TwoStep<R1, R2, C>, MODE, false>(p, nslab, st);
