@@ -387,6 +387,7 @@ __global__ void __launch_bounds__(kXInThreads, 1) tc_in32_kernel(const __grid_co
 struct TcOut32Params {
   const unsigned char* mats;
   int H, slab0, cnt;
+  int rest;              // L % 4096: rows t' below it exist in one more block n1 than the others
   int* status;
 };
 
@@ -396,7 +397,8 @@ struct TcOut32Params {
 // R k1 x S pieces per lane group and tile), so an item covers 16 S values of t' and R output rows n1 for each.
 template <bool F16, int R>
 __global__ void __launch_bounds__(kXOutThreads, 1) tc_out32_kernel(const __grid_constant__ CUtensorMap tm_res,
-                                                                  const __grid_constant__ CUtensorMap tm_out, const TcOut32Params p) {
+                                                                  const __grid_constant__ CUtensorMap tm_out,
+                                                                  const __grid_constant__ CUtensorMap tm_rest, const TcOut32Params p) {
   constexpr int S = 32 / R;
   static_assert(R == 32 || R == 16 || R == 8 || R == 4 || R == 2, "radix");
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -457,8 +459,14 @@ __global__ void __launch_bounds__(kXOutThreads, 1) tc_out32_kernel(const __grid_
             const int e2 = 2 * S * blk + S * m + s, k4 = e2 >> 5, row = 2 * (e2 & 31);
             const int tp = 64 * row + 4 * k4;
             const uint32_t src = smem_u32(Stg) + 32768 * m + s * (8 * R * 128);
-            tma_store_5d(&tm_out, 0, 0, tp, h, b, src);
-            tma_store_5d(&tm_out, 0, 0, tp + 64, h, b, src + 4 * R * 128);
+            // L % 4096 != 0: tm_rest has the partial block too and ends at t' = rest, tm_out has the whole blocks only; a box
+            // that straddles the end goes through both (the whole blocks' rows are written twice, alike)
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+              const int t = tp + 64 * half;
+              if (t < p.rest) tma_store_5d(&tm_rest, 0, 0, t, h, b, src + half * 4 * R * 128);
+              if (t + 4 > p.rest) tma_store_5d(&tm_out, 0, 0, t, h, b, src + half * 4 * R * 128);
+            }
           }
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -523,22 +531,21 @@ __global__ void __launch_bounds__(kXOutThreads, 1) tc_out32_kernel(const __grid_
 }
 
 // ---- host side ---------------------------------------------------------------------------
-// Shapes the tensor-core transpose kernels take: n = 4096 R with R = 32, 16 or 8, 64 channels per head (one
-// 128-byte line per row and head), whole 4096-row blocks, 16-byte aligned strides.
-bool tc32_supported(const spectre_ctx* ctx, const spectre_act* v, const spectre_act* y, int n) {
-  auto ok = [](const spectre_act* a) {
-    return (reinterpret_cast<uintptr_t>(a->ptr) & 15) == 0 && a->stride_l % 8 == 0 && a->stride_h % 8 == 0 &&
-           a->stride_b % 8 == 0 && a->stride_l > 0 && a->stride_h > 0 && a->stride_b > 0;
-  };
-  return n >= 8192 && n <= 131072 && (n & (n - 1)) == 0 && v->D == 64 && v->L % 4096 == 0 && ok(v) && ok(y) && ctx->dft32 != nullptr &&
-         ctx->tw_staged != nullptr && tensor_map_encoder() != nullptr;
+// Shapes the tensor-core transpose kernels take: n = 4096 R with R = 32 ... 2, 64 channels per head (one 128-byte line per row
+// and head), 16-byte aligned strides.  In: whole 4096-row blocks (a box of rows cannot be filled from two maps).  Out: any
+// number of rows from one block up.
+static bool tc32_shape(const spectre_ctx* ctx, const spectre_act* a, int n) {
+  return n >= 8192 && n <= 131072 && (n & (n - 1)) == 0 && a->D == 64 && (reinterpret_cast<uintptr_t>(a->ptr) & 15) == 0 &&
+         a->stride_l % 8 == 0 && a->stride_h % 8 == 0 && a->stride_b % 8 == 0 && a->stride_l > 0 && a->stride_h > 0 && a->stride_b > 0 &&
+         ctx->dft32 != nullptr && ctx->tw_staged != nullptr && tensor_map_encoder() != nullptr;
 }
+bool tc32_in_supported(const spectre_ctx* ctx, const spectre_act* v, int n) { return tc32_shape(ctx, v, n) && v->L % 4096 == 0; }
+bool tc32_out_supported(const spectre_ctx* ctx, const spectre_act* y, int n) { return tc32_shape(ctx, y, n) && y->L >= 4096; }
 
-// dims (column, n1, t', head, batch) over [B, L, H, 64]: row = 4096 n1 + t'
-static int make_act_map(CUtensorMap* tm, const spectre_act* a, unsigned box_n1, unsigned box_tp) {
+// dims (column, n1, t', head, batch) over [B, L, H, 64]: row = 4096 n1 + t', n1 < nb, t' < rows
+static int make_act_map(CUtensorMap* tm, const spectre_act* a, int nb, int rows, unsigned box_n1, unsigned box_tp) {
   const cuuint64_t sl = (cuuint64_t)a->stride_l * 2, sh = (cuuint64_t)a->stride_h * 2, sb = (cuuint64_t)a->stride_b * 2;
-  const cuuint64_t nb = (cuuint64_t)(a->L / 4096);
-  cuuint64_t dims[5] = {64, nb, 4096, (cuuint64_t)a->H, (cuuint64_t)a->B};
+  cuuint64_t dims[5] = {64, (cuuint64_t)nb, (cuuint64_t)rows, (cuuint64_t)a->H, (cuuint64_t)a->B};
   cuuint64_t strides[4] = {4096 * sl, sl, sh, sb};
   cuuint32_t box[5] = {64, box_n1, box_tp, 1, 1};
   cuuint32_t es[5] = {1, 1, 1, 1, 1};
@@ -556,7 +563,7 @@ static int launch_tc_in_r(const spectre_ctx* ctx, cudaStream_t st, const spectre
                           unsigned char* ws_in, unsigned char* gimg, float* gscale, float sc) {
   constexpr int S = 32 / R;
   CUtensorMap tm;
-  int rc = make_act_map(&tm, v, R, S == 1 ? 2 : S);
+  int rc = make_act_map(&tm, v, v->L / 4096, 4096, R, S == 1 ? 2 : S);
   if (rc != SPECTRE_OK) return rc;
   CUtensorMap tm_img;
   {
@@ -610,8 +617,10 @@ int launch_tc_in32(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v
 template <int R>
 static int launch_tc_out_r(const spectre_ctx* ctx, cudaStream_t st, const unsigned char* ws_out, const spectre_act* y, int slab0, int cnt) {
   constexpr int S = 32 / R;
-  CUtensorMap tm_res, tm_out;
-  int rc = make_act_map(&tm_out, y, R, 4);
+  CUtensorMap tm_res, tm_out, tm_rest;
+  const int nb = y->L / 4096, rest = y->L % 4096;
+  int rc = make_act_map(&tm_out, y, nb, 4096, R, 4);
+  if (rc == SPECTRE_OK) rc = make_act_map(&tm_rest, y, rest ? nb + 1 : nb, rest ? rest : 4096, R, 4);
   if (rc != SPECTRE_OK) return rc;
   {
     // the units' results as fp16: (128-byte piece, k1, piece index within the unit, tile, slab of the group)
@@ -626,15 +635,15 @@ static int launch_tc_out_r(const spectre_ctx* ctx, cudaStream_t st, const unsign
   }
   TcOut32Params p = {};
   p.mats = reinterpret_cast<const unsigned char*>(ctx->dft32) + (size_t)radix_index(R) * 4 * kXMat;
-  p.H = y->H; p.slab0 = slab0; p.cnt = cnt; p.status = ctx->status_dev;
+  p.H = y->H; p.slab0 = slab0; p.cnt = cnt; p.rest = rest; p.status = ctx->status_dev;
   const int nitems = cnt * (256 / S);
   int grid = nitems < ctx->sm_count ? nitems : ctx->sm_count;
   if (y->dtype == SPECTRE_F16) {
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_out32_kernel<true, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXOutSmem));
-    tc_out32_kernel<true, R><<<grid, kXOutThreads, kXOutSmem, st>>>(tm_res, tm_out, p);
+    tc_out32_kernel<true, R><<<grid, kXOutThreads, kXOutSmem, st>>>(tm_res, tm_out, tm_rest, p);
   } else {
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_out32_kernel<false, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXOutSmem));
-    tc_out32_kernel<false, R><<<grid, kXOutThreads, kXOutSmem, st>>>(tm_res, tm_out, p);
+    tc_out32_kernel<false, R><<<grid, kXOutThreads, kXOutSmem, st>>>(tm_res, tm_out, tm_rest, p);
   }
   SPECTRE_LAUNCH_OK("tc_out32_kernel");
   return SPECTRE_OK;

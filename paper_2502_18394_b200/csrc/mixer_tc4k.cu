@@ -645,8 +645,9 @@ size_t tc4k_workspace_bytes(const spectre_ctx* ctx, int n, int D, int nslab) {
   return g * per;
 }
 
-// mixer_tc32.cu: the radix-32 steps on the tensor cores (n = 131072, d_head = 64)
-bool tc32_supported(const spectre_ctx* ctx, const spectre_act* v, const spectre_act* y, int n);
+// mixer_tc32.cu: the radix-32 ... 2 steps on the tensor cores (d_head = 64)
+bool tc32_in_supported(const spectre_ctx* ctx, const spectre_act* v, int n);
+bool tc32_out_supported(const spectre_ctx* ctx, const spectre_act* y, int n);
 int launch_tc_in32(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, int n, int slab0, int cnt,
                    unsigned char* ws_in, unsigned char* gimg, float* gscale, float sc);
 int launch_tc_out32(const spectre_ctx* ctx, cudaStream_t st, const unsigned char* ws_out, const spectre_act* y, int n, int slab0, int cnt);
@@ -661,10 +662,10 @@ static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
   unsigned char* gimg = ws_out + nunits * k4OutBytes;
   float* gscale = reinterpret_cast<float*>(gimg + (size_t)cnt * R * k4GBytes);
 
-  const bool tc32 = R >= 2 && tc32_supported(ctx, v, y, n);       // radix-32 ... 2 steps on the tensor cores
+  const bool tc32_in = R >= 2 && tc32_in_supported(ctx, v, n), tc32_out = R >= 2 && tc32_out_supported(ctx, y, n);   // radix-32 ... 2 steps on the tensor cores
   TcGateParams gp = {reinterpret_cast<const float2*>(g), gimg, gscale, n, n / 2 + 1, R, slab0};
 
-  if (tc32) {
+  if (tc32_in) {
     int rc = launch_tc_in32(ctx, st, v, g, n, slab0, cnt, ws_in, gimg, gscale, in_scale(R));
     if (rc != SPECTRE_OK) return rc;
   } else {
@@ -699,7 +700,7 @@ static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
   tc_core_kernel<<<grid, k4CoreThreads, k4CoreSmem, st>>>(cp);
   SPECTRE_LAUNCH_OK("tc_core_kernel");
 
-  if (tc32) return launch_tc_out32(ctx, st, ws_out, y, n, slab0, cnt);
+  if (tc32_out) return launch_tc_out32(ctx, st, ws_out, y, n, slab0, cnt);
   constexpr int NT = 512 / R;
   TcOutParams op = {ws_out, reinterpret_cast<bf16*>(y->ptr), y->stride_b, y->stride_l, y->stride_h,
                     y->H, D, y->L, n, ntile, slab0, ctx->status_dev};
@@ -786,7 +787,7 @@ static int tc4k_readout_group(const spectre_ctx* ctx, cudaStream_t st, const flo
   tc_core_kernel<<<grid, k4CoreThreads, k4CoreSmem, st>>>(cp);
   SPECTRE_LAUNCH_OK("tc_core_kernel");
 
-  if (R >= 2 && tc32_supported(ctx, y, y, n)) return launch_tc_out32(ctx, st, ws_out, y, n, slab0, cnt);
+  if (R >= 2 && tc32_out_supported(ctx, y, n)) return launch_tc_out32(ctx, st, ws_out, y, n, slab0, cnt);
   constexpr int NT = 512 / R;
   TcOutParams op = {ws_out, reinterpret_cast<bf16*>(y->ptr), y->stride_b, y->stride_l, y->stride_h,
                     y->H, D, y->L, n, ntile, slab0, ctx->status_dev};

@@ -170,6 +170,20 @@ def test_mixer_4096_single_kernel(ctx, dt, L, D, monkeypatch):
     assert bool((wide[:, L:] == 7.0).all())                       # nothing beyond row L is written
 
 
+@pytest.mark.parametrize("dt,n,L", [("bf16", 16384, 4097), ("f16", 32768, 20011), ("bf16", 65536, 50002), ("f16", 131072, 69640),
+                                    ("bf16", 16384, 12290)])
+def test_mixer_staged_ragged_rows(ctx, dt, n, L):
+    # a partial 4096-row block through the second tensor map; rows beyond L stay untouched
+    w = W.Workload("t", B=2, L=L, H=2, D=64, dtype=dt, n_fft=n, seed=n + L)
+    x, g = W.activations(w), W.random_gate(w)
+    wide = torch.full((2, L + 5, 2, 64), 7.0, dtype=x.dtype, device="cuda")
+    S.spectre_mixer_forward(ctx, x.cuda(), g.cuda(), y=wide[:, :L], n_fft=n)
+    torch.cuda.synchronize()
+    ctx.poll_status()
+    assert_close(W.to_f64(wide[:, :L]), O.mixer(W.to_f64(x), gate_to_complex(g), n_fft=n), dt)
+    assert bool((wide[:, L:] == 7.0).all())
+
+
 @pytest.mark.parametrize("L", [64, 4160, 8128])
 def test_mixer_bf16_8192_short_sequences_through_the_tensor_maps(ctx, L):
     # whole 64-row blocks shorter than n: rows beyond L read as zero and are not written;
