@@ -180,6 +180,7 @@ struct TcIn32Params {
   float* gscale;                // [slab_local * R + k1]
   int H, slab0, cnt, n, K;
   float sc;                     // forward scale of the radix-R step
+  int rest;              // L % 4096: rows t' below it exist in one more block n1 than the others
   int* status;
 };
 
@@ -197,8 +198,10 @@ __device__ __forceinline__ float2 gate_ext(const float2* __restrict__ g, int k, 
 // R n1 x S t' lands a lane group's 32 rows set by set), so an accumulator m covers 2 S consecutive t2 and a
 // store box row (tile, k1, pair) is a run of 32 S bytes (at most 256: R = 2 stores two boxes of 128).
 template <bool F16, int R>
-__global__ void __launch_bounds__(kXInThreads, 1) tc_in32_kernel(const __grid_constant__ CUtensorMap tm_in,
-                                                                 const __grid_constant__ CUtensorMap tm_img, const TcIn32Params p) {
+__global__ void __launch_bounds__(kXInThreads, 1) tc_in32_kernel(const __grid_constant__ CUtensorMap tm_in, const __grid_constant__ CUtensorMap tm_rest,
+                                                                const __grid_constant__ CUtensorMap tm_in1,
+                                                                const __grid_constant__ CUtensorMap tm_rest1,
+                                                                const __grid_constant__ CUtensorMap tm_img, const TcIn32Params p) {
   constexpr int S = 32 / R, T2B = 16 / S;                      // sets per lane group; t2 blocks (of 4 S) per unit row
   static_assert(R == 32 || R == 16 || R == 8 || R == 4 || R == 2, "radix");
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -244,13 +247,23 @@ __global__ void __launch_bounds__(kXInThreads, 1) tc_in32_kernel(const __grid_co
     ok = load_warp_loop(bar, nitems, T, ok, [&](int item, int m, int slot) {
       const int slab = p.slab0 + item / (16 * T2B), a = (item / T2B) & 15, t2b = item % T2B;
       const int b = slab / p.H, h = slab - b * p.H;
+      constexpr int TB = S == 1 ? 2 : S;           // t' of a box
+      // L % 4096 != 0: tm_rest has the partial block n1 too and serves the t' below rest, tm_in the whole blocks; the box in
+      // which the partial block ends is loaded one t' at a time (R rows of 128 bytes: whole swizzle atoms from R = 8 on)
+      auto box = [&](uint32_t dst, int t) {
+        if (t < p.rest && t + TB > p.rest) {
+          for (int l = 0; l < TB; ++l)
+            tma_load_5d(dst + l * R * 128, t + l < p.rest ? &tm_rest1 : &tm_in1, 0, 0, t + l, h, b, bar.slotFull(slot));
+        } else {
+          tma_load_5d(dst, t < p.rest ? &tm_rest : &tm_in, 0, 0, t, h, b, bar.slotFull(slot));
+        }
+      };
       for (int u = 0; u < 4; ++u) {
         const int tp = 64 * (4 * a + u) + 4 * S * t2b + 2 * S * m;
         if (S == 1) {
-          tma_load_5d(smem_u32(Op) + slot * kXHalfOp + u * 2 * kXBox, &tm_in, 0, 0, tp, h, b, bar.slotFull(slot));
+          box(smem_u32(Op) + slot * kXHalfOp + u * 2 * kXBox, tp);
         } else {
-          for (int gq = 0; gq < 2; ++gq)
-            tma_load_5d(smem_u32(Op) + slot * kXHalfOp + (u * 2 + gq) * kXBox, &tm_in, 0, 0, tp + S * gq, h, b, bar.slotFull(slot));
+          for (int gq = 0; gq < 2; ++gq) box(smem_u32(Op) + slot * kXHalfOp + (u * 2 + gq) * kXBox, tp + S * gq);
         }
       }
     });
@@ -532,14 +545,17 @@ __global__ void __launch_bounds__(kXOutThreads, 1) tc_out32_kernel(const __grid_
 
 // ---- host side ---------------------------------------------------------------------------
 // Shapes the tensor-core transpose kernels take: n = 4096 R with R = 32 ... 2, 64 channels per head (one 128-byte line per row
-// and head), 16-byte aligned strides.  In: whole 4096-row blocks (a box of rows cannot be filled from two maps).  Out: any
-// number of rows from one block up.
+// and head), 16-byte aligned strides, any number of rows from one 4096-row block up; below R = 8 the partial block has to end
+// with a box on the way in (32 / R rows).
 static bool tc32_shape(const spectre_ctx* ctx, const spectre_act* a, int n) {
   return n >= 8192 && n <= 131072 && (n & (n - 1)) == 0 && a->D == 64 && (reinterpret_cast<uintptr_t>(a->ptr) & 15) == 0 &&
          a->stride_l % 8 == 0 && a->stride_h % 8 == 0 && a->stride_b % 8 == 0 && a->stride_l > 0 && a->stride_h > 0 && a->stride_b > 0 &&
          ctx->dft32 != nullptr && ctx->tw_staged != nullptr && tensor_map_encoder() != nullptr;
 }
-bool tc32_in_supported(const spectre_ctx* ctx, const spectre_act* v, int n) { return tc32_shape(ctx, v, n) && v->L % 4096 == 0; }
+bool tc32_in_supported(const spectre_ctx* ctx, const spectre_act* v, int n) { 
+  const int R = n / 4096;
+  return tc32_shape(ctx, v, n) && v->L >= 4096 && (R >= 8 || v->L % 4096 % (32 / R) == 0);
+}
 bool tc32_out_supported(const spectre_ctx* ctx, const spectre_act* y, int n) { return tc32_shape(ctx, y, n) && y->L >= 4096; }
 
 // dims (column, n1, t', head, batch) over [B, L, H, 64]: row = 4096 n1 + t', n1 < nb, t' < rows
@@ -562,8 +578,16 @@ template <int R>
 static int launch_tc_in_r(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, int n, int slab0, int cnt,
                           unsigned char* ws_in, unsigned char* gimg, float* gscale, float sc) {
   constexpr int S = 32 / R;
-  CUtensorMap tm;
-  int rc = make_act_map(&tm, v, v->L / 4096, 4096, R, S == 1 ? 2 : S);
+  constexpr int TB = S == 1 ? 2 : S;
+  CUtensorMap tm, tm_rest, tm1, tm_rest1;
+  const int nb = v->L / 4096, rest = v->L % 4096;
+  int rc = make_act_map(&tm, v, nb, 4096, R, TB);
+  tm_rest = tm1 = tm_rest1 = tm;
+  if (rest) {
+    if (rc == SPECTRE_OK) rc = make_act_map(&tm_rest, v, nb + 1, rest, R, TB);
+    if (rc == SPECTRE_OK) rc = make_act_map(&tm1, v, nb, 4096, R, 1);
+    if (rc == SPECTRE_OK) rc = make_act_map(&tm_rest1, v, nb + 1, rest, R, 1);
+  }
   if (rc != SPECTRE_OK) return rc;
   CUtensorMap tm_img;
   {
@@ -581,7 +605,7 @@ static int launch_tc_in_r(const spectre_ctx* ctx, cudaStream_t st, const spectre
   p.mats = reinterpret_cast<const unsigned char*>(ctx->dft32) + (size_t)radix_index(R) * 4 * kXMat;
   p.twr = reinterpret_cast<const float2*>(ctx->tw_staged) + (size_t)(R - 1) * 128;
   p.ws_in = ws_in; p.g = reinterpret_cast<const float2*>(g); p.gimg = gimg; p.gscale = gscale;
-  p.H = v->H; p.slab0 = slab0; p.cnt = cnt; p.n = n; p.K = n / 2 + 1; p.sc = sc;
+  p.H = v->H; p.slab0 = slab0; p.cnt = cnt; p.n = n; p.K = n / 2 + 1; p.sc = sc; p.rest = rest;
   p.status = ctx->status_dev;
   const int nitems = cnt * (256 / S);
   int grid = nitems < ctx->sm_count ? nitems : ctx->sm_count;
@@ -593,10 +617,10 @@ static int launch_tc_in_r(const spectre_ctx* ctx, cudaStream_t st, const spectre
   cfg.attrs = attr; cfg.numAttrs = 1;
   if (v->dtype == SPECTRE_F16) {
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_in32_kernel<true, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXInSmem));
-    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, tc_in32_kernel<true, R>, tm, tm_img, p));
+    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, tc_in32_kernel<true, R>, tm, tm_rest, tm1, tm_rest1, tm_img, p));
   } else {
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_in32_kernel<false, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXInSmem));
-    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, tc_in32_kernel<false, R>, tm, tm_img, p));
+    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, tc_in32_kernel<false, R>, tm, tm_rest, tm1, tm_rest1, tm_img, p));
   }
   SPECTRE_LAUNCH_OK("tc_in32_kernel");
   return SPECTRE_OK;
