@@ -7,6 +7,7 @@
 // column pairs that uses  conj(A^V) A^G + conj(B^V) B^G = ( conj(Z^V_k) Z^G_k + Z^V_{n-k} conj(Z^G_{n-k}) ) / 2.
 // Beyond one CTA's 2048 rows the passes leave the spectra of the N1 decimated sequences and the reduction
 // runs the last radix-N1 step itself.
+#include "fft_reg.cuh"
 #include "reg_fft.h"
 
 namespace spectre {
@@ -74,108 +75,82 @@ __global__ void __launch_bounds__(256) gate_grad_kernel(const float2* __restrict
 
 // Longer transforms, n = N1 M with token t = N1 n2 + n1: the workspaces hold Y[n1][k2], the M-point spectra of
 // the N1 decimated sequences (ws[slab_local][n1][k2][D/2]), and Z[k2 + M k1] = sum_n1 W_N1^{n1 k1} W_n^{n1 k2} Y[n1][k2].
-// A warp (or half of one) per (slab, k2 <= M/2): it forms Z at k2 + M k1 and at (M - k2) + M k1 for both tensors — each
-// family holds the mirror bins n - k of the other — and reduces the N1 (+1 at k2 = 0) bins k <= n/2 among them.
-// KW bins k2 per warp, 32 / KW lanes each; a lane takes KW adjacent column pairs per load (KW = 2: 16-byte loads).
-template <int N1, int KW>
-__device__ __forceinline__ void combine_bins(const float2* __restrict__ ws, size_t row0, int M, int half, int c, int k2,
-                                             int m2, const float2 (&wa)[N1], const float2 (&wb)[N1], float2 (&a)[KW][N1],
-                                             float2 (&b)[KW][N1]) {
-#pragma unroll
-  for (int n1 = 0; n1 < N1; ++n1) {
-    const float2* pa = ws + (row0 + (size_t)n1 * M + k2) * half + c;
-    const float2* pb = ws + (row0 + (size_t)n1 * M + m2) * half + c;
-    if (KW == 2) {
-      const float4 ta = *reinterpret_cast<const float4*>(pa), tb = *reinterpret_cast<const float4*>(pb);
-      a[0][n1] = make_float2(ta.x, ta.y); a[KW - 1][n1] = make_float2(ta.z, ta.w);
-      b[0][n1] = make_float2(tb.x, tb.y); b[KW - 1][n1] = make_float2(tb.z, tb.w);
-    } else {
-      a[0][n1] = *pa;
-      b[0][n1] = *pb;
-    }
-  }
-#pragma unroll
-  for (int v = 0; v < KW; ++v) {
-#pragma unroll
-    for (int q = 1; q < N1; ++q) {
-      a[v][q] = cmul(a[v][q], wa[q]);
-      b[v][q] = cmul(b[v][q], wb[q]);
-    }
-    Dft<N1, false>::run(a[v]);
-    Dft<N1, false>::run(b[v]);
-  }
-}
-
-template <int N1, int KW>
-__global__ void __launch_bounds__(256) gate_grad_combine_kernel(const float2* __restrict__ wsV, const float2* __restrict__ wsG,
+// A warp per (slab, k2 <= M/2).  Lanes 0-15 form Z of both tensors at k2 + M k1, lanes 16-31 at m2 + M k1, m2 = M - k2: each
+// family holds the mirror bins n - k of the other.  A lane takes two column pairs (16-byte loads), sums
+// S[k1] = conj(Z^V) Z^G over its pairs, the half-warp over its lanes, and dg_k = (w_k / 2n)(S_k + conj(S_{n-k})) takes one
+// exchange between the halves.  Bound by HBM; with both families and tensors in one lane (256 registers of spectra at
+// N1 = 8) the pass over 134 MB took 43 us.
+template <int N1>
+__global__ void __launch_bounds__(256, N1 <= 8 ? 2 : 1) gate_grad_combine_kernel(const float2* __restrict__ wsV, const float2* __restrict__ wsG,
                                                                 float2* __restrict__ dg, int n, int K, int D, int M,
                                                                 int slab0, int nslab) {
-  constexpr int LPK = 32 / KW;
   const size_t wid = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31, sub = lane % LPK;
-  const int nk2 = M / 2 + 1, wpk = (nk2 + KW - 1) / KW;      // warps per slab
-  if (wid >= (size_t)nslab * wpk) return;
-  const int slab_local = (int)(wid / wpk);
-  const int k2raw = (int)(wid % wpk) * KW + lane / LPK;
-  const bool valid = k2raw < nk2;                               // the last warp of a slab may own one bin only
-  const int k2 = valid ? k2raw : 0;
-  const int m2 = (M - k2) % M;
-  const int half = D / 2;
-  const bool own = k2 == 0 || k2 == m2;        // k2 = 0 and k2 = M/2 are their own mirror
-  float2 wa[N1], wb[N1];
-  wa[0] = wb[0] = make_float2(1.f, 0.f);
+  const int lane = threadIdx.x & 31, sub = lane & 15, s = sub % N1;
+  const int nk2 = M / 2 + 1, half = D / 2;
+  if (wid >= (size_t)nslab * nk2) return;
+  const int slab_local = (int)(wid / nk2), k2 = (int)(wid % nk2), m2 = (M - k2) % M;
+  const int mine = lane < 16 ? k2 : m2;
+  float2 w[N1];
+  w[0] = make_float2(1.f, 0.f);
 #pragma unroll
-  for (int q = 1; q < N1; ++q) {
-    wa[q] = (q == 1) ? twiddle_fwd((unsigned)k2, (unsigned)n) : cmul(wa[q / 2], wa[q - q / 2]);
-    wb[q] = (q == 1) ? twiddle_fwd((unsigned)m2, (unsigned)n) : cmul(wb[q / 2], wb[q - q / 2]);
-  }
-  float2 acc1[N1 / 2], acc2[N1 / 2], accn = make_float2(0.f, 0.f);
+  for (int q = 1; q < N1; ++q) w[q] = (q == 1) ? twiddle_fwd((unsigned)mine, (unsigned)n) : cmul(w[q / 2], w[q - q / 2]);
+  const size_t row0 = (size_t)slab_local * N1 * M + mine;
+  float2 acc[N1];
 #pragma unroll
-  for (int k1 = 0; k1 < N1 / 2; ++k1) acc1[k1] = acc2[k1] = make_float2(0.f, 0.f);
-  const size_t row0 = (size_t)slab_local * N1 * M;
-  for (int c = KW * sub; c < half; c += KW * LPK) {
-    float2 va[KW][N1], vb[KW][N1], ga[KW][N1], gb[KW][N1];
-    combine_bins<N1, KW>(wsV, row0, M, half, c, k2, m2, wa, wb, va, vb);
-    combine_bins<N1, KW>(wsG, row0, M, half, c, k2, m2, wa, wb, ga, gb);
+  for (int k1 = 0; k1 < N1; ++k1) acc[k1] = make_float2(0.f, 0.f);
+  for (int c = 2 * sub; c < half; c += 32) {                   // D is a multiple of 8: whole 16-byte pieces
+    float2 v[2][N1], g[2][N1];
 #pragma unroll
-    for (int v = 0; v < KW; ++v) {
+    for (int n1 = 0; n1 < N1; ++n1) {
+      const size_t at = (row0 + (size_t)n1 * M) * half + c;
+      const float4 tv = __ldcs(reinterpret_cast<const float4*>(wsV + at)), tg = __ldcs(reinterpret_cast<const float4*>(wsG + at));
+      v[0][n1] = make_float2(tv.x, tv.y); v[1][n1] = make_float2(tv.z, tv.w);
+      g[0][n1] = make_float2(tg.x, tg.y); g[1][n1] = make_float2(tg.z, tg.w);
+    }
 #pragma unroll
-      for (int k1 = 0; k1 < N1 / 2; ++k1) {
-        // bin k2 + M k1; its mirror is (N1 - k1) % N1 of the same family at k2 = 0, else N1 - 1 - k1 of the other
-        const float2 vm = k2 == 0 ? va[v][(N1 - k1) % N1] : vb[v][N1 - 1 - k1];
-        const float2 gm = k2 == 0 ? ga[v][(N1 - k1) % N1] : gb[v][N1 - 1 - k1];
-        acc1[k1] = cadd(acc1[k1], cadd(cmulc(ga[v][k1], va[v][k1]), cmulc(vm, gm)));
-        // bin (M - k2) + M k1, mirror N1 - 1 - k1 of the first family
-        acc2[k1] = cadd(acc2[k1], cadd(cmulc(gb[v][k1], vb[v][k1]), cmulc(va[v][N1 - 1 - k1], ga[v][N1 - 1 - k1])));
+    for (int i = 0; i < 2; ++i) {
+#pragma unroll
+      for (int q = 1; q < N1; ++q) {
+        v[i][q] = cmul(v[i][q], w[q]);
+        g[i][q] = cmul(g[i][q], w[q]);
       }
-      // bin n/2 (k2 = 0 only), its own mirror
-      accn = cadd(accn, cadd(cmulc(ga[v][N1 / 2], va[v][N1 / 2]), cmulc(va[v][N1 / 2], ga[v][N1 / 2])));
+      RegDft<N1, false>::run(v[i]);
+      RegDft<N1, false>::run(g[i]);
+#pragma unroll
+      for (int k1 = 0; k1 < N1; ++k1) acc[k1] = cadd(acc[k1], cmulc(g[i][k1], v[i][k1]));
     }
   }
-  float2* out = dg + (size_t)(slab0 + slab_local) * K;
-  const float w2 = 1.0f / (float)n, w1 = 0.5f / (float)n;      // bins other than 0 and n/2 count twice
+  // lane s of the half-warp: the sum of value s over its 16 lanes
 #pragma unroll
-  for (int k1 = 0; k1 <= N1; ++k1) {
-    float2 v = k1 < N1 / 2 ? acc1[k1 % (N1 / 2)] : (k1 < N1 ? acc2[k1 % (N1 / 2)] : accn);
+  for (int h = N1 / 2; h >= 1; h >>= 1) {
+    const bool up = s & h;
 #pragma unroll
-    for (int o = LPK / 2; o > 0; o >>= 1) {
-      v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-      v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    for (int i = 0; i < h; ++i) {
+      const float2 send = up ? acc[i] : acc[i + h], keep = up ? acc[i + h] : acc[i];
+      acc[i] = make_float2(keep.x + __shfl_xor_sync(0xffffffffu, send.x, h), keep.y + __shfl_xor_sync(0xffffffffu, send.y, h));
     }
-    if (sub == 0 && valid) {
-      if (k1 < N1 / 2) out[k2 + M * k1] = cscale(v, (k2 == 0 && k1 == 0) ? w1 : w2);
-      else if (k1 < N1) { if (!own) out[m2 + M * (k1 - N1 / 2)] = cscale(v, w2); }
-      else if (k2 == 0) out[M * (N1 / 2)] = cscale(v, w1);
-    }
+  }
+#pragma unroll
+  for (int h = N1; h < 16; h <<= 1) {
+    acc[0].x += __shfl_xor_sync(0xffffffffu, acc[0].x, h);
+    acc[0].y += __shfl_xor_sync(0xffffffffu, acc[0].y, h);
+  }
+  // the mirror of bin s of a family is bin N1 - 1 - s of the other, at k2 = 0 bin (N1 - s) % N1 of the same one
+  const int from = k2 == 0 ? (N1 - s) % N1 : (lane ^ 16) - s + (N1 - 1 - s);
+  const float mx = __shfl_sync(0xffffffffu, acc[0].x, from), my = __shfl_sync(0xffffffffu, acc[0].y, from);
+  const int k = mine + M * s;
+  const bool write = sub < N1 && (k2 == 0 ? lane < 16 && s <= N1 / 2 : s < N1 / 2 && (lane < 16 || k2 != m2));
+  if (write) {
+    const float wt = ((k == 0 || 2 * k == n) ? 0.5f : 1.0f) / (float)n;      // bins other than 0 and n/2 count twice
+    dg[(size_t)(slab0 + slab_local) * K + k] = make_float2((acc[0].x + mx) * wt, (acc[0].y - my) * wt);
   }
 }
 
 template <int N1>
 static void launch_gate_grad_combine(cudaStream_t st, const float2* wsV, const float2* wsG, float2* dg, int n, int K, int D,
                                      int M, int slab0, int cnt) {
-  constexpr int KW = N1 <= 8 ? 2 : 1;
-  const size_t nwarps = (size_t)cnt * ((M / 2 + 1 + KW - 1) / KW);
-  gate_grad_combine_kernel<N1, KW><<<(unsigned)((nwarps * 32 + 255) / 256), 256, 0, st>>>(wsV, wsG, dg, n, K, D, M, slab0, cnt);
+  const size_t nwarps = (size_t)cnt * (M / 2 + 1);
+  gate_grad_combine_kernel<N1><<<(unsigned)((nwarps * 32 + 255) / 256), 256, 0, st>>>(wsV, wsG, dg, n, K, D, M, slab0, cnt);
 }
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
