@@ -9,7 +9,6 @@ int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
                       float2* ws, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done);
 bool transform_supported(const spectre_ctx* ctx, int n);
 size_t transform_slab_bytes(int n, int D);
-int pool_sum(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* q, float* sums, int ncopy_max, int* ncopy_used);
 int pool_sum_ring(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* q, float* sums, void* ring, int N);
 size_t gate_min_workspace(int B, int H, int D, int n_fft, int r);
 size_t inverse_workspace_bytes(const spectre_ctx* ctx, int n, int D, int nslab);

@@ -77,13 +77,19 @@ template <> struct vec8<float> {
 template <typename T, bool RING>
 __global__ void __launch_bounds__(256, 4) pool_kernel(const T* __restrict__ q, int64_t sb, int64_t sl, int64_t sh, int L,
                                                    int H, int D, int rows_per, int ncopy, size_t copy_stride,
-                                                   float* __restrict__ sums, T* __restrict__ ring, int N) {
+                                                   float* __restrict__ sums, T* __restrict__ ring, int N,
+                                                   const char* __restrict__ warm, unsigned warm_per, size_t warm_bytes) {
   __shared__ float red[8][8][32];                              // [warp][channel][lane]
   // the gate kernels behind this one may start early: they stream weights before they need the sums
   asm volatile("griddepcontrol.launch_dependents;");
   constexpr int R = vec8<T>::kRows;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.z;
+  if (warm_per && threadIdx.x == 0) {                          // this CTA's part of the weights that the gate kernel reads next
+    const size_t at = (size_t)((b * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * warm_per;
+    if (at < warm_bytes)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(warm + at), "r"((unsigned)min((size_t)warm_per, warm_bytes - at)) : "memory");
+  }
   const int vec_per_head = D / 8, nvec = H * vec_per_head;
   const int vi = blockIdx.x * 32 + lane;
   const bool live = vi < nvec;
@@ -132,7 +138,7 @@ __global__ void __launch_bounds__(256) pool_clear_kernel(float4* __restrict__ su
 // Sums of q over the sequence into *ncopy_used <= ncopy_max partial copies (the consumer adds them up);
 // with `ring`, also the copy of q into ring[B][N][H][D] (zero rows from L on).
 static int pool_launch(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* q, float* sums, int ncopy_max,
-                       int* ncopy_used, void* ring, int N) {
+                       int* ncopy_used, void* ring, int N, const void* warm, size_t warm_bytes) {
   const int rows = ring ? N : q->L;
   const size_t copy_stride = (size_t)q->B * q->H * q->D;
   const int groups = (q->H * (q->D / 8) + 31) / 32;
@@ -172,28 +178,35 @@ static int pool_launch(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
       cfg.numAttrs = 1;
     }
   }
+  // Whole 16-byte pieces of `warm` per CTA into L2 on the side
+  const char* w0 = reinterpret_cast<const char*>((reinterpret_cast<uintptr_t>(warm) + 15) & ~(uintptr_t)15);
+  size_t wb = 0;
+  if (warm && warm_bytes >= 32) wb = (warm_bytes - (size_t)(w0 - reinterpret_cast<const char*>(warm))) & ~(size_t)15;
+  const size_t ctas = (size_t)groups * nslice * q->B;
+  const unsigned wper = (unsigned)(wb ? ((wb + ctas - 1) / ctas + 15) & ~(size_t)15 : 0);
   SPECTRE_IO_DISPATCH(q->dtype, {
     if (ring)
       SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, pool_kernel<T, true>, reinterpret_cast<const T*>(q->ptr), (int64_t)q->stride_b,
                                          (int64_t)q->stride_l, (int64_t)q->stride_h, (int)q->L, (int)q->H, (int)q->D, rows_per,
-                                         ncopy, copy_stride, sums, reinterpret_cast<T*>(ring), N));
+                                         ncopy, copy_stride, sums, reinterpret_cast<T*>(ring), N, w0, wper, wb));
     else
       SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, pool_kernel<T, false>, reinterpret_cast<const T*>(q->ptr), (int64_t)q->stride_b,
                                          (int64_t)q->stride_l, (int64_t)q->stride_h, (int)q->L, (int)q->H, (int)q->D, rows_per,
-                                         ncopy, copy_stride, sums, static_cast<T*>(nullptr), 0));
+                                         ncopy, copy_stride, sums, static_cast<T*>(nullptr), 0, w0, wper, wb));
   });
   SPECTRE_LAUNCH_OK("pool_kernel");
   return SPECTRE_OK;
 }
 
-int pool_sum(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* q, float* sums, int ncopy_max, int* ncopy_used) {
-  return pool_launch(ctx, st, q, sums, ncopy_max, ncopy_used, nullptr, 0);
+int pool_sum(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* q, float* sums, int ncopy_max, int* ncopy_used,
+             const void* warm, size_t warm_bytes) {
+  return pool_launch(ctx, st, q, sums, ncopy_max, ncopy_used, nullptr, 0, warm, warm_bytes);
 }
 
 // Prefill of the cache's query side in one pass over q: sum over the sequence into sums[B,H,D] and the ring copy.
 int pool_sum_ring(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* q, float* sums, void* ring, int N) {
   int used = 1;
-  return pool_launch(ctx, st, q, sums, 1, &used, ring, N);
+  return pool_launch(ctx, st, q, sums, 1, &used, ring, N, nullptr, 0);
 }
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -870,7 +883,11 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
     float* pooled = reinterpret_cast<float*>(reinterpret_cast<char*>(workspace) + sums_off);
     const size_t one_copy = (size_t)B * H * D * sizeof(float);
     size_t fit = (workspace_bytes - sums_off) / one_copy;
-    int rc = pool_sum(ctx, st, q, pooled, fit > (size_t)kPoolCopies ? kPoolCopies : (int)fit, &ncopy);
+    const size_t w2 = (size_t)(gp->shared_across_heads ? 1 : H) * gp->hidden * 2 * K * (gp->wdtype == SPECTRE_BF16 ? 2 : 4);
+    // Small weights are brought into L2 by the pooling pass: the gate kernel's chain of loads is latency then (2 heads, n = 1024:
+    // gate call 16.6 -> 15.4 us; 8 heads, n = 4096: 16.8 -> 16.2).  Larger ones take the pass's own bandwidth for no gain
+    // (8k: 21.9 -> 23.6 us).
+    int rc = pool_sum(ctx, st, q, pooled, fit > (size_t)kPoolCopies ? kPoolCopies : (int)fit, &ncopy, gp->W2, w2 <= ((size_t)4 << 20) ? w2 : 0);
     if (rc != SPECTRE_OK) return rc;
     sums = pooled;
   }
