@@ -66,6 +66,12 @@ def pool_launches(B, rows, H, D, sm_count=148):
     return 1 + (1 if -(-rows // rows_per) > 1 else 0)
 
 
+def gate_launches(w):
+    """Kernels of the gate's MLP: one, and the hidden layer's own when a single sequence's bins span >= 32 CTAs."""
+    batched = w.B >= 2 and w.wdtype == "bf16" and w.hidden == 64 and w.K >= 256
+    return 1 + (1 if not batched and (w.K + 255) // 256 >= 32 else 0)
+
+
 def measured_peak():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     try:
@@ -230,12 +236,12 @@ class MixerBench:
         elif ws_mix:
             per = w.n * (w.D // 2) * 8
             groups = math.ceil(w.B * w.H / max(1, ws_mix // per))
-            self.kernel_name, nk = "mixer (strided + onchip + strided per group)", 3 * groups
+            self.kernel_name, nk = "mixer (strided + register-resident + strided per group)", 3 * groups
         else:
-            self.kernel_name, nk = "mixer (onchip_kernel)", 1
+            self.kernel_name, nk = "mixer (register-resident fp32 kernel)", 1
         # pool (+ the kernel that clears its partial sums when it runs in several slices), gate_out (+ gate_hidden when a
         # head's bins span >= 32 CTAs), mixer kernels, wavelet
-        self.launches_per_step = (pool_launches(w.B, w.L, w.H, w.D) + 1 + (1 if (w.K + 255) // 256 >= 32 else 0) + nk +
+        self.launches_per_step = (pool_launches(w.B, w.L, w.H, w.D) + gate_launches(w) + nk +
                                   (1 if w.wavelet_levels and not fused_wrm else 0))
         self.h2d = w.B * w.L * w.H * w.D * (4 if w.dtype == "f32" else 2)
         self.d2h = self.h2d
@@ -252,7 +258,8 @@ class MixerBench:
             per = w.n * (w.D // 2) * 8
             gb = math.ceil(w.B * w.H / max(1, min(w.B * w.H, (128 << 20) // per)))
             # conjugate gate + forward kernels on dY; per group of heads two forward-only transforms and the reduction
-            self.launches_per_step += 1 + nk + gb * 3
+            # (a length one CTA transforms: one kernel for both gradients, and the sum of its partial gate gradients)
+            self.launches_per_step += 2 if w.n <= 2048 else 1 + nk + gb * 3
 
     def step(self, k: int, e0=None, e1=None):
         d = self.sets[k % self.nsets]
@@ -418,7 +425,7 @@ class AppendBench:
             wbytes = 2 if w.wdtype == "bf16" else 4
             self.alg_bytes += w.H * w.hidden * 2 * K * wbytes + 2 * w.B * w.H * K * 8   # + W2 stream, gate write + read
             self.kernel_name = "decode step (decode_spectrum_kernel dominant)"
-            self.launches_per_step = 5      # ring, gate_hidden, gate_out, decode_spectrum, decode_reduce
+            self.launches_per_step = 2 + gate_launches(W.scaled(w, n_fft=N))      # ring, gate, decode_spectrum
             self.d2h = w.B * w.H * w.D * es
 
     def _call(self, k):
