@@ -280,20 +280,24 @@ __device__ __forceinline__ void descriptor_and_hidden(const float* __restrict__ 
     }
   }
   __syncthreads();
-  for (int bb = warp; bb < nb; bb += nw) {                    // statistics: one warp per batch entry
-    float* qb = qbar + bb * D;
+  const int lw = NB > 1 && nb > nw ? 16 : 32, per = 32 / lw;   // statistics: a warp per batch entry, half a one where warps are fewer
+  const int sl = lane & (lw - 1);
+  for (int b0 = 0; b0 < nb; b0 += per * nw) {                  // every lane takes part in the shuffles
+    const int bb = b0 + per * warp + lane / lw;
+    float* qb = qbar + (bb < nb ? bb : 0) * D;
     float part = 0.f;
-    for (int c = lane; c < D; c += 32) part += qb[c];
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    for (int c = sl; c < D; c += lw) part += qb[c];
+    for (int o = lw / 2; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
     const float mean = part / (float)D;
     part = 0.f;
-    for (int c = lane; c < D; c += 32) {
+    for (int c = sl; c < D; c += lw) {
       float dlt = qb[c] - mean;
       part += dlt * dlt;
     }
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    for (int o = lw / 2; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
     const float rstd = 1.0f / sqrtf(part / (float)D + eps);
-    for (int c = lane; c < D; c += 32) qb[c] = gamma[c] * (qb[c] - mean) * rstd + beta[c];
+    if (bb < nb)
+      for (int c = sl; c < D; c += lw) qb[c] = gamma[c] * (qb[c] - mean) * rstd + beta[c];
   }
   __syncthreads();
   if constexpr (NB == 1) {
@@ -330,8 +334,21 @@ __device__ __forceinline__ void descriptor_and_hidden(const float* __restrict__ 
         const int bb = gi + sl * groups;
         if (bb < nb) {
           const float* qb = qbar + bb * D + c;
+          if (NB >= 4 && D % 4 == 0) {              // rows of q_bar start on 16 bytes: four inputs per broadcast, two per packed sum
+            uint64_t a2 = pk2(acc[sl], 0.f);
 #pragma unroll
-          for (int i = 0; i < 32; ++i) acc[sl] = fmaf(qb[i], wv[i], acc[sl]);
+            for (int i = 0; i < 32; i += 4) {
+              const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(qb + i);
+              a2 = fma2(t.x, pk2(wv[i], wv[i + 1]), a2);
+              a2 = fma2(t.y, pk2(wv[i + 2], wv[i + 3]), a2);
+            }
+            float lo, hi;
+            upk2(a2, lo, hi);
+            acc[sl] = lo + hi;
+          } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) acc[sl] = fmaf(qb[i], wv[i], acc[sl]);
+          }
         }
       }
     }
@@ -365,6 +382,24 @@ __device__ __forceinline__ void stage_weights(const void* src, void* dst, int by
     d4[i0] = v0;
     if (i1 < n16) d4[i1] = v1;
   }
+}
+
+// 16-byte asynchronous copies into shared memory; the caller commits and waits
+__device__ __forceinline__ void copy_async16(const void* src, void* dst, int bytes) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  for (int i = 16 * (int)threadIdx.x; i < bytes; i += 16 * (int)blockDim.x)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(d + i), "l"(reinterpret_cast<const char*>(src) + i) : "memory");
+}
+__device__ __forceinline__ void stage_vectors(const float* gamma, const float* beta, const float* b1, int D, int hidden, float* vec) {
+  for (int i = threadIdx.x; i < D; i += blockDim.x) { vec[i] = __ldg(gamma + i); vec[D + i] = __ldg(beta + i); }
+  for (int i = threadIdx.x; i < hidden; i += blockDim.x) vec[2 * D + i] = __ldg(b1 + i);
+}
+// A head's W1, LayerNorm weights and hidden bias into shared memory: W1, then gamma, beta, b1.  Requested before the wait
+// for the sums, the vectors' round trips are off the chain behind it.
+template <typename WT>
+__device__ __forceinline__ void stage_mlp(const WT* W1, const float* gamma, const float* beta, const float* b1, int D, int hidden, WT* w1s) {
+  stage_weights(W1, w1s, D * hidden * (int)sizeof(WT));
+  stage_vectors(gamma, beta, b1, D, hidden, reinterpret_cast<float*>(w1s + D * hidden));
 }
 
 // modReLU: max(|z| + b, 0) z / |z| = max(1 + b / |z|, 0) z   (0 at z = 0)
@@ -409,7 +444,7 @@ struct GateMlpParams {
   float* qbar_out;
   float* u_ws;            // [B,H,hidden] hidden activations (workspace)
   int post;               // 1: Toeplitz follows, skip modReLU/phase here
-  int stage_w1;           // W1 of a head is copied to shared memory before the wait (size and alignment allow)
+  int stage_w1;           // W1, gamma, beta and b1 of a head are copied to shared memory before the wait (size and alignment allow)
 };
 
 // raw (re, im) weight pair of one bin in one hidden row
@@ -444,12 +479,12 @@ __global__ void __launch_bounds__(256) gate_hidden_kernel(const GateMlpParams p)
   float* qbar = u + BB * p.hidden;
   const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
   WT* w1s = reinterpret_cast<WT*>(u + ((BB * (p.hidden + p.D) + 3) & ~3));
-  if (p.stage_w1) stage_weights(W1, w1s, p.D * p.hidden * (int)sizeof(WT));
+  const float* vec = reinterpret_cast<const float*>(w1s + p.D * p.hidden);
+  if (p.stage_w1) stage_mlp(W1, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D, p.hidden, w1s);
   asm volatile("griddepcontrol.wait;" ::: "memory");        // the sums come from the kernel before
   if (p.stage_w1)
     descriptor_and_hidden<WT, BB, true>(p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
-                                        p.inv_count, p.D, p.hidden, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, w1s,
-                                        p.b1 + h * p.hs_b1, qbar, u, BB);
+                                        p.inv_count, p.D, p.hidden, vec, vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, BB);
   else
     descriptor_and_hidden<WT, BB, false>(p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                          p.inv_count, p.D, p.hidden, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, W1,
@@ -543,7 +578,7 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
   const WT* col = reinterpret_cast<const WT*>(p.W2) + h * p.hs_w2 + 2 * (size_t)(live ? k : 0);
   const size_t ld = 2 * (size_t)p.K;
   WT* w1s = reinterpret_cast<WT*>(u + ((BB * (p.hidden + p.D) + 3) & ~3));
-  if (!PRE && p.stage_w1) stage_weights(reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1, w1s, p.D * p.hidden * (int)sizeof(WT));
+  const float* vec = reinterpret_cast<const float*>(w1s + p.D * p.hidden);
   typename wraw<WT>::type w[R];
   const int n0 = min(R, p.hidden);
   if (live) {
@@ -551,6 +586,12 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
     for (int i = 0; i < R; ++i)
       if (i < n0) w[i] = wraw<WT>::load(col + (size_t)i * ld);
   }
+  const int kc = live ? k : 0;
+  const float2 b2 = make_float2(__ldg(p.b2 + h * p.hs_b2 + 2 * kc), __ldg(p.b2 + h * p.hs_b2 + 2 * kc + 1));
+  const float bias = (!p.post && p.modrelu_bias) ? __ldg(p.modrelu_bias + h * p.hs_mb + kc) : 0.f;
+  if (!PRE && p.stage_w1)
+    stage_mlp(reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D,
+              p.hidden, w1s);
   // everything above reads only weights; the sums / hidden activations come from the kernel before
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (PRE) {
@@ -566,8 +607,7 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
     const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
     if (p.stage_w1)
       descriptor_and_hidden<WT, BB, true>(p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
-                                          p.inv_count, p.D, p.hidden, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, w1s,
-                                          p.b1 + h * p.hs_b1, qbar, u, BB);
+                                          p.inv_count, p.D, p.hidden, vec, vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, BB);
     else
       descriptor_and_hidden<WT, BB, false>(p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                            p.inv_count, p.D, p.hidden, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, W1,
@@ -579,10 +619,9 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
       }
   }
   if (!live) return;
-  const float* b2 = p.b2 + h * p.hs_b2;
   float2 acc[BB];
 #pragma unroll
-  for (int bb = 0; bb < BB; ++bb) acc[bb] = make_float2(b2[2 * k], b2[2 * k + 1]);
+  for (int bb = 0; bb < BB; ++bb) acc[bb] = b2;
   // BB >= 4: the sums of two batch entries share a packed fp32 pair (one instruction per pair and
   // component; each half rounds like a scalar fmaf, so the results do not change)
   constexpr int NP = BB >= 4 ? BB / 2 : 1;
@@ -598,7 +637,6 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
       upk2(ay[pp], acc[2 * pp].y, acc[2 * pp + 1].y);
     }
   }
-  const float bias = (!p.post && p.modrelu_bias) ? p.modrelu_bias[h * p.hs_mb + k] : 0.f;
   // one positional phase for the whole batch unless per-entry shifts are given
   float2 ph = make_float2(1.f, 0.f);
   if (!p.post && !p.shift) ph = phase_reduced(k, p.n, p.pm_all);
@@ -610,6 +648,74 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
       if (!p.post) {
         if (p.modrelu_bias) a = modrelu(a, bias);         // without a bias modReLU is the identity (|z| z / |z| = z, exactly, in this arithmetic too)
         a = cmul(a, p.shift ? phase_factor(k, p.n, p.shift_all + p.shift[b]) : ph);
+      }
+      p.g_out[((size_t)b * p.H + h) * p.K + k] = a;
+    }
+  }
+}
+
+// ---- the whole gate of a short transform, several batch entries ----
+// One CTA per head and BB entries, one bin per thread.  All of a head's weights go to shared memory (cp.async) ahead of the wait
+// for the sums.  What bounds it is the chain of short phases behind that wait, and in a chain of kernels the first pass over
+// their code: fetched once per SM and launch, so the loops here are rolled up (gate_out_kernel's 32 rows per thread are 600 instructions).
+template <typename WT, int BB>
+__global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams p) {
+  extern __shared__ __align__(16) float u[];       // [hidden][BB], q_bar [BB][D], W1, gamma, beta, b1, W2
+  asm volatile("griddepcontrol.launch_dependents;");
+  const int nbg = (p.B + BB - 1) / BB;
+  const int h = blockIdx.x / nbg, b0 = (blockIdx.x - h * nbg) * BB;
+  const int nb = min(BB, p.B - b0), k = threadIdx.x;
+  const bool live = k < p.K;
+  WT* w1s = reinterpret_cast<WT*>(u + ((BB * (p.hidden + p.D) + 3) & ~3));
+  float* vec = reinterpret_cast<float*>(w1s + p.D * p.hidden);
+  WT* w2s = reinterpret_cast<WT*>(vec + ((2 * p.D + p.hidden + 3) & ~3));
+  copy_async16(reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1, w1s, p.D * p.hidden * (int)sizeof(WT));
+  copy_async16(reinterpret_cast<const WT*>(p.W2) + h * p.hs_w2, w2s, p.hidden * 2 * p.K * (int)sizeof(WT));
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  stage_vectors(p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D, p.hidden, vec);
+  const int kc = live ? k : 0;
+  const float2 b2 = make_float2(__ldg(p.b2 + h * p.hs_b2 + 2 * kc), __ldg(p.b2 + h * p.hs_b2 + 2 * kc + 1));
+  const float bias = (!p.post && p.modrelu_bias) ? __ldg(p.modrelu_bias + h * p.hs_mb + kc) : 0.f;
+  asm volatile("cp.async.wait_group 0;" ::: "memory");       // every thread's copies; the barriers below make them the CTA's
+  asm volatile("griddepcontrol.wait;" ::: "memory");         // the sums come from the kernel before
+  float* qbar = u + BB * p.hidden;
+  descriptor_and_hidden<WT, BB, true>(p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
+                                      p.inv_count, p.D, p.hidden, vec, vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, BB);
+  if (p.qbar_out)
+    for (int e = threadIdx.x; e < nb * p.D; e += blockDim.x) {
+      const int bb = e / p.D, c = e - bb * p.D;
+      p.qbar_out[((size_t)(b0 + bb) * p.H + h) * p.D + c] = qbar[e];
+    }
+  if (!live) return;
+  uint64_t ax[BB / 2], ay[BB / 2];                           // two entries per packed fp32 pair
+#pragma unroll
+  for (int i = 0; i < BB / 2; ++i) { ax[i] = pk2(b2.x, b2.x); ay[i] = pk2(b2.y, b2.y); }
+  const typename wraw<WT>::type* wk = reinterpret_cast<const typename wraw<WT>::type*>(w2s) + k;
+#pragma unroll 4
+  for (int j = 0; j < p.hidden; ++j) {
+    const float2 wv = wraw<WT>::cvt(wk[j * p.K]);
+    const uint64_t wx = pk2(wv.x, wv.x), wy = pk2(wv.y, wv.y);
+#pragma unroll
+    for (int v = 0; v < BB / 4; ++v) {
+      const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(u + j * BB + 4 * v);   // entries 4v .. 4v + 3 (absent ones: stale, never stored)
+      ax[2 * v] = fma2(t.x, wx, ax[2 * v]);         ay[2 * v] = fma2(t.x, wy, ay[2 * v]);
+      ax[2 * v + 1] = fma2(t.y, wx, ax[2 * v + 1]); ay[2 * v + 1] = fma2(t.y, wy, ay[2 * v + 1]);
+    }
+  }
+  float2 ph = make_float2(1.f, 0.f);                         // one positional phase for the whole batch unless per-entry shifts are given
+  if (!p.post && !p.shift) ph = phase_reduced(k, p.n, p.pm_all);
+#pragma unroll
+  for (int bb = 0; bb < BB; ++bb) {
+    if (bb < nb) {
+      const int b = b0 + bb;
+      float x0, x1, y0, y1;
+      upk2(ax[bb / 2], x0, x1);
+      upk2(ay[bb / 2], y0, y1);
+      float2 a = bb & 1 ? make_float2(x1, y1) : make_float2(x0, y0);
+      if (!p.post) {
+        if (p.modrelu_bias) a = modrelu(a, bias);
+        if (p.shift) ph = phase_factor(k, p.n, p.shift_all + p.shift[b]);
+        a = cmul(a, ph);
       }
       p.g_out[((size_t)b * p.H + h) * p.K + k] = a;
     }
@@ -718,7 +824,9 @@ __global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p)
   const float2* b2 = reinterpret_cast<const float2*>(p.b2 + h * p.hs_b2);
   const float* mb = !p.post && p.modrelu_bias ? p.modrelu_bias + h * p.hs_mb : nullptr;
   bf16* w1s = reinterpret_cast<bf16*>(u + ((NB * (p.hidden + p.D) + 3) & ~3));
-  if (p.stage_w1) stage_weights(reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, w1s, p.D * p.hidden * 2);
+  const float* vec = reinterpret_cast<const float*>(w1s + p.D * p.hidden);
+  const float *gamma = p.gamma + h * p.hs_ln, *beta = p.beta + h * p.hs_ln, *b1 = p.b1 + h * p.hs_b1;
+  if (p.stage_w1) stage_mlp(reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, gamma, beta, b1, p.D, p.hidden, w1s);
   // a CTA's chunks are contiguous, its warps take neighbouring ones
   const int nchunk = (p.K + 15) / 16, per = (nchunk + (int)gridDim.x - 1) / (int)gridDim.x;
   const int c0 = blockIdx.x * per + warp, c1 = min(nchunk, (int)(blockIdx.x + 1) * per);
@@ -728,10 +836,9 @@ __global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   float* qbar = u + NB * p.hidden;
   const float* sums = p.sums + ((size_t)b0 * p.H + h) * p.D;
-  const float *gamma = p.gamma + h * p.hs_ln, *beta = p.beta + h * p.hs_ln, *b1 = p.b1 + h * p.hs_b1;
   if (p.stage_w1)
-    descriptor_and_hidden<bf16, NB, true>(sums, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, gamma, beta,
-                                          p.eps, w1s, b1, qbar, u, NB);
+    descriptor_and_hidden<bf16, NB, true>(sums, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, vec,
+                                          vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, NB);
   else
     descriptor_and_hidden<bf16, NB, false>(sums, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, gamma, beta,
                                            p.eps, reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, b1, qbar, u, NB);
@@ -923,8 +1030,15 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   if (grid_out.y > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "H * ceil(B / 8) exceeds 65535");
   const bool wb = gp->wdtype == SPECTRE_BF16;
   const size_t w1_bytes = (size_t)D * gp->hidden * (wb ? 2 : 4);
-  mp.stage_w1 = w1_bytes <= 16384 && w1_bytes % 16 == 0 && !(reinterpret_cast<uintptr_t>(gp->W1) & 15);
-  const size_t smem = (((size_t)BB * (D + gp->hidden) + 3) & ~(size_t)3) * sizeof(float) + (mp.stage_w1 ? w1_bytes : 0);
+  const size_t act_bytes = (((size_t)BB * (D + gp->hidden) + 3) & ~(size_t)3) * sizeof(float);
+  const size_t staged_bytes = w1_bytes + (2 * (size_t)D + gp->hidden) * sizeof(float);
+  mp.stage_w1 = w1_bytes <= 16384 && w1_bytes % 16 == 0 && !(reinterpret_cast<uintptr_t>(gp->W1) & 15) && act_bytes + staged_bytes <= 49152;
+  const size_t smem = act_bytes + (mp.stage_w1 ? staged_bytes : 0);
+  // One CTA holds all bins and a head's weights fit beside its activations: all of them staged, one short kernel
+  const size_t w2_bytes = (size_t)gp->hidden * 2 * K * (wb ? 2 : 4);
+  const size_t short_bytes = act_bytes + w1_bytes + ((2 * (size_t)D + gp->hidden + 3) & ~(size_t)3) * sizeof(float) + w2_bytes;
+  const bool all_staged = BB >= 4 && !mma && grid_out.x == 1 && w1_bytes % 16 == 0 && w2_bytes % 16 == 0 && short_bytes <= 49152 &&
+                          !((reinterpret_cast<uintptr_t>(gp->W1) | reinterpret_cast<uintptr_t>(gp->W2)) & 15);
   const bool pre = grid_out.x >= 32;               // many CTAs per head: compute the hidden layer once
   // Programmatic dependent launch: the weight stream of the output layer may overlap the kernel
   // before it (the pooling pass here, or whatever produced sum_q); each kernel waits for its
@@ -944,6 +1058,8 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
     cfg_mma.gridDim = dim3((unsigned)(fit < 1 ? 1 : (blocks < fit ? blocks : fit)), grid_out.y, 1);
     cfg_mma.blockDim = dim3(256, 1, 1);
   }
+  cudaLaunchConfig_t cfg_short = cfg_out;
+  cfg_short.gridDim = dim3(grid_out.y, 1, 1); cfg_short.dynamicSmemBytes = short_bytes;
 #define SPECTRE_GATE_LAUNCH(WT, NB)                                                              \
   do {                                                                                           \
     if (pre) {                                                                                   \
@@ -960,6 +1076,9 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   } while (0)
   if (mma) {
     if (BB == 8) SPECTRE_GATE_MMA(8); else SPECTRE_GATE_MMA(4);
+  } else if (all_staged) {
+    if (wb) SPECTRE_CUDA_OK(BB == 8 ? cudaLaunchKernelEx(&cfg_short, gate_short_kernel<bf16, 8>, mp) : cudaLaunchKernelEx(&cfg_short, gate_short_kernel<bf16, 4>, mp));
+    else SPECTRE_CUDA_OK(BB == 8 ? cudaLaunchKernelEx(&cfg_short, gate_short_kernel<float, 8>, mp) : cudaLaunchKernelEx(&cfg_short, gate_short_kernel<float, 4>, mp));
   } else switch (BB) {
     case 8: if (wb) SPECTRE_GATE_LAUNCH(bf16, 8); else SPECTRE_GATE_LAUNCH(float, 8); break;
     case 4: if (wb) SPECTRE_GATE_LAUNCH(bf16, 4); else SPECTRE_GATE_LAUNCH(float, 4); break;

@@ -126,18 +126,11 @@ __device__ __forceinline__ float to_float(bf16 x) { return __bfloat162float(x); 
 template <typename WT>
 __global__ void __launch_bounds__(256, 3) level_gates_kernel(const LevelGateParams p) {
   __shared__ __align__(16) float qs[kLgBatch][64];
-  extern __shared__ float part_raw[];                        // [4][kLgBatch][hidden]: hidden-layer partial sums per input quarter
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  extern __shared__ __align__(16) float part_raw[];          // [4][kLgBatch][hidden]: hidden-layer partial sums per input quarter; [hidden][kLgBatch]
   const int tid = threadIdx.x, h = blockIdx.x, b0 = blockIdx.y * kLgBatch;
   const WT* W1 = reinterpret_cast<const WT*>(p.Ww1) + h * p.hs_w1;
   const WT* W2 = reinterpret_cast<const WT*>(p.Ww2) + h * p.hs_w2;
   const int nitems = 4 * p.hidden;
-  float qv[2];
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int e = tid + 256 * i, b = b0 + (e >> 6);
-    qv[i] = b < p.B ? p.qbar[((size_t)b * p.H + h) * 64 + (e & 63)] : 0.f;
-  }
   WT w1[16], w2[32];
   {
     const int it = min(tid, nitems - 1), jj = it % p.hidden, cq = it / p.hidden;
@@ -147,8 +140,17 @@ __global__ void __launch_bounds__(256, 3) level_gates_kernel(const LevelGatePara
   const int ii = min(tid, p.NG - 1);
 #pragma unroll
   for (int u = 0; u < 32; ++u) w2[u] = W2[(size_t)min(u, p.hidden - 1) * p.NG + ii];
+  float b1v = __ldg(p.bw1 + h * p.hs_b1 + tid % p.hidden);
+  const float b2v = __ldg(p.bw2 + h * p.hs_b2 + ii);
+  // Everything above reads only weights; q_bar comes from the kernel before.  The mixer behind this one may start only now:
+  // it reads the tokens without a wait of its own.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 2; ++i) qs[(tid + 256 * i) >> 6][(tid + 256 * i) & 63] = qv[i];
+  for (int i = 0; i < 2; ++i) {
+    const int e = tid + 256 * i, b = b0 + (e >> 6);
+    qs[e >> 6][e & 63] = b < p.B ? p.qbar[((size_t)b * p.H + h) * 64 + (e & 63)] : 0.f;
+  }
   __syncthreads();
   for (int it = tid; it < nitems; it += 256) {
     const int jj = it % p.hidden, cq = it / p.hidden;
@@ -174,17 +176,19 @@ __global__ void __launch_bounds__(256, 3) level_gates_kernel(const LevelGatePara
     for (int e = 0; e < kLgBatch; ++e) part_raw[(cq * kLgBatch + e) * p.hidden + jj] = acc[e];
   }
   __syncthreads();
-  for (int i = tid; i < kLgBatch * p.hidden; i += 256) {       // u = GELU(sum of the quarters + bias), kept in part[0]
+  // u = GELU(sum of the quarters + bias), kept behind the quarters with the 8 entries of a unit side by side
+  float* us = part_raw + 4 * kLgBatch * p.hidden;
+  for (int i = tid; i < kLgBatch * p.hidden; i += 256) {
     const int e = i / p.hidden, jj = i - e * p.hidden;
     const int st = kLgBatch * p.hidden;
-    part_raw[i] = gelu_erf(p.bw1[h * p.hs_b1 + jj] + ((part_raw[i] + part_raw[st + i]) + (part_raw[2 * st + i] + part_raw[3 * st + i])));
+    us[jj * kLgBatch + e] = gelu_erf(b1v + ((part_raw[i] + part_raw[st + i]) + (part_raw[2 * st + i] + part_raw[3 * st + i])));
+    if (i + 256 < kLgBatch * p.hidden) b1v = __ldg(p.bw1 + h * p.hs_b1 + (i + 256) % p.hidden);
   }
   __syncthreads();
   if (tid < p.NG) {
-    float acc[kLgBatch];
-    const float b2 = p.bw2[h * p.hs_b2 + ii];
+    uint64_t acc2[kLgBatch / 2];                               // two entries per packed fp32 pair
 #pragma unroll
-    for (int e = 0; e < kLgBatch; ++e) acc[e] = b2;
+    for (int e = 0; e < kLgBatch / 2; ++e) acc2[e] = pk2(b2v, b2v);
     for (int j0 = 0; j0 < p.hidden; j0 += 32) {
       if (j0 > 0) {
 #pragma unroll
@@ -194,11 +198,20 @@ __global__ void __launch_bounds__(256, 3) level_gates_kernel(const LevelGatePara
       for (int u = 0; u < 32; ++u) {
         if (j0 + u < p.hidden) {
           const float wv = to_float(w2[u]);
+          const uint64_t ww = pk2(wv, wv);
+          const ulonglong2* ur = reinterpret_cast<const ulonglong2*>(us + (j0 + u) * kLgBatch);
 #pragma unroll
-          for (int e = 0; e < kLgBatch; ++e) acc[e] = fmaf(part_raw[e * p.hidden + j0 + u], wv, acc[e]);
+          for (int e = 0; e < kLgBatch / 4; ++e) {
+            const ulonglong2 t = ur[e];
+            acc2[2 * e] = fma2(t.x, ww, acc2[2 * e]);
+            acc2[2 * e + 1] = fma2(t.y, ww, acc2[2 * e + 1]);
+          }
         }
       }
     }
+    float acc[kLgBatch];
+#pragma unroll
+    for (int e = 0; e < kLgBatch / 2; ++e) upk2(acc2[e], acc[2 * e], acc[2 * e + 1]);
 #pragma unroll
     for (int e = 0; e < kLgBatch; ++e)
       if (b0 + e < p.B) p.out[((size_t)(b0 + e) * p.H + h) * p.NG + ii] = acc[e];
@@ -660,6 +673,9 @@ int launch_mixer_tc196(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
   p.F = reinterpret_cast<const __half*>(ctx->dft49);
   p.H = v->H; p.L = v->L; p.B = v->B;
   p.status = ctx->status_dev;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
   bool dependent = false;            // the mixer kernel follows a kernel of ours whose output it reads
   if (wrm) {
     const int J = wrm->levels;
@@ -676,17 +692,17 @@ int launch_mixer_tc196(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
       lp.out = level_gate_scratch;
       lp.B = v->B; lp.H = v->H; lp.hidden = hid; lp.NG = (J + 1) * 64;
       const dim3 lgrid((unsigned)v->H, (unsigned)((v->B + kLgBatch - 1) / kLgBatch));
-      const size_t lsmem = (size_t)4 * kLgBatch * hid * sizeof(float);       // <= 32 KB
-      if (wrm->wdtype == SPECTRE_BF16) level_gates_kernel<bf16><<<lgrid, 256, lsmem, st>>>(lp);
-      else level_gates_kernel<float><<<lgrid, 256, lsmem, st>>>(lp);
+      const size_t lsmem = (size_t)5 * kLgBatch * hid * sizeof(float);       // <= 40 KB
+      cudaLaunchConfig_t lcfg = {};                            // its weight loads overlap the kernel that makes q_bar
+      lcfg.gridDim = lgrid; lcfg.blockDim = dim3(256); lcfg.dynamicSmemBytes = lsmem; lcfg.stream = st;
+      lcfg.attrs = attr; lcfg.numAttrs = 1;
+      if (wrm->wdtype == SPECTRE_BF16) SPECTRE_CUDA_OK(cudaLaunchKernelEx(&lcfg, level_gates_kernel<bf16>, lp));
+      else SPECTRE_CUDA_OK(cudaLaunchKernelEx(&lcfg, level_gates_kernel<float>, lp));
       SPECTRE_LAUNCH_OK("level_gates_kernel");
       p.level_gates = level_gate_scratch;
       dependent = true;
     }
   }
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
   const unsigned nwork = (unsigned)(p.H * ((p.B + k196Heads - 1) / k196Heads)), slots = 2u * (unsigned)ctx->sm_count;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nwork < slots ? nwork : slots);        // persistent: two CTAs per SM
