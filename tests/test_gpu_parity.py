@@ -319,6 +319,21 @@ def test_gate_batches_on_tensor_cores(ctx, B, H, n, r, shifts):
     assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
 
 
+@pytest.mark.parametrize("B,n,D,hid,wdt,r,shifts", [(4, 2, 64, 64, "bf16", 0, False), (8, 196, 64, 64, "bf16", 0, True), (13, 64, 24, 32, "f32", 2, False),
+                                                     (9, 254, 64, 40, "bf16", 0, False), (5, 510, 8, 8, "f32", 0, True), (11, 100, 128, 64, "bf16", 1, False)])
+def test_gate_short_transforms(ctx, B, n, D, hid, wdt, r, shifts):
+    # one CTA per head and 4 or 8 entries with all weights staged: two bins up to as many as a block has threads, the last
+    # group of entries ragged, inputs of the hidden layer not a multiple of 32, phases per entry
+    w = W.Workload("t", B=B, L=min(n, 33), H=3, D=D, dtype="bf16", wdtype=wdt, n_fft=n, hidden=hid, seed=n + B)
+    p = W.gate_params(w, modrelu_bias_std=0.01, toeplitz_r=r, bias_std=0.1)
+    x = W.activations(w, structured=True)
+    shift = torch.arange(B, dtype=torch.int64) * 7 - 3 if shifts else None
+    g = S.spectre_gate(ctx, to_dev(p), n, q=x.cuda(), shift=shift.cuda() if shifts else None, shift_all=11)
+    ref = O.gate(W.to_f64(x).sum(axis=1), 1.0 / w.L, n, shift=(shift.numpy() if shifts else np.zeros(B, dtype=np.int64)) + 11,
+                 **gate_params_np(p))
+    assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
+
+
 def test_gate_from_running_sum_and_shared_heads(ctx):
     w = W.Workload("t", B=2, L=64, H=4, D=32, dtype="f32", wdtype="f32", n_fft=64, seed=13)
     p = W.gate_params(w)
