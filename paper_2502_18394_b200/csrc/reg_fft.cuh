@@ -43,6 +43,11 @@ enum RegMode { kRegMix = 0, kRegForward = 1, kRegInverse = 2, kRegGrad = 3 };
 template <int R1, int R2, int C_>
 struct TwoStep {
   static constexpr int C = C_, M = R1 * R2, E = R1, S = R2, U = R1 / R2;
+  // mix() runs the steps as a loop over one copy of the DFT.  From 32 points on, straight-line code (four DFTs) waits for
+  // instructions: 1024 = 32 x 32 at 12.6 M elements takes 35.9 us in the loop against 38.6 (fp32), 27.3 against 30.1 (bf16).
+  // 28 x 28 and smaller ones lose 1 - 10 % to its extra barrier and moves, and so does the gradient (55 -> 58 us), whose loop over
+  // three transforms carries more state; the forward transform alone gains nothing.
+  static constexpr bool kLoop = R1 == R2 && R1 >= 32;
   static constexpr int kActive = S * C, kThreads = (kActive + 31) / 32 * 32;
   static constexpr int kExch = R1 * (R2 + 1) * C;                   // elements of the exchange buffer
   static constexpr int kGate = M;
@@ -60,15 +65,31 @@ struct TwoStep {
   template <bool HALF, class Before = Nothing>
   __device__ __forceinline__ void forward(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before = Before()) const {
     RegDft<R1, false>::run(x);
-#pragma unroll
-    for (int a = 0; a < R1 / 2; ++a) {
-      const float4 w = tw_load4(tw + a * R1 + m);
-      if (a > 0) x[2 * a] = cmul(x[2 * a], make_float2(w.x, w.y));
-      x[2 * a + 1] = cmul(x[2 * a + 1], make_float2(w.z, w.w));
-    }
-    exchange<HALF, true>(x, buf, act, before);
+    turn<HALF>(x, buf, tw, act, before);
 #pragma unroll
     for (int u = 0; u < U; ++u) sub<false>(x, u);
+  }
+  static __device__ __forceinline__ void swap_parts(float2 (&x)[E]) {
+#pragma unroll
+    for (int i = 0; i < E; ++i) x[i] = make_float2(x[i].y, x[i].x);
+  }
+  // kLoop: forward transform, gate(x), inverse transform.  The inverse is the forward one of the values with real and
+  // imaginary parts swapped, its exchange the same one, so all four DFTs are one piece of code.
+  template <class Before, class Gate>
+  __device__ __forceinline__ void mix(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before, Gate gate) const {
+#pragma unroll 1
+    for (int step = 0; step < 4; ++step) {
+      RegDft<R1, false>::run(x);
+      settle(x);
+      if (!(step & 1)) {
+        turn<false>(x, buf, tw, act, [&] { if (step == 0) before(); });
+      } else if (step == 1) {
+        gate(x);
+        swap_parts(x);
+        __syncthreads();                                   // every thread has read the exchange buffer: it may be written again
+      }
+    }
+    swap_parts(x);
   }
   template <bool HALF>
   __device__ __forceinline__ void inverse(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act) const {
@@ -87,6 +108,17 @@ struct TwoStep {
   }
 
  private:
+  // between the steps: twiddles and exchange
+  template <bool HALF, class Before>
+  __device__ __forceinline__ void turn(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before) const {
+#pragma unroll
+    for (int a = 0; a < R1 / 2; ++a) {
+      const float4 w = tw_load4(tw + a * R1 + m);
+      if (a > 0) x[2 * a] = cmul(x[2 * a], make_float2(w.x, w.y));
+      x[2 * a + 1] = cmul(x[2 * a + 1], make_float2(w.z, w.w));
+    }
+    exchange<HALF, true>(x, buf, act, before);
+  }
   template <bool INV>
   __device__ __forceinline__ void sub(float2 (&x)[E], int u) const {
     float2 y[R2];
@@ -148,6 +180,7 @@ struct TwoStep {
 template <int C_>
 struct ThreeStep2048 {
   static constexpr int C = C_, M = 2048, E = 32, S = 64, PW = C / 4;
+  static constexpr bool kLoop = false;
   static constexpr int kActive = S * C, kThreads = kActive;
   static constexpr int kExch = (2048 + 256) * C;
   static constexpr int kGate = 2048 + 64;
@@ -397,15 +430,20 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
       extra[P::gate_slot(i)] = v;
     }
   }
-  if constexpr (MODE != kRegInverse) pl.template forward<HALF>(x, buf, p.tw, act);
-
-  settle(x);
-  if constexpr (MODE == kRegMix) {                         // the gate table is complete: the exchange had a barrier
+  auto gate = [&](float2 (&z)[E]) {                        // the gate table is complete: the exchange had a barrier
 #pragma unroll
     for (int i = 0; i < E; ++i) {
-      x[i] = cmul(x[i], extra[P::gate_slot(pl.bin(i))]);
+      z[i] = cmul(z[i], extra[P::gate_slot(pl.bin(i))]);
       if (i % 4 == 3) asm volatile("" ::: "memory");        // four gates at a time: there are no registers for more
     }
+  };
+  constexpr bool kRolled = MODE == kRegMix && P::kLoop;
+  if constexpr (kRolled) {
+    pl.mix(x, buf, p.tw, act, [] {}, gate);
+  } else if constexpr (MODE != kRegInverse) {
+    pl.template forward<HALF>(x, buf, p.tw, act);
+    settle(x);
+    if constexpr (MODE == kRegMix) gate(x);
   }
   if constexpr (MODE == kRegForward) {
     float2* out = p.ws + wrow * half + pout;
@@ -458,8 +496,10 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
     }
   }
 
-  settle(x);
-  pl.template inverse<HALF>(x, buf, p.tw, act);
+  if constexpr (!kRolled) {
+    settle(x);
+    pl.template inverse<HALF>(x, buf, p.tw, act);
+  }
   if (!live) return;
   if constexpr (WS) {
     char* base = reinterpret_cast<char*>(p.ws + wrow * half);
@@ -528,7 +568,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_stream_k
     for (int i = 0; i < E; ++i) x[i] = PairIo<T>::cvt(rows[(pl.m + P::S * i) * 8 + pl.p]);
     if (__syncthreads_or(!ok)) break;
     if (threadIdx.x == 0 && w + (int)gridDim.x < ntotal) fetch(w + gridDim.x);     // every thread has its rows: the buffer is free
-    pl.template forward<false>(x, buf, p.tw, act, [&] {
+    auto fill = [&] {
 #pragma unroll
       for (int i = 0; i < kGv; ++i) {
         const int k = threadIdx.x + i * P::kThreads;
@@ -537,15 +577,23 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_stream_k
         if (k == 0 || 2 * k == P::M) v.y = 0.f;
         if (k < P::M) gs[P::gate_slot(k)] = v;
       }
-    });
-    settle(x);
+    };
+    auto gate = [&](float2 (&z)[E]) {
 #pragma unroll
-    for (int i = 0; i < E; ++i) {
-      x[i] = cmul(x[i], gs[P::gate_slot(pl.bin(i))]);
-      if (i % 4 == 3) asm volatile("" ::: "memory");
+      for (int i = 0; i < E; ++i) {
+        z[i] = cmul(z[i], gs[P::gate_slot(pl.bin(i))]);
+        if (i % 4 == 3) asm volatile("" ::: "memory");
+      }
+    };
+    if constexpr (P::kLoop) {
+      pl.mix(x, buf, p.tw, act, fill, gate);
+    } else {
+      pl.template forward<false>(x, buf, p.tw, act, fill);
+      settle(x);
+      gate(x);
+      settle(x);
+      pl.template inverse<false>(x, buf, p.tw, act);
     }
-    settle(x);
-    pl.template inverse<false>(x, buf, p.tw, act);
     reg_store_tokens<T, P>(x, p, b, h, 2 * pair, pl.m, act && pair < p.D / 2);
   }
   if (!ok) {                                       // do not leave with copies in flight (bounded again)
@@ -612,6 +660,9 @@ static int reg_launch_stream(RegParams p, int nslab, cudaStream_t st, int sm_cou
 // same tiles are 20 % slower (batch of 16 x 12 heads, n = 1024: fp32 45 us against 38, workspace rows 35 against 32): a
 // request covers more rows, and each row costs the load/store unit a cycle.
 constexpr int kRegPairs = 8;
+// The mixer of 1024 and 2048 points with tiles for at most half the SMs: 4 pairs per CTA, so that the few warps there are have
+// twice the SMs (up to 16 heads of one sequence: n = 1024 7.5 -> 6.1 us, 2048 15.0 -> 10.1; 512 and less are slower, 5.2 -> 5.4,
+// and with 2 pairs 1024 is too, 8.0).
 
 template <typename T, int MODE>
 static int reg_launch_tokens(const spectre_ctx* ctx, const RegParams& q, int M, int nslab, cudaStream_t st) {
@@ -627,10 +678,18 @@ static int reg_launch_tokens(const spectre_ctx* ctx, const RegParams& q, int M, 
       const int rc = reg_launch_stream<T, TwoStep<R1, R2, C>>(p, nslab, st, ctx->sm_count, &done); \
       if (rc != SPECTRE_OK || done) return rc;                                                       \
     }                                                                                                \
+    if constexpr (MODE == kRegMix && R1 == 32 && R2 == 32) {                                         \
+      if (2 * tiles <= ctx->sm_count) return reg_launch<T, TwoStep<R1, R2, 4>, MODE, false>(p, nslab, st); \
+    }                                                                                                \
     return reg_launch<T, TwoStep<R1, R2, C>, MODE, false>(p, nslab, st);
+  const long long tiles = (long long)nslab * ((p.D / 2 + C - 1) / C);
   switch (M) {
     SPECTRE_REG_TWO_STEP(SPECTRE_REG_CASE)
-    case 2048: return reg_launch<T, ThreeStep2048<C>, MODE, false>(p, nslab, st);
+    case 2048:
+      if constexpr (MODE == kRegMix) {
+        if (2 * tiles <= ctx->sm_count) return reg_launch<T, ThreeStep2048<4>, MODE, false>(p, nslab, st);
+      }
+      return reg_launch<T, ThreeStep2048<C>, MODE, false>(p, nslab, st);
     default: return fail(SPECTRE_ERR_UNSUPPORTED, "transform length not supported");
   }
 #undef SPECTRE_REG_CASE

@@ -69,7 +69,8 @@ def test_register_transforms(ctx, dt, n, L, D):
         assert slab_err(W.to_f64(dv), rv) < TOL[dt] and rel_err(gate_to_complex(dg), rg) < TOL["f32"]
 
 
-@pytest.mark.parametrize("dt,B,H,n,L,D", [("bf16", 20, 8, 1024, 1000, 40), ("f16", 64, 8, 256, 255, 64), ("bf16", 40, 8, 784, 784, 24)])
+@pytest.mark.parametrize("dt,B,H,n,L,D", [("bf16", 20, 8, 1024, 1000, 40), ("f16", 64, 8, 256, 255, 64), ("bf16", 40, 8, 784, 784, 24),
+                                               ("f32", 10, 8, 1024, 1000, 24), ("f32", 10, 8, 2048, 1025, 24)])
 def test_register_transforms_more_tiles_than_resident(ctx, dt, B, H, n, L, D):
     # persistent CTAs, rows of the next tile by TMA: column tiles beyond D, rows beyond L, several tiles per CTA
     assert run_mixer(ctx, W.Workload("t", B=B, L=L, H=H, D=D, dtype=dt, n_fft=n, seed=n + L), n_fft=n) < TOL[dt]
