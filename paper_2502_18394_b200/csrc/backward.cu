@@ -19,6 +19,7 @@ bool transform_supported(const spectre_ctx* ctx, int n);
 size_t transform_slab_bytes(int n, int D);
 
 __global__ void __launch_bounds__(256) conj_gate_kernel(const float2* __restrict__ g, float2* __restrict__ gc, size_t total) {
+  after_previous();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < total) {
     float2 v = g[i];
@@ -30,6 +31,7 @@ __global__ void __launch_bounds__(256) conj_gate_kernel(const float2* __restrict
 // leave per group of pairs: dg_k = (w_k / 2n) (S_k + conj(S_{n-k})).
 __global__ void __launch_bounds__(256) gate_grad_sum_kernel(const float2* __restrict__ sums, float2* __restrict__ dg, int n, int K,
                                                             int parts, int slab0, int nslab) {
+  after_previous();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (size_t)nslab * K) return;
   const int k = (int)(i % K), slab_local = (int)(i / K), km = k == 0 ? 0 : n - k;
@@ -84,6 +86,7 @@ template <int N1>
 __global__ void __launch_bounds__(256, N1 <= 8 ? 2 : 1) gate_grad_combine_kernel(const float2* __restrict__ wsV, const float2* __restrict__ wsG,
                                                                 float2* __restrict__ dg, int n, int K, int D, int M,
                                                                 int slab0, int nslab) {
+  after_previous();
   const size_t wid = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31, sub = lane & 15, s = sub % N1;
   const int nk2 = M / 2 + 1, half = D / 2;
@@ -150,7 +153,8 @@ template <int N1>
 static void launch_gate_grad_combine(cudaStream_t st, const float2* wsV, const float2* wsG, float2* dg, int n, int K, int D,
                                      int M, int slab0, int cnt) {
   const size_t nwarps = (size_t)cnt * (M / 2 + 1);
-  gate_grad_combine_kernel<N1><<<(unsigned)((nwarps * 32 + 255) / 256), 256, 0, st>>>(wsV, wsG, dg, n, K, D, M, slab0, cnt);
+  (void)launch_after(gate_grad_combine_kernel<N1>, (unsigned)((nwarps * 32 + 255) / 256), 256, 0, st, wsV, wsG, dg, n, K, D, M, slab0,
+                     cnt);                                     // the caller asks for the error
 }
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -184,7 +188,8 @@ static int backward_reg(const spectre_ctx* ctx, cudaStream_t st, const spectre_a
     p.slab0 = s0;
     int rc = reg_grad(ctx, st, p, n, cnt, v->dtype);
     if (rc != SPECTRE_OK) return rc;
-    gate_grad_sum_kernel<<<(unsigned)(((size_t)cnt * K + 255) / 256), 256, 0, st>>>(p.sums, reinterpret_cast<float2*>(dg), n, K, parts, s0, cnt);
+    SPECTRE_CUDA_OK(launch_after(gate_grad_sum_kernel, (unsigned)(((size_t)cnt * K + 255) / 256), 256, 0, st, p.sums,
+                                 reinterpret_cast<float2*>(dg), n, K, parts, s0, cnt));
     SPECTRE_LAUNCH_OK("gate_grad_sum_kernel");
   }
   return SPECTRE_OK;
@@ -241,7 +246,7 @@ extern "C" int spectre_mixer_backward(spectre_ctx* ctx, void* stream, const spec
   if (dv) {
     float2* gc = reinterpret_cast<float2*>(base);
     const size_t total = (size_t)nslab * K;
-    conj_gate_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(reinterpret_cast<const float2*>(g), gc, total);
+    SPECTRE_CUDA_OK(launch_after(conj_gate_kernel, (unsigned)((total + 255) / 256), 256, 0, st, reinterpret_cast<const float2*>(g), gc, total));
     SPECTRE_LAUNCH_OK("conj_gate_kernel");
     rc = spectre_mixer_forward(ctx, stream, dy, reinterpret_cast<const float*>(gc), dv, n_fft, nullptr,
                                mix_bytes ? base + gc_bytes : nullptr, mix_bytes);

@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(256) split_kernel(const float2* __restrict__ w
 template <int N1>
 __global__ void __launch_bounds__(256) combine_split_kernel(const float2* __restrict__ ws, float* __restrict__ prefix, int n,
                                                             int K, int D, int M, int slab0, int nslab) {
+  after_previous();
   const int half = D / 2;
   const int nk2 = M / 2 + 1;
   const size_t total = (size_t)nslab * nk2 * half;
@@ -109,7 +110,8 @@ template <int N1>
 static void launch_combine_split(cudaStream_t st, const float2* ws, float* prefix, int n, int K, int D, int M, int slab0,
                                  int cnt) {
   const size_t total = (size_t)cnt * (M / 2 + 1) * (D / 2);
-  combine_split_kernel<N1><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(ws, prefix, n, K, D, M, slab0, cnt);
+  (void)launch_after(combine_split_kernel<N1>, (unsigned)((total + 255) / 256), 256, 0, st, ws, prefix, n, K, D, M, slab0,
+                     cnt);                                     // the caller asks for the error
 }
 
 // Ring buffers: rows 0..L-1 <- tokens, rows L..N-1 <- 0 (Alg. 1 PreFill).  A CTA copies kRingRows

@@ -51,6 +51,26 @@ bool is_pow2(int64_t x);
 // stages (0 for n = 1) or -1 if n has another prime factor or needs > 8 stages.
 int radix_plan(int n, int* radices);
 
+#ifdef __CUDACC__
+// A short kernel in a chain: launched as the programmatic dependent of the one before it and waiting for it as its first
+// action, its launch overlaps that kernel's end (2 us less between the two than after an ordinary launch).
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+cudaError_t launch_after(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+#endif
+
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // ---- device helpers --------------------------------------------------------

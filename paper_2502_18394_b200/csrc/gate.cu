@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(256, 4) pool_kernel(const T* __restrict__ q, i
 
 // Clears the partial sums ahead of a pooling pass with several slices; lets that pass start at once.
 __global__ void __launch_bounds__(256) pool_clear_kernel(float4* __restrict__ sums, size_t n4) {
+  after_previous();                                            // the pass behind reads its rows without a wait of its own
   asm volatile("griddepcontrol.launch_dependents;");
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n4) sums[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -173,7 +174,7 @@ static int pool_launch(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
     if ((reinterpret_cast<uintptr_t>(sums) & 15) || (copy_stride * ncopy) % 4) {
       SPECTRE_CUDA_OK(cudaMemsetAsync(sums, 0, copy_stride * ncopy * sizeof(float), st));
     } else {
-      pool_clear_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(reinterpret_cast<float4*>(sums), n4);
+      SPECTRE_CUDA_OK(launch_after(pool_clear_kernel, (unsigned)((n4 + 255) / 256), 256, 0, st, reinterpret_cast<float4*>(sums), n4));
       SPECTRE_LAUNCH_OK("pool_clear_kernel");
       cfg.numAttrs = 1;
     }
@@ -898,6 +899,7 @@ struct GatePostParams {
 // Toeplitz update along the bin axis ('same' window, zero boundary, reads the
 // pre-update gate), then modReLU and phase (Sec. 3.2 steps 3b-3c).
 __global__ void __launch_bounds__(256) gate_post_kernel(const GatePostParams p) {
+  after_previous();
   asm volatile("griddepcontrol.launch_dependents;");
   const int bh = blockIdx.y, b = bh / p.H, h = bh - b * p.H;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1097,7 +1099,7 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
     pp.H = H; pp.K = K; pp.n = n_fft;
     dim3 grid((K + 255) / 256, B * H);
     if (grid.y > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "B*H exceeds 65535");
-    gate_post_kernel<<<grid, 256, 0, st>>>(pp);
+    SPECTRE_CUDA_OK(launch_after(gate_post_kernel, grid, 256, 0, st, pp));
     SPECTRE_LAUNCH_OK("gate_post_kernel");
   }
   return SPECTRE_OK;

@@ -465,6 +465,7 @@ struct StridedParams {
 // A thread takes PP column pairs of one n2: two up to N1 = 16, one at 32, whose 32 points fill the registers.
 template <typename T, int N1, bool INV>
 __global__ void __launch_bounds__(256) strided_kernel(const StridedParams p) {
+  after_previous();
   constexpr int PP = N1 <= 16 ? 2 : 1;
   const int npg = p.D / (2 * PP);
   const size_t total = (size_t)p.nslab * p.M * npg;
@@ -610,11 +611,11 @@ static int launch_strided(const StridedParams& p, int N1, cudaStream_t st) {
   size_t total = (size_t)p.nslab * p.M * (N1 <= 16 ? p.D / 4 : p.D / 2);
   unsigned blocks = (unsigned)((total + 255) / 256);
   switch (N1) {
-    case 2: strided_kernel<T, 2, INV><<<blocks, 256, 0, st>>>(p); break;
-    case 4: strided_kernel<T, 4, INV><<<blocks, 256, 0, st>>>(p); break;
-    case 8: strided_kernel<T, 8, INV><<<blocks, 256, 0, st>>>(p); break;
-    case 16: strided_kernel<T, 16, INV><<<blocks, 256, 0, st>>>(p); break;
-    case 32: strided_kernel<T, 32, INV><<<blocks, 256, 0, st>>>(p); break;
+    case 2: SPECTRE_CUDA_OK(launch_after(strided_kernel<T, 2, INV>, blocks, 256, 0, st, p)); break;
+    case 4: SPECTRE_CUDA_OK(launch_after(strided_kernel<T, 4, INV>, blocks, 256, 0, st, p)); break;
+    case 8: SPECTRE_CUDA_OK(launch_after(strided_kernel<T, 8, INV>, blocks, 256, 0, st, p)); break;
+    case 16: SPECTRE_CUDA_OK(launch_after(strided_kernel<T, 16, INV>, blocks, 256, 0, st, p)); break;
+    case 32: SPECTRE_CUDA_OK(launch_after(strided_kernel<T, 32, INV>, blocks, 256, 0, st, p)); break;
     default: return fail(SPECTRE_ERR_UNSUPPORTED, "outer factor not supported");
   }
   SPECTRE_LAUNCH_OK("strided_kernel");
@@ -678,6 +679,7 @@ static int reg_mixer_multi(const spectre_ctx* ctx, cudaStream_t st, const spectr
   int group = (int)(ws_bytes / slab_ws_bytes(n, v->D));
   const int pref = preferred_group(ctx, n, v->D, nslab);
   if (group > pref) group = pref;
+  group = (nslab + (nslab + group - 1) / group - 1) / ((nslab + group - 1) / group);      // equal groups, not full ones and a remainder
   for (int s0 = 0; s0 < nslab; s0 += group) {
     const int cnt = nslab - s0 < group ? nslab - s0 : group;
     int rc = launch_strided<T, false>(strided_params(v, false, n, kRegM, p.ws, s0, cnt), p.N1, st);

@@ -412,6 +412,7 @@ template <bool F16, int R>
 __global__ void __launch_bounds__(kXOutThreads, 1) tc_out32_kernel(const __grid_constant__ CUtensorMap tm_res,
                                                                   const __grid_constant__ CUtensorMap tm_out,
                                                                   const __grid_constant__ CUtensorMap tm_rest, const TcOut32Params p) {
+  after_previous();
   constexpr int S = 32 / R;
   static_assert(R == 32 || R == 16 || R == 8 || R == 4 || R == 2, "radix");
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -664,10 +665,10 @@ static int launch_tc_out_r(const spectre_ctx* ctx, cudaStream_t st, const unsign
   int grid = nitems < ctx->sm_count ? nitems : ctx->sm_count;
   if (y->dtype == SPECTRE_F16) {
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_out32_kernel<true, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXOutSmem));
-    tc_out32_kernel<true, R><<<grid, kXOutThreads, kXOutSmem, st>>>(tm_res, tm_out, tm_rest, p);
+    SPECTRE_CUDA_OK(launch_after(tc_out32_kernel<true, R>, grid, kXOutThreads, kXOutSmem, st, tm_res, tm_out, tm_rest, p));
   } else {
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_out32_kernel<false, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXOutSmem));
-    tc_out32_kernel<false, R><<<grid, kXOutThreads, kXOutSmem, st>>>(tm_res, tm_out, tm_rest, p);
+    SPECTRE_CUDA_OK(launch_after(tc_out32_kernel<false, R>, grid, kXOutThreads, kXOutSmem, st, tm_res, tm_out, tm_rest, p));
   }
   SPECTRE_LAUNCH_OK("tc_out32_kernel");
   return SPECTRE_OK;

@@ -309,6 +309,7 @@ __device__ __forceinline__ void core_store(uint32_t tmem_d, unsigned char* out, 
 // Operand images (tc_stage.cuh): stages 0-2 have columns 64 c + digit, the last operand has columns
 // 16 (s1 / 4) + 8 (c / 2) + 2 (s1 % 4) + c % 2.
 __global__ void __launch_bounds__(k4CoreThreads, 2) tc_core_kernel(const TcCoreParams p) {
+  after_previous();
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* Fsm = smem;
   unsigned char* Bsm = smem + k4FBytes;
@@ -445,6 +446,7 @@ struct TcOutParams {
 // results arrive ready for the inverse radix-R step (conjugated, scaled, times conj(W_n^{k1 t'})).
 template <int R, bool F16>
 __global__ void __launch_bounds__(256, 3) tc_out_kernel(const TcOutParams p) {
+  after_previous();
   constexpr int NT = 512 / R;
   extern __shared__ __align__(128) uint32_t stage[];            // [R][NT][D/2 words]
   const int nblk = 4096 / NT;
@@ -531,6 +533,7 @@ struct TcSpecParams {
 
 // one CTA per head of the group: m for all its R units
 __global__ void __launch_bounds__(256) tc_gate_amax_kernel(const TcSpecParams p) {
+  after_previous();
   __shared__ float red[8];
   const float2* g = p.g + (size_t)(p.slab0 + blockIdx.x) * p.K;
   float m = 0.f;
@@ -595,6 +598,7 @@ __device__ __forceinline__ void spec_in_bins(const TcSpecParams& p, const float4
 }
 
 __global__ void __launch_bounds__(256, 3) tc_spec_in_kernel(const TcSpecParams p) {
+  after_previous();
   extern __shared__ __align__(16) uint32_t spec_stage[];        // [D / 2][kSpecPitch]
   const int tid = threadIdx.x, warp = tid >> 5, l = tid & 31;
   const int j = blockIdx.x & 15, sk = blockIdx.x >> 4;
@@ -697,7 +701,7 @@ static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
   SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_core_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, k4CoreSmem));
   int grid = 2 * ctx->sm_count;                     // two resident CTAs per SM, a contiguous range of units each
   if ((size_t)grid > nunits) grid = (int)nunits;
-  tc_core_kernel<<<grid, k4CoreThreads, k4CoreSmem, st>>>(cp);
+  SPECTRE_CUDA_OK(launch_after(tc_core_kernel, grid, k4CoreThreads, k4CoreSmem, st, cp));
   SPECTRE_LAUNCH_OK("tc_core_kernel");
 
   if (tc32_out) return launch_tc_out32(ctx, st, ws_out, y, n, slab0, cnt);
@@ -707,7 +711,7 @@ static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
   const size_t smem_out = (size_t)R * NT * (D / 2) * 4;
   if (smem_out > 48 * 1024)
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_out_kernel<R, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_out));
-  tc_out_kernel<R, F16><<<cnt * (4096 / NT), 256, smem_out, st>>>(op);
+  SPECTRE_CUDA_OK(launch_after(tc_out_kernel<R, F16>, cnt * (4096 / NT), 256, smem_out, st, op));
   SPECTRE_LAUNCH_OK("tc_out_kernel");
   return SPECTRE_OK;
 }
@@ -771,10 +775,10 @@ static int tc4k_readout_group(const spectre_ctx* ctx, cudaStream_t st, const flo
 
   TcSpecParams sp = {reinterpret_cast<const float2*>(spec), reinterpret_cast<const float2*>(g), ws_in, gscale,
                      n, n / 2 + 1, R, D, ntile, slab0, in_scale(R) / 64.0f};
-  tc_gate_amax_kernel<<<cnt, 256, 0, st>>>(sp);
+  SPECTRE_CUDA_OK(launch_after(tc_gate_amax_kernel, cnt, 256, 0, st, sp));
   SPECTRE_LAUNCH_OK("tc_gate_amax_kernel");
   const size_t smem_spec = (size_t)(D / 2) * kSpecPitch * 4;
-  tc_spec_in_kernel<<<cnt * R * 16, 256, smem_spec, st>>>(sp);
+  SPECTRE_CUDA_OK(launch_after(tc_spec_in_kernel, cnt * R * 16, 256, smem_spec, st, sp));
   SPECTRE_LAUNCH_OK("tc_spec_in_kernel");
 
   TcCoreParams cp = {ws_in, gimg, ws_out, reinterpret_cast<const __half*>(ctx->dft64),
@@ -784,7 +788,7 @@ static int tc4k_readout_group(const spectre_ctx* ctx, cudaStream_t st, const flo
   SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_core_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, k4CoreSmem));
   int grid = 2 * ctx->sm_count;
   if ((size_t)grid > nunits) grid = (int)nunits;
-  tc_core_kernel<<<grid, k4CoreThreads, k4CoreSmem, st>>>(cp);
+  SPECTRE_CUDA_OK(launch_after(tc_core_kernel, grid, k4CoreThreads, k4CoreSmem, st, cp));
   SPECTRE_LAUNCH_OK("tc_core_kernel");
 
   if (R >= 2 && tc32_out_supported(ctx, y, n)) return launch_tc_out32(ctx, st, ws_out, y, n, slab0, cnt);
@@ -794,7 +798,7 @@ static int tc4k_readout_group(const spectre_ctx* ctx, cudaStream_t st, const flo
   const size_t smem_out = (size_t)R * NT * (D / 2) * 4;
   if (smem_out > 48 * 1024)
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_out_kernel<R, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_out));
-  tc_out_kernel<R, F16><<<cnt * (4096 / NT), 256, smem_out, st>>>(op);
+  SPECTRE_CUDA_OK(launch_after(tc_out_kernel<R, F16>, cnt * (4096 / NT), 256, smem_out, st, op));
   SPECTRE_LAUNCH_OK("tc_out_kernel");
   return SPECTRE_OK;
 }
