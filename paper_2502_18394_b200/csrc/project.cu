@@ -26,6 +26,8 @@ template <> __device__ __forceinline__ float pj_wload<bf16>(const bf16* p) { ret
 template <typename WT>
 __global__ void __launch_bounds__(256) proj_weights_kernel(const WT* __restrict__ Wq, const WT* __restrict__ Wv,
                                                            bf16* __restrict__ wt, int H, float* __restrict__ sum_q, size_t nsum) {
+  after_previous();                             // the projection kernel's set-up runs meanwhile
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx < nsum) sum_q[idx] = 0.f;             // the projection kernel adds its token sums into these (no memset node in the stream)
   if (idx >= (size_t)H * 128 * 64) return;
@@ -94,6 +96,7 @@ __global__ void __launch_bounds__(kPpThreads, 1) project_qv_persistent_kernel(co
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  after_previous();
   const int per = (p.nitems + (int)gridDim.x - 1) / (int)gridDim.x;
   const int i0 = (int)blockIdx.x * per, i1 = min(p.nitems, i0 + per);
   bool ok = true;
@@ -305,11 +308,11 @@ extern "C" int spectre_project_qv(spectre_ctx* ctx, void* stream, const spectre_
   const size_t nsum = sum_q ? (size_t)x->B * x->H * 64 : 0, nw = (size_t)x->H * 128 * 64;
   const unsigned wblocks = (unsigned)(((nsum > nw ? nsum : nw) + 255) / 256);
   if (wdtype == SPECTRE_BF16)
-    proj_weights_kernel<bf16><<<wblocks, 256, 0, st>>>(reinterpret_cast<const bf16*>(Wq), reinterpret_cast<const bf16*>(Wv), wt, x->H,
-                                                       sum_q, nsum);
+    SPECTRE_CUDA_OK(launch_after(proj_weights_kernel<bf16>, wblocks, 256, 0, st, reinterpret_cast<const bf16*>(Wq),
+                                 reinterpret_cast<const bf16*>(Wv), wt, x->H, sum_q, nsum));
   else
-    proj_weights_kernel<float><<<wblocks, 256, 0, st>>>(reinterpret_cast<const float*>(Wq), reinterpret_cast<const float*>(Wv), wt, x->H,
-                                                        sum_q, nsum);
+    SPECTRE_CUDA_OK(launch_after(proj_weights_kernel<float>, wblocks, 256, 0, st, reinterpret_cast<const float*>(Wq),
+                                 reinterpret_cast<const float*>(Wv), wt, x->H, sum_q, nsum));
   SPECTRE_LAUNCH_OK("proj_weights_kernel");
   if (tensor_map_encoder() == nullptr) return fail(SPECTRE_ERR_UNSUPPORTED, "the driver does not provide cuTensorMapEncodeTiled");
   CUtensorMap tm_x, tm_q, tm_v;
@@ -320,7 +323,7 @@ extern "C" int spectre_project_qv(spectre_ctx* ctx, void* stream, const spectre_
   ProjPersistParams pp = {wt, sum_q, x->H, tiles, (int)((size_t)x->B * x->H * tiles), ctx->status_dev};
   SPECTRE_CUDA_OK(cudaFuncSetAttribute(project_qv_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPpSmem));
   const int grid = pp.nitems < ctx->sm_count ? pp.nitems : ctx->sm_count;
-  project_qv_persistent_kernel<<<grid, kPpThreads, kPpSmem, st>>>(tm_x, tm_q, tm_v, pp);
+  SPECTRE_CUDA_OK(launch_after(project_qv_persistent_kernel, grid, kPpThreads, kPpSmem, st, tm_x, tm_q, tm_v, pp));
   SPECTRE_LAUNCH_OK("project_qv_persistent_kernel");
   return SPECTRE_OK;
 }
