@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(256) gate_grad_sum_kernel(const float2* __rest
 // ws[slab_local][k][D/2] (transforms that fit one CTA).
 __global__ void __launch_bounds__(256) gate_grad_kernel(const float2* __restrict__ wsV, const float2* __restrict__ wsG,
                                                         float2* __restrict__ dg, int n, int K, int D, int slab0, int nslab) {
+  after_previous();
   const size_t wid = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (wid >= (size_t)nslab * K) return;
@@ -269,7 +270,8 @@ extern "C" int spectre_mixer_backward(spectre_ctx* ctx, void* stream, const spec
       switch (N1) {
         case 1: {
           const size_t nwarps = (size_t)cnt * K;
-          gate_grad_kernel<<<(unsigned)((nwarps * 32 + 255) / 256), 256, 0, st>>>(wsV, wsG, dgc, n_fft, (int)K, D, s0, cnt);
+          SPECTRE_CUDA_OK(launch_after(gate_grad_kernel, (unsigned)((nwarps * 32 + 255) / 256), 256, 0, st, wsV, wsG, dgc, n_fft, (int)K,
+                                       D, s0, cnt));
           break;
         }
         case 2: launch_gate_grad_combine<2>(st, wsV, wsG, dgc, n_fft, (int)K, D, M, s0, cnt); break;

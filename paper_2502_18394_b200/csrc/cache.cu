@@ -34,6 +34,7 @@ __device__ __forceinline__ void store_split(float* __restrict__ prefix, size_t s
 constexpr int kSplitBins = 4;
 __global__ void __launch_bounds__(256) split_kernel(const float2* __restrict__ ws, float* __restrict__ prefix, int n,
                                                     int K, int D, int slab0, int nslab) {
+  after_previous();
   const int half = D / 2;
   const int kblocks = (K + kSplitBins - 1) / kSplitBins;
   const size_t total = (size_t)nslab * kblocks * half;
@@ -120,6 +121,7 @@ constexpr int kRingRows = 8;
 template <typename T>
 __global__ void __launch_bounds__(256) ring_fill_kernel(const T* __restrict__ src, int64_t sb, int64_t sl, int64_t sh,
                                                         T* __restrict__ buf, int B, int N, int H, int D, int L) {
+  after_previous();
   constexpr int V = 16 / sizeof(T);
   const int vec_per_row = H * D / V;
   const int chunks = (N + kRingRows - 1) / kRingRows;
@@ -147,6 +149,7 @@ __global__ void __launch_bounds__(256) append_spectrum_kernel(float* __restrict_
                                                               const T* __restrict__ v_t, int H, int D, int N, int K,
                                                               int slot, unsigned tm, int evict, int warps_per_slab,
                                                               size_t nwarps_total) {
+  after_previous();
   const size_t wid = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (wid >= nwarps_total) return;
@@ -201,6 +204,7 @@ __global__ void __launch_bounds__(256) append_ring_kernel(T* __restrict__ V_buf,
                                                           float* __restrict__ sum_q, const T* __restrict__ q_t,
                                                           const T* __restrict__ v_t, int B, int H, int D, int N,
                                                           int slot, int evict) {
+  after_previous();
   const int total = B * H * D;
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= total) return;
@@ -223,6 +227,7 @@ __global__ void __launch_bounds__(256) decode_ring_kernel(T* __restrict__ V_buf,
                                                           int* __restrict__ done, const T* __restrict__ q_t,
                                                           const T* __restrict__ v_t, int B, int H, int D, int N, int slot,
                                                           int evict) {
+  after_previous();                                       // first: the spectrum pass behind the gate reads bins without a wait of its own
   asm volatile("griddepcontrol.launch_dependents;");      // the gate kernel behind streams weights before it needs sum_q
   const int total = B * H * D;
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -436,7 +441,7 @@ extern "C" int spectre_prefix_cache_prefill(spectre_ctx* ctx, void* stream, cons
     switch (N1) {
       case 1: {
         size_t total = (size_t)cnt * ((K + kSplitBins - 1) / kSplitBins) * (D / 2);
-        split_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(ws, cache->prefix_fft, N, K, D, s0, cnt);
+        SPECTRE_CUDA_OK(launch_after(split_kernel, (unsigned)((total + 255) / 256), 256, 0, st, ws, cache->prefix_fft, N, K, D, s0, cnt));
         break;
       }
       case 2: launch_combine_split<2>(st, ws, cache->prefix_fft, N, K, D, M, s0, cnt); break;
@@ -453,8 +458,8 @@ extern "C" int spectre_prefix_cache_prefill(spectre_ctx* ctx, void* stream, cons
   unsigned blocks = (unsigned)nblocks;
   if (!v_ring_done) {
     SPECTRE_IO_DISPATCH(cache->buf_dtype, {
-      ring_fill_kernel<T><<<blocks, 256, 0, st>>>(reinterpret_cast<const T*>(v->ptr), v->stride_b, v->stride_l, v->stride_h,
-                                                  reinterpret_cast<T*>(cache->V_buf), B, N, H, D, v->L);
+      SPECTRE_CUDA_OK(launch_after(ring_fill_kernel<T>, blocks, 256, 0, st, reinterpret_cast<const T*>(v->ptr), v->stride_b, v->stride_l,
+                                   v->stride_h, reinterpret_cast<T*>(cache->V_buf), B, N, H, D, v->L));
     });
     SPECTRE_LAUNCH_OK("ring_fill_kernel");
   }
@@ -481,12 +486,12 @@ extern "C" int spectre_prefix_cache_append(spectre_ctx* ctx, void* stream, const
   const unsigned blocks = (unsigned)((nwarps * 32 + 255) / 256);
   const unsigned blocks2 = (unsigned)(((size_t)B * H * D + 255) / 256);
   SPECTRE_IO_DISPATCH(cache->buf_dtype, {
-    append_spectrum_kernel<T><<<blocks, 256, 0, st>>>(cache->prefix_fft, reinterpret_cast<const T*>(cache->V_buf),
-                                                      reinterpret_cast<const T*>(v_t), H, D, N, K, slot, (unsigned)slot,
-                                                      evict, wps, nwarps);
-    append_ring_kernel<T><<<blocks2, 256, 0, st>>>(reinterpret_cast<T*>(cache->V_buf), reinterpret_cast<T*>(cache->Q_buf),
-                                                   cache->sum_q, reinterpret_cast<const T*>(q_t),
-                                                   reinterpret_cast<const T*>(v_t), B, H, D, N, slot, evict);
+    SPECTRE_CUDA_OK(launch_after(append_spectrum_kernel<T>, blocks, 256, 0, st, cache->prefix_fft,
+                                 reinterpret_cast<const T*>(cache->V_buf), reinterpret_cast<const T*>(v_t), H, D, N, K, slot,
+                                 (unsigned)slot, evict, wps, nwarps));
+    SPECTRE_CUDA_OK(launch_after(append_ring_kernel<T>, blocks2, 256, 0, st, reinterpret_cast<T*>(cache->V_buf),
+                                 reinterpret_cast<T*>(cache->Q_buf), cache->sum_q, reinterpret_cast<const T*>(q_t),
+                                 reinterpret_cast<const T*>(v_t), B, H, D, N, slot, evict));
   });
   SPECTRE_LAUNCH_OK("append kernels");
   return SPECTRE_OK;
@@ -540,9 +545,10 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   // (a)-(b) ring buffers, running sum, delta
   const unsigned blocks_r = (unsigned)(((size_t)B * H * D + 255) / 256);
   SPECTRE_IO_DISPATCH(cache->buf_dtype,
-                      decode_ring_kernel<T><<<blocks_r, 256, 0, st>>>(reinterpret_cast<T*>(cache->V_buf), reinterpret_cast<T*>(cache->Q_buf),
-                                                                      cache->sum_q, delta, done, reinterpret_cast<const T*>(q_t),
-                                                                      reinterpret_cast<const T*>(v_t), B, H, D, N, slot, evict));
+                      SPECTRE_CUDA_OK(launch_after(decode_ring_kernel<T>, blocks_r, 256, 0, st, reinterpret_cast<T*>(cache->V_buf),
+                                                   reinterpret_cast<T*>(cache->Q_buf), cache->sum_q, delta, done,
+                                                   reinterpret_cast<const T*>(q_t), reinterpret_cast<const T*>(v_t), B, H, D, N, slot,
+                                                   evict)));
   SPECTRE_LAUNCH_OK("decode_ring_kernel");
   // (c)-(d) gate from the running sum with phase p = t
   rc = spectre_gate(ctx, stream, nullptr, cache->sum_q, B, H, D, 1.0f / (float)N, params, N, nullptr, t, g_out, nullptr,

@@ -36,6 +36,7 @@ __device__ __forceinline__ void wavelet_pass_through(const WaveletParams& p, int
 
 template <typename T, typename WT>
 __global__ void __launch_bounds__(256) wavelet_kernel(const WaveletParams p) {
+  after_previous();
   extern __shared__ float smw[];
   float* tile = smw;                               // [rows][D]
   float* sg = tile + (size_t)p.rows * p.D;         // [(J+1)][D]  holds 1 + s
@@ -146,6 +147,7 @@ template <> struct pair_io<float> {
 
 template <typename T, typename WT, int J>
 __global__ void __launch_bounds__(256) wavelet_reg_kernel(const WaveletParams p) {
+  after_previous();
   extern __shared__ float smw[];
   float* sg = smw;                                 // [(J+1)][D]  holds 1 + s
   float* u = sg + (size_t)(J + 1) * p.D;           // [hidden]
@@ -217,10 +219,10 @@ __global__ void __launch_bounds__(256) wavelet_reg_kernel(const WaveletParams p)
 template <typename T, typename WT>
 static int launch_wavelet_reg(const WaveletParams& p, int J, unsigned grid, size_t smem, cudaStream_t st) {
   switch (J) {
-    case 1: wavelet_reg_kernel<T, WT, 1><<<grid, 256, smem, st>>>(p); break;
-    case 2: wavelet_reg_kernel<T, WT, 2><<<grid, 256, smem, st>>>(p); break;
-    case 3: wavelet_reg_kernel<T, WT, 3><<<grid, 256, smem, st>>>(p); break;
-    default: wavelet_reg_kernel<T, WT, 4><<<grid, 256, smem, st>>>(p); break;
+    case 1: SPECTRE_CUDA_OK(launch_after(wavelet_reg_kernel<T, WT, 1>, grid, 256, smem, st, p)); break;
+    case 2: SPECTRE_CUDA_OK(launch_after(wavelet_reg_kernel<T, WT, 2>, grid, 256, smem, st, p)); break;
+    case 3: SPECTRE_CUDA_OK(launch_after(wavelet_reg_kernel<T, WT, 3>, grid, 256, smem, st, p)); break;
+    default: SPECTRE_CUDA_OK(launch_after(wavelet_reg_kernel<T, WT, 4>, grid, 256, smem, st, p)); break;
   }
   SPECTRE_LAUNCH_OK("wavelet_reg_kernel");
   return SPECTRE_OK;
@@ -298,7 +300,7 @@ extern "C" int spectre_wavelet_refine(spectre_ctx* ctx, void* stream, const spec
     if (smem > 48 * 1024)                                                                                       \
       SPECTRE_CUDA_OK(cudaFuncSetAttribute(wavelet_kernel<T, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
                                            (int)smem));                                                         \
-    wavelet_kernel<T, WT><<<grid, 256, smem, st>>>(p);                                                          \
+    SPECTRE_CUDA_OK(launch_after(wavelet_kernel<T, WT>, grid, 256, smem, st, p));                               \
   } while (0)
   SPECTRE_IO_DISPATCH(y_in->dtype, {
     if (wbf) SPECTRE_WAVELET_LAUNCH(T, bf16);
