@@ -19,8 +19,8 @@ namespace spectre {
 // [H*D] row, so a warp reads 512 contiguous bytes of a row; the CTA's 8 warps take rows 8 apart with
 // up to 8 rows per thread in flight and four CTAs per SM.  The warps' partial sums meet in shared memory, and the CTA adds
 // one value per channel with float atomics into copy (slice mod ncopy) of sums[ncopy][B,H,D] (zeroed
-// by the caller on the same stream), which keeps the contention per address low; a CTA that holds the
-// whole sequence stores its sums instead.
+// by the caller on the same stream), which keeps the contention per address low; where there are as many copies
+// as slices it stores its sums instead.
 template <typename T> struct vec8;
 template <> struct vec8<bf16> {
   typedef uint4 raw;
@@ -80,6 +80,8 @@ __global__ void __launch_bounds__(256, 4) pool_kernel(const T* __restrict__ q, i
                                                    float* __restrict__ sums, T* __restrict__ ring, int N,
                                                    const char* __restrict__ warm, unsigned warm_per, size_t warm_bytes) {
   __shared__ float red[8][8][32];                              // [warp][channel][lane]
+  const bool own = (int)gridDim.y <= ncopy;                    // a copy of the sums per slice: stored, nothing was cleared
+  if (own) after_previous();
   // the gate kernels behind this one may start early: they stream weights before they need the sums
   asm volatile("griddepcontrol.launch_dependents;");
   constexpr int R = vec8<T>::kRows;
@@ -118,12 +120,12 @@ __global__ void __launch_bounds__(256, 4) pool_kernel(const T* __restrict__ q, i
   float s = 0.f;                                               // thread (channel = warp, lane) adds up the 8 warps
 #pragma unroll
   for (int w = 0; w < 8; ++w) s += red[w][warp][lane];
-  // with several slices the kernel runs as the programmatic dependent of the kernel that clears the sums:
+  // with more slices than copies the kernel runs as the programmatic dependent of the kernel that clears the sums:
   // everything above overlaps it, the additions wait for it (no effect in an ordinary launch)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (live) {
     float* dst = sums + (size_t)(blockIdx.y % ncopy) * copy_stride + ((size_t)b * H + h) * D + c + warp;
-    if (gridDim.y == 1) *dst = s;                              // the only slice: no other CTA adds to this address
+    if (own) *dst = s;
     else atomicAdd(dst, s);
   }
 }
@@ -151,8 +153,15 @@ static int pool_launch(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
   if (slices < 1) slices = 1;
   int rows_per = (int)((rows + slices - 1) / slices);
   if (rows_per < 8) rows_per = 8;
-  const int nslice = (rows + rows_per - 1) / rows_per;
-  int ncopy = (nslice + 15) / 16;                              // <= 16 CTAs add into one address
+  int nslice = (rows + rows_per - 1) / rows_per;
+  // Sequences of up to 1024 rows: a slice per copy instead, stored without a kernel that clears them (2 us of host time, and
+  // the second's launch; one warp's 16 rows take 2 or 4 rounds of loads)
+  if (nslice > 8 && ncopy_max >= 8 && rows <= 1024) {
+    rows_per = (rows + 7) / 8;
+    nslice = (rows + rows_per - 1) / rows_per;
+  }
+  const bool own = nslice <= ncopy_max && nslice <= 8;
+  int ncopy = own ? nslice : (nslice + 15) / 16;               // <= 16 CTAs add into one address
   if (ncopy > 8) ncopy = 8;                                    // one batch of loads for the consumer
   if (ncopy > ncopy_max) ncopy = ncopy_max;
   if (ncopy < 1) ncopy = 1;
@@ -168,15 +177,14 @@ static int pool_launch(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
   cfg.blockDim = dim3(256);
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = 0;
-  if (nslice > 1) {
+  cfg.numAttrs = 1;
+  if (!own) {
     const size_t n4 = copy_stride * ncopy / 4;
     if ((reinterpret_cast<uintptr_t>(sums) & 15) || (copy_stride * ncopy) % 4) {
       SPECTRE_CUDA_OK(cudaMemsetAsync(sums, 0, copy_stride * ncopy * sizeof(float), st));
+      cfg.numAttrs = 0;
     } else {
       SPECTRE_CUDA_OK(launch_after(pool_clear_kernel, (unsigned)((n4 + 255) / 256), 256, 0, st, reinterpret_cast<float4*>(sums), n4));
-      SPECTRE_LAUNCH_OK("pool_clear_kernel");
-      cfg.numAttrs = 1;
     }
   }
   // Whole 16-byte pieces of `warm` per CTA into L2 on the side
@@ -655,6 +663,69 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
   }
 }
 
+// ---- the whole gate of one batch entry when its CTAs leave room ----
+// kParts threads share a bin, each with kRows rows of W2: with the usual 64 hidden units every weight is requested ahead of the
+// wait for the sums, where gate_out_kernel's thread takes 2 (bf16) or 4 (fp32) dependent rounds of loads.  The chain behind the wait is
+// all that is left.
+template <typename WT>
+__global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams p) {
+  constexpr int R = wraw<WT>::kRows, kParts = 64 / R, kBins = 256 / kParts;
+  extern __shared__ __align__(16) float u[];       // [hidden], q_bar [D], W1, gamma, beta, b1
+  __shared__ float2 part[kParts][kBins];
+  asm volatile("griddepcontrol.launch_dependents;");
+  const int h = blockIdx.y % p.H, b = blockIdx.y / p.H;
+  const int q = threadIdx.x / kBins, t = threadIdx.x % kBins, k = blockIdx.x * kBins + t, kc = min(k, p.K - 1);
+  const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
+  const WT* col = reinterpret_cast<const WT*>(p.W2) + h * p.hs_w2 + 2 * (size_t)kc;
+  const size_t ld = 2 * (size_t)p.K;
+  WT* w1s = reinterpret_cast<WT*>(u + ((p.hidden + p.D + 3) & ~3));
+  const float* vec = reinterpret_cast<const float*>(w1s + p.D * p.hidden);
+  typename wraw<WT>::type w[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) w[i] = wraw<WT>::load(col + (size_t)min(q * R + i, p.hidden - 1) * ld);
+  const float2 b2 = make_float2(__ldg(p.b2 + h * p.hs_b2 + 2 * kc), __ldg(p.b2 + h * p.hs_b2 + 2 * kc + 1));
+  const float bias = (!p.post && p.modrelu_bias) ? __ldg(p.modrelu_bias + h * p.hs_mb + kc) : 0.f;
+  if (p.stage_w1) stage_mlp(W1, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D, p.hidden, w1s);
+  asm volatile("griddepcontrol.wait;" ::: "memory");         // the sums come from the kernel before
+  float* qbar = u + p.hidden;
+  const float* sums = p.sums + ((size_t)b * p.H + h) * p.D;
+  if (p.stage_w1)
+    descriptor_and_hidden<WT, 1, true>(sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, vec, vec + p.D,
+                                       p.eps, w1s, vec + 2 * p.D, qbar, u, 1);
+  else
+    descriptor_and_hidden<WT, 1, false>(sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden,
+                                        p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, W1, p.b1 + h * p.hs_b1, qbar, u, 1);
+  if (p.qbar_out && blockIdx.x == 0)
+    for (int c = threadIdx.x; c < p.D; c += blockDim.x) p.qbar_out[((size_t)b * p.H + h) * p.D + c] = qbar[c];
+  float2 acc = make_float2(0.f, 0.f);
+  for (int j0 = q * R; j0 < p.hidden; j0 += kParts * R) {
+    if (j0 != q * R) {                                       // more than 64 hidden units
+#pragma unroll
+      for (int i = 0; i < R; ++i) w[i] = wraw<WT>::load(col + (size_t)min(j0 + i, p.hidden - 1) * ld);
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      if (j0 + i < p.hidden) {
+        const float2 wv = wraw<WT>::cvt(w[i]);
+        const float uv = u[j0 + i];
+        acc.x = fmaf(uv, wv.x, acc.x);
+        acc.y = fmaf(uv, wv.y, acc.y);
+      }
+    }
+  }
+  part[q][t] = acc;
+  __syncthreads();
+  if (q > 0 || k >= p.K) return;
+  acc = b2;
+#pragma unroll
+  for (int i = 0; i < kParts; ++i) acc = cadd(acc, part[i][t]);
+  if (!p.post) {
+    if (p.modrelu_bias) acc = modrelu(acc, bias);
+    acc = cmul(acc, p.shift ? phase_factor(k, p.n, p.shift_all + p.shift[b]) : phase_reduced(k, p.n, p.pm_all));
+  }
+  p.g_out[((size_t)b * p.H + h) * p.K + k] = acc;
+}
+
 // ---- the whole gate of a short transform, several batch entries ----
 // One CTA per head and BB entries, one bin per thread.  All of a head's weights go to shared memory (cp.async) ahead of the wait
 // for the sums.  What bounds it is the chain of short phases behind that wait, and in a chain of kernels the first pass over
@@ -1060,6 +1131,12 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
     cfg_mma.gridDim = dim3((unsigned)(fit < 1 ? 1 : (blocks < fit ? blocks : fit)), grid_out.y, 1);
     cfg_mma.blockDim = dim3(256, 1, 1);
   }
+  // One entry per CTA and 2 (bf16) or 4 (fp32) threads per bin where every CTA has an SM to itself (1024 points, 2 heads, fp32: the chain
+  // of three kernels 14.0 -> 12.8 us); with three CTAs per SM they crowd out the kernel behind (4k decode step 16.6 -> 19.0)
+  const int split_bins = wb ? 128 : 64;
+  const bool split = BB == 1 && !pre && (long long)((K + split_bins - 1) / split_bins) * B * H <= ctx->sm_count;
+  cudaLaunchConfig_t cfg_split = cfg_out;
+  cfg_split.gridDim = dim3((unsigned)((K + split_bins - 1) / split_bins), (unsigned)(B * H), 1); cfg_split.blockDim = dim3(256, 1, 1);
   cudaLaunchConfig_t cfg_short = cfg_out;
   cfg_short.gridDim = dim3(grid_out.y, 1, 1); cfg_short.dynamicSmemBytes = short_bytes;
 #define SPECTRE_GATE_LAUNCH(WT, NB)                                                              \
@@ -1081,6 +1158,8 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   } else if (all_staged) {
     if (wb) SPECTRE_CUDA_OK(BB == 8 ? cudaLaunchKernelEx(&cfg_short, gate_short_kernel<bf16, 8>, mp) : cudaLaunchKernelEx(&cfg_short, gate_short_kernel<bf16, 4>, mp));
     else SPECTRE_CUDA_OK(BB == 8 ? cudaLaunchKernelEx(&cfg_short, gate_short_kernel<float, 8>, mp) : cudaLaunchKernelEx(&cfg_short, gate_short_kernel<float, 4>, mp));
+  } else if (split) {
+    SPECTRE_CUDA_OK(wb ? cudaLaunchKernelEx(&cfg_split, gate_split_kernel<bf16>, mp) : cudaLaunchKernelEx(&cfg_split, gate_split_kernel<float>, mp));
   } else switch (BB) {
     case 8: if (wb) SPECTRE_GATE_LAUNCH(bf16, 8); else SPECTRE_GATE_LAUNCH(float, 8); break;
     case 4: if (wb) SPECTRE_GATE_LAUNCH(bf16, 4); else SPECTRE_GATE_LAUNCH(float, 4); break;

@@ -335,6 +335,20 @@ def test_gate_short_transforms(ctx, B, n, D, hid, wdt, r, shifts):
     assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
 
 
+@pytest.mark.parametrize("B,H,L,n,D,hid,wdt,r", [(1, 2, 1024, 1024, 64, 64, "f32", 0), (1, 3, 77, 500, 64, 100, "bf16", 2), (2, 2, 9, 128, 32, 300, "f32", 0),
+                                                 (1, 1, 1, 2, 8, 8, "bf16", 0), (1, 2, 1023, 4094, 64, 64, "bf16", 0), (1, 1, 1025, 1026, 24, 17, "f32", 0)])
+def test_gate_few_blocks(ctx, B, H, L, n, D, hid, wdt, r):
+    # several threads per bin: hidden widths below and above the rows they hold, the last block of bins partial; pooled sums in a
+    # copy per slice up to 1024 rows and beyond
+    w = W.Workload("t", B=B, L=L, H=H, D=D, dtype="bf16", wdtype=wdt, n_fft=n, hidden=hid, seed=n + hid)
+    p = W.gate_params(w, modrelu_bias_std=0.01, toeplitz_r=r, bias_std=0.1)
+    x = W.activations(w, structured=True)
+    qbar = torch.empty(B, H, D, device="cuda")
+    g = S.spectre_gate(ctx, to_dev(p), n, q=x.cuda(), shift_all=11, qbar_out=qbar)
+    ref = O.gate(W.to_f64(x).sum(axis=1), 1.0 / w.L, n, shift=np.full(B, 11, dtype=np.int64), **gate_params_np(p))
+    assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
+
+
 def test_gate_from_running_sum_and_shared_heads(ctx):
     w = W.Workload("t", B=2, L=64, H=4, D=32, dtype="f32", wdtype="f32", n_fft=64, seed=13)
     p = W.gate_params(w)
