@@ -57,13 +57,15 @@ NCU_TRAFFIC_VARIANT = {("c4", "prefill"): (10208e6, "profiles/launches_c4_prefil
                        ("c4", "readout"): (7015e6, "profiles/launches_c4_readout.md (ncu capture at B = 2, x4; not this run)")}
 
 
-def pool_launches(B, rows, H, D, sm_count=148):
-    """Kernels of one pooling pass: the pass itself and, when it runs in several slices of the sequence that add
-    into the same sums (the library's rule, restated), the small kernel that clears them."""
+def pool_launches(B, rows, H, D, sm_count=148, copies=16):
+    """Kernels of one pooling pass: the pass itself and, when it runs in more slices of the sequence than there are
+    copies of the sums to store (the library's rule, restated), the small kernel that clears them."""
     groups = (H * (D // 8) + 31) // 32
     slices = max(1, (4 * sm_count) // (groups * B))
     rows_per = max(8, -(-rows // slices))
-    return 1 + (1 if -(-rows // rows_per) > 1 else 0)
+    if -(-rows // rows_per) > 8 and copies >= 8 and rows <= 1024:
+        rows_per = -(-rows // 8)
+    return 1 + (1 if -(-rows // rows_per) > min(copies, 8) else 0)
 
 
 def gate_launches(w):
