@@ -5,6 +5,8 @@
 //                      stream over W2, 1-8 batch entries per pass; with the Toeplitz update off it also applies modReLU and
 //                      the positional phase
 //   gate_mma_kernel    the same on the tensor cores, several batch entries with bf16 weights
+//   gate_short_kernel  the same for few bins and several batch entries, all weights staged
+//   gate_split_kernel  the same for one batch entry and few bins, several threads per bin
 //   gate_post_kernel Toeplitz update, modReLU, phase (only when r > 0)
 #include "tc_common.cuh"
 
