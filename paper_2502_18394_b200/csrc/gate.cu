@@ -1098,8 +1098,10 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   // batch entries per CTA: the weights of a head are fetched once for all of them
   // Tensor cores for bf16 weights and the usual 64 hidden units (the fragments of A fill the registers): 4 or 8 entries (5 ... 7
   // would need two passes over W2 with 4).  With under 256 bins the 8 warps of its CTAs have no chunk each and the
-  // narrower CTAs below, more of them per SM, are faster (99 bins, 256 entries: 15 us against 16).
-  const bool mma = gp->wdtype == SPECTRE_BF16 && gp->hidden == 64 && K >= 256 && B >= 2;
+  // narrower CTAs below, more of them per SM, are faster (99 bins, 256 entries: 15 us against 16).  It reads a bin's two output
+  // biases as one 8-byte word: an array that starts at an odd float (part of a flat parameter buffer) goes to the kernels that
+  // read single floats.
+  const bool mma = gp->wdtype == SPECTRE_BF16 && gp->hidden == 64 && K >= 256 && B >= 2 && !(reinterpret_cast<uintptr_t>(gp->b2) & 7);
   const int BB = mma ? (B <= 4 ? 4 : 8) : (gp->hidden > 256 || B < 2) ? 1 : (B < 4 ? 2 : (B < 8 ? 4 : 8));
   dim3 grid_out((K + thr_out - 1) / thr_out, (unsigned)(H * ((B + BB - 1) / BB)));
   if (grid_out.y > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "H * ceil(B / 8) exceeds 65535");

@@ -320,6 +320,24 @@ def test_gate_batches_on_tensor_cores(ctx, B, H, n, r, shifts):
     assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
 
 
+@pytest.mark.parametrize("B,n", [(2, 510), (4, 4096), (8, 1000), (9, 32768), (8, 196), (1, 1024)])
+def test_gate_parameters_at_odd_floats_of_a_flat_buffer(ctx, B, n):
+    # the header asks for float pointers only: every fp32 parameter starts 4 bytes past an 8-byte boundary, at shapes of every
+    # output-layer kernel
+    w = W.Workload("t", B=B, L=33, H=2, D=64, dtype="bf16", n_fft=n, seed=n + B)
+    p = W.gate_params(w, modrelu_bias_std=0.01, bias_std=0.1)
+    x = W.activations(w, structured=True)
+    dev = to_dev(p)
+    for k in ("ln_gamma", "ln_beta", "b1", "b2", "modrelu_bias"):
+        flat = torch.empty(dev[k].numel() + 1, device="cuda")
+        flat[1:].copy_(dev[k].reshape(-1))
+        dev[k] = flat[1:].view(dev[k].shape)
+        assert dev[k].data_ptr() % 8 == 4
+    g = S.spectre_gate(ctx, dev, n, q=x.cuda(), shift_all=11)
+    ref = O.gate(W.to_f64(x).sum(axis=1), 1.0 / w.L, n, shift=np.full(B, 11, dtype=np.int64), **gate_params_np(p))
+    assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
+
+
 @pytest.mark.parametrize("B,n,D,hid,wdt,r,shifts", [(4, 2, 64, 64, "bf16", 0, False), (8, 196, 64, 64, "bf16", 0, True), (13, 64, 24, 32, "f32", 2, False),
                                                      (9, 254, 64, 40, "bf16", 0, False), (5, 510, 8, 8, "f32", 0, True), (11, 100, 128, 64, "bf16", 1, False)])
 def test_gate_short_transforms(ctx, B, n, D, hid, wdt, r, shifts):
