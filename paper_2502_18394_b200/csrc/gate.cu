@@ -963,7 +963,7 @@ __global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p)
 
 struct GatePostParams {
   const float2* g_raw; float2* g_out;
-  const float2* taps; size_t hs_t; int r;
+  const float* taps; size_t hs_t; int r;          // (re, im) pairs, read as single floats: the array may start at an odd one
   const float* modrelu_bias; size_t hs_mb;
   const long long* shift; long long shift_all;
   int H, K, n;
@@ -978,11 +978,11 @@ __global__ void __launch_bounds__(256) gate_post_kernel(const GatePostParams p) 
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= p.K) return;
   const float2* g = p.g_raw + (size_t)bh * p.K;
-  const float2* t = p.taps + h * p.hs_t;
+  const float* t = p.taps + 2 * (h * p.hs_t + p.r);
   float2 acc = g[k];
   for (int m = -p.r; m <= p.r; ++m) {
     int src = k - m;
-    if (src >= 0 && src < p.K) acc = cadd(acc, cmul(t[m + p.r], g[src]));
+    if (src >= 0 && src < p.K) acc = cadd(acc, cmul(make_float2(t[2 * m], t[2 * m + 1]), g[src]));
   }
   long long sh = p.shift_all + (p.shift ? p.shift[b] : 0);
   long long pm = sh % p.n; if (pm < 0) pm += p.n;
@@ -1176,7 +1176,7 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   if (r > 0) {
     GatePostParams pp = {};
     pp.g_raw = raw; pp.g_out = reinterpret_cast<float2*>(g_out);
-    pp.taps = reinterpret_cast<const float2*>(gp->toeplitz); pp.hs_t = one * (2 * r + 1); pp.r = r;
+    pp.taps = gp->toeplitz; pp.hs_t = one * (2 * r + 1); pp.r = r;
     pp.modrelu_bias = gp->modrelu_bias; pp.hs_mb = one * K;
     pp.shift = mp.shift; pp.shift_all = shift_all;
     pp.H = H; pp.K = K; pp.n = n_fft;

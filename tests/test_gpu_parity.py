@@ -320,15 +320,15 @@ def test_gate_batches_on_tensor_cores(ctx, B, H, n, r, shifts):
     assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
 
 
-@pytest.mark.parametrize("B,n", [(2, 510), (4, 4096), (8, 1000), (9, 32768), (8, 196), (1, 1024)])
-def test_gate_parameters_at_odd_floats_of_a_flat_buffer(ctx, B, n):
+@pytest.mark.parametrize("B,n,r", [(2, 510, 0), (4, 4096, 0), (8, 1000, 2), (9, 32768, 0), (8, 196, 1), (1, 1024, 0)])
+def test_gate_parameters_at_odd_floats_of_a_flat_buffer(ctx, B, n, r):
     # the header asks for float pointers only: every fp32 parameter starts 4 bytes past an 8-byte boundary, at shapes of every
-    # output-layer kernel
+    # output-layer kernel and in the Toeplitz update
     w = W.Workload("t", B=B, L=33, H=2, D=64, dtype="bf16", n_fft=n, seed=n + B)
-    p = W.gate_params(w, modrelu_bias_std=0.01, bias_std=0.1)
+    p = W.gate_params(w, modrelu_bias_std=0.01, toeplitz_r=r, bias_std=0.1)
     x = W.activations(w, structured=True)
     dev = to_dev(p)
-    for k in ("ln_gamma", "ln_beta", "b1", "b2", "modrelu_bias"):
+    for k in ("ln_gamma", "ln_beta", "b1", "b2", "modrelu_bias") + (("toeplitz",) if r else ()):
         flat = torch.empty(dev[k].numel() + 1, device="cuda")
         flat[1:].copy_(dev[k].reshape(-1))
         dev[k] = flat[1:].view(dev[k].shape)
