@@ -18,7 +18,7 @@ int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
 bool transform_supported(const spectre_ctx* ctx, int n);
 size_t transform_slab_bytes(int n, int D);
 
-__global__ void __launch_bounds__(256) conj_gate_kernel(const float2* __restrict__ g, float2* __restrict__ gc, size_t total) {
+__global__ void __launch_bounds__(256) conj_gate_kernel(const float2* g, float2* gc, size_t total) {
   after_previous();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < total) {
@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(256) conj_gate_kernel(const float2* __restrict
 
 // dg from the partial sums S_k = sum over the pairs of conj(Z^V_k) Z^G_k of all n bins, which the transform kernels
 // leave per group of pairs: dg_k = (w_k / 2n) (S_k + conj(S_{n-k})).
-__global__ void __launch_bounds__(256) gate_grad_sum_kernel(const float2* __restrict__ sums, float2* __restrict__ dg, int n, int K,
+__global__ void __launch_bounds__(256) gate_grad_sum_kernel(const float2* sums, float2* dg, int n, int K,
                                                             int parts, int slab0, int nslab) {
   after_previous();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(256) gate_grad_sum_kernel(const float2* __rest
   float2 acc = make_float2(0.f, 0.f);
 #pragma unroll 4
   for (int p = 0; p < parts; ++p) {
-    const float2 a = __ldg(s + (size_t)p * n + k), b = __ldg(s + (size_t)p * n + km);
+    const float2 a = s[(size_t)p * n + k], b = s[(size_t)p * n + km];
     acc.x += a.x + b.x;
     acc.y += a.y - b.y;
   }
@@ -49,8 +49,8 @@ __global__ void __launch_bounds__(256) gate_grad_sum_kernel(const float2* __rest
 
 // One warp per (slab, bin): lanes over the column pairs, both workspaces hold the spectrum itself,
 // ws[slab_local][k][D/2] (transforms that fit one CTA).
-__global__ void __launch_bounds__(256) gate_grad_kernel(const float2* __restrict__ wsV, const float2* __restrict__ wsG,
-                                                        float2* __restrict__ dg, int n, int K, int D, int slab0, int nslab) {
+__global__ void __launch_bounds__(256) gate_grad_kernel(const float2* wsV, const float2* wsG,
+                                                        float2* dg, int n, int K, int D, int slab0, int nslab) {
   after_previous();
   const size_t wid = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -84,8 +84,8 @@ __global__ void __launch_bounds__(256) gate_grad_kernel(const float2* __restrict
 // exchange between the halves.  Bound by HBM; with both families and tensors in one lane (256 registers of spectra at
 // N1 = 8) the pass over 134 MB took 43 us.
 template <int N1>
-__global__ void __launch_bounds__(256, N1 <= 8 ? 2 : 1) gate_grad_combine_kernel(const float2* __restrict__ wsV, const float2* __restrict__ wsG,
-                                                                float2* __restrict__ dg, int n, int K, int D, int M,
+__global__ void __launch_bounds__(256, N1 <= 8 ? 2 : 1) gate_grad_combine_kernel(const float2* wsV, const float2* wsG,
+                                                                float2* dg, int n, int K, int D, int M,
                                                                 int slab0, int nslab) {
   after_previous();
   const size_t wid = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;

@@ -19,7 +19,7 @@ int inverse_from_spectrum(const spectre_ctx* ctx, cudaStream_t st, const float* 
 // With Z = fft_n(a + jb) for each column pair (a, b), the half spectra of the two real columns follow
 // from Hermitian symmetry (App. B):
 //   A_k = (Z_k + conj(Z_{n-k})) / 2,   B_k = (Z_k - conj(Z_{n-k})) / (2j).
-__device__ __forceinline__ void store_split(float* __restrict__ prefix, size_t slab, int K, int D, int k, int c, float2 z,
+__device__ __forceinline__ void store_split(float* prefix, size_t slab, int K, int D, int k, int c, float2 z,
                                             float2 zm) {
   float4 out;
   out.x = 0.5f * (z.x + zm.x);
@@ -32,7 +32,7 @@ __device__ __forceinline__ void store_split(float* __restrict__ prefix, size_t s
 // Transforms that fit the on-chip kernel (N1 = 1) leave Z in ws[slab_local][k][D/2].  A thread takes
 // kSplitBins consecutive bins of one column pair, all their loads in flight together.
 constexpr int kSplitBins = 4;
-__global__ void __launch_bounds__(256) split_kernel(const float2* __restrict__ ws, float* __restrict__ prefix, int n,
+__global__ void __launch_bounds__(256) split_kernel(const float2* ws, float* prefix, int n,
                                                     int K, int D, int slab0, int nslab) {
   after_previous();
   const int half = D / 2;
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(256) split_kernel(const float2* __restrict__ w
 // M - k2 of one column pair holds both sides of every Hermitian pair it stores: the bins k2 + M k1 and
 // (M - k2) + M k1 for k1 < N1/2 (and, at k2 = 0, bin n/2); the packed spectrum never goes back to memory.
 template <int N1>
-__global__ void __launch_bounds__(256) combine_split_kernel(const float2* __restrict__ ws, float* __restrict__ prefix, int n,
+__global__ void __launch_bounds__(256) combine_split_kernel(const float2* ws, float* prefix, int n,
                                                             int K, int D, int M, int slab0, int nslab) {
   after_previous();
   const int half = D / 2;
@@ -119,8 +119,8 @@ static void launch_combine_split(cudaStream_t st, const float2* ws, float* prefi
 // consecutive rows of one batch entry, a thread one 16-byte piece of each with all of them in flight.
 constexpr int kRingRows = 8;
 template <typename T>
-__global__ void __launch_bounds__(256) ring_fill_kernel(const T* __restrict__ src, int64_t sb, int64_t sl, int64_t sh,
-                                                        T* __restrict__ buf, int B, int N, int H, int D, int L) {
+__global__ void __launch_bounds__(256) ring_fill_kernel(const T* src, int64_t sb, int64_t sl, int64_t sh,
+                                                        T* buf, int B, int N, int H, int D, int L) {
   after_previous();
   constexpr int V = 16 / sizeof(T);
   const int vec_per_row = H * D / V;
@@ -145,8 +145,7 @@ __global__ void __launch_bounds__(256) ring_fill_kernel(const T* __restrict__ sr
 // twiddle of bin k0 + l once, then the warp walks the 32 bins with every lane
 // updating 2 channels (one 16-byte complex pair) of the bin's contiguous row.
 template <typename T>
-__global__ void __launch_bounds__(256) append_spectrum_kernel(float* __restrict__ prefix, const T* __restrict__ V_buf,
-                                                              const T* __restrict__ v_t, int H, int D, int N, int K,
+__global__ void __launch_bounds__(256) append_spectrum_kernel(float* prefix, const T* V_buf, const T* v_t, int H, int D, int N, int K,
                                                               int slot, unsigned tm, int evict, int warps_per_slab,
                                                               size_t nwarps_total) {
   after_previous();
@@ -200,9 +199,8 @@ __global__ void __launch_bounds__(256) append_spectrum_kernel(float* __restrict_
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) append_ring_kernel(T* __restrict__ V_buf, T* __restrict__ Q_buf,
-                                                          float* __restrict__ sum_q, const T* __restrict__ q_t,
-                                                          const T* __restrict__ v_t, int B, int H, int D, int N,
+__global__ void __launch_bounds__(256) append_ring_kernel(T* V_buf, T* Q_buf,
+                                                          float* sum_q, const T* q_t, const T* v_t, int B, int H, int D, int N,
                                                           int slot, int evict) {
   after_previous();
   const int total = B * H * D;
@@ -222,10 +220,9 @@ __global__ void __launch_bounds__(256) append_ring_kernel(T* __restrict__ V_buf,
 // Ring buffers and running sum as in the append, plus delta = v_t - v_old in fp32 for the
 // spectrum pass (which then no longer needs the ring buffer).
 template <typename T>
-__global__ void __launch_bounds__(256) decode_ring_kernel(T* __restrict__ V_buf, T* __restrict__ Q_buf,
-                                                          float* __restrict__ sum_q, float* __restrict__ delta,
-                                                          int* __restrict__ done, const T* __restrict__ q_t,
-                                                          const T* __restrict__ v_t, int B, int H, int D, int N, int slot,
+__global__ void __launch_bounds__(256) decode_ring_kernel(T* V_buf, T* Q_buf,
+                                                          float* sum_q, float* delta,
+                                                          int* done, const T* q_t, const T* v_t, int B, int H, int D, int N, int slot,
                                                           int evict) {
   after_previous();                                       // first: the spectrum pass behind the gate reads bins without a wait of its own
   asm volatile("griddepcontrol.launch_dependents;");      // the gate kernel behind streams weights before it needs sum_q
@@ -257,9 +254,8 @@ struct DecodeRows { int r[SPECTRE_DECODE_MAX_ROWS]; };
 // Bound by HBM (16 bytes per bin and channel).  Launched as a programmatic dependent of the gate kernel: the first bins are
 // on their way before the gate is complete (the spectrum itself was written by kernels in front of the ring kernel).
 template <typename T, int NR>
-__global__ void __launch_bounds__(256) decode_spectrum_kernel(float* __restrict__ prefix, const float* __restrict__ delta,
-                                                              const float2* __restrict__ g, float* __restrict__ partial,
-                                                              int* __restrict__ done, T* __restrict__ y, int H, int D, int N, int K,
+__global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, const float* delta, const float2* g, float* partial,
+                                                              int* done, T* y, int H, int D, int N, int K,
                                                               unsigned tm, DecodeRows rows, int nrows, int nblk) {
   __shared__ float red[8][NR][64];
   __shared__ int last;

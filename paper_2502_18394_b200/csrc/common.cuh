@@ -52,6 +52,11 @@ bool is_pow2(int64_t x);
 int radix_plan(int n, int* radices);
 
 #ifdef __CUDACC__
+// What other kernels write - the caller's tensors and weights, workspaces, cache state - is read by plain loads through pointers
+// without __restrict__.  A kernel of a chain is resident while the one before it still writes, so a const __restrict__ pointer or
+// __ldg, which say that nothing changes while this kernel runs, would let a load go through the read-only path, and any
+// __restrict__ parameter, which says that nothing else reaches that memory, would let it move in front of the wait.  Both are for
+// the context's tables, which nothing writes after spectre_create.
 // A short kernel in a chain: launched as the programmatic dependent of the one before it and waiting for it as its first
 // action, its launch overlaps that kernel's end (2 us less between the two than after an ordinary launch).
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -27,7 +27,7 @@ template <typename T> struct vec8;
 template <> struct vec8<bf16> {
   typedef uint4 raw;
   static constexpr int kRows = 8;
-  static __device__ __forceinline__ raw load(const bf16* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
+  static __device__ __forceinline__ raw load(const bf16* p) { return *reinterpret_cast<const uint4*>(p); }
   static __device__ __forceinline__ raw zero() { return make_uint4(0u, 0u, 0u, 0u); }
   static __device__ __forceinline__ void add(const raw& r, float (&a)[8]) {
     const uint32_t u[4] = {r.x, r.y, r.z, r.w};
@@ -41,7 +41,7 @@ template <> struct vec8<bf16> {
 template <> struct vec8<f16> {
   typedef uint4 raw;
   static constexpr int kRows = 8;
-  static __device__ __forceinline__ raw load(const f16* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
+  static __device__ __forceinline__ raw load(const f16* p) { return *reinterpret_cast<const uint4*>(p); }
   static __device__ __forceinline__ raw zero() { return make_uint4(0u, 0u, 0u, 0u); }
   static __device__ __forceinline__ void add(const raw& r, float (&a)[8]) {
     const uint32_t u[4] = {r.x, r.y, r.z, r.w};
@@ -58,8 +58,8 @@ template <> struct vec8<float> {
   static constexpr int kRows = 4;
   static __device__ __forceinline__ raw load(const float* p) {
     raw r;
-    r.lo = __ldg(reinterpret_cast<const float4*>(p));
-    r.hi = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    r.lo = *reinterpret_cast<const float4*>(p);
+    r.hi = *(reinterpret_cast<const float4*>(p) + 1);
     return r;
   }
   static __device__ __forceinline__ raw zero() {
@@ -77,10 +77,10 @@ template <> struct vec8<float> {
 // RING: the rows also go, as loaded, into the dense copy ring[B][N][H][D]; rows L..N-1 of it are zeroed
 // (the ring buffer of the Prefix-FFT cache, Alg. 1 PreFill), and the slices cover N rows instead of L.
 template <typename T, bool RING>
-__global__ void __launch_bounds__(256, 4) pool_kernel(const T* __restrict__ q, int64_t sb, int64_t sl, int64_t sh, int L,
+__global__ void __launch_bounds__(256, 4) pool_kernel(const T* q, int64_t sb, int64_t sl, int64_t sh, int L,
                                                    int H, int D, int rows_per, int ncopy, size_t copy_stride,
-                                                   float* __restrict__ sums, T* __restrict__ ring, int N,
-                                                   const char* __restrict__ warm, unsigned warm_per, size_t warm_bytes) {
+                                                   float* sums, T* ring, int N,
+                                                   const char* warm, unsigned warm_per, size_t warm_bytes) {
   __shared__ float red[8][8][32];                              // [warp][channel][lane]
   const bool own = (int)gridDim.y <= ncopy;                    // a copy of the sums per slice: stored, nothing was cleared
   if (own) after_previous();
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(256, 4) pool_kernel(const T* __restrict__ q, i
 }
 
 // Clears the partial sums ahead of a pooling pass with several slices; lets that pass start at once.
-__global__ void __launch_bounds__(256) pool_clear_kernel(float4* __restrict__ sums, size_t n4) {
+__global__ void __launch_bounds__(256) pool_clear_kernel(float4* sums, size_t n4) {
   after_previous();                                            // the pass behind reads its rows without a wait of its own
   asm volatile("griddepcontrol.launch_dependents;");
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -227,15 +227,9 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4],
 
 // ---- MLP ---------------------------------------------------------------------
 template <typename WT> __device__ __forceinline__ float wload(const WT* p);
-template <> __device__ __forceinline__ float wload<float>(const float* p) { return __ldg(p); }
+template <> __device__ __forceinline__ float wload<float>(const float* p) { return *p; }
 template <> __device__ __forceinline__ float wload<bf16>(const bf16* p) {
-  return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p)) << 16);
-}
-template <typename WT> __device__ __forceinline__ float2 wload2(const WT* p);
-template <> __device__ __forceinline__ float2 wload2<float>(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
-template <> __device__ __forceinline__ float2 wload2<bf16>(const bf16* p) {
-  unsigned r = __ldg(reinterpret_cast<const unsigned*>(p));
-  return make_float2(__uint_as_float(r << 16), __uint_as_float(r & 0xffff0000u));
+  return __uint_as_float((uint32_t)*reinterpret_cast<const unsigned short*>(p) << 16);
 }
 
 // q_bar = LN(inv_count * sum) into shared memory (Sec. 3.2 step 3a), then the hidden layer
@@ -255,10 +249,10 @@ template <typename WT, bool STAGED> __device__ __forceinline__ float wget(const 
 }
 
 template <typename WT, int NB, bool STAGED>
-__device__ __forceinline__ void descriptor_and_hidden(const float* __restrict__ sums, size_t bstride, int nb, int ncopy,
+__device__ __forceinline__ void descriptor_and_hidden(const float* sums, size_t bstride, int nb, int ncopy,
                                                       size_t copy_stride, float inv_count, int D, int hidden,
-                                                      const float* __restrict__ gamma, const float* __restrict__ beta,
-                                                      float eps, const WT* __restrict__ W1, const float* __restrict__ b1,
+                                                      const float* gamma, const float* beta,
+                                                      float eps, const WT* W1, const float* b1,
                                                       float* qbar, float* u, int ustride) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
   if (NB > 1 && ncopy == 1) {                                // means, one copy: up to 4 channels per thread in flight
@@ -387,9 +381,9 @@ __device__ __forceinline__ void stage_weights(const void* src, void* dst, int by
   const int n16 = bytes >> 4;
   for (int i0 = threadIdx.x; i0 < n16; i0 += 2 * blockDim.x) {
     const int i1 = i0 + (int)blockDim.x;
-    const uint4 v0 = __ldg(s4 + i0);
+    const uint4 v0 = s4[i0];
     uint4 v1 = make_uint4(0u, 0u, 0u, 0u);
-    if (i1 < n16) v1 = __ldg(s4 + i1);
+    if (i1 < n16) v1 = s4[i1];
     d4[i0] = v0;
     if (i1 < n16) d4[i1] = v1;
   }
@@ -402,8 +396,8 @@ __device__ __forceinline__ void copy_async16(const void* src, void* dst, int byt
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(d + i), "l"(reinterpret_cast<const char*>(src) + i) : "memory");
 }
 __device__ __forceinline__ void stage_vectors(const float* gamma, const float* beta, const float* b1, int D, int hidden, float* vec) {
-  for (int i = threadIdx.x; i < D; i += blockDim.x) { vec[i] = __ldg(gamma + i); vec[D + i] = __ldg(beta + i); }
-  for (int i = threadIdx.x; i < hidden; i += blockDim.x) vec[2 * D + i] = __ldg(b1 + i);
+  for (int i = threadIdx.x; i < D; i += blockDim.x) { vec[i] = gamma[i]; vec[D + i] = beta[i]; }
+  for (int i = threadIdx.x; i < hidden; i += blockDim.x) vec[2 * D + i] = b1[i];
 }
 // A head's W1, LayerNorm weights and hidden bias into shared memory: W1, then gamma, beta, b1.  Requested before the wait
 // for the sums, the vectors' round trips are off the chain behind it.
@@ -462,13 +456,13 @@ struct GateMlpParams {
 template <typename WT> struct wraw;
 template <> struct wraw<bf16> {
   typedef unsigned type;
-  static __device__ __forceinline__ type load(const bf16* p) { return __ldg(reinterpret_cast<const unsigned*>(p)); }
+  static __device__ __forceinline__ type load(const bf16* p) { return *reinterpret_cast<const unsigned*>(p); }
   static __device__ __forceinline__ float2 cvt(type r) { return make_float2(__uint_as_float(r << 16), __uint_as_float(r & 0xffff0000u)); }
   static constexpr int kRows = 32;
 };
 template <> struct wraw<float> {
   typedef float2 type;
-  static __device__ __forceinline__ type load(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
+  static __device__ __forceinline__ type load(const float* p) { return *reinterpret_cast<const float2*>(p); }
   static __device__ __forceinline__ float2 cvt(type r) { return r; }
   static constexpr int kRows = 16;
 };
@@ -542,7 +536,7 @@ __device__ __forceinline__ void gate_use_rows(const typename wraw<WT>::type (&wc
   }
 }
 template <typename WT, bool FULL, int N>
-__device__ __forceinline__ void gate_fetch_rows(typename wraw<WT>::type (&wc)[wraw<WT>::kRows], int o, const WT* __restrict__ col,
+__device__ __forceinline__ void gate_fetch_rows(typename wraw<WT>::type (&wc)[wraw<WT>::kRows], int o, const WT* col,
                                                 size_t ld, int j, int hidden) {
   const int nr = FULL ? N : min(N, hidden - j);
 #pragma unroll
@@ -554,7 +548,7 @@ __device__ __forceinline__ void gate_fetch_rows(typename wraw<WT>::type (&wc)[wr
 // the latency of a whole block to show): the two halves of w alternate, each refilled with the rows R
 // further on as soon as it has been used, so R / 2 to R rows are in flight throughout.
 template <typename WT, int BB, bool FULL>
-__device__ __forceinline__ void gate_stream(typename wraw<WT>::type (&w)[wraw<WT>::kRows], const WT* __restrict__ col, size_t ld,
+__device__ __forceinline__ void gate_stream(typename wraw<WT>::type (&w)[wraw<WT>::kRows], const WT* col, size_t ld,
                                             int hidden, const float* __restrict__ u, float2 (&acc)[BB],
                                             uint64_t (&ax)[BB >= 4 ? BB / 2 : 1], uint64_t (&ay)[BB >= 4 ? BB / 2 : 1]) {
   constexpr int R = wraw<WT>::kRows, Hf = R / 2;
@@ -598,8 +592,8 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
       if (i < n0) w[i] = wraw<WT>::load(col + (size_t)i * ld);
   }
   const int kc = live ? k : 0;
-  const float2 b2 = make_float2(__ldg(p.b2 + h * p.hs_b2 + 2 * kc), __ldg(p.b2 + h * p.hs_b2 + 2 * kc + 1));
-  const float bias = (!p.post && p.modrelu_bias) ? __ldg(p.modrelu_bias + h * p.hs_mb + kc) : 0.f;
+  const float2 b2 = make_float2(p.b2[h * p.hs_b2 + 2 * kc], p.b2[h * p.hs_b2 + 2 * kc + 1]);
+  const float bias = (!p.post && p.modrelu_bias) ? p.modrelu_bias[h * p.hs_mb + kc] : 0.f;
   if (!PRE && p.stage_w1)
     stage_mlp(reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D,
               p.hidden, w1s);
@@ -685,8 +679,8 @@ __global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams 
   typename wraw<WT>::type w[R];
 #pragma unroll
   for (int i = 0; i < R; ++i) w[i] = wraw<WT>::load(col + (size_t)min(q * R + i, p.hidden - 1) * ld);
-  const float2 b2 = make_float2(__ldg(p.b2 + h * p.hs_b2 + 2 * kc), __ldg(p.b2 + h * p.hs_b2 + 2 * kc + 1));
-  const float bias = (!p.post && p.modrelu_bias) ? __ldg(p.modrelu_bias + h * p.hs_mb + kc) : 0.f;
+  const float2 b2 = make_float2(p.b2[h * p.hs_b2 + 2 * kc], p.b2[h * p.hs_b2 + 2 * kc + 1]);
+  const float bias = (!p.post && p.modrelu_bias) ? p.modrelu_bias[h * p.hs_mb + kc] : 0.f;
   if (p.stage_w1) stage_mlp(W1, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D, p.hidden, w1s);
   asm volatile("griddepcontrol.wait;" ::: "memory");         // the sums come from the kernel before
   float* qbar = u + p.hidden;
@@ -748,8 +742,8 @@ __global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams 
   asm volatile("cp.async.commit_group;" ::: "memory");
   stage_vectors(p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D, p.hidden, vec);
   const int kc = live ? k : 0;
-  const float2 b2 = make_float2(__ldg(p.b2 + h * p.hs_b2 + 2 * kc), __ldg(p.b2 + h * p.hs_b2 + 2 * kc + 1));
-  const float bias = (!p.post && p.modrelu_bias) ? __ldg(p.modrelu_bias + h * p.hs_mb + kc) : 0.f;
+  const float2 b2 = make_float2(p.b2[h * p.hs_b2 + 2 * kc], p.b2[h * p.hs_b2 + 2 * kc + 1]);
+  const float bias = (!p.post && p.modrelu_bias) ? p.modrelu_bias[h * p.hs_mb + kc] : 0.f;
   asm volatile("cp.async.wait_group 0;" ::: "memory");       // every thread's copies; the barriers below make them the CTA's
   asm volatile("griddepcontrol.wait;" ::: "memory");         // the sums come from the kernel before
   float* qbar = u + BB * p.hidden;
@@ -830,23 +824,22 @@ struct GateChunk {
 // before it get the same values twice).
 __device__ __forceinline__ int gate_chunk_bin(int chunk, int K) { return min(16 * chunk, K - 16); }
 // src: W2 of the head at row 2 q, bin i8
-__device__ __forceinline__ void gate_fetch_chunk(GateChunk& x, const unsigned* __restrict__ src, const float2* __restrict__ b2,
-                                                 const float* __restrict__ mb, int K, int chunk, int lane) {
+__device__ __forceinline__ void gate_fetch_chunk(GateChunk& x, const unsigned* src, const float2* b2, const float* mb, int K, int chunk, int lane) {
   const int k0 = gate_chunk_bin(chunk, K);
   const unsigned* r = src + k0;
   const size_t far = 7 * (size_t)K;
 #pragma unroll
   for (int s = 0; s < 16; ++s) {
-    x.w[0][s] = __ldg(r);
-    x.w[1][s] = __ldg(r + 8);
+    x.w[0][s] = r[0];
+    x.w[1][s] = r[8];
     r += (s & 1) ? far : (size_t)K;
   }
-  x.b2 = __ldg(b2 + k0 + (lane & 15));
-  x.mb = mb ? __ldg(mb + k0 + (lane & 15)) : 0.f;
+  x.b2 = b2[k0 + (lane & 15)];
+  x.mb = mb ? mb[k0 + (lane & 15)] : 0.f;
 }
 // out: g_out of the lane's entry (i8) at bin 2 q; pm: the positional phase (per lane where entries differ)
 template <int NB, bool SHIFTS>
-__device__ __forceinline__ void gate_use_chunk(const GateChunk& x, const uint32_t (&A)[4][MmaRows<NB>::kSets][4], float2* __restrict__ out,
+__device__ __forceinline__ void gate_use_chunk(const GateChunk& x, const uint32_t (&A)[4][MmaRows<NB>::kSets][4], float2* out,
                                                int n, int k0, bool write, bool relu, unsigned pm, int q, int lane) {
   // the phase of bin k0 + lane % 16, handed round below (per-entry shifts: evaluated where they are used)
   float2 ph = make_float2(1.f, 0.f);

@@ -142,9 +142,9 @@ __device__ __forceinline__ void store_elem(const OnchipParams& p, const TileCoor
 }
 
 // Hermitian extension of the half-spectrum gate at full-spectrum index k.
-__device__ __forceinline__ float2 gate_at(const float2* __restrict__ g, int k, int n) {
+__device__ __forceinline__ float2 gate_at(const float2* g, int k, int n) {
   int kk = (2 * k <= n) ? k : n - k;
-  float2 v = __ldg(g + kk);
+  float2 v = g[kk];
   if (kk != k) v.y = -v.y;
   if (k == 0 || 2 * k == n) v.y = 0.f;
   return v;
@@ -265,7 +265,7 @@ __device__ __forceinline__ void middle(const OnchipParams& p, const TileCoord& t
         xa[q] = xb[q] = make_float2(0.f, 0.f);
         if (col < p.D) {
           const float2* row = p.spec + ((size_t)slab * p.K + kk) * p.D + col;
-          const float2 gk = cscale(__ldg(g + kk), p.scale);
+          const float2 gk = cscale(g[kk], p.scale);
           xa[q] = pair_from_half(gk, *reinterpret_cast<const float4*>(row), k, kk, p.n);
           xb[q] = pair_from_half(gk, *reinterpret_cast<const float4*>(row + 2), k, kk, p.n);
         }

@@ -140,8 +140,8 @@ __global__ void __launch_bounds__(256, 3) level_gates_kernel(const LevelGatePara
   const int ii = min(tid, p.NG - 1);
 #pragma unroll
   for (int u = 0; u < 32; ++u) w2[u] = W2[(size_t)min(u, p.hidden - 1) * p.NG + ii];
-  float b1v = __ldg(p.bw1 + h * p.hs_b1 + tid % p.hidden);
-  const float b2v = __ldg(p.bw2 + h * p.hs_b2 + ii);
+  float b1v = p.bw1[h * p.hs_b1 + tid % p.hidden];
+  const float b2v = p.bw2[h * p.hs_b2 + ii];
   // Everything above reads only weights; q_bar comes from the kernel before.  The mixer behind this one may start only now:
   // it reads the tokens without a wait of its own.
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(256, 3) level_gates_kernel(const LevelGatePara
     const int e = i / p.hidden, jj = i - e * p.hidden;
     const int st = kLgBatch * p.hidden;
     us[jj * kLgBatch + e] = gelu_erf(b1v + ((part_raw[i] + part_raw[st + i]) + (part_raw[2 * st + i] + part_raw[3 * st + i])));
-    if (i + 256 < kLgBatch * p.hidden) b1v = __ldg(p.bw1 + h * p.hs_b1 + (i + 256) % p.hidden);
+    if (i + 256 < kLgBatch * p.hidden) b1v = p.bw1[h * p.hs_b1 + (i + 256) % p.hidden];
   }
   __syncthreads();
   if (tid < p.NG) {
@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(128 * NH + 32, NH == 2 ? 2 : 1) mixer_tc196_ke
       float2 v = make_float2(0.f, 0.f);
       if (kM < 49 && b < p.B) {
         const int k = k1 + 4 * kM, kk = k <= 98 ? k : 196 - k;
-        v = __ldg(p.g + ((size_t)b * p.H + hh) * 99 + kk);
+        v = p.g[((size_t)b * p.H + hh) * 99 + kk];
         if (kk != k) v.y = -v.y;
         if (k == 0 || k == 98) v.y = 0.f;
       }

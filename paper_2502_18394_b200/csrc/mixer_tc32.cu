@@ -185,9 +185,9 @@ struct TcIn32Params {
 };
 
 // bins k = k1 + R kM, kM < 4096, of the Hermitian extension of one head's gate
-__device__ __forceinline__ float2 gate_ext(const float2* __restrict__ g, int k, int n) {
+__device__ __forceinline__ float2 gate_ext(const float2* g, int k, int n) {
   const int kk = (2 * k <= n) ? k : n - k;
-  float2 v = __ldg(g + kk);
+  float2 v = g[kk];
   if (kk != k) v.y = -v.y;
   if (k == 0 || 2 * k == n) v.y = 0.f;
   return v;

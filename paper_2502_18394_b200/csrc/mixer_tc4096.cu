@@ -38,9 +38,9 @@ struct Tc4096Params {
   int* status;
 };
 
-__device__ __forceinline__ float2 gate4096(const float2* __restrict__ g, int k) {
+__device__ __forceinline__ float2 gate4096(const float2* g, int k) {
   const int kk = k <= 2048 ? k : 4096 - k;
-  float2 v = __ldg(g + kk);
+  float2 v = g[kk];
   if (kk != k) v.y = -v.y;
   if (k == 0 || k == 2048) v.y = 0.f;
   return v;

@@ -91,7 +91,7 @@ __device__ __forceinline__ void tc_gate_body(const TcGateParams& p, int sk, floa
   for (int i = 0; i < 16; ++i) {                                 // 16 strided loads in flight per thread
     const int k = k1 + p.R * (threadIdx.x + 256 * i);
     const int kk = (2 * k <= p.n) ? k : p.n - k;
-    float2 v = __ldg(g + kk);
+    float2 v = g[kk];
     if (kk != k) v.y = -v.y;
     if (k == 0 || 2 * k == p.n) v.y = 0.f;
     gv[i] = v;
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256, 3) tc_in_kernel(const TcInParams p, const
       float2 x[R];
 #pragma unroll
       for (int n1 = 0; n1 < R; ++n1) {
-        const uint32_t v = n1 < nvalid ? __ldg(pl + n1 * lstride) : 0u;
+        const uint32_t v = n1 < nvalid ? pl[n1 * lstride] : 0u;
         x[n1] = F16 ? unpack_h2(v) : make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
       }
       Dft<R, false>::run(x);
@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(k4CoreThreads, 2) tc_core_kernel(const TcCoreP
         if (stage == 3) {
           const int gi = unit / p.ntile;                         // slab_local * R + k1
           core_store(tmem, p.ws_out + (size_t)unit * k4OutBytes, q, wh, T, p.twr + 128 * (gi % p.R),
-                     __ldg(p.gscale + gi) * p.out_scale);
+                     p.gscale[gi] * p.out_scale);
         } else {
           if (stage == 0) epilogue_twiddle2<k4Lbo, k4Sbo, 1>(tmem, Bsm, q, 2 * wh, T, twh, wr0, wr1);
           else if (stage == 2) epilogue_twiddle2<k4Lbo, k4Sbo, 2>(tmem, Bsm, q, 2 * wh, T, twh, wr0, wr1);
@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(256, 3) tc_out_kernel(const TcOutParams p) {
         const int tile = item % p.ntile, tl = (item / p.ntile) * 8 + t8;
         const uint32_t* pu = wsl + tile * (k4OutBytes / 4) + unit_row_slot(tb * NT + tl) * 4 + c4;
 #pragma unroll
-        for (int k1 = 0; k1 < R; ++k1) raw[u][k1] = __ldg(pu + k1 * ustride);   // scaled and twiddled by the core
+        for (int k1 = 0; k1 < R; ++k1) raw[u][k1] = pu[k1 * ustride];   // scaled and twiddled by the core
       }
     }
 #pragma unroll
@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(256) tc_gate_amax_kernel(const TcSpecParams p)
   const float2* g = p.g + (size_t)(p.slab0 + blockIdx.x) * p.K;
   float m = 0.f;
   for (int k = threadIdx.x; k < p.K; k += 256) {
-    const float2 v = __ldg(g + k);
+    const float2 v = g[k];
     m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
   }
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -562,7 +562,7 @@ constexpr int kSpecPitch = 260;
 // j < 8 means k < n/2 and j >= 8 means k > n/2, except for the two real bins k = 0 (j = 0) and k = n/2 (j = 8)
 // of the first unit row, which the caller patches.  MIRROR is therefore a property of the CTA.
 template <bool MIRROR>
-__device__ __forceinline__ void spec_in_bins(const TcSpecParams& p, const float4* __restrict__ spec, const float2* __restrict__ g,
+__device__ __forceinline__ void spec_in_bins(const TcSpecParams& p, const float4* spec, const float2* g,
                                              uint32_t* spec_stage, int j, int k1, int warp, int l, bool live, float s) {
   const unsigned rowq = (unsigned)(p.D / 2);                    // float4 per bin row
   const int kbase = k1 + p.R * (warp + 256 * j), r8 = 8 * p.R, r64 = 64 * p.R;
@@ -576,8 +576,8 @@ __device__ __forceinline__ void spec_in_bins(const TcSpecParams& p, const float4
       for (int u = 0; u < 4; ++u) {
         const int k = kbase + (it + a) * r8 + u * r64;
         const unsigned kk = (unsigned)(MIRROR ? p.n - k : k);
-        ab[a][u] = __ldg(spec + kk * rowq);
-        gk[a][u] = __ldg(g + kk);
+        ab[a][u] = spec[kk * rowq];
+        gk[a][u] = g[kk];
       }
     }
 #pragma unroll
@@ -614,8 +614,8 @@ __global__ void __launch_bounds__(256, 3) tc_spec_in_kernel(const TcSpecParams p
   if (k1 == 0 && warp == 0 && (j == 0 || j == 8) && live) {
     // the real bins k = 0 and k = n/2 (kA = 0, first kB of the group): only Re(gA) and Re(gB) survive (App. B)
     const unsigned kk = j == 0 ? 0u : (unsigned)(p.n / 2);
-    const float4 v = __ldg(spec + kk * (unsigned)(p.D / 2));
-    const float2 gs = cscale(__ldg(g + kk), s);
+    const float4 v = spec[kk * (unsigned)(p.D / 2)];
+    const float2 gs = cscale(g[kk], s);
     spec_stage[l * kSpecPitch] = pack_h2(gs.x * v.x - gs.y * v.y, -(gs.x * v.z - gs.y * v.w));
   }
   __syncthreads();

@@ -50,9 +50,9 @@ struct Tc8kParams {
 };
 
 // Hermitian extension of the half-spectrum gate (n = 8192).
-__device__ __forceinline__ float2 gate8192(const float2* __restrict__ g, int k) {
+__device__ __forceinline__ float2 gate8192(const float2* g, int k) {
   int kk = k <= 4096 ? k : 8192 - k;
-  float2 v = __ldg(g + kk);
+  float2 v = g[kk];
   if (kk != k) v.y = -v.y;
   if (k == 0 || k == 4096) v.y = 0.f;
   return v;

@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
   if constexpr (MODE == kRegMix) {
     for (int i = threadIdx.x; i < P::M; i += P::kThreads) {
       const int k = k1 + p.N1 * i, kk = 2 * k <= p.n ? k : p.n - k;
-      float2 v = cscale(__ldg(g + kk), p.scale);
+      float2 v = cscale(g[kk], p.scale);
       if (kk != k) v.y = -v.y;
       if (k == 0 || 2 * k == p.n) v.y = 0.f;
       extra[P::gate_slot(i)] = v;
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
       x[i] = make_float2(0.f, 0.f);
       if (live_out) {
         const float4 ab = *reinterpret_cast<const float4*>(spec + (size_t)kk * p.D);
-        x[i] = pair_from_half(cscale(__ldg(g + kk), p.scale), ab, k, kk, p.n);
+        x[i] = pair_from_half(cscale(g[kk], p.scale), ab, k, kk, p.n);
       }
     }
   }
@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
 #pragma unroll
     for (int i = 0; i < E; ++i) {
       const int k = pl.bin(i), kk = 2 * k <= p.n ? k : p.n - k;
-      float2 v = cscale(__ldg(g + kk), p.scale);
+      float2 v = cscale(g[kk], p.scale);
       if (kk == k) v.y = -v.y;
       if (k == 0 || 2 * k == p.n) v.y = 0.f;
       x[i] = cmul(x[i], v);
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_stream_k
 #pragma unroll
     for (int i = 0; i < kGv; ++i) {
       const int k = threadIdx.x + i * P::kThreads;
-      gv[i] = k < P::M ? __ldg(g + (2 * k <= P::M ? k : P::M - k)) : make_float2(0.f, 0.f);
+      gv[i] = k < P::M ? g[2 * k <= P::M ? k : P::M - k] : make_float2(0.f, 0.f);
     }
     ok = mbar_wait(bar, par);
     float2 x[E];

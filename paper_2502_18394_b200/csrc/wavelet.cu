@@ -7,7 +7,7 @@
 namespace spectre {
 
 template <typename WT> __device__ __forceinline__ float wl(const WT* p);
-template <> __device__ __forceinline__ float wl<float>(const float* p) { return __ldg(p); }
+template <> __device__ __forceinline__ float wl<float>(const float* p) { return *p; }
 template <> __device__ __forceinline__ float wl<bf16>(const bf16* p) { return __bfloat162float(*p); }
 
 struct WaveletParams {
