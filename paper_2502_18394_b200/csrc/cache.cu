@@ -11,6 +11,9 @@ bool transform_supported(const spectre_ctx* ctx, int n);
 size_t transform_slab_bytes(int n, int D);
 int pool_sum_ring(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* q, float* sums, void* ring, int N);
 size_t gate_min_workspace(int B, int H, int D, int n_fft, int r);
+int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float* sum_q, int B, int H, int D, float inv_count,
+              const spectre_gate_params* gp, int n_fft, const int64_t* shift, int64_t shift_all, float* g_out, float* qbar_out,
+              void* workspace, size_t workspace_bytes, bool early);
 size_t inverse_workspace_bytes(const spectre_ctx* ctx, int n, int D, int nslab);
 int inverse_from_spectrum(const spectre_ctx* ctx, cudaStream_t st, const float* spec, const float* g, const spectre_act* y,
                           int n, void* ws, size_t ws_bytes);
@@ -547,8 +550,8 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
                                                    evict)));
   SPECTRE_LAUNCH_OK("decode_ring_kernel");
   // (c)-(d) gate from the running sum with phase p = t
-  rc = spectre_gate(ctx, stream, nullptr, cache->sum_q, B, H, D, 1.0f / (float)N, params, N, nullptr, t, g_out, nullptr,
-                    gate_ws, gate_bytes);
+  rc = gate_call(ctx, stream, nullptr, cache->sum_q, B, H, D, 1.0f / (float)N, params, N, nullptr, t, g_out, nullptr, gate_ws,
+                 gate_bytes, true);
   if (rc != SPECTRE_OK) return rc;
   // (b) + (e) one pass over the spectrum
   DecodeRows dr;

@@ -450,7 +450,14 @@ struct GateMlpParams {
   float* u_ws;            // [B,H,hidden] hidden activations (workspace)
   int post;               // 1: Toeplitz follows, skip modReLU/phase here
   int stage_w1;           // W1, gamma, beta and b1 of a head are copied to shared memory before the wait (size and alignment allow)
+  int early;              // the kernel in front is of the same call and has waited for the caller's work: the weights, which the caller's
+                          // last kernel may have written, are read ahead of the wait.  Otherwise the wait comes first
 };
+// In front of the trigger: what triggers before it has waited lets its dependents start beside the caller's kernel too
+__device__ __forceinline__ void gate_start(const GateMlpParams& p) {
+  if (!p.early) after_previous();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // raw (re, im) weight pair of one bin in one hidden row
 template <typename WT> struct wraw;
@@ -480,7 +487,7 @@ __global__ void __launch_bounds__(256) gate_hidden_kernel(const GateMlpParams p)
   const int nbg = (p.B + BB - 1) / BB;
   const int h = blockIdx.x / nbg, b0 = (blockIdx.x - h * nbg) * BB;
   const int nb = min(BB, p.B - b0);
-  asm volatile("griddepcontrol.launch_dependents;");
+  gate_start(p);
   float* qbar = u + BB * p.hidden;
   const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
   WT* w1s = reinterpret_cast<WT*>(u + ((BB * (p.hidden + p.D) + 3) & ~3));
@@ -572,8 +579,7 @@ __device__ __forceinline__ void gate_stream(typename wraw<WT>::type (&w)[wraw<WT
 template <typename WT, int BB, bool PRE>
 __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const GateMlpParams p) {
   extern __shared__ __align__(16) float u[];       // [hidden][BB], then q_bar [BB][D]
-  // a kernel launched behind this one as a programmatic dependent may do its set-up meanwhile
-  asm volatile("griddepcontrol.launch_dependents;");
+  gate_start(p);                                   // a kernel launched behind this one as a programmatic dependent may do its set-up meanwhile
   constexpr int R = wraw<WT>::kRows;
   const int nbg = (p.B + BB - 1) / BB;
   const int h = blockIdx.y / nbg, b0 = (blockIdx.y - h * nbg) * BB;
@@ -668,7 +674,7 @@ __global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams 
   constexpr int R = wraw<WT>::kRows, kParts = 64 / R, kBins = 256 / kParts;
   extern __shared__ __align__(16) float u[];       // [hidden], q_bar [D], W1, gamma, beta, b1
   __shared__ float2 part[kParts][kBins];
-  asm volatile("griddepcontrol.launch_dependents;");
+  gate_start(p);
   const int h = blockIdx.y % p.H, b = blockIdx.y / p.H;
   const int q = threadIdx.x / kBins, t = threadIdx.x % kBins, k = blockIdx.x * kBins + t, kc = min(k, p.K - 1);
   const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
@@ -729,7 +735,7 @@ __global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams 
 template <typename WT, int BB>
 __global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams p) {
   extern __shared__ __align__(16) float u[];       // [hidden][BB], q_bar [BB][D], W1, gamma, beta, b1, W2
-  asm volatile("griddepcontrol.launch_dependents;");
+  gate_start(p);
   const int nbg = (p.B + BB - 1) / BB;
   const int h = blockIdx.x / nbg, b0 = (blockIdx.x - h * nbg) * BB;
   const int nb = min(BB, p.B - b0), k = threadIdx.x;
@@ -882,7 +888,7 @@ __device__ __forceinline__ void gate_use_chunk(const GateChunk& x, const uint32_
 template <int NB, bool SHIFTS>
 __global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p) {
   extern __shared__ __align__(16) float u[];       // [hidden][NB], then q_bar [NB][D], then W1
-  asm volatile("griddepcontrol.launch_dependents;");
+  gate_start(p);
   constexpr int kSets = MmaRows<NB>::kSets;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane & 3, i8 = lane >> 2, nw = blockDim.x >> 5;
   const int nbg = (p.B + NB - 1) / NB;
@@ -1014,10 +1020,11 @@ extern "C" size_t spectre_gate_workspace_bytes(const spectre_ctx* ctx, int32_t B
   return gate_ws_layout(B, H, D, n_fft, toeplitz_r, 1024, kPoolCopies, &off, &off2);   // any hidden width
 }
 
-extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q, const float* sum_q, int32_t B,
-                            int32_t H, int32_t D, float inv_count, const spectre_gate_params* gp, int32_t n_fft,
-                            const int64_t* shift, int64_t shift_all, float* g_out, float* qbar_out, void* workspace,
-                            size_t workspace_bytes) {
+namespace spectre {
+// spectre_gate; `early`: see GateMlpParams
+int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float* sum_q, int B, int H, int D, float inv_count,
+              const spectre_gate_params* gp, int n_fft, const int64_t* shift, int64_t shift_all, float* g_out, float* qbar_out,
+              void* workspace, size_t workspace_bytes, bool early) {
   if (!ctx) return fail(SPECTRE_ERR_INVALID_ARG, "ctx is NULL");
   if (!gp) return fail(SPECTRE_ERR_INVALID_ARG, "gate parameters are NULL");
   if ((q != nullptr) == (sum_q != nullptr)) return fail(SPECTRE_ERR_INVALID_ARG, "give exactly one of q and sum_q");
@@ -1044,12 +1051,9 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   const int r = gp->toeplitz_r;
   size_t sums_off, u_off;
   const size_t need = gate_ws_layout(B, H, D, n_fft, r, gp->hidden, 1, &u_off, &sums_off);   // one copy is enough
-  const bool need_ws = true;
-  if (need_ws) {
-    if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 15))
-      return fail(SPECTRE_ERR_WORKSPACE, "workspace is NULL or not 16-byte aligned");
-    if (workspace_bytes < need) return fail(SPECTRE_ERR_WORKSPACE, "gate workspace too small");
-  }
+  if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 15))
+    return fail(SPECTRE_ERR_WORKSPACE, "workspace is NULL or not 16-byte aligned");
+  if (workspace_bytes < need) return fail(SPECTRE_ERR_WORKSPACE, "gate workspace too small");
   SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const float* sums = sum_q;
@@ -1084,6 +1088,7 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   mp.qbar_out = qbar_out;
   mp.u_ws = reinterpret_cast<float*>(reinterpret_cast<char*>(workspace) + u_off);
   mp.post = r > 0;
+  mp.early = early;
   float2* raw = r > 0 ? reinterpret_cast<float2*>(workspace) : nullptr;
   mp.g_out = r > 0 ? raw : reinterpret_cast<float2*>(g_out);
   // block sized to the bin count for short transforms (K = 99 does not need 256 threads)
@@ -1110,9 +1115,9 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   const bool all_staged = BB >= 4 && !mma && grid_out.x == 1 && w1_bytes % 16 == 0 && w2_bytes % 16 == 0 && short_bytes <= 49152 &&
                           !((reinterpret_cast<uintptr_t>(gp->W1) | reinterpret_cast<uintptr_t>(gp->W2)) & 15);
   const bool pre = grid_out.x >= 32;               // many CTAs per head: compute the hidden layer once
-  // Programmatic dependent launch: the weight stream of the output layer may overlap the kernel
-  // before it (the pooling pass here, or whatever produced sum_q); each kernel waits for its
-  // predecessor (griddepcontrol.wait) before it touches the sums.
+  // Programmatic dependent launch: the weight stream of the output layer overlaps the kernel before it where that is one of
+  // this call (the pooling pass, the decode step's ring kernel); each kernel waits for its predecessor
+  // (griddepcontrol.wait) before it touches the sums, and first of all where the caller's own kernel precedes it.
   cudaLaunchAttribute pdl[1];
   pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   pdl[0].val.programmaticStreamSerializationAllowed = 1;
@@ -1140,6 +1145,7 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
   do {                                                                                           \
     if (pre) {                                                                                   \
       SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_hid, gate_hidden_kernel<WT, NB>, mp));             \
+      mp.early = 1;                                                                              \
       SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_out, gate_out_kernel<WT, NB, true>, mp));          \
     } else {                                                                                     \
       SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_out, gate_out_kernel<WT, NB, false>, mp));         \
@@ -1179,6 +1185,16 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
     SPECTRE_LAUNCH_OK("gate_post_kernel");
   }
   return SPECTRE_OK;
+}
+}  // namespace spectre
+
+// With q the pooling pass is in front of the gate kernels; with sum_q whatever the caller launched last is.
+extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q, const float* sum_q, int32_t B,
+                            int32_t H, int32_t D, float inv_count, const spectre_gate_params* gp, int32_t n_fft,
+                            const int64_t* shift, int64_t shift_all, float* g_out, float* qbar_out, void* workspace,
+                            size_t workspace_bytes) {
+  return gate_call(ctx, stream, q, sum_q, B, H, D, inv_count, gp, n_fft, shift, shift_all, g_out, qbar_out, workspace, workspace_bytes,
+                   q != nullptr);
 }
 
 // ---- gate without any caller- or library-side allocation -----------------------

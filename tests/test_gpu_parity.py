@@ -367,6 +367,29 @@ def test_gate_few_blocks(ctx, B, H, L, n, D, hid, wdt, r):
     assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
 
 
+@pytest.mark.parametrize("B,n,wdt", [(1, 1024, "f32"), (1, 32768, "bf16"), (1, 4096, "bf16"), (2, 1024, "bf16"), (8, 196, "bf16"), (8, 1000, "f32"),
+                                     (3, 32768, "f32")])
+def test_gate_from_running_sum_sees_weights_that_the_kernel_in_front_wrote(ctx, B, n, wdt):
+    # every output-layer kernel; the weights change between calls, by the kernel right in front of the gate
+    w = W.Workload("t", B=B, L=8, H=4, D=64, dtype="bf16", wdtype=wdt, n_fft=n, seed=n + B)
+    p = to_dev(W.gate_params(w, modrelu_bias_std=0.01, bias_std=0.1))
+    base = {k: p[k].clone() for k in ("W1", "W2")}
+    sum_q = torch.randn(B, 4, 64, generator=torch.Generator().manual_seed(1)).cuda() * 9
+    scales = [1.0, -3.0, 0.25, 2.0]
+    want = []
+    for s in scales:
+        for k in base:
+            torch.mul(base[k], s, out=p[k])
+        torch.cuda.synchronize()
+        want.append(S.spectre_gate(ctx, p, n, sum_q=sum_q, inv_count=1.0 / n))
+        torch.cuda.synchronize()
+    for rep in range(40):
+        i = rep % len(scales)
+        torch.mul(base["W1"], scales[i], out=p["W1"])
+        torch.mul(base["W2"], scales[i], out=p["W2"])
+        assert torch.equal(S.spectre_gate(ctx, p, n, sum_q=sum_q, inv_count=1.0 / n), want[i])
+
+
 def test_gate_from_running_sum_and_shared_heads(ctx):
     w = W.Workload("t", B=2, L=64, H=4, D=32, dtype="f32", wdtype="f32", n_fft=64, seed=13)
     p = W.gate_params(w)

@@ -25,3 +25,14 @@ def test_read_only_loads_and_restrict_are_for_the_contexts_tables(name, text):
             assert "__restrict__" not in m.group(2), f"{name}: {m.group(1)}"
     for m in re.finditer(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", text):
         assert m.group(1) in TABLES | {"Gtab", "u"}, f"{name}: const __restrict__ {m.group(1)}"      # Gtab, u: shared memory
+
+
+@pytest.mark.parametrize("name,text", [pytest.param(n, t, id=n) for n, t in sources() if "launch_dependents" in t])
+def test_kernels_wait_before_they_let_their_dependents_start(name, text):
+    # What a dependent reads ahead of its own wait (weights, the cached spectrum, tokens) was written in front of the call at the
+    # latest.  So no kernel triggers before it has waited, unless it is told that the kernel in front of it has.
+    for body in re.split(r"(?=__global__ void|__device__ __forceinline__ void)", text)[1:]:
+        first = body.find("launch_dependents")
+        if first >= 0:
+            before = body[:first]
+            assert "after_previous()" in before or "griddepcontrol.wait" in before, f"{name}: {body[:90]}"
