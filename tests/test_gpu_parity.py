@@ -497,6 +497,25 @@ def test_mixer_196_with_refinement_in_the_store_phase(ctx, J, L, B, H, wdt, hid,
     assert slab_err(W.to_f64(y), ref) < TOL["bf16"]
 
 
+def test_mixer_196_refinement_sees_weights_that_the_kernel_in_front_wrote(ctx):
+    w = W.Workload("t", B=16, L=196, H=3, D=64, dtype="bf16", seed=5)
+    v, g = W.activations(w).cuda(), W.random_gate(w).cuda()
+    gen = torch.Generator().manual_seed(2)
+    wrm = {"levels": 2, "hidden": 64, "qbar": torch.randn(16, 3, 64, generator=gen).cuda(),
+           "Ww1": (torch.randn(3, 64, 64, generator=gen) * 0.1).bfloat16().cuda(), "bw1": torch.zeros(3, 64, device="cuda"),
+           "Ww2": (torch.randn(3, 64, 192, generator=gen) * 0.1).bfloat16().cuda(), "bw2": torch.zeros(3, 192, device="cuda")}
+    base, scales, want = {k: wrm[k].clone() for k in ("Ww1", "Ww2")}, [1.0, -3.0, 0.25, 2.0], []
+    for rep in range(44):
+        i = rep % 4
+        for k in base:
+            torch.mul(base[k], scales[i], out=wrm[k])
+        if rep < 4:
+            torch.cuda.synchronize()
+            want.append(S.spectre_mixer_forward(ctx, v, g, wrm=wrm))
+        else:
+            assert torch.equal(S.spectre_mixer_forward(ctx, v, g, wrm=wrm), want[i])
+
+
 def test_mixer_196_refinement_without_workspace(ctx):
     # the MLP's level gates need scratch: without it the call must still be right (separate refinement kernel)
     w = W.Workload("t", B=2, L=196, H=3, D=64, dtype="bf16", wdtype="bf16", n_fft=196, seed=31, wavelet_levels=2)

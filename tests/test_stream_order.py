@@ -36,3 +36,10 @@ def test_kernels_wait_before_they_let_their_dependents_start(name, text):
         if first >= 0:
             before = body[:first]
             assert "after_previous()" in before or "griddepcontrol.wait" in before, f"{name}: {body[:90]}"
+
+
+def test_level_gates_read_nothing_ahead_of_their_wait():
+    # the first kernel of its call: any kernel of the caller's may be in front
+    text = dict(sources())["mixer_tc.cu"]
+    body = text[text.index("level_gates_kernel(const"):]
+    assert not re.search(r"\bW[12]\[|p\.(bw1|bw2|qbar)\[", body[:body.index("after_previous()")])
