@@ -200,9 +200,10 @@ template <class F> int released(F f) {
   return rc;
 }
 
-template <PyObject* (*F)(PyObject* const*)>
+// ARGS: the number of arguments F reads; the wrappers in binding.py pass every one
+template <PyObject* (*F)(PyObject* const*), int ARGS>
 PyObject* guarded(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  (void)n;                                         // the wrappers in binding.py pass every argument
+  if (n != ARGS) return PyErr_Format(PyExc_TypeError, "expected %d arguments, got %zd", ARGS, n);
   try {
     return F(a);
   } catch (const Failed&) {
@@ -405,10 +406,11 @@ PyObject* set_error(PyObject*, PyObject* type) {
   Py_RETURN_NONE;
 }
 
-#define SPECTRE_METHOD(name) {#name, (PyCFunction)(void (*)(void))guarded<name>, METH_FASTCALL, nullptr}
-PyMethodDef g_methods[] = {SPECTRE_METHOD(gate), SPECTRE_METHOD(mixer_forward), SPECTRE_METHOD(wavelet_refine), SPECTRE_METHOD(prefill),
-                           SPECTRE_METHOD(append), SPECTRE_METHOD(decode_step), SPECTRE_METHOD(readout), SPECTRE_METHOD(project_qv),
-                           SPECTRE_METHOD(mixer_backward), {"set_error", set_error, METH_O, nullptr}, {nullptr, nullptr, 0, nullptr}};
+#define SPECTRE_METHOD(name, args) {#name, (PyCFunction)(void (*)(void))guarded<name, args>, METH_FASTCALL, nullptr}
+PyMethodDef g_methods[] = {SPECTRE_METHOD(gate, 13), SPECTRE_METHOD(mixer_forward, 8), SPECTRE_METHOD(wavelet_refine, 5),
+                           SPECTRE_METHOD(prefill, 6), SPECTRE_METHOD(append, 6), SPECTRE_METHOD(decode_step, 11),
+                           SPECTRE_METHOD(readout, 6), SPECTRE_METHOD(project_qv, 10), SPECTRE_METHOD(mixer_backward, 9),
+                           {"set_error", set_error, METH_O, nullptr}, {nullptr, nullptr, 0, nullptr}};
 PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, g_methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

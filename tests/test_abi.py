@@ -3,6 +3,8 @@ host-side validation answers without a GPU; the N>1 'replicas only' layout of be
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -51,3 +53,16 @@ def test_null_arguments_fail_without_a_device(lib):
     assert b"no CPU fallback" in lib.spectre_last_error()
     assert lib.spectre_mixer_forward(None, None, None, None, None, 8, None, None, 0) == 1
     assert lib.spectre_prefix_cache_append(None, None, None, None, None, 0) == 1
+
+
+def test_native_calls_with_another_number_of_arguments_are_refused():
+    # in a process of its own: a call that reads beyond its argument array ends the process
+    code = ("from paper_2502_18394_b200 import build, binding\nbuild.build()\next = binding._native()\n"
+            "for name in ('gate', 'mixer_forward', 'wavelet_refine', 'prefill', 'append', 'decode_step', 'readout', 'project_qv', "
+            "'mixer_backward'):\n"
+            "    for n in (0, 1, 4, 30):\n"
+            "        try:\n            getattr(ext, name)(*[None] * n)\n"
+            "        except TypeError as e:\n            assert 'arguments, got %d' % n in str(e), (name, n, e)\n"
+            "        else:\n            raise SystemExit(name)\n")
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr
