@@ -78,6 +78,11 @@ long long integer(PyObject* o) {
   return v;
 }
 int32_t integer32(PyObject* o) { return (int32_t)integer(o); }
+bool truth(PyObject* o) {
+  const int t = PyObject_IsTrue(o);
+  if (t < 0) throw Failed{};
+  return t == 1;
+}
 double real(PyObject* o) {
   const double v = PyFloat_AsDouble(o);
   if (v == -1.0 && PyErr_Occurred()) throw Failed{};
@@ -365,7 +370,7 @@ PyObject* project_qv(PyObject* const* a) {
     raise(PyExc_ValueError, "Wq and Wv must be contiguous and of one dtype");
   at::Tensor q = none(a[4]) ? at::empty_like(x) : tensor(a[4]), v = none(a[5]) ? at::empty_like(x) : tensor(a[5]), sum;
   if (!none(a[6])) sum = tensor(a[6]);
-  else if (PyObject_IsTrue(a[7]) == 1) sum = empty({ax.B, ax.H, ax.D}, x, at::kFloat);
+  else if (truth(a[7])) sum = empty({ax.B, ax.H, ax.D}, x, at::kFloat);
   const spectre_act aq = act(q), av = act(v);
   const Workspace w(a[8], x, [&] { return spectre_project_workspace_bytes(ctx, ax.H, ax.D); });
   void* st = stream(a[9]);
@@ -383,7 +388,7 @@ PyObject* mixer_backward(PyObject* const* a) {
   const spectre_act av = act(v), ady = act(dy);
   const float* g = (const float*)pointer(a[3]);
   const int32_t n = none(a[4]) ? av.L : integer32(a[4]);
-  const bool want_dv = PyObject_IsTrue(a[5]) == 1, want_dg = PyObject_IsTrue(a[6]) == 1;
+  const bool want_dv = truth(a[5]), want_dg = truth(a[6]);
   at::Tensor dv, dg;
   spectre_act adv = {};
   if (want_dv) {

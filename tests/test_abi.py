@@ -66,3 +66,15 @@ def test_native_calls_with_another_number_of_arguments_are_refused():
             "        else:\n            raise SystemExit(name)\n")
     res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert res.returncode == 0, res.stderr
+
+
+def test_a_flag_without_a_truth_value_raises_its_own_error(lib):
+    import torch
+    from paper_2502_18394_b200 import binding
+    x, w = torch.zeros(1, 8, 1, 64, dtype=torch.bfloat16), torch.zeros(1, 64, 64)
+    both = torch.zeros(2)                                    # bool() of it raises
+    ext = binding._native()
+    with pytest.raises(RuntimeError, match="[Bb]oolean value"):
+        ext.mixer_backward(None, x, x, torch.zeros(1, 1, 5, 2), None, both, True, None, None)
+    with pytest.raises(RuntimeError, match="[Bb]oolean value"):
+        ext.project_qv(None, x, w, w, None, None, None, both, None, None)
