@@ -14,6 +14,7 @@ LIB = os.path.join(PKG, "libspectre.so")
 NATIVE = os.path.join(PKG, "_native.so")
 NATIVE_SRC = os.path.join(CSRC, "native.cpp")
 OBJ = os.path.join(PKG, "build")
+NATIVE_ABI = os.path.join(OBJ, "native_abi")
 SOURCES = ["reg_grad.cu", "reg_mix.cu", "reg_inverse.cu", "reg_forward.cu", "api.cu", "mixer.cu", "mixer_tc.cu", "mixer_tc8k.cu",
            "mixer_tc4k.cu", "gate.cu", "cache.cu", "wavelet.cu", "backward.cu", "project.cu"]
 FLAGS = ["-std=c++17", "-O3", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -51,9 +52,20 @@ def _compile(src: str, obj: str, verbose: bool) -> str:
     return res.stderr
 
 
+def native_abi() -> str:
+    """What the extension is compiled against beside its sources: another torch or Python has another ABI."""
+    import sysconfig
+
+    import torch
+    return f"torch {torch.__version__} {sysconfig.get_config_var('SOABI')}"
+
+
 def native_is_stale() -> bool:
-    if not os.path.exists(NATIVE):
+    if not os.path.exists(NATIVE) or not os.path.exists(NATIVE_ABI):
         return True
+    with open(NATIVE_ABI) as f:
+        if f.read() != native_abi():
+            return True
     return os.path.getmtime(NATIVE) < max(os.path.getmtime(f) for f in (NATIVE_SRC, os.path.join(ROOT, "include", "spectre.h")))
 
 
@@ -73,6 +85,9 @@ def build_native(force: bool = False) -> str:
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError("g++ failed on " + NATIVE_SRC + ":\n" + res.stdout + res.stderr)
+    os.makedirs(OBJ, exist_ok=True)
+    with open(NATIVE_ABI, "w") as f:
+        f.write(native_abi())
     return NATIVE
 
 

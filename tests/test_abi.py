@@ -78,3 +78,11 @@ def test_a_flag_without_a_truth_value_raises_its_own_error(lib):
         ext.mixer_backward(None, x, x, torch.zeros(1, 1, 5, 2), None, both, True, None, None)
     with pytest.raises(RuntimeError, match="[Bb]oolean value"):
         ext.project_qv(None, x, w, w, None, None, None, both, None, None)
+
+
+def test_the_extension_is_rebuilt_for_another_torch(lib, monkeypatch):
+    import torch
+    from paper_2502_18394_b200 import build
+    assert not build.native_is_stale()
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert build.native_is_stale()
