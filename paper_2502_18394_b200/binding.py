@@ -4,7 +4,9 @@ Argument marshalling only: every step of the path runs in the CUDA kernels.
 Function names are those of include/spectre.h.  The per-step calls are marshalled
 in native code (csrc/native.cpp, the _native extension), contexts, queries and
 pre-marshalled calls through ctypes.  PyTorch appears here for device memory
-(tensors, workspace) and the current stream, nothing else.  If the shared library
+(tensors, workspace) and the current stream, nothing else.  What a call with a
+`stream` argument allocates belongs to that stream, as under torch.cuda.stream:
+a program that uses it on another one orders the two.  If the shared library
 or the extension is missing every call raises: there is no CPU or PyTorch fallback.
 """
 from __future__ import annotations

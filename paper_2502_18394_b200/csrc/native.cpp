@@ -5,10 +5,13 @@
 // tensors are unpacked, outputs and workspaces come from torch's allocator and the C ABI is called, without another Python
 // object in between.  The C ABI is the only thing that touches the device.
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <optional>
 #include <string>
+#include <vector>
 
 #include "spectre.h"
 
@@ -109,13 +112,23 @@ struct Attr {                                      // owned attribute
   Attr(const Attr&) = delete;
 };
 
-void* stream(PyObject* s) {
-  if (none(s)) return c10::cuda::getCurrentCUDAStream().stream();
-  Attr a(s, kAttrStream);
-  void* p = PyLong_AsVoidPtr(a.o);
-  if (!p && PyErr_Occurred()) throw Failed{};
-  return p;
-}
+// The stream of a call: the current one, or the `cuda_stream` of the object given.  Outputs and workspaces of the call are
+// allocated on it too: torch's allocator hands a freed block on in the order of the stream that it was allocated on.
+struct Stream {
+  std::optional<c10::cuda::CUDAStreamGuard> guard;
+  void* st;
+  Stream(PyObject* s, const at::Tensor& like) {
+    if (none(s)) {
+      st = c10::cuda::getCurrentCUDAStream().stream();
+      return;
+    }
+    Attr a(s, kAttrStream);
+    st = PyLong_AsVoidPtr(a.o);
+    if (!st && PyErr_Occurred()) throw Failed{};
+    if (like.is_cuda() && c10::cuda::getCurrentCUDAStream(like.get_device()).stream() != st)
+      guard.emplace(c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(st), like.get_device()));
+  }
+};
 spectre_ctx* context(PyObject* o) {
   if (none(o)) return nullptr;
   void* p = PyLong_AsVoidPtr(o);
@@ -239,15 +252,15 @@ PyObject* gate(PyObject* const* a) {
   const float inv = (float)real(a[5]);
   const int64_t* shift = (const int64_t*)pointer(a[6]);
   const int64_t shift_all = integer(a[7]);
+  const Stream on(a[11], ref);
   at::Tensor g = none(a[8]) ? empty({B, H, n / 2 + 1, 2}, ref, at::kFloat) : tensor(a[8]);
   float *out = (float*)g.data_ptr(), *qbar = (float*)pointer(a[9]);
-  void* st = stream(a[11]);
   if (fixed) {
-    check(released([&] { return spectre_gate_static(ctx, st, from_q ? &q : nullptr, sum_q, B, H, D, inv, &p, n, shift, shift_all, out, qbar); }));
+    check(released([&] { return spectre_gate_static(ctx, on.st, from_q ? &q : nullptr, sum_q, B, H, D, inv, &p, n, shift, shift_all, out, qbar); }));
   } else {
     const Workspace w(a[10], ref, [&] { return spectre_gate_workspace_bytes(ctx, B, H, D, n, p.toeplitz_r); });
     check(released([&] {
-      return spectre_gate(ctx, st, from_q ? &q : nullptr, sum_q, B, H, D, inv, &p, n, shift, shift_all, out, qbar, w.ptr, w.bytes);
+      return spectre_gate(ctx, on.st, from_q ? &q : nullptr, sum_q, B, H, D, inv, &p, n, shift, shift_all, out, qbar, w.ptr, w.bytes);
     }));
   }
   return THPVariable_Wrap(g);
@@ -259,14 +272,14 @@ PyObject* mixer_forward(PyObject* const* a) {
   const at::Tensor& v = tensor(a[1]);
   const spectre_act av = act(v);
   const int32_t n = none(a[4]) ? av.L : integer32(a[4]);
+  const Stream on(a[7], v);
   at::Tensor y = none(a[3]) ? at::empty_like(v) : tensor(a[3]);
   const spectre_act ay = act(y);
   const float* g = (const float*)pointer(a[2]);
   spectre_wavelet wrm = {};
   if (!none(a[5])) wrm = wavelet(a[5]);
   const Workspace w(a[6], v, [&] { return spectre_mixer_workspace_bytes(ctx, av.B, av.L, av.H, av.D, n, av.dtype); });
-  void* st = stream(a[7]);
-  check(released([&] { return spectre_mixer_forward(ctx, st, &av, g, &ay, n, none(a[5]) ? nullptr : &wrm, w.ptr, w.bytes); }));
+  check(released([&] { return spectre_mixer_forward(ctx, on.st, &av, g, &ay, n, none(a[5]) ? nullptr : &wrm, w.ptr, w.bytes); }));
   return THPVariable_Wrap(y);
 }
 
@@ -274,11 +287,11 @@ PyObject* mixer_forward(PyObject* const* a) {
 PyObject* wavelet_refine(PyObject* const* a) {
   spectre_ctx* ctx = context(a[0]);
   const at::Tensor& x = tensor(a[1]);
+  const Stream on(a[4], x);
   at::Tensor y = none(a[3]) ? at::empty_like(x) : tensor(a[3]);
   const spectre_wavelet w = wavelet(a[2]);
   const spectre_act ax = act(x), ay = act(y);
-  void* st = stream(a[4]);
-  check(released([&] { return spectre_wavelet_refine(ctx, st, &ax, &ay, &w); }));
+  check(released([&] { return spectre_wavelet_refine(ctx, on.st, &ax, &ay, &w); }));
   return THPVariable_Wrap(y);
 }
 
@@ -289,9 +302,9 @@ PyObject* prefill(PyObject* const* a) {
   const spectre_cache c = cache_state(a[1], &vb);
   const at::Tensor& v = tensor(a[3]);
   const spectre_act aq = act(tensor(a[2])), av = act(v);
+  const Stream on(a[5], v);
   const Workspace w(a[4], v, [&] { return spectre_prefill_workspace_bytes(ctx, c.B, c.H, c.D, c.N_max); });
-  void* st = stream(a[5]);
-  check(released([&] { return spectre_prefix_cache_prefill(ctx, st, &c, &aq, &av, w.ptr, w.bytes); }));
+  check(released([&] { return spectre_prefix_cache_prefill(ctx, on.st, &c, &aq, &av, w.ptr, w.bytes); }));
   Py_RETURN_NONE;
 }
 
@@ -304,11 +317,11 @@ PyObject* append(PyObject* const* a) {
   spectre_ctx* ctx = context(a[0]);
   const at::Tensor &q = tensor(a[2]), &v = tensor(a[3]);
   contiguous_tokens(q, v);
+  const Stream on(a[5], q);
   at::Tensor vb;
   const spectre_cache c = cache_state(a[1], &vb);
   const int64_t t = integer(a[4]);
-  void* st = stream(a[5]);
-  check(released([&] { return spectre_prefix_cache_append(ctx, st, &c, q.data_ptr(), v.data_ptr(), t); }));
+  check(released([&] { return spectre_prefix_cache_append(ctx, on.st, &c, q.data_ptr(), v.data_ptr(), t); }));
   Py_RETURN_NONE;
 }
 
@@ -333,15 +346,15 @@ PyObject* decode_step(PyObject* const* a) {
   at::Tensor vb;
   const spectre_cache c = cache_state(a[1], &vb);
   const int64_t t = integer(a[4]);
+  const Stream on(a[10], v);
   at::Tensor y = none(a[7]) ? empty({c.B, nrows, c.H, c.D}, v, v.scalar_type()) : tensor(a[7]);
   at::Tensor g = none(a[8]) ? empty({c.B, c.H, c.N_max / 2 + 1, 2}, v, at::kFloat) : tensor(a[8]);
   const Workspace w(a[9], v, [&] {
     const int32_t r = nrows < 1 ? 1 : (nrows > SPECTRE_DECODE_MAX_ROWS ? SPECTRE_DECODE_MAX_ROWS : nrows);
     return spectre_decode_workspace_bytes(ctx, c.B, c.H, c.D, c.N_max, r, p.toeplitz_r);
   });
-  void* st = stream(a[10]);
   check(released([&] {
-    return spectre_prefix_cache_decode_step(ctx, st, &c, q.data_ptr(), v.data_ptr(), t, &p, rows.data(), nrows, y.data_ptr(),
+    return spectre_prefix_cache_decode_step(ctx, on.st, &c, q.data_ptr(), v.data_ptr(), t, &p, rows.data(), nrows, y.data_ptr(),
                                             (float*)g.data_ptr(), w.ptr, w.bytes);
   }));
   return Py_BuildValue("NN", THPVariable_Wrap(y), THPVariable_Wrap(g));
@@ -353,11 +366,11 @@ PyObject* readout(PyObject* const* a) {
   at::Tensor vb;
   const spectre_cache c = cache_state(a[1], &vb);
   const at::Tensor& g = tensor(a[2]);
+  const Stream on(a[5], g);
   at::Tensor y = none(a[3]) ? empty({c.B, c.N_max, c.H, c.D}, g, vb.scalar_type()) : tensor(a[3]);
   const spectre_act ay = act(y);
   const Workspace w(a[4], g, [&] { return spectre_readout_workspace_bytes(ctx, c.B, c.H, c.D, c.N_max); });
-  void* st = stream(a[5]);
-  check(released([&] { return spectre_prefix_cache_readout(ctx, st, &c, (const float*)g.data_ptr(), &ay, w.ptr, w.bytes); }));
+  check(released([&] { return spectre_prefix_cache_readout(ctx, on.st, &c, (const float*)g.data_ptr(), &ay, w.ptr, w.bytes); }));
   return THPVariable_Wrap(y);
 }
 
@@ -368,15 +381,15 @@ PyObject* project_qv(PyObject* const* a) {
   const spectre_act ax = act(x);
   if (wq.scalar_type() != wv.scalar_type() || !(wq.is_contiguous() && wv.is_contiguous()))
     raise(PyExc_ValueError, "Wq and Wv must be contiguous and of one dtype");
+  const Stream on(a[9], x);
   at::Tensor q = none(a[4]) ? at::empty_like(x) : tensor(a[4]), v = none(a[5]) ? at::empty_like(x) : tensor(a[5]), sum;
   if (!none(a[6])) sum = tensor(a[6]);
   else if (truth(a[7])) sum = empty({ax.B, ax.H, ax.D}, x, at::kFloat);
   const spectre_act aq = act(q), av = act(v);
   const Workspace w(a[8], x, [&] { return spectre_project_workspace_bytes(ctx, ax.H, ax.D); });
-  void* st = stream(a[9]);
   float* s = sum.defined() ? (float*)sum.data_ptr() : nullptr;
   const int32_t wd = dtype_code(wq);
-  check(released([&] { return spectre_project_qv(ctx, st, &ax, wq.data_ptr(), wv.data_ptr(), wd, &aq, &av, s, w.ptr, w.bytes); }));
+  check(released([&] { return spectre_project_qv(ctx, on.st, &ax, wq.data_ptr(), wv.data_ptr(), wd, &aq, &av, s, w.ptr, w.bytes); }));
   PyObject* so = sum.defined() ? THPVariable_Wrap(sum) : Py_NewRef(Py_None);
   return Py_BuildValue("NNN", THPVariable_Wrap(q), THPVariable_Wrap(v), so);
 }
@@ -389,6 +402,7 @@ PyObject* mixer_backward(PyObject* const* a) {
   const float* g = (const float*)pointer(a[3]);
   const int32_t n = none(a[4]) ? av.L : integer32(a[4]);
   const bool want_dv = truth(a[5]), want_dg = truth(a[6]);
+  const Stream on(a[8], v);
   at::Tensor dv, dg;
   spectre_act adv = {};
   if (want_dv) {
@@ -397,9 +411,8 @@ PyObject* mixer_backward(PyObject* const* a) {
   }
   if (want_dg) dg = empty({av.B, av.H, n / 2 + 1, 2}, v, at::kFloat);
   const Workspace w(a[7], v, [&] { return spectre_mixer_backward_workspace_bytes(ctx, av.B, av.L, av.H, av.D, n, av.dtype); });
-  void* st = stream(a[8]);
   float* pg = want_dg ? (float*)dg.data_ptr() : nullptr;
-  check(released([&] { return spectre_mixer_backward(ctx, st, &av, &ady, g, want_dv ? &adv : nullptr, pg, n, w.ptr, w.bytes); }));
+  check(released([&] { return spectre_mixer_backward(ctx, on.st, &av, &ady, g, want_dv ? &adv : nullptr, pg, n, w.ptr, w.bytes); }));
   PyObject* ov = want_dv ? THPVariable_Wrap(dv) : Py_NewRef(Py_None);
   PyObject* og = want_dg ? THPVariable_Wrap(dg) : Py_NewRef(Py_None);
   return Py_BuildValue("NN", ov, og);

@@ -958,6 +958,39 @@ def test_fp16_io_gate_wavelet_cache_decode_backward(ctx):
     assert max(rel_err(gate_to_complex(dg)[b, h], rg[b, h]) for b in range(B) for h in range(H)) < TOL["f32"]
 
 
+# ------------------------------------------------------------------ streams
+def test_what_a_call_on_a_given_stream_allocates_belongs_to_that_stream(ctx):
+    # torch's allocator reuses a freed block in the order of the stream it was allocated on: a workspace of another stream's would
+    # be handed on while the call's kernels still use it, and an output could be written before that stream is done with the block
+    w = W.Workload("t", B=1, L=16384, H=2, D=64, dtype="bf16", seed=3)
+    p = to_dev(W.gate_params(w))
+    x = W.activations(w).cuda()
+    wq = (torch.randn(2, 64, 64) * 0.1).cuda()
+    cache = S.PrefixCache(1, 2, 64, 16384)
+    wrm = {"levels": 2, "level_gates": torch.zeros(1, 2, 3, 64, device="cuda")}
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    torch.cuda.memory._record_memory_history(context=None, max_entries=10000)
+    try:
+        g = S.spectre_gate(ctx, p, w.n, q=x, stream=side)
+        y = S.spectre_mixer_forward(ctx, x, g, stream=side)
+        S.spectre_wavelet_refine(ctx, y, wrm, stream=side)
+        S.spectre_prefix_cache_prefill(ctx, cache, x, x, stream=side)
+        S.spectre_prefix_cache_readout(ctx, cache, g, stream=side)
+        S.spectre_prefix_cache_decode_step(ctx, cache, x[:, 0].contiguous(), x[:, 1].contiguous(), 16384, p, [5], stream=side)
+        S.spectre_project_qv(ctx, x, wq, wq, stream=side)
+        S.spectre_mixer_backward(ctx, x, x, g, stream=side)
+        events = [e for e in torch.cuda.memory._snapshot()["device_traces"][torch.cuda.current_device()] if e["action"] == "alloc"]
+    finally:
+        torch.cuda.memory._record_memory_history(enabled=None)
+    torch.cuda.synchronize()
+    mine = [e for e in events if e["stream"] == side.cuda_stream]
+    assert len(mine) >= 12, [(e["size"], e["stream"]) for e in events]
+    assert len(events) - len(mine) <= 2                      # x[:, 0] and x[:, 1] of the decode step, made here
+    ref = O.mixer(W.to_f64(x), gate_to_complex(g))
+    assert slab_err(W.to_f64(y), ref) < TOL["bf16"]
+
+
 # ------------------------------------------------------------------ errors
 def test_invalid_arguments_are_rejected_before_launch(ctx):
     x = torch.zeros(1, 64, 2, 16, device="cuda")
