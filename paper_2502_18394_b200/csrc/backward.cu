@@ -244,16 +244,7 @@ extern "C" int spectre_mixer_backward(spectre_ctx* ctx, void* stream, const spec
   auto pitch_ok = [](const spectre_act* a) { return !a || (a->stride_l >= 0 && a->stride_l <= (1 << 18)); };   // 32-bit row offsets
   if (dg && reg_supported(n_fft) && pitch_ok(v) && pitch_ok(dy) && pitch_ok(dv))
     return backward_reg(ctx, st, v, dy, g, dv, dg, n_fft, base + gc_bytes + mix_bytes, workspace_bytes - gc_bytes - mix_bytes);
-  if (dv) {
-    float2* gc = reinterpret_cast<float2*>(base);
-    const size_t total = (size_t)nslab * K;
-    SPECTRE_CUDA_OK(launch_after(conj_gate_kernel, (unsigned)((total + 255) / 256), 256, 0, st, reinterpret_cast<const float2*>(g), gc, total));
-    SPECTRE_LAUNCH_OK("conj_gate_kernel");
-    rc = spectre_mixer_forward(ctx, stream, dy, reinterpret_cast<const float*>(gc), dv, n_fft, nullptr,
-                               mix_bytes ? base + gc_bytes : nullptr, mix_bytes);
-    if (rc != SPECTRE_OK) return rc;
-  }
-  if (dg) {
+  if (dg) {                                  // first: dv may alias dy, which this reads
     size_t group = (workspace_bytes - gc_bytes - mix_bytes) / (2 * per);
     if (group > (size_t)nslab) group = (size_t)nslab;
     float2* wsV = reinterpret_cast<float2*>(base + gc_bytes + mix_bytes);
@@ -282,6 +273,15 @@ extern "C" int spectre_mixer_backward(spectre_ctx* ctx, void* stream, const spec
       }
       SPECTRE_LAUNCH_OK("gate_grad kernel");
     }
+  }
+  if (dv) {
+    float2* gc = reinterpret_cast<float2*>(base);
+    const size_t total = (size_t)nslab * K;
+    SPECTRE_CUDA_OK(launch_after(conj_gate_kernel, (unsigned)((total + 255) / 256), 256, 0, st, reinterpret_cast<const float2*>(g), gc, total));
+    SPECTRE_LAUNCH_OK("conj_gate_kernel");
+    rc = spectre_mixer_forward(ctx, stream, dy, reinterpret_cast<const float*>(gc), dv, n_fft, nullptr,
+                               mix_bytes ? base + gc_bytes : nullptr, mix_bytes);
+    if (rc != SPECTRE_OK) return rc;
   }
   return SPECTRE_OK;
 }

@@ -894,6 +894,20 @@ def test_mixer_backward(ctx, dt, L, n, D):
     assert torch.equal(only_dg, dg)
 
 
+@pytest.mark.parametrize("dt,n", [("bf16", 8192), ("f16", 4096), ("f32", 4096), ("f32", 90), ("bf16", 1024), ("bf16", 196)])
+def test_mixer_backward_in_place(ctx, dt, n):
+    # dv over dy, with the gate's gradient wanted too: one kernel for both and two passes
+    w = W.Workload("t", B=1, L=n, H=2, D=64, dtype=dt, seed=n)
+    v, dy, g = W.activations(w).cuda(), W.activations(w, stream=1).cuda(), W.random_gate(w).cuda()
+    ref_dv, ref_dg = O.mixer_backward(W.to_f64(v), W.to_f64(dy), gate_to_complex(g))
+    dg = torch.empty(1, 2, n // 2 + 1, 2, device="cuda")
+    ws = torch.empty(max(16, S.spectre_mixer_backward_workspace_bytes(ctx, 1, n, 2, 64, n, S._dtype_code(v))), dtype=torch.uint8, device="cuda")
+    S.prepare_mixer_backward(ctx, v, dy, g, dy, dg, ws)()
+    torch.cuda.synchronize()
+    assert slab_err(W.to_f64(dy), ref_dv) < TOL[dt]
+    assert rel_err(gate_to_complex(dg), ref_dg) < 1e-5
+
+
 # ------------------------------------------------------------------ fp16 I/O
 @pytest.mark.parametrize("n,L,D", [(64, 64, 16), (196, 196, 64), (1000, 1000, 24), (4096, 4096, 16), (8192, 8192, 64),
                                    (8192, 6000, 64), (16384, 16384, 16), (65536, 65536, 64)])
