@@ -381,10 +381,11 @@ PyObject* project_qv(PyObject* const* a) {
   const spectre_act ax = act(x);
   if (wq.scalar_type() != wv.scalar_type() || !(wq.is_contiguous() && wv.is_contiguous()))
     raise(PyExc_ValueError, "Wq and Wv must be contiguous and of one dtype");
+  const bool want_sum = none(a[6]) && truth(a[7]);
   const Stream on(a[9], x);
   at::Tensor q = none(a[4]) ? at::empty_like(x) : tensor(a[4]), v = none(a[5]) ? at::empty_like(x) : tensor(a[5]), sum;
   if (!none(a[6])) sum = tensor(a[6]);
-  else if (truth(a[7])) sum = empty({ax.B, ax.H, ax.D}, x, at::kFloat);
+  else if (want_sum) sum = empty({ax.B, ax.H, ax.D}, x, at::kFloat);
   const spectre_act aq = act(q), av = act(v);
   const Workspace w(a[8], x, [&] { return spectre_project_workspace_bytes(ctx, ax.H, ax.D); });
   float* s = sum.defined() ? (float*)sum.data_ptr() : nullptr;
