@@ -11,6 +11,8 @@ bool transform_supported(const spectre_ctx* ctx, int n);
 size_t transform_slab_bytes(int n, int D);
 int pool_sum_ring(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* q, float* sums, void* ring, int N);
 size_t gate_min_workspace(int B, int H, int D, int n_fft, int r);
+int gate_check(const spectre_ctx* ctx, const spectre_act* q, const float* sum_q, int B, int H, int D, float inv_count,
+               const spectre_gate_params* gp, int n_fft, const float* g_out, const void* workspace, size_t workspace_bytes);
 int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float* sum_q, int B, int H, int D, float inv_count,
               const spectre_gate_params* gp, int n_fft, const int64_t* shift, int64_t shift_all, float* g_out, float* qbar_out,
               void* workspace, size_t workspace_bytes, bool early);
@@ -533,12 +535,15 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   const size_t done_bytes = round256((size_t)B * H * sizeof(int));
   const size_t gate_bytes = gate_min_workspace(B, H, D, N, params->toeplitz_r < 0 ? 0 : params->toeplitz_r);
   if (workspace_bytes < delta_bytes + part_bytes + done_bytes + gate_bytes) return fail(SPECTRE_ERR_WORKSPACE, "decode workspace too small");
-  SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   float* delta = reinterpret_cast<float*>(workspace);
   float* partial = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(workspace) + delta_bytes);
   int* done = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes);
   void* gate_ws = reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes + done_bytes;
+  // a gate that would be refused below must not leave the cache with the token in it
+  rc = gate_check(ctx, nullptr, cache->sum_q, B, H, D, 1.0f / (float)N, params, N, g_out, gate_ws, gate_bytes);
+  if (rc != SPECTRE_OK) return rc;
+  SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int slot = (int)(t % N);
   const int evict = t >= N ? 1 : 0;
   // (a)-(b) ring buffers, running sum, delta

@@ -1021,10 +1021,23 @@ extern "C" size_t spectre_gate_workspace_bytes(const spectre_ctx* ctx, int32_t B
 }
 
 namespace spectre {
-// spectre_gate; `early`: see GateMlpParams
-int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float* sum_q, int B, int H, int D, float inv_count,
-              const spectre_gate_params* gp, int n_fft, const int64_t* shift, int64_t shift_all, float* g_out, float* qbar_out,
-              void* workspace, size_t workspace_bytes, bool early) {
+// Tensor cores for bf16 weights and the usual 64 hidden units (the fragments of A fill the registers): 4 or 8 entries (5 ... 7
+// would need two passes over W2 with 4).  With under 256 bins the 8 warps of its CTAs have no chunk each and the
+// narrower CTAs of the other kernels, more of them per SM, are faster (99 bins, 256 entries: 15 us against 16).  It reads a bin's two
+// output biases as one 8-byte word: an array that starts at an odd float (part of a flat parameter buffer) goes to the kernels that
+// read single floats.
+static bool gate_on_mma(const spectre_gate_params* gp, int B, int K) {
+  return gp->wdtype == SPECTRE_BF16 && gp->hidden == 64 && K >= 256 && B >= 2 && !(reinterpret_cast<uintptr_t>(gp->b2) & 7);
+}
+// batch entries per CTA: the weights of a head are fetched once for all of them
+static int gate_entries(const spectre_gate_params* gp, int B, int K) {
+  if (gate_on_mma(gp, B, K)) return B <= 4 ? 4 : 8;
+  return (gp->hidden > 256 || B < 2) ? 1 : (B < 4 ? 2 : (B < 8 ? 4 : 8));
+}
+
+// Everything that spectre_gate refuses, so that the decode step can ask before it changes the cache.
+int gate_check(const spectre_ctx* ctx, const spectre_act* q, const float* sum_q, int B, int H, int D, float inv_count,
+               const spectre_gate_params* gp, int n_fft, const float* g_out, const void* workspace, size_t workspace_bytes) {
   if (!ctx) return fail(SPECTRE_ERR_INVALID_ARG, "ctx is NULL");
   if (!gp) return fail(SPECTRE_ERR_INVALID_ARG, "gate parameters are NULL");
   if ((q != nullptr) == (sum_q != nullptr)) return fail(SPECTRE_ERR_INVALID_ARG, "give exactly one of q and sum_q");
@@ -1043,17 +1056,31 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
     int rc = check_act(q, "q");
     if (rc != SPECTRE_OK) return rc;
     if (q->B != B || q->H != H || q->D != D) return fail(SPECTRE_ERR_INVALID_ARG, "q shape differs from B, H, D");
-    if (!(inv_count > 0.f)) inv_count = 1.0f / (float)q->L;
   } else if (!(inv_count > 0.f)) {
     return fail(SPECTRE_ERR_INVALID_ARG, "inv_count must be positive with sum_q");
   }
-  const int K = n_fft / 2 + 1;
-  const int r = gp->toeplitz_r;
+  const int K = n_fft / 2 + 1, BB = gate_entries(gp, B, K);
+  if ((long long)H * ((B + BB - 1) / BB) > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "H * ceil(B / 8) exceeds 65535");
+  if (gp->toeplitz_r > 0 && (long long)B * H > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "B*H exceeds 65535");
   size_t sums_off, u_off;
-  const size_t need = gate_ws_layout(B, H, D, n_fft, r, gp->hidden, 1, &u_off, &sums_off);   // one copy is enough
+  const size_t need = gate_ws_layout(B, H, D, n_fft, gp->toeplitz_r, gp->hidden, 1, &u_off, &sums_off);   // one copy is enough
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 15))
     return fail(SPECTRE_ERR_WORKSPACE, "workspace is NULL or not 16-byte aligned");
   if (workspace_bytes < need) return fail(SPECTRE_ERR_WORKSPACE, "gate workspace too small");
+  return SPECTRE_OK;
+}
+
+// spectre_gate; `early`: see GateMlpParams
+int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float* sum_q, int B, int H, int D, float inv_count,
+              const spectre_gate_params* gp, int n_fft, const int64_t* shift, int64_t shift_all, float* g_out, float* qbar_out,
+              void* workspace, size_t workspace_bytes, bool early) {
+  int rc = gate_check(ctx, q, sum_q, B, H, D, inv_count, gp, n_fft, g_out, workspace, workspace_bytes);
+  if (rc != SPECTRE_OK) return rc;
+  if (q && !(inv_count > 0.f)) inv_count = 1.0f / (float)q->L;
+  const int K = n_fft / 2 + 1;
+  const int r = gp->toeplitz_r;
+  size_t sums_off, u_off;
+  gate_ws_layout(B, H, D, n_fft, r, gp->hidden, 1, &u_off, &sums_off);
   SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const float* sums = sum_q;
@@ -1066,7 +1093,7 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
     // Small weights are brought into L2 by the pooling pass: the gate kernel's chain of loads is latency then (2 heads, n = 1024:
     // gate call 16.6 -> 15.4 us; 8 heads, n = 4096: 16.8 -> 16.2).  Larger ones take the pass's own bandwidth for no gain
     // (8k: 21.9 -> 23.6 us).
-    int rc = pool_sum(ctx, st, q, pooled, fit > (size_t)kPoolCopies ? kPoolCopies : (int)fit, &ncopy, gp->W2, w2 <= ((size_t)4 << 20) ? w2 : 0);
+    rc = pool_sum(ctx, st, q, pooled, fit > (size_t)kPoolCopies ? kPoolCopies : (int)fit, &ncopy, gp->W2, w2 <= ((size_t)4 << 20) ? w2 : 0);
     if (rc != SPECTRE_OK) return rc;
     sums = pooled;
   }
@@ -1093,16 +1120,9 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
   mp.g_out = r > 0 ? raw : reinterpret_cast<float2*>(g_out);
   // block sized to the bin count for short transforms (K = 99 does not need 256 threads)
   const int thr_out = K >= 256 ? 256 : ((K + 31) / 32 * 32 < 64 ? 64 : (K + 31) / 32 * 32);
-  // batch entries per CTA: the weights of a head are fetched once for all of them
-  // Tensor cores for bf16 weights and the usual 64 hidden units (the fragments of A fill the registers): 4 or 8 entries (5 ... 7
-  // would need two passes over W2 with 4).  With under 256 bins the 8 warps of its CTAs have no chunk each and the
-  // narrower CTAs below, more of them per SM, are faster (99 bins, 256 entries: 15 us against 16).  It reads a bin's two output
-  // biases as one 8-byte word: an array that starts at an odd float (part of a flat parameter buffer) goes to the kernels that
-  // read single floats.
-  const bool mma = gp->wdtype == SPECTRE_BF16 && gp->hidden == 64 && K >= 256 && B >= 2 && !(reinterpret_cast<uintptr_t>(gp->b2) & 7);
-  const int BB = mma ? (B <= 4 ? 4 : 8) : (gp->hidden > 256 || B < 2) ? 1 : (B < 4 ? 2 : (B < 8 ? 4 : 8));
+  const bool mma = gate_on_mma(gp, B, K);
+  const int BB = gate_entries(gp, B, K);
   dim3 grid_out((K + thr_out - 1) / thr_out, (unsigned)(H * ((B + BB - 1) / BB)));
-  if (grid_out.y > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "H * ceil(B / 8) exceeds 65535");
   const bool wb = gp->wdtype == SPECTRE_BF16;
   const size_t w1_bytes = (size_t)D * gp->hidden * (wb ? 2 : 4);
   const size_t act_bytes = (((size_t)BB * (D + gp->hidden) + 3) & ~(size_t)3) * sizeof(float);
@@ -1180,7 +1200,6 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
     pp.shift = mp.shift; pp.shift_all = shift_all;
     pp.H = H; pp.K = K; pp.n = n_fft;
     dim3 grid((K + 255) / 256, B * H);
-    if (grid.y > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "B*H exceeds 65535");
     SPECTRE_CUDA_OK(launch_after(gate_post_kernel, grid, 256, 0, st, pp));
     SPECTRE_LAUNCH_OK("gate_post_kernel");
   }

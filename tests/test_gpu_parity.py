@@ -777,6 +777,25 @@ def test_decode_step_leaves_the_same_state_as_append(ctx):
     assert torch.equal(a.V_buf, b.V_buf) and torch.equal(a.Q_buf, b.Q_buf)
 
 
+def test_a_refused_decode_step_leaves_the_cache_as_it_was(ctx):
+    w = W.Workload("t", B=1, L=40, H=2, D=64, dtype="f32", wdtype="f32", n_fft=64, seed=2)
+    cache = S.PrefixCache(1, 2, 64, 64, dtype=torch.float32)
+    x = W.activations(w).cuda()
+    S.spectre_prefix_cache_prefill(ctx, cache, x, x)
+    p = to_dev(W.gate_params(w))
+    state = ("prefix_fft", "V_buf", "Q_buf", "sum_q")
+    before = [getattr(cache, k).clone() for k in state]
+    odd = torch.empty(p["W2"].numel() + 1, device="cuda")[1:].view(p["W2"].shape)
+    odd_g = torch.empty(2 * 33 * 2 + 1, device="cuda")[1:].view(1, 2, 33, 2)
+    for params, g_out, status in ((dict(p, W2=odd), None, S.SPECTRE_ERR_INVALID_ARG), (dict(p, hidden=2000), None, S.SPECTRE_ERR_UNSUPPORTED),
+                                  (dict(p, ln_eps=-1.0), None, S.SPECTRE_ERR_INVALID_ARG), (p, odd_g, S.SPECTRE_ERR_INVALID_ARG)):
+        with pytest.raises(S.SpectreError) as e:
+            S.spectre_prefix_cache_decode_step(ctx, cache, x[:, 0].contiguous(), x[:, 1].contiguous(), 70, params, [63], g_out=g_out)
+        assert e.value.status == status
+        torch.cuda.synchronize()
+        assert all(torch.equal(getattr(cache, k), b) for k, b in zip(state, before))
+
+
 def test_decode_step_rejects_bad_rows(ctx):
     N = 64
     w = W.Workload("t", B=1, L=8, H=2, D=16, dtype="f32", wdtype="f32", n_fft=N, seed=2, N_max=N)
