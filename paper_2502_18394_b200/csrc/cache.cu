@@ -160,6 +160,20 @@ __global__ void __launch_bounds__(256) append_spectrum_kernel(float* prefix, con
   const int slab = (int)(wid / warps_per_slab);
   const int k0 = (int)(wid % warps_per_slab) * 32;
   const int b = slab / H, h = slab - b * H;
+  const int half = D / 2;
+  auto difference = [&](int c, float& d0, float& d1) {
+    d0 = d1 = 0.f;
+    if (c >= half) return;
+    d0 = io<T>::load1(v_t + (size_t)slab * D + 2 * c);
+    d1 = io<T>::load1(v_t + (size_t)slab * D + 2 * c + 1);
+    if (evict) {
+      const T* old = V_buf + (((size_t)b * N + slot) * H + h) * D + 2 * c;
+      d0 -= io<T>::load1(old);
+      d1 -= io<T>::load1(old + 1);
+    }
+  };
+  float d0, d1;
+  difference(lane, d0, d1);                    // on its way while the twiddle is evaluated
   // twiddle exp(-j 2 pi k t / N) of bin k0 + lane, angle reduced in integers
   float2 my = make_float2(1.f, 0.f);
   if (k0 + lane < K) {
@@ -167,21 +181,11 @@ __global__ void __launch_bounds__(256) append_spectrum_kernel(float* prefix, con
     my = twiddle_fwd(kk, (unsigned)N);
   }
   const int nb = min(32, K - k0);
-  const int half = D / 2;
   float* base = prefix + (((size_t)slab * K + k0) * D) * 2;
   for (int c0 = 0; c0 < half; c0 += 32) {      // uniform trip count: every lane takes part in the shuffles
     const int c = c0 + lane;
     const bool live = c < half;
-    float d0 = 0.f, d1 = 0.f;
-    if (live) {
-      d0 = io<T>::load1(v_t + (size_t)slab * D + 2 * c);
-      d1 = io<T>::load1(v_t + (size_t)slab * D + 2 * c + 1);
-      if (evict) {
-        const T* old = V_buf + (((size_t)b * N + slot) * H + h) * D + 2 * c;
-        d0 -= io<T>::load1(old);
-        d1 -= io<T>::load1(old + 1);
-      }
-    }
+    if (c0 > 0) difference(c, d0, d1);
     // four bins per round, their loads issued together (the compiler cannot move a load of this array
     // above the store before it)
     for (int i0 = 0; i0 < nb; i0 += 4) {
@@ -213,11 +217,11 @@ __global__ void __launch_bounds__(256) append_ring_kernel(T* V_buf, T* Q_buf,
   if (idx >= total) return;
   int b = idx / (H * D), hd = idx - b * (H * D);
   size_t o = ((size_t)b * N + slot) * H * D + hd;
-  float qn = io<T>::load1(q_t + idx);
-  float qo = evict ? io<T>::load1(Q_buf + o) : 0.f;
-  sum_q[idx] += qn - qo;
-  Q_buf[o] = q_t[idx];
-  V_buf[o] = v_t[idx];
+  const T q = q_t[idx], v = v_t[idx];          // all loads in front of the stores, which none may pass
+  const float s = sum_q[idx], qo = evict ? io<T>::load1(Q_buf + o) : 0.f;
+  sum_q[idx] = s + (io<T>::load1(&q) - qo);
+  Q_buf[o] = q;
+  V_buf[o] = v;
 }
 
 
@@ -237,13 +241,12 @@ __global__ void __launch_bounds__(256) decode_ring_kernel(T* V_buf, T* Q_buf,
   if (idx < B * H) done[idx] = 0;                          // the spectrum pass counts a slab's finished blocks here
   int b = idx / (H * D), hd = idx - b * (H * D);
   size_t o = ((size_t)b * N + slot) * H * D + hd;
-  float qn = io<T>::load1(q_t + idx), vn = io<T>::load1(v_t + idx);
-  float qo = evict ? io<T>::load1(Q_buf + o) : 0.f;
-  float vo = evict ? io<T>::load1(V_buf + o) : 0.f;
-  sum_q[idx] += qn - qo;
-  delta[idx] = vn - vo;
-  Q_buf[o] = q_t[idx];
-  V_buf[o] = v_t[idx];
+  const T q = q_t[idx], v = v_t[idx];                      // all loads in front of the stores, which none may pass
+  const float s = sum_q[idx], qo = evict ? io<T>::load1(Q_buf + o) : 0.f, vo = evict ? io<T>::load1(V_buf + o) : 0.f;
+  sum_q[idx] = s + (io<T>::load1(&q) - qo);
+  delta[idx] = io<T>::load1(&v) - vo;
+  Q_buf[o] = q;
+  V_buf[o] = v;
 }
 
 struct DecodeRows { int r[SPECTRE_DECODE_MAX_ROWS]; };
