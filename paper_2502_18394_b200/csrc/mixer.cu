@@ -33,6 +33,8 @@ namespace cg = cooperative_groups;
 
 namespace spectre {
 
+int wavelet_check(const spectre_ctx* ctx, int L, int D, const spectre_wavelet* w);   // wavelet.cu
+
 int launch_mixer_tc8192(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g,
                         const spectre_act* y);   // mixer_tc.cu
 bool tc8192_supported(const spectre_act* v, const spectre_act* y);                     // mixer_tc8k.cu
@@ -929,8 +931,8 @@ extern "C" int spectre_mixer_forward(spectre_ctx* ctx, void* stream, const spect
     if (overlap && (staged || pl.N1 > 1)) return fail(SPECTRE_ERR_INVALID_ARG, "y may not overlap v on the multi-pass path");
   }
   if (wrm) {
-    if (wrm->levels < 1 || wrm->levels > 10 || (v->L % (1 << wrm->levels)) != 0)
-      return fail(SPECTRE_ERR_INVALID_ARG, "wavelet levels: 2^J must divide L");
+    rc = wavelet_check(ctx, v->L, v->D, wrm);                // a refinement that would be refused behind the mixer
+    if (rc != SPECTRE_OK) return rc;
   }
   SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

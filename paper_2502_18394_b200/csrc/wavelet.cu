@@ -228,6 +228,31 @@ static int launch_wavelet_reg(const WaveletParams& p, int J, unsigned grid, size
   return SPECTRE_OK;
 }
 
+// Rows of a shared-memory tile (J > 4) and the kernel's shared memory: about 32 KB of fp32 per CTA
+static int wavelet_rows(int L, int D, int J) {
+  const int span = 1 << J, rows = (8192 / D) / span * span;
+  return rows < span ? (span < L ? span : L) : (rows < L ? rows : L);
+}
+static size_t wavelet_smem(int L, int D, const spectre_wavelet* w) {
+  return ((size_t)wavelet_rows(L, D, w->levels) * D + (size_t)(w->levels + 1) * D + (w->level_gates ? 0 : w->hidden)) * sizeof(float);
+}
+
+// Everything that the refinement of an [.., L, .., D] tensor refuses, so that spectre_mixer_forward can ask before it writes one.
+int wavelet_check(const spectre_ctx* ctx, int L, int D, const spectre_wavelet* w) {
+  const int J = w->levels;
+  if (J < 1 || J > 10) return fail(SPECTRE_ERR_INVALID_ARG, "wavelet levels must be in 1..10");
+  if (L % (1 << J)) return fail(SPECTRE_ERR_INVALID_ARG, "2^J must divide L");
+  if (!w->level_gates) {
+    if (!w->qbar || !w->Ww1 || !w->bw1 || !w->Ww2 || !w->bw2)
+      return fail(SPECTRE_ERR_INVALID_ARG, "level_gates is NULL and the MLP inputs are incomplete");
+    if (w->hidden < 1 || w->hidden > 1024) return fail(SPECTRE_ERR_UNSUPPORTED, "wavelet hidden width must be in 1..1024");
+    if (w->wdtype != SPECTRE_F32 && w->wdtype != SPECTRE_BF16) return fail(SPECTRE_ERR_INVALID_ARG, "unknown weight dtype");
+  }
+  if (J > 4 && wavelet_smem(L, D, w) > (size_t)ctx->max_smem_optin)
+    return fail(SPECTRE_ERR_UNSUPPORTED, "2^J * D exceeds the shared-memory tile");
+  return SPECTRE_OK;
+}
+
 }  // namespace spectre
 
 using namespace spectre;
@@ -244,14 +269,8 @@ extern "C" int spectre_wavelet_refine(spectre_ctx* ctx, void* stream, const spec
       y_in->dtype != y_out->dtype)
     return fail(SPECTRE_ERR_INVALID_ARG, "y_in and y_out differ in shape or dtype");
   const int J = w->levels, L = y_in->L, D = y_in->D;
-  if (J < 1 || J > 10) return fail(SPECTRE_ERR_INVALID_ARG, "wavelet levels must be in 1..10");
-  if (L % (1 << J)) return fail(SPECTRE_ERR_INVALID_ARG, "2^J must divide L");
-  if (!w->level_gates) {
-    if (!w->qbar || !w->Ww1 || !w->bw1 || !w->Ww2 || !w->bw2)
-      return fail(SPECTRE_ERR_INVALID_ARG, "level_gates is NULL and the MLP inputs are incomplete");
-    if (w->hidden < 1 || w->hidden > 1024) return fail(SPECTRE_ERR_UNSUPPORTED, "wavelet hidden width must be in 1..1024");
-    if (w->wdtype != SPECTRE_F32 && w->wdtype != SPECTRE_BF16) return fail(SPECTRE_ERR_INVALID_ARG, "unknown weight dtype");
-  }
+  rc = wavelet_check(ctx, L, D, w);
+  if (rc != SPECTRE_OK) return rc;
   if (J <= 4) {                              // register-resident streaming kernel
     SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
     cudaStream_t st0 = reinterpret_cast<cudaStream_t>(stream);
@@ -274,13 +293,8 @@ extern "C" int spectre_wavelet_refine(spectre_ctx* ctx, void* stream, const spec
       return launch_wavelet_reg<T, float>(p0, J, grid0, smem0, st0);
     });
   }
-  const int span = 1 << J;
-  int rows = (8192 / D) / span * span;      // about 32 KB of fp32 per CTA
-  if (rows < span) rows = span;
-  if (rows > L) rows = L;
-  const int hidden = w->level_gates ? 0 : w->hidden;
-  size_t smem = ((size_t)rows * D + (size_t)(J + 1) * D + hidden) * sizeof(float);
-  if (smem > (size_t)ctx->max_smem_optin) return fail(SPECTRE_ERR_UNSUPPORTED, "2^J * D exceeds the shared-memory tile");
+  const int rows = wavelet_rows(L, D, J), hidden = w->level_gates ? 0 : w->hidden;
+  const size_t smem = wavelet_smem(L, D, w);
   SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   WaveletParams p = {};
