@@ -157,7 +157,10 @@ static int pool_launch(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
   if (rows_per < 8) rows_per = 8;
   int nslice = (rows + rows_per - 1) / rows_per;
   // Sequences of up to 1024 rows: a slice per copy instead, stored without a kernel that clears them (2 us of host time, and
-  // the second's launch; one warp's 16 rows take 2 or 4 rounds of loads)
+  // the second's launch; one warp's 16 rows take 2 or 4 rounds of loads).  Gate call alone, many slices -> 8: at 1024 rows it gains
+  // throughout (1 x 8 heads bf16 7.9 -> 6.8 us, 8 x 8 13.9 -> 12.5, fp32 1 x 32 13.2 -> 11.8), at 2048 in bf16 only (10.9 -> 9.1,
+  // 15.1 -> 14.9; fp32 14.5 -> 15.3, 4 x 4 13.2 -> 14.1), at 4096 hardly anywhere (12.0 -> 13.5, 19.4 -> 21.5, 18.5 -> 23.1).  With
+  // the mixer behind it 2048 rows gain nothing on the whole (bf16 4 x 4 30.5 -> 31.0, 8 x 8 48.7 -> 49.2, fp32 4 x 4 31.9 -> 34.3).
   if (nslice > 8 && ncopy_max >= 8 && rows <= 1024) {
     rows_per = (rows + 7) / 8;
     nslice = (rows + rows_per - 1) / rows_per;
@@ -665,7 +668,7 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
   }
 }
 
-// ---- the whole gate of one batch entry when its CTAs leave room ----
+// ---- the whole gate of one batch entry in few CTAs ----
 // kParts threads share a bin, each with kRows rows of W2: with the usual 64 hidden units every weight is requested ahead of the
 // wait for the sums, where gate_out_kernel's thread takes 2 (bf16) or 4 (fp32) dependent rounds of loads.  The chain behind the wait is
 // all that is left.
@@ -1021,11 +1024,13 @@ extern "C" size_t spectre_gate_workspace_bytes(const spectre_ctx* ctx, int32_t B
 }
 
 namespace spectre {
-// Tensor cores for bf16 weights and the usual 64 hidden units (the fragments of A fill the registers): 4 or 8 entries (5 ... 7
-// would need two passes over W2 with 4).  With under 256 bins the 8 warps of its CTAs have no chunk each and the
-// narrower CTAs of the other kernels, more of them per SM, are faster (99 bins, 256 entries: 15 us against 16).  It reads a bin's two
-// output biases as one 8-byte word: an array that starts at an odd float (part of a flat parameter buffer) goes to the kernels that
-// read single floats.
+// Tensor cores for bf16 weights and 64 hidden units, the width of every workload here: the kernel's loops over the hidden units
+// are written for it, and the fragments of A fill the registers then.  Narrower widths stay on the other kernels, which at 32 are
+// no slower than this one would be at 64 (8 entries x 32 heads x 32768: 43.8 us against 54.0; 8 x 8 x 1024 9.7 : 9.8), but at 48 are
+// (65.6 against 54.0): a form for multiples of 16 would gain there.  4 or 8 entries (5 ... 7 would need two passes over W2 with
+// 4).  With under 256 bins the 8 warps of its CTAs have no chunk each and the narrower CTAs of the other kernels, more of them per
+// SM, are faster (99 bins, 256 entries: 15 us against 16).  It reads a bin's two output biases as one 8-byte word: an array that
+// starts at an odd float (part of a flat parameter buffer) goes to the kernels that read single floats.
 static bool gate_on_mma(const spectre_gate_params* gp, int B, int K) {
   return gp->wdtype == SPECTRE_BF16 && gp->hidden == 64 && K >= 256 && B >= 2 && !(reinterpret_cast<uintptr_t>(gp->b2) & 7);
 }
@@ -1153,10 +1158,15 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
     cfg_mma.gridDim = dim3((unsigned)(fit < 1 ? 1 : (blocks < fit ? blocks : fit)), grid_out.y, 1);
     cfg_mma.blockDim = dim3(256, 1, 1);
   }
-  // One entry per CTA and 2 (bf16) or 4 (fp32) threads per bin where every CTA has an SM to itself (1024 points, 2 heads, fp32: the chain
-  // of three kernels 14.0 -> 12.8 us); with three CTAs per SM they crowd out the kernel behind (4k decode step 16.6 -> 19.0)
+  // One entry and 2 (bf16) or 4 (fp32) threads per bin where its CTAs are few: a quarter of the SMs in bf16, three eighths in fp32.
+  // The gate by itself gains beyond that (fp32, 14 heads x 1024: 10.4 -> 9.2 us), but the kernel behind starts beside these CTAs
+  // and shares SMs that it would have had to itself.  Gate and mixer together, one sequence of 512 ... 8192 points: every number of
+  // heads below the line gains, 0.25 ... 2.1 us (bf16 4 x 2048 23.1 -> 22.0, fp32 4 x 1024 17.7 -> 16.0); between it and one CTA per SM
+  // it is -2.4 ... +6.7 (bf16 8 x 4096 27.9 -> 34.6, fp32 12 x 1024 21.2 -> 26.0).  A decode step gains 0.1 ... 1.6 us below the line and
+  // loses up to 1.7 with more CTAs than SMs (bf16 12 x 4096 15.3 -> 17.0).
   const int split_bins = wb ? 128 : 64;
-  const bool split = BB == 1 && !pre && (long long)((K + split_bins - 1) / split_bins) * B * H <= ctx->sm_count;
+  const long long split_ctas = (long long)((K + split_bins - 1) / split_bins) * B * H;
+  const bool split = BB == 1 && !pre && 8 * split_ctas <= (wb ? 2 : 3) * (long long)ctx->sm_count;
   cudaLaunchConfig_t cfg_split = cfg_out;
   cfg_split.gridDim = dim3((unsigned)((K + split_bins - 1) / split_bins), (unsigned)(B * H), 1); cfg_split.blockDim = dim3(256, 1, 1);
   cudaLaunchConfig_t cfg_short = cfg_out;

@@ -354,10 +354,11 @@ def test_gate_short_transforms(ctx, B, n, D, hid, wdt, r, shifts):
 
 
 @pytest.mark.parametrize("B,H,L,n,D,hid,wdt,r", [(1, 2, 1024, 1024, 64, 64, "f32", 0), (1, 3, 77, 500, 64, 100, "bf16", 2), (2, 2, 9, 128, 32, 300, "f32", 0),
-                                                 (1, 1, 1, 2, 8, 8, "bf16", 0), (1, 2, 1023, 4094, 64, 64, "bf16", 0), (1, 1, 1025, 1026, 24, 17, "f32", 0)])
+                                                 (1, 1, 1, 2, 8, 8, "bf16", 0), (1, 2, 1023, 4094, 64, 64, "bf16", 0), (1, 1, 1025, 1026, 24, 17, "f32", 0),
+                                                 (1, 18, 33, 510, 64, 64, "bf16", 0), (1, 19, 33, 510, 64, 64, "bf16", 0), (1, 6, 33, 1022, 64, 64, "f32", 0), (1, 7, 33, 1022, 64, 64, "f32", 0)])
 def test_gate_few_blocks(ctx, B, H, L, n, D, hid, wdt, r):
-    # several threads per bin: hidden widths below and above the rows they hold, the last block of bins partial; pooled sums in a
-    # copy per slice up to 1024 rows and beyond
+    # several threads per bin: hidden widths below and above the rows they hold, the last block of bins partial, heads on both sides
+    # of its line; pooled sums in a copy per slice up to 1024 rows and beyond
     w = W.Workload("t", B=B, L=L, H=H, D=D, dtype="bf16", wdtype=wdt, n_fft=n, hidden=hid, seed=n + hid)
     p = W.gate_params(w, modrelu_bias_std=0.01, toeplitz_r=r, bias_std=0.1)
     x = W.activations(w, structured=True)
