@@ -160,39 +160,42 @@ __global__ void __launch_bounds__(256) append_spectrum_kernel(float* prefix, con
   const int slab = (int)(wid / warps_per_slab);
   const int k0 = (int)(wid % warps_per_slab) * 32;
   const int b = slab / H, h = slab - b * H;
-  const int half = D / 2;
-  auto difference = [&](int c, float& d0, float& d1) {
-    d0 = d1 = 0.f;
-    if (c >= half) return;
-    d0 = io<T>::load1(v_t + (size_t)slab * D + 2 * c);
-    d1 = io<T>::load1(v_t + (size_t)slab * D + 2 * c + 1);
-    if (evict) {
-      const T* old = V_buf + (((size_t)b * N + slot) * H + h) * D + 2 * c;
-      d0 -= io<T>::load1(old);
-      d1 -= io<T>::load1(old + 1);
-    }
+  const int half = D / 2, nb = min(32, K - k0);
+  float* base = prefix + (((size_t)slab * K + k0) * D) * 2;
+  // four bins per round, their loads issued together (the compiler cannot move a load of this array
+  // above the store before it)
+  float4 v[4];
+  auto fetch = [&](int i0, int c) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c < half && i0 + u < nb) v[u] = *reinterpret_cast<const float4*>(base + ((size_t)(i0 + u) * D + 2 * c) * 2);
   };
-  float d0, d1;
-  difference(lane, d0, d1);                    // on its way while the twiddle is evaluated
+  T tok[2], old[2];                            // as loaded, so that nothing waits for them yet
+  auto token = [&](int c) {
+    if (c >= half) return;
+    const T *a = v_t + (size_t)slab * D + 2 * c, *o = evict ? V_buf + (((size_t)b * N + slot) * H + h) * D + 2 * c : a;
+    tok[0] = a[0]; tok[1] = a[1];
+    old[0] = o[0]; old[1] = o[1];
+  };
+  token(lane);
+  fetch(0, lane);
   // twiddle exp(-j 2 pi k t / N) of bin k0 + lane, angle reduced in integers
   float2 my = make_float2(1.f, 0.f);
   if (k0 + lane < K) {
     unsigned kk = (unsigned)(((unsigned long long)(k0 + lane) * tm) % (unsigned)N);
     my = twiddle_fwd(kk, (unsigned)N);
   }
-  const int nb = min(32, K - k0);
-  float* base = prefix + (((size_t)slab * K + k0) * D) * 2;
   for (int c0 = 0; c0 < half; c0 += 32) {      // uniform trip count: every lane takes part in the shuffles
     const int c = c0 + lane;
     const bool live = c < half;
-    if (c0 > 0) difference(c, d0, d1);
-    // four bins per round, their loads issued together (the compiler cannot move a load of this array
-    // above the store before it)
+    if (c0 > 0) token(c);
+    float d0 = 0.f, d1 = 0.f;
+    if (live) {
+      d0 = io<T>::load1(tok) - (evict ? io<T>::load1(old) : 0.f);
+      d1 = io<T>::load1(tok + 1) - (evict ? io<T>::load1(old + 1) : 0.f);
+    }
     for (int i0 = 0; i0 < nb; i0 += 4) {
-      float4 v[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (live && i0 + u < nb) v[u] = *reinterpret_cast<const float4*>(base + ((size_t)(i0 + u) * D + 2 * c) * 2);
+      if (c0 + i0 > 0) fetch(i0, c);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int i = min(i0 + u, 31);
