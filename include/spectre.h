@@ -53,7 +53,7 @@ typedef struct spectre_ctx spectre_ctx;   /* opaque: device properties, launch l
  * tables (the 64-point and 49-point DFT matrices of the tensor-core mixers, 32 KiB each; the
  * twiddles between two 64-point stages and a quarter-wave twiddle table, 16 KiB each; the twiddles
  * of the four-step splits n = 4096 R, 63 KiB; the DFT matrices of the tensor-core radix-32 ... 2
- * kernels, 320 KiB; the twiddles of the register-resident fp32 transforms, 52 KiB)
+ * kernels, 320 KiB; the twiddles of the register-resident fp32 transforms, 64 KiB)
  * and one pinned status word, all released by spectre_destroy.  No other call allocates. */
 int spectre_create(spectre_ctx** out, int device);
 int spectre_destroy(spectre_ctx* ctx);

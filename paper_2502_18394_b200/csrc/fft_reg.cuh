@@ -160,12 +160,18 @@ template <bool INV> struct RegDft<4, INV> {
 SPECTRE_REG_ODD(3)
 SPECTRE_REG_ODD(5)
 SPECTRE_REG_ODD(7)
+SPECTRE_REG_CT(6, 2, 3)
 SPECTRE_REG_CT(8, 2, 4)
+SPECTRE_REG_CT(9, 3, 3)
+SPECTRE_REG_CT(10, 2, 5)
+SPECTRE_REG_CT(12, 3, 4)
 SPECTRE_REG_CT(14, 2, 7)
 SPECTRE_REG_CT(16, 4, 4)
+SPECTRE_REG_CT(18, 2, 9)
 SPECTRE_REG_CT(20, 4, 5)
 SPECTRE_REG_CT(24, 3, 8)
 SPECTRE_REG_CT(28, 4, 7)
+SPECTRE_REG_CT(30, 5, 6)
 SPECTRE_REG_CT(32, 4, 8)
 #undef SPECTRE_REG_ODD
 #undef SPECTRE_REG_CT

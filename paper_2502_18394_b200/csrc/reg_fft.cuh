@@ -517,7 +517,11 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
 // rows N1 tokens apart).
 //   map   dims (column, row, head, batch) of the tokens; boxes of 16 columns x reg_box_rows() rows land as [row][8 pairs],
 //         from which the threads of a warp read 128 contiguous bytes; rows and columns beyond the tensor are zeros
-template <class P> __host__ __device__ constexpr int reg_box_rows() { return P::M / ((P::M + 255) / 256); }     // at most 256, dividing M
+template <class P> __host__ __device__ constexpr int reg_box_rows() {                  // the most that divide M: at most 256, whole 128-byte pieces
+  int r = 256;
+  while (P::M % r || r % 4) --r;
+  return r;
+}
 template <class P> __host__ __device__ constexpr size_t reg_stream_bytes() {            // rows, exchange, gate table, barrier
   return (size_t)P::M * P::C * 4 + reg_exch_bytes<P, kRegMix>() + (size_t)P::kGate * 8 + 16;
 }

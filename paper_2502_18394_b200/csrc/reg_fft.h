@@ -25,8 +25,15 @@ struct RegParams {
   float scale;              // 1/n, folded into the gate
 };
 
-// Lengths M that one CTA transforms: powers of two 64 ... 2048 and the squares of 14, 20, 24, 28 (patch grids).
-#define SPECTRE_REG_TWO_STEP(X) X(8, 8) X(16, 8) X(16, 16) X(32, 16) X(32, 32) X(14, 14) X(20, 20) X(24, 24) X(28, 28)
+// Lengths M that one CTA transforms: the powers of two 64 ... 2048 and, for patch grids, the square of every even side from 8 to 32
+// whose prime factors are 2, 3, 5, 7 (the others are no supported lengths).  Even, because the twiddle tables hold pairs of
+// factors; the first step is at least the second and a multiple of it, so that a thread holds as many points on either side of
+// the exchange: odd sides and most rectangles have no such plan and run on onchip_kernel.  Mixer of 12.6 M elements there and
+// here, fp32 / bf16, us: 100 89 / 106 -> 28 / 25, 144 102 / 113 -> 25 / 20, 324 129 / 149 -> 33 / 30, 900 119 / 135 -> 36 / 35 (its backward
+// 236 ... 368 -> 38 ... 62), one sequence of 900 19 -> 7; what stays there: 225 96 / 111, 441 113 / 130, 192 71 / 88, 384 86 / 105.
+#define SPECTRE_REG_TWO_STEP(X)                                  \
+  X(8, 8) X(16, 8) X(16, 16) X(32, 16) X(32, 32) X(10, 10)       \
+  X(12, 12) X(14, 14) X(18, 18) X(20, 20) X(24, 24) X(28, 28) X(30, 30)
 bool reg_supported(int M);
 constexpr int kRegWsM = 1024;    // the length whose rows may also come from the complex workspace
 // partial sums per (batch, head) and bin that the gradient leaves, one per group of pairs summed inside a warp

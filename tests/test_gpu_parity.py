@@ -51,7 +51,8 @@ def test_mixer_f32_four_step(ctx, n):
 @pytest.mark.parametrize("dt,n,L,D", [("f32", 64, 1, 8), ("bf16", 128, 127, 24), ("f16", 256, 129, 40), ("bf16", 400, 400, 64),
                                       ("f32", 576, 290, 16), ("f16", 784, 784, 24), ("bf16", 512, 511, 8), ("f32", 1024, 1000, 24),
                                       ("bf16", 2048, 1025, 40), ("f32", 4096, 2049, 24), ("f16", 8192, 5003, 40), ("f32", 16384, 9001, 8),
-                                      ("f32", 32768, 20011, 24)])
+                                      ("f32", 32768, 20011, 24), ("bf16", 100, 99, 64), ("f32", 144, 144, 24), ("f16", 324, 300, 40),
+                                      ("f32", 900, 900, 16), ("f32", 324, 324, 8), ("f32", 100, 1, 8), ("bf16", 900, 899, 24)])
 def test_register_transforms(ctx, dt, n, L, D):
     # partial column tiles, idle threads, rows cut anywhere; the workspace route and, at 4096 / 8192, in place without one
     w = W.Workload("t", B=2, L=L, H=3, D=D, dtype=dt, n_fft=n, seed=n + L)
@@ -70,7 +71,8 @@ def test_register_transforms(ctx, dt, n, L, D):
 
 
 @pytest.mark.parametrize("dt,B,H,n,L,D", [("bf16", 20, 8, 1024, 1000, 40), ("f16", 64, 8, 256, 255, 64), ("bf16", 40, 8, 784, 784, 24),
-                                               ("f32", 10, 8, 1024, 1000, 24), ("f32", 10, 8, 2048, 1025, 24)])
+                                               ("f32", 10, 8, 1024, 1000, 24), ("f32", 10, 8, 2048, 1025, 24), ("bf16", 300, 8, 100, 99, 24),
+                                               ("f16", 300, 8, 144, 144, 40), ("bf16", 60, 8, 324, 323, 64), ("f16", 40, 8, 900, 900, 24)])
 def test_register_transforms_more_tiles_than_resident(ctx, dt, B, H, n, L, D):
     # persistent CTAs, rows of the next tile by TMA: column tiles beyond D, rows beyond L, several tiles per CTA
     assert run_mixer(ctx, W.Workload("t", B=B, L=L, H=H, D=D, dtype=dt, n_fft=n, seed=n + L), n_fft=n) < TOL[dt]
