@@ -57,23 +57,6 @@ NCU_TRAFFIC_VARIANT = {("c4", "prefill"): (10208e6, "profiles/launches_c4_prefil
                        ("c4", "readout"): (7015e6, "profiles/launches_c4_readout.md (ncu capture at B = 2, x4; not this run)")}
 
 
-def pool_launches(B, rows, H, D, sm_count=148, copies=16):
-    """Kernels of one pooling pass: the pass itself and, when it runs in more slices of the sequence than there are
-    copies of the sums to store (the library's rule, restated), the small kernel that clears them."""
-    groups = (H * (D // 8) + 31) // 32
-    slices = max(1, (4 * sm_count) // (groups * B))
-    rows_per = max(8, -(-rows // slices))
-    if -(-rows // rows_per) > 8 and copies >= 8 and rows <= 1024:
-        rows_per = -(-rows // 8)
-    return 1 + (1 if -(-rows // rows_per) > min(copies, 8) else 0)
-
-
-def gate_launches(w):
-    """Kernels of the gate's MLP: one, and the hidden layer's own when a single sequence's bins span >= 32 CTAs."""
-    batched = w.B >= 2 and w.wdtype == "bf16" and w.hidden == 64 and w.K >= 256
-    return 1 + (1 if not batched and (w.K + 255) // 256 >= 32 else 0)
-
-
 def measured_peak():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     try:
@@ -224,44 +207,28 @@ class MixerBench:
         import math
         fused_wrm = w.dtype in ("bf16", "f16") and w.n == 196 and w.D == 64 and w.wavelet_levels in (1, 2) and w.wavelet_hidden <= 256
         if w.dtype in ("bf16", "f16") and w.n == 8192:
-            self.kernel_name, nk = "mixer_tc8192_kernel (single-kernel tcgen05 mixer)", 1
+            self.kernel_name = "mixer_tc8192_kernel (single-kernel tcgen05 mixer)"
         elif w.dtype in ("bf16", "f16") and w.n == 196 and w.D == 64:
             # level gates of the fused refinement (own small kernel) + the persistent mixer kernel
-            self.kernel_name, nk = "mixer_tc196_kernel (single-kernel tcgen05 mixer, refinement in the store phase) + level_gates_kernel", (2 if fused_wrm else 1)
+            self.kernel_name = "mixer_tc196_kernel (single-kernel tcgen05 mixer" + (", refinement in the store phase) + level_gates_kernel" if fused_wrm else ")")
         elif w.dtype in ("bf16", "f16") and ws_mix and w.n >= 4096:
-            R, ntile = w.n // 4096, w.D // 8
-            per = R * ntile * (65536 + 65536) + R * 16384 + 256
-            groups = math.ceil(w.B * w.H / max(1, ws_mix // per))
-            tc32 = R == 32 and w.D == 64 and w.L % 4096 == 0
-            self.kernel_name, nk = ("mixer, staged tcgen05 path (" + ("tc_in32 incl. gate images + tc_core + tc_out32" if tc32 else
-                                    "tc_in incl. gate images + tc_core + tc_out") + " per group)"), 3 * groups
+            tc32 = w.n >= 8192 and w.D == 64
+            self.kernel_name = ("mixer, staged tcgen05 path (" + ("tc_in32 incl. gate images + tc_core + tc_out32" if tc32 else
+                                "tc_in incl. gate images + tc_core + tc_out") + " per group)")
         elif ws_mix:
-            per = w.n * (w.D // 2) * 8
-            groups = math.ceil(w.B * w.H / max(1, ws_mix // per))
-            self.kernel_name, nk = "mixer (strided + register-resident + strided per group)", 3 * groups
+            self.kernel_name = "mixer (strided + register-resident + strided per group)"
         else:
-            self.kernel_name, nk = "mixer (register-resident fp32 kernel)", 1
-        # pool (+ the kernel that clears its partial sums when it runs in several slices), gate_out (+ gate_hidden when a
-        # head's bins span >= 32 CTAs), mixer kernels, wavelet
-        self.launches_per_step = (pool_launches(w.B, w.L, w.H, w.D) + gate_launches(w) + nk +
-                                  (1 if w.wavelet_levels and not fused_wrm else 0))
+            self.kernel_name = "mixer (register-resident fp32 kernel)"
         self.h2d = w.B * w.L * w.H * w.D * (4 if w.dtype == "f32" else 2)
         self.d2h = self.h2d
         if project:
             es = 2
             self.kernel_name = "spectre_project_qv (proj_weights_kernel + project_qv_persistent_kernel, tcgen05 + TMA)"
             self.alg_bytes = 3 * w.B * w.L * w.H * w.D * es + 2 * w.H * w.D * w.D * es     # read X, write Q and V, read weights
-            # weights transpose + projection replace the pooling pass
-            self.launches_per_step += 2 - pool_launches(w.B, w.L, w.H, w.D)
         if backward:
             # timed call = spectre_mixer_backward: dV (read dY, write dV, read g) + gate gradient (read V and dY, write dg)
             self.kernel_name = "spectre_mixer_backward (dV through the forward kernels, dg through two fp32 transforms)"
             self.alg_bytes = 2 * mixer_algorithmic_bytes(w)
-            per = w.n * (w.D // 2) * 8
-            gb = math.ceil(w.B * w.H / max(1, min(w.B * w.H, (128 << 20) // per)))
-            # conjugate gate + forward kernels on dY; per group of heads two forward-only transforms and the reduction
-            # (a length one CTA transforms: one kernel for both gradients, and the sum of its partial gate gradients)
-            self.launches_per_step += 2 if w.n <= 2048 else 1 + nk + gb * 3
 
     def step(self, k: int, e0=None, e1=None):
         d = self.sets[k % self.nsets]
@@ -375,10 +342,6 @@ class AppendBench:
             tok = w.B * w.N_max * w.H * w.D * es
             self.alg_bytes = 4 * tok + w.B * w.H * K * w.D * 8            # read q, v; write both rings; write the spectrum
             self.kernel_name = "spectre_prefix_cache_prefill (per group of heads fp32 transforms of the decimated sequences, filling V_buf, + last radix step with the Hermitian split; one pass over q for sum_q and Q_buf)"
-            per = w.N_max * (w.D // 2) * 8
-            groups = -(-(w.B * w.H) // max(1, min(w.B * w.H, ws.numel() // per)))
-            # (transforms, combine + split) per group; the query pass (pooling + ring) and the kernel that clears its sums
-            self.launches_per_step = 2 * groups + pool_launches(w.B, w.N_max, w.H, w.D)
             self.h2d, self.d2h = 2 * tok, w.B * w.H * w.D * 4
             self.q_host = self.v_host = None
             return
@@ -396,9 +359,6 @@ class AppendBench:
                 self.arith_dtype = "f16 tensor-core operands, f32 accumulate (f32 spectrum in, " + w.dtype + " rows out)"
             self.kernel_name = ("spectre_prefix_cache_readout (gated operand images from the fp32 spectra, inverse half of the staged "
                                 "tcgen05 path)" if w.dtype != "f32" else "spectre_prefix_cache_readout (fp32 transform kernels)")
-            per = 2 * (N // 4096) * (w.D // 8) * 65536
-            groups = -(-(w.B * w.H) // max(1, min(w.B * w.H, self.ro_ws.numel() // max(per, 1))))
-            self.launches_per_step = 4 * groups                           # (gate maximum, spectrum-in, core, transpose-out) per group
             self.h2d, self.d2h = w.B * w.H * K * 8, w.B * N * w.H * w.D * es
             self.q_host = self.v_host = None
             return
@@ -410,7 +370,6 @@ class AppendBench:
         self.units_per_step = w.B                                         # tokens appended
         self.alg_bytes = append_algorithmic_bytes(w)
         self.kernel_name = "append_spectrum_kernel"
-        self.launches_per_step = 2
         es = 4 if w.dtype == "f32" else 2
         self.h2d = 2 * w.B * w.H * w.D * es
         self.d2h = w.B * w.H * w.D * 4
@@ -427,7 +386,6 @@ class AppendBench:
             wbytes = 2 if w.wdtype == "bf16" else 4
             self.alg_bytes += w.H * w.hidden * 2 * K * wbytes + 2 * w.B * w.H * K * 8   # + W2 stream, gate write + read
             self.kernel_name = "decode step (decode_spectrum_kernel dominant)"
-            self.launches_per_step = 2 + gate_launches(W.scaled(w, n_fft=N))      # ring, gate, decode_spectrum
             self.d2h = w.B * w.H * w.D * es
 
     def _call(self, k):
@@ -703,8 +661,10 @@ def measure(bench, K, Wm, local_rank, dev, e2e_steps):
     R.barrier()
     torch.cuda.synchronize()
     sampler.start()
+    from paper_2502_18394_b200 import binding as S
     windows, kern = [], []
     step0 = Wm
+    launched = S.lib().spectre_launch_count()
     while True:
         e0 = [torch.cuda.Event(enable_timing=True) if k % ev_stride == 0 else None for k in range(K)]
         e1 = [torch.cuda.Event(enable_timing=True) if k % ev_stride == 0 else None for k in range(K)]
@@ -723,6 +683,7 @@ def measure(bench, K, Wm, local_rank, dev, e2e_steps):
         total = sum(x[0] for x in windows)
         if len(windows) >= 15 or (len(windows) == 1 and tot_ms >= 50.0) or total >= 400.0:
             break
+    launched = S.lib().spectre_launch_count() - launched                       # the library's own count, all windows
     clocks = sampler.stop()
     order = sorted(range(len(windows)), key=lambda i: windows[i][0])
     mid = order[len(order) // 2]
@@ -745,9 +706,9 @@ def measure(bench, K, Wm, local_rank, dev, e2e_steps):
     torch.cuda.synchronize()
     R.barrier()
     e2e_ms, e2e_units = R.aggregate(ev_a.elapsed_time(ev_b), bench.units_per_step * Ke, dev)
-    info = {k: getattr(bench, k) for k in ("alg_bytes", "kernel_name", "launches_per_step", "h2d", "d2h", "nsets", "units_per_step")}
+    info = {k: getattr(bench, k) for k in ("alg_bytes", "kernel_name", "h2d", "d2h", "nsets", "units_per_step")}
     info["arith_dtype"] = getattr(bench, "arith_dtype", None)
-    return {"tot_ms": tot_ms, "tot_units": tot_units, "kern_ms": kern_ms, "clocks": clocks, "windows": len(windows),
+    return {"tot_ms": tot_ms, "tot_units": tot_units, "kern_ms": kern_ms, "clocks": clocks, "windows": len(windows), "launched": launched,
             "window_ms": [round(x[0], 4) for x in windows], "kern_events": len([e for e in e0 if e is not None]) * len(windows),
             "e2e_ms": e2e_ms, "e2e_units": e2e_units, "e2e_steps": Ke, "bench_info": info}
 
@@ -770,7 +731,7 @@ def result_block(w, info, m, K, Wm, world, cpu, label="", variant=False, variant
         "clocks": m["clocks"],
         "e2e": {"value": m["e2e_units"] / (m["e2e_ms"] * 1e-3), "unit": "tokens/s", "h2d_bytes_per_step": info["h2d"],
                 "d2h_bytes_per_step": info["d2h"], "steps": m["e2e_steps"]},
-        "gpu_launches": info["launches_per_step"] * K * m["windows"],
+        "gpu_launches": m["launched"],
         "roofline": {"bound": "hbm", "kernel": info["kernel_name"], "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "peak_source": peak_src, "algorithmic_bytes_per_launch": info["alg_bytes"],
                      "kernel_ms": m["kern_ms"], "kernel_timed_steps": m["kern_events"],

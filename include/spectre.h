@@ -78,6 +78,10 @@ const char* spectre_status_string(int status);
 /* Text of the most recent failure on the calling thread ("" if none). */
 const char* spectre_last_error(void);
 
+/* Diagnostic: kernels that the compute calls of this process have launched (under stream capture:
+ * recorded) since the library was loaded, on every device and stream. */
+uint64_t spectre_launch_count(void);
+
 /* A [B, L, H, D] activation; D contiguous; strides in elements. */
 typedef struct {
   void* ptr;

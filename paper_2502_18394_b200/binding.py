@@ -32,7 +32,7 @@ SPECTRE_F16 = 2
 
 EXPORTS = [
     "spectre_create", "spectre_destroy", "spectre_status_string", "spectre_last_error", "spectre_poll_status",
-    "spectre_selftest_wait_timeout",
+    "spectre_selftest_wait_timeout", "spectre_launch_count",
     "spectre_gate_workspace_bytes", "spectre_gate", "spectre_gate_static_max_bytes", "spectre_gate_static",
     "spectre_mixer_workspace_bytes", "spectre_mixer_forward",
     "spectre_wavelet_refine",
@@ -94,6 +94,7 @@ def lib():
     L.spectre_status_string.argtypes = [C.c_int]
     L.spectre_status_string.restype = C.c_char_p
     L.spectre_last_error.restype = C.c_char_p
+    L.spectre_launch_count.restype = C.c_uint64
     L.spectre_gate_workspace_bytes.argtypes = [C.c_void_p] + [C.c_int32] * 5
     L.spectre_gate_workspace_bytes.restype = C.c_size_t
     L.spectre_gate.argtypes = [C.c_void_p, C.c_void_p, C.POINTER(Act), C.c_void_p, C.c_int32, C.c_int32, C.c_int32,

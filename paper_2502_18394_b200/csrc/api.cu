@@ -1,4 +1,5 @@
 // Context, status strings and host-side argument checks of the C ABI.
+#include <atomic>
 #include <cstdio>
 #include <new>
 
@@ -15,6 +16,9 @@ int build_tw_staged(float2* tab, cudaStream_t st);   // mixer_tc4k.cu
 int build_dft32(void* mats, cudaStream_t st);        // mixer_tc32.cu
 
 static thread_local std::string g_last_error;
+static std::atomic<uint64_t> g_launches{0};
+
+void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
 int fail(int status, const std::string& msg) {
   g_last_error = msg;
@@ -197,5 +201,7 @@ extern "C" const char* spectre_status_string(int status) {
     default: return "unknown status";
   }
 }
+
+extern "C" uint64_t spectre_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
 extern "C" const char* spectre_last_error(void) { return g_last_error.c_str(); }

@@ -580,7 +580,7 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   cfg.numAttrs = 1;
   SPECTRE_IO_DISPATCH(cache->buf_dtype, {
     auto kern = NR == 1 ? decode_spectrum_kernel<T, 1> : (NR == 2 ? decode_spectrum_kernel<T, 2> : decode_spectrum_kernel<T, SPECTRE_DECODE_MAX_ROWS>);
-    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, cache->prefix_fft, static_cast<const float*>(delta), g2, partial, done,
+    SPECTRE_CUDA_OK(launch_kernel(&cfg, kern, cache->prefix_fft, static_cast<const float*>(delta), g2, partial, done,
                                        reinterpret_cast<T*>(y_rows), H, D, N, K, (unsigned)slot, dr, (int)nrows, nblk));
   });
   return SPECTRE_OK;

@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 
 #include "spectre.h"
 
@@ -52,6 +53,14 @@ bool is_pow2(int64_t x);
 int radix_plan(int n, int* radices);
 
 #ifdef __CUDACC__
+// Every launch of the entry points goes through here and is counted (spectre_launch_count).
+void count_launch();
+template <class... P, class... A>
+cudaError_t launch_kernel(const cudaLaunchConfig_t* cfg, void (*kern)(P...), A&&... args) {
+  const cudaError_t e = cudaLaunchKernelEx(cfg, kern, std::forward<A>(args)...);
+  if (e == cudaSuccess) count_launch();
+  return e;
+}
 // What other kernels write - the caller's tensors and weights, workspaces, cache state - is read by plain loads through pointers
 // without __restrict__.  A kernel of a chain is resident while the one before it still writes, so a const __restrict__ pointer or
 // __ldg, which say that nothing changes while this kernel runs, would let a load go through the read-only path, and any
@@ -72,7 +81,7 @@ cudaError_t launch_after(void (*kern)(P...), dim3 grid, int block, size_t smem, 
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+  return launch_kernel(&cfg, kern, P(args)...);
 }
 #endif
 

@@ -200,11 +200,11 @@ static int pool_launch(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
   const unsigned wper = (unsigned)(wb ? ((wb + ctas - 1) / ctas + 15) & ~(size_t)15 : 0);
   SPECTRE_IO_DISPATCH(q->dtype, {
     if (ring)
-      SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, pool_kernel<T, true>, reinterpret_cast<const T*>(q->ptr), (int64_t)q->stride_b,
+      SPECTRE_CUDA_OK(launch_kernel(&cfg, pool_kernel<T, true>, reinterpret_cast<const T*>(q->ptr), (int64_t)q->stride_b,
                                          (int64_t)q->stride_l, (int64_t)q->stride_h, (int)q->L, (int)q->H, (int)q->D, rows_per,
                                          ncopy, copy_stride, sums, reinterpret_cast<T*>(ring), N, w0, wper, wb));
     else
-      SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, pool_kernel<T, false>, reinterpret_cast<const T*>(q->ptr), (int64_t)q->stride_b,
+      SPECTRE_CUDA_OK(launch_kernel(&cfg, pool_kernel<T, false>, reinterpret_cast<const T*>(q->ptr), (int64_t)q->stride_b,
                                          (int64_t)q->stride_l, (int64_t)q->stride_h, (int)q->L, (int)q->H, (int)q->D, rows_per,
                                          ncopy, copy_stride, sums, static_cast<T*>(nullptr), 0, w0, wper, wb));
   });
@@ -1162,25 +1162,25 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
 #define SPECTRE_GATE_LAUNCH(WT, NB)                                                              \
   do {                                                                                           \
     if (pre) {                                                                                   \
-      SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_hid, gate_hidden_kernel<WT, NB>, mp));             \
+      SPECTRE_CUDA_OK(launch_kernel(&cfg_hid, gate_hidden_kernel<WT, NB>, mp));             \
       mp.early = 1;                                                                              \
-      SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_out, gate_out_kernel<WT, NB, true>, mp));          \
+      SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, true>, mp));          \
     } else {                                                                                     \
-      SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_out, gate_out_kernel<WT, NB, false>, mp));         \
+      SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, false>, mp));         \
     }                                                                                            \
   } while (0)
 #define SPECTRE_GATE_MMA(NB)                                                                     \
   do {                                                                                           \
-    if (mp.shift && !mp.post) SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_mma, gate_mma_kernel<NB, true>, mp)); \
-    else SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg_mma, gate_mma_kernel<NB, false>, mp));          \
+    if (mp.shift && !mp.post) SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, true>, mp)); \
+    else SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, false>, mp));          \
   } while (0)
   if (mma) {
     if (BB == 8) SPECTRE_GATE_MMA(8); else SPECTRE_GATE_MMA(4);
   } else if (all_staged) {
-    if (wb) SPECTRE_CUDA_OK(BB == 8 ? cudaLaunchKernelEx(&cfg_short, gate_short_kernel<bf16, 8>, mp) : cudaLaunchKernelEx(&cfg_short, gate_short_kernel<bf16, 4>, mp));
-    else SPECTRE_CUDA_OK(BB == 8 ? cudaLaunchKernelEx(&cfg_short, gate_short_kernel<float, 8>, mp) : cudaLaunchKernelEx(&cfg_short, gate_short_kernel<float, 4>, mp));
+    if (wb) SPECTRE_CUDA_OK(BB == 8 ? launch_kernel(&cfg_short, gate_short_kernel<bf16, 8>, mp) : launch_kernel(&cfg_short, gate_short_kernel<bf16, 4>, mp));
+    else SPECTRE_CUDA_OK(BB == 8 ? launch_kernel(&cfg_short, gate_short_kernel<float, 8>, mp) : launch_kernel(&cfg_short, gate_short_kernel<float, 4>, mp));
   } else if (split) {
-    SPECTRE_CUDA_OK(wb ? cudaLaunchKernelEx(&cfg_split, gate_split_kernel<bf16>, mp) : cudaLaunchKernelEx(&cfg_split, gate_split_kernel<float>, mp));
+    SPECTRE_CUDA_OK(wb ? launch_kernel(&cfg_split, gate_split_kernel<bf16>, mp) : launch_kernel(&cfg_split, gate_split_kernel<float>, mp));
   } else switch (BB) {
     case 8: if (wb) SPECTRE_GATE_LAUNCH(bf16, 8); else SPECTRE_GATE_LAUNCH(float, 8); break;
     case 4: if (wb) SPECTRE_GATE_LAUNCH(bf16, 4); else SPECTRE_GATE_LAUNCH(float, 4); break;

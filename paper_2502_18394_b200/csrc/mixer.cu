@@ -594,7 +594,7 @@ static int launch_onchip_cf(const OnchipParams& p, const TransformPlan& pl, int 
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = (C > 1) ? 1 : 0;
-  SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, p));
+  SPECTRE_CUDA_OK(launch_kernel(&cfg, kern, p));
   return SPECTRE_OK;
 }
 

@@ -697,8 +697,8 @@ int launch_mixer_tc196(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
       cudaLaunchConfig_t lcfg = {};
       lcfg.gridDim = lgrid; lcfg.blockDim = dim3(256); lcfg.dynamicSmemBytes = lsmem; lcfg.stream = st;
       lcfg.attrs = attr; lcfg.numAttrs = 1;
-      if (wrm->wdtype == SPECTRE_BF16) SPECTRE_CUDA_OK(cudaLaunchKernelEx(&lcfg, level_gates_kernel<bf16>, lp));
-      else SPECTRE_CUDA_OK(cudaLaunchKernelEx(&lcfg, level_gates_kernel<float>, lp));
+      if (wrm->wdtype == SPECTRE_BF16) SPECTRE_CUDA_OK(launch_kernel(&lcfg, level_gates_kernel<bf16>, lp));
+      else SPECTRE_CUDA_OK(launch_kernel(&lcfg, level_gates_kernel<float>, lp));
       SPECTRE_LAUNCH_OK("level_gates_kernel");
       p.level_gates = level_gate_scratch;
       dependent = true;
@@ -716,7 +716,7 @@ int launch_mixer_tc196(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
   do {                                                                                                            \
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(mixer_tc196_kernel<k196Heads, JJ, FH>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                          k196_smem(k196Heads)));                                                  \
-    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, mixer_tc196_kernel<k196Heads, JJ, FH>, p));                          \
+    SPECTRE_CUDA_OK(launch_kernel(&cfg, mixer_tc196_kernel<k196Heads, JJ, FH>, p));                          \
   } while (0)
   const bool f16 = v->dtype == SPECTRE_F16;
   if (p.J == 2) { if (f16) SPECTRE_TC196_LAUNCH(2, true); else SPECTRE_TC196_LAUNCH(2, false); }

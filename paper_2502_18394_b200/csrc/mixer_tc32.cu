@@ -618,10 +618,10 @@ static int launch_tc_in_r(const spectre_ctx* ctx, cudaStream_t st, const spectre
   cfg.attrs = attr; cfg.numAttrs = 1;
   if (v->dtype == SPECTRE_F16) {
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_in32_kernel<true, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXInSmem));
-    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, tc_in32_kernel<true, R>, tm, tm_rest, tm1, tm_rest1, tm_img, p));
+    SPECTRE_CUDA_OK(launch_kernel(&cfg, tc_in32_kernel<true, R>, tm, tm_rest, tm1, tm_rest1, tm_img, p));
   } else {
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_in32_kernel<false, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXInSmem));
-    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, tc_in32_kernel<false, R>, tm, tm_rest, tm1, tm_rest1, tm_img, p));
+    SPECTRE_CUDA_OK(launch_kernel(&cfg, tc_in32_kernel<false, R>, tm, tm_rest, tm1, tm_rest1, tm_img, p));
   }
   SPECTRE_LAUNCH_OK("tc_in32_kernel");
   return SPECTRE_OK;

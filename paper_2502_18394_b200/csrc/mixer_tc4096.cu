@@ -308,7 +308,7 @@ int launch_mixer_tc4096(const spectre_ctx* ctx, cudaStream_t st, const spectre_a
   cfg.numAttrs = 1;
   auto kern = v->dtype == SPECTRE_F16 ? mixer_tc4096_kernel<true> : mixer_tc4096_kernel<false>;
   SPECTRE_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, k40Smem));
-  SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, tm_in, tm_out, p));
+  SPECTRE_CUDA_OK(launch_kernel(&cfg, kern, tm_in, tm_out, p));
   return SPECTRE_OK;
 }
 

@@ -690,7 +690,7 @@ static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, tc_in_kernel<R, F16>, ip, gp, cnt * R));
+  SPECTRE_CUDA_OK(launch_kernel(&cfg, tc_in_kernel<R, F16>, ip, gp, cnt * R));
   SPECTRE_LAUNCH_OK("tc_in_kernel");
   }
 

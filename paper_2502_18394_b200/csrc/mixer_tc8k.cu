@@ -380,10 +380,10 @@ int launch_mixer_tc8192(const spectre_ctx* ctx, cudaStream_t st, const spectre_a
   cfg.numAttrs = 1;
   if (v->dtype == SPECTRE_F16) {
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(mixer_tc8192_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, k8Smem));
-    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, mixer_tc8192_kernel<true>, tm_in, tm_out, p));
+    SPECTRE_CUDA_OK(launch_kernel(&cfg, mixer_tc8192_kernel<true>, tm_in, tm_out, p));
   } else {
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(mixer_tc8192_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, k8Smem));
-    SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, mixer_tc8192_kernel<false>, tm_in, tm_out, p));
+    SPECTRE_CUDA_OK(launch_kernel(&cfg, mixer_tc8192_kernel<false>, tm_in, tm_out, p));
   }
   SPECTRE_LAUNCH_OK("mixer_tc8192_kernel");
   return SPECTRE_OK;

@@ -622,7 +622,7 @@ static int reg_launch(RegParams p, int nslab, cudaStream_t st) {
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, p));
+  SPECTRE_CUDA_OK(launch_kernel(&cfg, kern, p));
   return SPECTRE_OK;
 }
 
@@ -655,7 +655,7 @@ static int reg_launch_stream(RegParams p, int nslab, cudaStream_t st, int sm_cou
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  SPECTRE_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, map, p, (int)total));
+  SPECTRE_CUDA_OK(launch_kernel(&cfg, kern, map, p, (int)total));
   *done = true;
   return SPECTRE_OK;
 }

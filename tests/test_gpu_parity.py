@@ -994,6 +994,18 @@ def test_fp16_io_gate_wavelet_cache_decode_backward(ctx):
     assert max(rel_err(gate_to_complex(dg)[b, h], rg[b, h]) for b in range(B) for h in range(H)) < TOL["f32"]
 
 
+def test_launch_count_follows_the_calls(ctx):
+    w = W.Workload("t", B=1, L=64, H=2, D=16, dtype="f32", seed=1)
+    x, g = W.activations(w).cuda(), W.random_gate(w).cuda()
+    c0 = S.lib().spectre_launch_count()
+    S.spectre_mixer_forward(ctx, x, g)                       # one kernel
+    c1 = S.lib().spectre_launch_count()
+    S.spectre_wavelet_refine(ctx, x, {"levels": 2, "level_gates": torch.zeros(1, 2, 3, 16, device="cuda")})
+    cache = S.PrefixCache(1, 2, 16, 64, dtype=torch.float32)
+    S.spectre_prefix_cache_append(ctx, cache, x[:, 0].contiguous(), x[:, 1].contiguous(), 0)   # spectrum and ring
+    assert c1 - c0 == 1 and S.lib().spectre_launch_count() - c1 == 3
+
+
 # ------------------------------------------------------------------ streams
 def test_what_a_call_on_a_given_stream_allocates_belongs_to_that_stream(ctx):
     # torch's allocator reuses a freed block in the order of the stream it was allocated on: a workspace of another stream's would
