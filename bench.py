@@ -53,7 +53,7 @@ NCU_TRAFFIC = {"c1": None,
 
 # The same for the variant legs of c4 that have a capture (per call; both taken at B = 2 and scaled by 4, the
 # traffic being proportional to the batch).
-NCU_TRAFFIC_VARIANT = {("c4", "prefill"): (10208e6, "profiles/launches_c4_prefill.md (ncu capture at B = 2, x4; not this run)"),
+NCU_TRAFFIC_VARIANT = {("c4", "prefill"): (10131e6, "profiles/launches_c4_prefill.md (ncu capture at B = 2, x4; not this run)"),
                        ("c4", "readout"): (7015e6, "profiles/launches_c4_readout.md (ncu capture at B = 2, x4; not this run)")}
 
 

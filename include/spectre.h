@@ -130,6 +130,7 @@ typedef struct {
  *              to one copy (4*B*H*D bytes of sums, 4*B*H*hidden of hidden activations, plus
  *              8*B*H*K with the Toeplitz update on, each rounded up to 256) is accepted;
  *              with sum_q given the sums part is still counted but unused
+ * W2 and g_out start on 8 bytes, every other array of floats on 4.
  */
 size_t spectre_gate_workspace_bytes(const spectre_ctx* ctx, int32_t B, int32_t H, int32_t D,
                                     int32_t n_fft, int32_t toeplitz_r);
@@ -312,8 +313,9 @@ int spectre_prefix_cache_append(spectre_ctx* ctx, void* stream, const spectre_ca
  *   y_rows    [B, nrows, H, D] contiguous, dtype buf_dtype (device), written
  *   g_out     [B, H, K, 2] float32 (device), written: the gate of this step
  *   workspace >= spectre_decode_workspace_bytes(...) bytes, 16-byte aligned
- * Errors: as spectre_prefix_cache_append and spectre_gate; a row outside the
- * window or nrows out of range is SPECTRE_ERR_INVALID_ARG before any launch.
+ * Errors: as spectre_prefix_cache_append and spectre_gate, a row outside the window or
+ * nrows out of range is SPECTRE_ERR_INVALID_ARG; all before any launch: a refused step
+ * leaves the cache as it was.
  */
 size_t spectre_decode_workspace_bytes(const spectre_ctx* ctx, int32_t B, int32_t H, int32_t D,
                                       int32_t N_max, int32_t nrows, int32_t toeplitz_r);
@@ -356,8 +358,10 @@ int spectre_prefix_cache_readout(spectre_ctx* ctx, void* stream, const spectre_c
  *   dg_k = dL/dRe g_k + j dL/dIm g_k = (w_k / n) sum_c conj(Vhat_{k,c}) Ghat_{k,c}
  * v, dy, dv: activations of identical shape and dtype; dv may alias dy where
  * spectre_mixer_forward allows y to alias v.  dv or dg may be NULL to skip that
- * gradient (not both).  dg: [B, H, K, 2] float32.  dv runs on the same kernels as
- * the forward pass; dg uses two forward-only fp32 transforms and a reduction.
+ * gradient (not both).  dg: [B, H, K, 2] float32.  Lengths that one CTA transforms in registers
+ * (powers of two 64 ... 2048, squares of even sides): one fp32 kernel for both.  Others: dv runs on
+ * the same kernels as the forward pass; dg, computed first, uses two forward-only fp32 transforms
+ * and a reduction.
  * workspace >= spectre_mixer_backward_workspace_bytes(...), 16-byte aligned; any size
  * down to the conjugate gate + the forward workspace + two (batch, head) slabs of
  * spectrum (n_fft * D/2 * 8 bytes each) is accepted.

@@ -7,9 +7,10 @@
 // operand and is converted (four rows x four pairs transposed) in place, and the last epilogue stages whole 16-byte pieces
 // of 8 t1 x 32 t2 rows per warp, which that warp alone hands to the TMA engine.
 //
-// Why: the staged path spends three kernels and two fp16 intermediates on it (transpose-in 32 us, core 31 us, transpose-out
-// 45 us at B = 4, H = 16, D = 64; this kernel: 42 us).  Bound now by the 16-byte row requests (4096 in and out per CTA, about 1.2 cycles each on
-// the SM's request path) and the epilogues, one CTA's requests running under the other's arithmetic.
+// Why: the staged path spends three kernels and two fp16 intermediates on it (100 us at B = 4, H = 16, D = 64, rotating buffers;
+// this kernel: 46 us, 48 with cold caches).  What bounds it is the latency of the epilogues: the 16-byte row requests (4096 in and 4096 out per CTA,
+// about 1.2 cycles each on the SM's request path, 3.5 CTAs per SM) are 17 us of it, the rest is TMEM and twiddle loads in front
+// of their use with only the other CTA of the SM to hide them, and 512 CTAs are 1.73 waves of the 296 that are resident.
 //
 // Rows beyond L are zero: the map ends at the last whole block of 64, TMA fills and clips the rest, and the L % 64 rows of
 // a partial block are read by the conversion and written by the last epilogue with plain 16-byte accesses.
