@@ -250,6 +250,8 @@ int wavelet_check(const spectre_ctx* ctx, int L, int D, const spectre_wavelet* w
   }
   if (J > 4 && wavelet_smem(L, D, w) > (size_t)ctx->max_smem_optin)
     return fail(SPECTRE_ERR_UNSUPPORTED, "2^J * D exceeds the shared-memory tile");
+  if (J <= 4 && ((size_t)(J + 1) * D + (w->level_gates ? 0 : w->hidden)) * sizeof(float) > 48 * 1024)      // the launch would fail
+    return fail(SPECTRE_ERR_UNSUPPORTED, "(J + 1) * D exceeds the shared memory of the level gates");
   return SPECTRE_OK;
 }
 

@@ -1070,15 +1070,18 @@ def test_invalid_arguments_are_rejected_before_launch(ctx):
     assert float(S.spectre_mixer_forward(ctx, x, g).abs().max()) == 0.0
 
 
-@pytest.mark.parametrize("dt,n,J", [("f32", 64, 2), ("bf16", 196, 2), ("f32", 4096, 10)])
+@pytest.mark.parametrize("dt,n,J", [("f32", 64, 2), ("bf16", 196, 2), ("f32", 4096, 10), ("f32", 16, 4)])
 def test_a_refused_refinement_leaves_the_tensor_as_it_was(ctx, dt, n, J):
     # mixer in place with a refinement that the wavelet entry point would refuse: nothing is written
-    w = W.Workload("t", B=1, L=n, H=2, D=64, dtype=dt, seed=2)
+    D = 2560 if J == 4 else 64
+    w = W.Workload("t", B=1, L=n, H=2, D=D, dtype=dt, seed=2)
     x, g = W.activations(w).cuda(), W.random_gate(w).cuda()
     before = x.clone()
     wrms = [{"levels": J, "hidden": 64}]                                      # neither level gates nor the MLP
     if J == 10:                                                               # 1024 x 64 floats exceed the shared-memory tile
         wrms.append({"levels": J, "level_gates": torch.zeros(1, 2, J + 1, 64, device="cuda")})
+    if J == 4:                                                                # 5 x 2560 level gates exceed a launch's 48 KB
+        wrms.append({"levels": J, "level_gates": torch.zeros(1, 2, J + 1, D, device="cuda")})
     for wrm in wrms:
         with pytest.raises(S.SpectreError):
             S.spectre_mixer_forward(ctx, x, g, y=x, wrm=wrm)
