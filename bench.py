@@ -37,7 +37,7 @@ L2_BYTES = 126e6
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from the ncu
 # captures summarised under profiles/ (None until a capture exists for that workload).
-# c2: mixer_tc8192_kernel 35.0 MB read + 1.2 MB written inside the launch (its 33.6 MB output was still
+# c2: the mixer kernel before the present one: 35.0 MB read + 1.2 MB written inside the launch (its 33.6 MB output was still
 #     dirty in L2 when the launch ended, so this understates the traffic; nothing is re-read)
 # c3: the three kernels of one staged mixer call at full size (intermediates spill from L2)
 # c4: append_spectrum_kernel measured at B = 2 (1015.3 MB), scaled by 4 to B = 8
@@ -207,7 +207,7 @@ class MixerBench:
         import math
         fused_wrm = w.dtype in ("bf16", "f16") and w.n == 196 and w.D == 64 and w.wavelet_levels in (1, 2) and w.wavelet_hidden <= 256
         if w.dtype in ("bf16", "f16") and w.n == 8192:
-            self.kernel_name = "mixer_tc8192_kernel (single-kernel tcgen05 mixer)"
+            self.kernel_name = "mixer_tc64_kernel (single-kernel tcgen05 mixer)"
         elif w.dtype in ("bf16", "f16") and w.n == 196 and w.D == 64:
             # level gates of the fused refinement (own small kernel) + the persistent mixer kernel
             self.kernel_name = "mixer_tc196_kernel (single-kernel tcgen05 mixer" + (", refinement in the store phase) + level_gates_kernel" if fused_wrm else ")")

@@ -15,7 +15,7 @@ NATIVE = os.path.join(PKG, "_native.so")
 NATIVE_SRC = os.path.join(CSRC, "native.cpp")
 OBJ = os.path.join(PKG, "build")
 NATIVE_ABI = os.path.join(OBJ, "native_abi")
-SOURCES = ["reg_grad.cu", "reg_mix.cu", "reg_inverse.cu", "reg_forward.cu", "api.cu", "mixer.cu", "mixer_tc.cu", "mixer_tc8k.cu",
+SOURCES = ["reg_grad.cu", "reg_mix.cu", "reg_inverse.cu", "reg_forward.cu", "api.cu", "mixer.cu", "mixer_tc.cu", "mixer_tc64.cu",
            "mixer_tc4k.cu", "gate.cu", "cache.cu", "wavelet.cu", "backward.cu", "project.cu"]
 FLAGS = ["-std=c++17", "-O3", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
          "-Xcompiler", "-fPIC", "-shared"]

@@ -36,9 +36,9 @@ namespace spectre {
 int wavelet_check(const spectre_ctx* ctx, int L, int D, const spectre_wavelet* w);   // wavelet.cu
 
 int launch_mixer_tc8192(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g,
-                        const spectre_act* y);   // mixer_tc.cu
-bool tc8192_supported(const spectre_act* v, const spectre_act* y);                     // mixer_tc8k.cu
-bool tc4096_supported(const spectre_act* v, const spectre_act* y);                     // mixer_tc4096.cu
+                        const spectre_act* y);   // mixer_tc64.cu
+bool tc8192_supported(const spectre_act* v, const spectre_act* y);                     // mixer_tc64.cu
+bool tc4096_supported(const spectre_act* v, const spectre_act* y);                     // mixer_tc64.cu
 int launch_mixer_tc4096(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, const spectre_act* y);
 int launch_mixer_tc196(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g,
                        const spectre_act* y, const spectre_wavelet* wrm, float* level_gate_scratch);

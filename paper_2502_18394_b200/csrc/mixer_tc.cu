@@ -1,5 +1,5 @@
 // Tensor-core kernels shared by the blocked-DFT mixers: the DFT-matrix and twiddle-table builders
-// (owned by the context) and the n = 196 mixer.  The n = 8192 mixer lives in mixer_tc8k.cu, the
+// (owned by the context) and the n = 196 mixer.  The n = 4096 and 8192 mixers live in mixer_tc64.cu, the
 // multi-kernel path for longer transforms in mixer_tc4k.cu.
 #include "tc_common.cuh"
 

@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(256, 3) tc_in_kernel(const TcInParams p, const
   // copy out: per (k1, tile) unit and pair c4 the CTA holds NT2 consecutive t2 x 4 t1 = NT2 16-byte
   // chunks, contiguous in the unit's image (column 64 c4 + t2, K group t1g).  The skew permutes the
   // words inside a chunk (low two bits) and the chunks among their neighbours (next three bits).
-  unsigned char* img0 = p.ws_in + (size_t)slab_local * R * p.ntile * k4ImgBytes + (size_t)t1g * k8Lbo0 +
+  unsigned char* img0 = p.ws_in + (size_t)slab_local * R * p.ntile * k4ImgBytes + (size_t)t1g * k4Lbo +
                         (size_t)(t2b * NT2) * 16;
   const bool pow2 = (p.ntile & (p.ntile - 1)) == 0;
   const int nchunk = R * p.ntile * 4 * NT2;

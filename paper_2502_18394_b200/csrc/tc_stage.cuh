@@ -1,23 +1,10 @@
-// The 64 x 64 stages of a 4096-point transform on the tensor cores, shared by the n = 8192 kernel
-// (two such problems per tile) and the core kernel of the longer transforms (one per unit): operand
-// strides per stage and the epilogues between the stages.  Conventions as in mixer_tc8k.cu: the
-// accumulator of a stage has the new digit along its rows and, along its columns, the column pair c
-// and the digit that is contracted next.
+// Epilogues between the 64 x 64 stages of a 4096-point transform on the tensor cores, for the core kernel of the longer
+// transforms (mixer_tc4k.cu): the accumulator of a stage has the new digit along its rows and, along its columns, the column
+// pair c and the digit that is contracted next.
 #pragma once
 #include "tc_common.cuh"
 
 namespace spectre {
-
-// Operand strides (bytes) per stage: LBO between core matrices along K, SBO between 8-column
-// groups.  Stage 0 is the TMA landing image (dense).  The others are chosen so that the stores
-// of the epilogue that writes them spread over all 32 banks.
-constexpr int k8Lbo0 = 4096, k8Sbo0 = 128;       // columns 64 c + t2, K = t1
-constexpr int k8Lbo1 = 4160, k8Sbo1 = 128;       // columns 64 c + k1, K = t2
-constexpr int k8Lbo2 = 4112, k8Sbo2 = 128;       // columns 64 c + k1, K = k2
-constexpr int k8Lbo3 = 144, k8Sbo3 = 2336;       // columns 4 s1 + c,  K = k1
-constexpr int k8BBytes = 32 * k8Sbo3;            // largest of the four images (74752)
-constexpr int k8GStride = 72;                    // gate table: entry (k1, k2) at 72 k2 + k1
-constexpr int k8GBytes = 64 * k8GStride * 4;     // per half, fp16 (re, im)
 
 // Epilogue after a stage whose accumulator has columns 64 c + d (d = the digit still to be
 // contracted), for one warp: TMEM lane quadrant q, pair c.  A thread owns rows (new digit)
@@ -32,41 +19,7 @@ constexpr int k8GBytes = 64 * k8GStride * 4;     // per half, fp16 (re, im)
 //   2 (row % 4) + c % 2, which keeps the four rows a half-warp writes at once in four different
 //   16-byte slots of a core matrix even when LBO and SBO are multiples of 128 (dense images), and
 //   leaves all four pairs of a row in one thread of the epilogue that reads the next accumulator.
-template <int LBO, int SBO, int COLS>
-__device__ __forceinline__ void epilogue_twiddle(uint32_t tmem_d, unsigned char* Bout, int q, int c, int T,
-                                                 const float2* __restrict__ tw, float2 wr0, float2 wr1) {
-  const int i = T >> 2, tq = T & 3;
-  uint32_t r[2][16];
-  const uint32_t taddr0 = tmem_d + ((uint32_t)(32 * q) << 16) + 64 * c;
-  tmem_ld_16x256b_x4(taddr0, r[0]);
-  tw += q * 512 + T;
-#pragma unroll
-  for (int step = 0; step < 4; ++step) {                      // step = 2 j + chunk
-    const int j = step >> 1, chunk = step & 1;
-    const int row = 8 * (2 * q + j) + i;
-    float2 w[4];
-#pragma unroll
-    for (int x = 0; x < 4; ++x) w[x] = __ldg(tw + (4 * step + x) * 32);
-    tmem_ld_wait();
-    if (step < 3) {
-      const int nj = (step + 1) >> 1, nchunk = (step + 1) & 1;
-      tmem_ld_16x256b_x4(taddr0 + ((uint32_t)(16 * nj) << 16) + 32 * nchunk, r[(step + 1) & 1]);
-    }
-    const uint32_t (&rr)[16] = r[step & 1];
-    const uint32_t colpart = COLS == 1 ? (uint32_t)((8 * c + (row >> 3)) * SBO + (row & 7) * 16)
-                           : COLS == 0 ? (uint32_t)((row >> 1) * SBO + (4 * (row & 1) + c) * 16)
-                                       : (uint32_t)((2 * (row >> 2) + (c >> 1)) * SBO + (2 * (row & 3) + (c & 1)) * 16);
-    const uint32_t base = colpart + (uint32_t)((8 * chunk + (tq >> 1)) * LBO + 8 * (tq & 1));
-#pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      const float2 w1 = cmul(w[x], j ? wr1 : wr0);
-      *reinterpret_cast<uint2*>(Bout + base + 2 * x * LBO) =
-          cmul2_pack_h2(pk2u(rr[4 * x], rr[4 * x + 1]), pk2u(rr[4 * x + 2], rr[4 * x + 3]), pk2(w[x].x, w1.x), pk2(w[x].y, w1.y));
-    }
-  }
-}
-
-// The same for the two pairs c0 and c0 + 1 of one warp: the twiddles depend on (row, d) only, so each
+// Both pairs c0 and c0 + 1 of one warp: the twiddles depend on (row, d) only, so each
 // table entry is fetched once and used for both pairs.  The eight (step, pair) accumulator chunks are
 // walked in the order (step, pair) with the TMEM loads one chunk ahead.
 template <int LBO, int SBO, int COLS>
@@ -139,10 +92,6 @@ __device__ __forceinline__ void epilogue_gate_t(uint32_t tmem_d, unsigned char* 
       *reinterpret_cast<uint32_t*>(Bout + base + x * SBO + 16) = pack_h2(v1.x, -v1.y);
     }
   }
-}
-__device__ __forceinline__ void epilogue_gate(uint32_t tmem_d, unsigned char* Bout, int q, int c, int T,
-                                              const uint32_t* __restrict__ Gtab) {
-  epilogue_gate_t<k8Lbo2, k8Sbo2, k8GStride, false>(tmem_d, Bout, q, c, T, Gtab);
 }
 
 }  // namespace spectre

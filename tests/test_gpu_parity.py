@@ -187,6 +187,26 @@ def test_mixer_staged_ragged_rows(ctx, dt, n, L):
     assert bool((wide[:, L:] == 7.0).all())
 
 
+@pytest.mark.parametrize("dt,n,B,L,H,D", [("bf16", 4096, 1, 4096, 1, 8), ("f16", 4096, 5, 4096, 31, 64), ("bf16", 4096, 7, 2047, 43, 24),
+                                          ("f16", 8192, 1, 8192, 1, 8), ("bf16", 8192, 3, 8192, 33, 64), ("f16", 8192, 5, 4160, 37, 40)])
+def test_mixer_single_kernel_tiles_per_cta(ctx, dt, n, B, L, H, D):
+    # one tile, and persistent CTAs with several: the next tile's rows land where the last one's results left, gates change
+    # from tile to tile.  All slabs against an fp64 transform; the fp16 operand images keep 1e-3 of a slab's norm
+    x = W.activations(W.Workload("t", B=B, L=L, H=H, D=D, dtype=dt, seed=n + B)).cuda()
+    g = torch.randn(B, H, n // 2 + 1, 2, generator=torch.Generator().manual_seed(n + H)).cuda()
+    g *= torch.exp(torch.arange(B * H, device="cuda").view(B, H, 1, 1) % 7 - 3.0)          # scales differ between neighbours
+    y = S.spectre_mixer_forward(ctx, x, g, n_fft=n)
+    torch.cuda.synchronize()
+    ctx.poll_status()
+    for b in range(B):
+        G = torch.view_as_complex(g[b].double())
+        G[:, 0].imag = 0
+        G[:, -1].imag = 0
+        ref = torch.fft.irfft(torch.fft.rfft(x[b].double(), n=n, dim=0) * G.t()[:, :, None], n=n, dim=0)[:L]
+        err = (y[b].double() - ref).norm(dim=(0, 2)) / ref.norm(dim=(0, 2))
+        assert float(err.max()) < (3e-3 if dt == "bf16" else 2e-3)      # + the output's rounding: 2^-9 / sqrt(3) and 2^-12 / sqrt(3)
+
+
 @pytest.mark.parametrize("L", [64, 4160, 8128])
 def test_mixer_bf16_8192_short_sequences_through_the_tensor_maps(ctx, L):
     # whole 64-row blocks shorter than n: rows beyond L read as zero and are not written;
