@@ -410,34 +410,36 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
         for (int e = 0; e < 4; ++e)
           *reinterpret_cast<uint4*>(p0 + 256 * e) = make_uint4(to_h2(at(r[0], e)), to_h2(at(r[1], e)), to_h2(at(r[2], e)), to_h2(at(r[3], e)));
       } else {
-        // radix-2 step: lanes with bit 3 clear form the even bins' inputs, the others the odd bins'
-        const int odd = (T >> 3) & 1;
+        // radix-2 step: a lane takes two of the four pairs, the even bins' inputs into the lower half, the odd ones' into the upper
+        const int hp = (T >> 3) & 1;
         unsigned char* p0 = ring + a * 512 + t2l * 16;
-        uint4 lo[4], hi[4];
+        uint2 lo[4], hi[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          lo[u] = *reinterpret_cast<const uint4*>(p0 + 128 * u);
-          hi[u] = *reinterpret_cast<const uint4*>(p0 + 8192 + 128 * u);
+          lo[u] = *reinterpret_cast<const uint2*>(p0 + 128 * u + 8 * hp);
+          hi[u] = *reinterpret_cast<const uint2*>(p0 + 8192 + 128 * u + 8 * hp);
         }
         const float2 w0 = cmul(wconv, W8[c]);
         const float2 w64[4] = {make_float2(1.f, 0.f), make_float2(0.998795456f, -0.049067674f),
                                make_float2(0.995184727f, -0.098017140f), make_float2(0.989176510f, -0.146730474f)};
-        const float sg = odd ? -1.f : 1.f;
         float2 w[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) w[u] = odd ? cmul(w0, w64[u]) : make_float2(1.f, 0.f);
+        for (int u = 0; u < 4; ++u) w[u] = cmul(w0, w64[u]);
         __syncwarp();                                            // every lane has read: the slots may be written
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          uint32_t o[4];
+        for (int e = 0; e < 2; ++e) {
+          uint32_t ev[4], od[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const uint32_t ua = at(lo[u], e), ub = at(hi[u], e);
+            const uint32_t ua = e ? lo[u].y : lo[u].x, ub = e ? hi[u].y : hi[u].x;
             const float2 va = F16 ? unpack_h2(ua) : unpack_bf2(ua), vb = F16 ? unpack_h2(ub) : unpack_bf2(ub);
-            const float2 s = cmul(make_float2(fmaf(sg, vb.x, va.x), fmaf(sg, vb.y, va.y)), w[u]);
-            o[u] = pack_h2(s.x, s.y);
+            const float2 s = cadd(va, vb), d = cmul(csub(va, vb), w[u]);
+            ev[u] = pack_h2(s.x, s.y);
+            od[u] = pack_h2(d.x, d.y);
           }
-          *reinterpret_cast<uint4*>(p0 + odd * 8192 + 128 * e) = make_uint4(o[0], o[1], o[2], o[3]);
+          unsigned char* out = p0 + 128 * (2 * hp + e);
+          *reinterpret_cast<uint4*>(out) = make_uint4(ev[0], ev[1], ev[2], ev[3]);
+          *reinterpret_cast<uint4*>(out + 8192) = make_uint4(od[0], od[1], od[2], od[3]);
         }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -579,7 +581,7 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
     auto epilogue3 = [&](int tile, int c, int job, float gs) {
       float2 w[2];
       if (HALVES == 2) {
-        w[0] = cmul(wout, W8[c]);                                // W_8192^{64 s1 + 8 c}
+        w[0] = cscale(cmul(wout, W8[c]), gs);                    // W_8192^{64 s1 + 8 c}
         w[1] = cmul(w[0], make_float2(0.99999529380957617f, -0.0030679567629659761f));
       }
       wait_acc(job);
@@ -595,15 +597,19 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
       for (int x = 0; x < 8; ++x) {
         float re[2] = {__uint_as_float(r[4 * x]), __uint_as_float(r[4 * x + 1])};
         float im[2] = {__uint_as_float(r[4 * x + 2]), __uint_as_float(r[4 * x + 3])};
-        if (HALVES == 2) {                                       // (even, odd) -> rows t and t + 4096
-          const float2 v = cmul(make_float2(re[1], im[1]), w[x >> 2]);
-          if (x != 3 && x != 7) w[x >> 2] = cmul(w[x >> 2], make_float2(kStepX, kStepY));
-          const float er = re[0], ei = im[0];
-          re[0] = er + v.x; re[1] = er - v.x; im[0] = ei + v.y; im[1] = ei - v.y;
-        }
         uint32_t o[2];
+        if (HALVES == 2) {                                       // (even, odd) -> rows t and t + 4096
+          const float2 v = cmul(make_float2(re[1], im[1]), w[x >> 2]);      // scaled with w
+          if (x != 3 && x != 7) w[x >> 2] = cmul(w[x >> 2], make_float2(kStepX, kStepY));
 #pragma unroll
-        for (int e = 0; e < 2; ++e) o[e] = F16 ? pack_h2(gs * re[e], -gs * im[e]) : pack_bf2(gs * re[e], -gs * im[e]);
+          for (int e = 0; e < 2; ++e) {
+            const float a = fmaf(gs, re[0], e ? -v.x : v.x), b = fmaf(-gs, im[0], e ? v.y : -v.y);
+            o[e] = F16 ? pack_h2(a, b) : pack_bf2(a, b);
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) o[e] = F16 ? pack_h2(gs * re[e], -gs * im[e]) : pack_bf2(gs * re[e], -gs * im[e]);
+        }
         // an overflow anywhere in a column makes every row of it non-finite: one row per thread is enough
         if (x == 0) bad |= nonfinite16x2<F16>(o[0]) | nonfinite16x2<F16>(o[1]);
         if (HALVES == 1) {                                       // [s2 % 8][s1][32 bytes]
