@@ -10,6 +10,8 @@
 // tile, run-time radices) -> 30 us = 1.7 TB/s of its rows; its backward 287 us (four transforms and a reduction) -> 57 us;
 // n = 2048 86 -> 43 us at the same size.
 #pragma once
+#include <type_traits>
+
 #include "fft_reg.cuh"
 #include "reg_fft.h"
 
@@ -27,6 +29,25 @@ __device__ __forceinline__ float2 tw_load2(const float2* p) {
   asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
   return v;
 }
+struct TwGlobal {
+  const float4* p;
+  __device__ __forceinline__ float4 load4(int i) const { return tw_load4(p + i); }
+  __device__ __forceinline__ float2 load2(int i) const { return tw_load2(reinterpret_cast<const float2*>(p) + i); }
+};
+// The same from a copy of the table in shared memory
+struct TwShared {
+  uint32_t p;
+  __device__ __forceinline__ float4 load4(int i) const {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(p + 16u * (uint32_t)i));
+    return v;
+  }
+  __device__ __forceinline__ float2 load2(int i) const {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(p + 8u * (uint32_t)i));
+    return v;
+  }
+};
 
 // Keeps the work in front of this point in front of it: without it the compiler interleaves the end of the forward
 // transform with the start of the inverse one and runs out of registers.
@@ -50,7 +71,7 @@ struct TwoStep {
   static constexpr bool kLoop = R1 == R2 && R1 >= 32;
   static constexpr int kActive = S * C, kThreads = (kActive + 31) / 32 * 32;
   static constexpr int kExch = R1 * (R2 + 1) * C;                   // elements of the exchange buffer
-  static constexpr int kGate = M;
+  static constexpr int kGate = M, kTw = 0;                       // twiddles in shared memory: none
   static constexpr int kParts = 1, kRed = C, kRedShift = 0;         // pairs side by side in a warp after the transform
   int p, m;
   __device__ __forceinline__ explicit TwoStep(int tid) : p(tid % C), m(tid / C) {}
@@ -184,6 +205,12 @@ struct ThreeStep2048 {
   static constexpr int kActive = S * C, kThreads = kActive;
   static constexpr int kExch = (2048 + 256) * C;
   static constexpr int kGate = 2048 + 64;
+  // Mixer and gradient take the twiddles from a copy in shared memory: the one CTA of an SM leaves room for it, and its loads take no 64-bit addresses, with
+  // which the mixer spilled 300 bytes a thread (public calls, us: layer of 8 x 2048 x 8 heads fp32 60.1 -> 56.0, of 16 x 2048 x 12 fp16
+  // 116.3 -> 109.3, forward and backward of 4 x 2048 x 8 bf16 62.6 -> 58.5).  The other modes spill nothing and lose by the copy
+  // (prompt of 4 x 1800 x 16 102.9 -> 103.5), and so do the two-step plans, whose exchanges take the same path (forward and backward
+  // of 16 x 1024 x 12 105 -> 117).
+  static constexpr int kTw = 16 * 64 + 32;
   static constexpr int kParts = PW, kRed = 4, kRedShift = 3;
   int p, m, p2, kg, l8;
   int o1, ojb, oka, q;                                    // offsets of the three access patterns, slot of row digit 0
@@ -204,22 +231,21 @@ struct ThreeStep2048 {
   __device__ __forceinline__ int bin(int i) const { return kg + 8 * (i >> 3) + 32 * l8 + 256 * (i & 7); }
   static __device__ __forceinline__ int gate_slot(int k) { return k + (k >> 5); }
 
-  template <bool HALF>
-  __device__ __forceinline__ void forward(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool) const {
+  template <bool HALF, class TW>
+  __device__ __forceinline__ void forward(float2 (&x)[E], void* buf, const TW& tw, bool) const {
     RegDft<32, false>::run(x);
 #pragma unroll
     for (int a = 0; a < 16; ++a) {
-      const float4 w = tw_load4(tw + a * 64 + m);
+      const float4 w = tw.load4(a * 64 + m);
       if (a > 0) x[2 * a] = cmul(x[2 * a], make_float2(w.x, w.y));
       x[2 * a + 1] = cmul(x[2 * a + 1], make_float2(w.z, w.w));
     }
     move<HALF, 0, 1>(x, buf);
-    const float2* w64 = reinterpret_cast<const float2*>(tw + 16 * 64);
 #pragma unroll
     for (int u = 0; u < 4; ++u) sub<false>(x, u);
 #pragma unroll
     for (int a = 1; a < 8; ++a) {
-      const float2 w = tw_load2(w64 + 8 * a + l8);
+      const float2 w = tw.load2(2 * 16 * 64 + 8 * a + l8);
 #pragma unroll
       for (int u = 0; u < 4; ++u) x[8 * u + a] = cmul(x[8 * u + a], w);
     }
@@ -227,15 +253,14 @@ struct ThreeStep2048 {
 #pragma unroll
     for (int u = 0; u < 4; ++u) sub<false>(x, u);
   }
-  template <bool HALF>
-  __device__ __forceinline__ void inverse(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool) const {
-    const float2* w64 = reinterpret_cast<const float2*>(tw + 16 * 64);
+  template <bool HALF, class TW>
+  __device__ __forceinline__ void inverse(float2 (&x)[E], void* buf, const TW& tw, bool) const {
 #pragma unroll
     for (int u = 0; u < 4; ++u) sub<true>(x, u);
     move<HALF, 2, 1>(x, buf);
 #pragma unroll
     for (int a = 1; a < 8; ++a) {
-      const float2 w = tw_load2(w64 + 8 * a + l8);
+      const float2 w = tw.load2(2 * 16 * 64 + 8 * a + l8);
 #pragma unroll
       for (int u = 0; u < 4; ++u) x[8 * u + a] = cmulc(x[8 * u + a], w);
     }
@@ -244,7 +269,7 @@ struct ThreeStep2048 {
     move<HALF, 1, 0>(x, buf);
 #pragma unroll
     for (int a = 0; a < 16; ++a) {
-      const float4 w = tw_load4(tw + a * 64 + m);
+      const float4 w = tw.load4(a * 64 + m);
       if (a > 0) x[2 * a] = cmulc(x[2 * a], make_float2(w.x, w.y));
       x[2 * a + 1] = cmulc(x[2 * a + 1], make_float2(w.z, w.w));
     }
@@ -383,8 +408,10 @@ template <class P> constexpr int reg_min_blocks() {
   return b < 1 ? 1 : (b > 16 ? 16 : b);
 }
 template <class P, int MODE> __host__ __device__ constexpr size_t reg_exch_bytes() { return ((size_t)P::kExch * (MODE == kRegGrad ? 4 : 8) + 15) / 16 * 16; }
-template <class P, int MODE> constexpr size_t reg_smem_bytes() {
-  return reg_exch_bytes<P, MODE>() + (MODE == kRegGrad ? (size_t)P::E * P::kThreads * 8 : 0) + (MODE == kRegMix ? (size_t)P::kGate * 8 : 0);
+template <class P, int MODE> __host__ __device__ constexpr bool reg_tw_shared() { return P::kTw != 0 && (MODE == kRegMix || MODE == kRegGrad); }
+template <class P, int MODE> __host__ __device__ constexpr size_t reg_smem_bytes() {
+  return reg_exch_bytes<P, MODE>() + (MODE == kRegGrad ? (size_t)P::E * P::kThreads * 8 : 0) + (MODE == kRegMix ? (size_t)P::kGate * 8 : 0) +
+         (reg_tw_shared<P, MODE>() ? (size_t)P::kTw * 16 : 0);
 }
 
 // MODE kRegMix      rows -> forward, gate, inverse -> rows
@@ -413,6 +440,17 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
   const bool live = act && pin < half, live_out = act && pout < half;
   const size_t wrow = ((size_t)slab_local * p.N1 + k1) * P::M;                    // first workspace row of the sequence
   const float2* g = p.g + (size_t)slab * p.K;
+  typename std::conditional<P::kTw == 0, const float4*, typename std::conditional<reg_tw_shared<P, MODE>(), TwShared, TwGlobal>::type>::type tw;
+  if constexpr (reg_tw_shared<P, MODE>()) {                // the table is the context's: not behind the wait
+    float4* dst = reinterpret_cast<float4*>(reg_smem + reg_smem_bytes<P, MODE>() - P::kTw * 16);
+    for (int i = threadIdx.x; i < P::kTw; i += P::kThreads) dst[i] = __ldg(p.tw + i);
+    tw.p = smem_u32(dst);
+    __syncthreads();
+  } else if constexpr (P::kTw != 0) {
+    tw.p = p.tw;
+  } else {
+    tw = p.tw;
+  }
   // a programmatic dependent of the kernel before it: the set-up overlaps that kernel's end, nothing is read earlier
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -439,9 +477,9 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
   };
   constexpr bool kRolled = MODE == kRegMix && P::kLoop;
   if constexpr (kRolled) {
-    pl.mix(x, buf, p.tw, act, [] {}, gate);
+    pl.mix(x, buf, tw, act, [] {}, gate);
   } else if constexpr (MODE != kRegInverse) {
-    pl.template forward<HALF>(x, buf, p.tw, act);
+    pl.template forward<HALF>(x, buf, tw, act);
     settle(x);
     if constexpr (MODE == kRegMix) gate(x);
   }
@@ -470,7 +508,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
     for (int i = 0; i < E; ++i) extra[i * P::kThreads + threadIdx.x] = x[i];
     reg_load_tokens<T, P, MODE>(x, p.src2, p.s2_sb, p.s2_sl, p.s2_sh, p, b, h, k1, 2 * pin, pl.m, live);
     __syncthreads();
-    pl.template forward<HALF>(x, buf, p.tw, act);
+    pl.template forward<HALF>(x, buf, tw, act);
     if (p.sums) {
       constexpr int RL = P::kRed;
       const int s = (threadIdx.x >> P::kRedShift) % RL;
@@ -498,7 +536,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
 
   if constexpr (!kRolled) {
     settle(x);
-    pl.template inverse<HALF>(x, buf, p.tw, act);
+    pl.template inverse<HALF>(x, buf, tw, act);
   }
   if (!live) return;
   if constexpr (WS) {
