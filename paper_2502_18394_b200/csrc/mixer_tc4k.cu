@@ -11,12 +11,10 @@
 //   (gate images)   per (head, k1): the 4096 gate values the unit needs (Hermitian extension,
 //                   normalised by their maximum, fp16) in the order the core reads them; written by
 //                   the first CTAs of the tc_in_kernel launch
-//   tc_core_kernel  persistent, one CTA per SM, units taken in pairs: 16 epilogue warps alternate
-//                   between the two units while a producer warp fetches the operand images with
-//                   bulk async copies and issues the MMAs (64-point DFT matrix as the A operand,
-//                   see mixer_tc.cu for the formulation), so one unit's epilogue on the ALUs
-//                   overlaps the other unit's stage on the tensor core; 4 x [MMA -> epilogue] per
-//                   unit.  Result: the unit's 4096 x 4 complex outputs in fp16, tile-major
+//   the units       4 x [MMA with the 64-point DFT matrix -> epilogue] per unit (see mixer_tc64.cu for the
+//                   formulation).  More units than SMs: mixer_tc64_kernel, two units a tile; otherwise, for an odd
+//                   number of units a head and for the read-out tc_core_kernel, one unit at a time on each
+//                   of two CTAs per SM.  Result: the unit's 4096 x 4 complex outputs in fp16, tile-major
 //   tc_out_kernel   inverse radix-R over k1 with conj twiddles, 1/n and gate scale, bf16,
 //                   transposed through shared memory into whole-row stores
 //
@@ -656,6 +654,10 @@ int launch_tc_in32(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v
                    unsigned char* ws_in, unsigned char* gimg, float* gscale, float sc);
 int launch_tc_out32(const spectre_ctx* ctx, cudaStream_t st, const unsigned char* ws_out, const spectre_act* y, int n, int slab0, int cnt);
 
+// mixer_tc64.cu
+int launch_units_tc64(const spectre_ctx* ctx, cudaStream_t st, const unsigned char* ws_in, const unsigned char* gimg, const float* gscale,
+                      unsigned char* ws_out, int nunits, int ntile, int R, float out_scale);
+
 template <int R, bool F16>
 static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g,
                       const spectre_act* y, int n, int slab0, int cnt, unsigned char* ws) {
@@ -694,15 +696,24 @@ static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
   SPECTRE_LAUNCH_OK("tc_in_kernel");
   }
 
+  const float out_scale = 1.0f / ((float)R * in_scale(R));
+  // More units than SMs: two a tile on one CTA per SM (mixer_tc64.cu).  Fewer are better spread over the SMs one by one.  Mixer call of one
+  // sequence, bf16, us, tc_core_kernel -> there: 16384 points 2 heads (64 units) 26.9 -> 27.9, 4 (128) 28.2 -> 29.0, 6 (192) 39.3 -> 36.6,
+  // 9 43.5 -> 39.7, 16 70.9 -> 65.7, 28 111.8 -> 105.7; 32768 points 5 heads 58.9 -> 55.2; 131072 points 1 head 40.8 -> 37.2, 3 87.3 -> 81.6.
+  if (ntile % 2 == 0 && nunits > (size_t)ctx->sm_count && tensor_map_encoder()) {
+    const int rc = launch_units_tc64(ctx, st, ws_in, gimg, gscale, ws_out, (int)nunits, ntile, R, out_scale);
+    if (rc != SPECTRE_OK) return rc;
+  } else {
   TcCoreParams cp = {ws_in, gimg, ws_out, reinterpret_cast<const __half*>(ctx->dft64),
                      reinterpret_cast<const float2*>(ctx->tw64x64),
                      reinterpret_cast<const float2*>(ctx->tw_staged) + (size_t)(R - 1) * 128, gscale,
-                     1.0f / ((float)R * in_scale(R)), (int)nunits, ntile, R, ctx->status_dev, 0};
+                     out_scale, (int)nunits, ntile, R, ctx->status_dev, 0};
   SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_core_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, k4CoreSmem));
   int grid = 2 * ctx->sm_count;                     // two resident CTAs per SM, a contiguous range of units each
   if ((size_t)grid > nunits) grid = (int)nunits;
   SPECTRE_CUDA_OK(launch_after(tc_core_kernel, grid, k4CoreThreads, k4CoreSmem, st, cp));
   SPECTRE_LAUNCH_OK("tc_core_kernel");
+  }
 
   if (tc32_out) return launch_tc_out32(ctx, st, ws_out, y, n, slab0, cnt);
   constexpr int NT = 512 / R;

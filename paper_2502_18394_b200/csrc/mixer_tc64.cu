@@ -1,7 +1,9 @@
-// Tensor-core spectral mixer for n = 4096 and n = 8192, bf16 or fp16 I/O (Sec. 3.2 steps 2 and 4), one persistent kernel.
+// Tensor-core spectral mixer for n = 4096 and n = 8192, bf16 or fp16 I/O (Sec. 3.2 steps 2 and 4), one persistent kernel, which also
+// transforms the 4096-point units of longer sequences (HALVES = 0).
 //
 // A tile is eight 4096-point problems that share a 32-byte piece of every row: n = 4096 the eight column pairs of one piece,
-// n = 8192 the even and the odd output bins of four column pairs (radix-2 step on the ALUs; HALVES = 2).  A 4096-point problem
+// n = 8192 the even and the odd output bins of four column pairs (radix-2 step on the ALUs; HALVES = 2), units two adjacent ones
+// of a (head, k1), whose chunks land as operands from their images in the workspace and whose results return there.  A 4096-point problem
 // is 64 x 64: four contractions with the 64-point DFT matrix F (128 x 128 in real form, scaled by 1/8, rows ordered so that Re
 // and Im of a bin sit 8 TMEM lanes apart), the inverse as conj(FFT(conj(.))).  Row index t = 64 t1 + t2, bin k1 + 64 k2:
 //
@@ -34,7 +36,10 @@
 // What bounds it now is the epilogues' latency: a tile of n = 4096 takes 13 k cycles to land and pass stage 0, 7.5 k in stages 1 and 2
 // (MMAs 4.1 k, arithmetic 3 k) and 16 k in stage 3 side by side with the next tile's stage 0, of which the pieces are 11 k; a step of an
 // epilogue is some 300 cycles of waits and fences around 200 of arithmetic, with four warps per scheduler to overlap them.
-// Measured and not kept: F in TMEM for stages 0 and 3, too (31 -> 33), the first gate table by the epilogue warps (31 -> 33),
+// A set waits for a job only when the job before it in the same accumulator is known to be complete (its own last job was a later one):
+// a wait for a phase whose predecessor is still under way would be answered by the phase before that.
+// Measured and not kept: chunks of 16 t2 with accumulators of 128 columns in stages 0 and 3, too (n = 4096 31 -> 33), four sets of
+// four warps (31 -> 33), F in TMEM for stages 0 and 3, too (31 -> 33), the first gate table by the epilogue warps (31 -> 33),
 // accumulators read one group ahead into registers (31 -> 33), two chunks of lookahead instead of three (31 -> 43).
 #include <cuda.h>
 
@@ -52,9 +57,11 @@ constexpr int k64Chunk = 16384, k64Op = 8 * k64Chunk, k64F = 128 * 128 * 2;
 constexpr int k64TmAcc = 256;
 constexpr int k64Rows = 33;                      // gate table: rows k2 = 0 ... 31 and, for k1 = 0, 32
 template <int HALVES> struct Tc64 {
+  static constexpr bool kUnits = HALVES == 0;
   static constexpr int n = 4096 * HALVES, kRing = HALVES == 1 ? 3 : 2;
-  static constexpr int kFOff = k64Op + kRing * k64Chunk, kGateOff = kFOff + k64F, kTwOff = kGateOff + HALVES * k64Rows * 256;
-  static constexpr int kBarOff = kTwOff + 8192 + 64, kSmem = kBarOff + 512;
+  static constexpr int kGate = kUnits ? 16384 : HALVES * k64Rows * 256, kRowTw = kUnits ? 2048 : 0;
+  static constexpr int kFOff = k64Op + kRing * k64Chunk, kGateOff = kFOff + k64F, kTwOff = kGateOff + kGate;
+  static constexpr int kBarOff = kTwOff + 8192 + 64 + kRowTw, kSmem = kBarOff + 512;
   static_assert(kSmem <= 232448 && kBarOff % 8 == 0, "shared memory");
   // Where chunk c of a tile's rows lands, in chunks: the first ones behind the operand space, the others in the part of it that
   // the last tile's chunk c - kRing left through
@@ -70,6 +77,12 @@ struct Tc64Params {
   int64_t s_sb, s_sl, s_sh, d_sb, d_sl, d_sh;
   int H, ntile, L, D, total;
   int* status;
+  // units of a longer transform
+  const unsigned char* gimg;   // gate tables [head, k1][16 KB]
+  const float* gscale;         // and their bounds
+  const float2* twr;           // [R][128]: W_n^{64 k1 t1}, W_n^{k1 t2}
+  float out_scale;
+  int R;
 };
 
 #define SPECTRE_R16(r) "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), \
@@ -149,6 +162,7 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
   float2* T8 = reinterpret_cast<float2*>(smem + C::kTwOff);      // W_4096^{8 c k1} at [c (8)][k1 (64)]
   float2* T1 = T8 + 512;                                         // W_4096^{r k1} at [r (8)][k1 (64)]
   float2* W8 = T8 + 1024;                                        // W_8192^{8 c}
+  const float2* Rtw = T8 + 1032;                                 // units: the 128 factors of even and odd tiles' k1
   const uint32_t bars = smem_u32(smem + C::kBarOff);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::kBarOff + 424);
   float* gmax = reinterpret_cast<float*>(smem + C::kBarOff + 432);   // bound of the gates of even and odd tiles, the two warps' maxima
@@ -177,7 +191,7 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
     for (int i = 0; i < 4; ++i) { mbar_init(accFull(i), 1); mbar_init(accFree(i), 8); mbar_init(a2Full(i), 16); }
     for (int i = 0; i < 2; ++i) { mbar_init(yFull(i), 1); mbar_init(yFree(i), 16); }
     for (int i = 0; i < 3; ++i) mbar_init(landFree(i), 1);
-    mbar_init(gFull, 2);
+    mbar_init(gFull, C::kUnits ? 1 : 2);
     mbar_init(gFree, 16);
     mbar_init(aFull, 64);
     mbar_init(opFull, 16);
@@ -204,15 +218,32 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
   if (warp == k64Warps + 1) {
     // ---- rows in and out.  Chunk c of a tile: 8 values of t2 of all t1 ----
     auto load = [&](int tile, int c) {
-      const int slab = tile / p.ntile, b = slab / p.H, h = slab - b * p.H, col0 = (tile - slab * p.ntile) * (16 / HALVES);
       mbar_expect_tx(landFull(c), k64Chunk);
-      for (int half = 0; half < HALVES; ++half)
-        tma_load_5d(smem_u32(smem) + C::land_slot(c) * k64Chunk + half * 8192, &tm_in, col0, 8 * c, 64 * half, h, b, landFull(c));
+      if constexpr (C::kUnits) {                                 // both units' columns of these t2, all K groups: an operand as it lands
+        tma_load_5d(smem_u32(smem) + C::land_slot(c) * k64Chunk, &tm_in, 0, 0, 2 * tile, 0, c, landFull(c));
+      } else {
+        const int slab = tile / p.ntile, b = slab / p.H, h = slab - b * p.H, col0 = (tile - slab * p.ntile) * (16 / (HALVES ? HALVES : 1));
+        for (int half = 0; half < HALVES; ++half)
+          tma_load_5d(smem_u32(smem) + C::land_slot(c) * k64Chunk + half * 8192, &tm_in, col0, 8 * c, 64 * half, h, b, landFull(c));
+      }
     };
+    auto load_gate = [&](int tile, int it) {                     // units: gate table and row factors of (head, k1)
+      const int gi = tile / p.ntile;
+      mbar_expect_tx(gFull, 16384 + 1024);
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                   :: "r"(smem_u32(Gsm)), "l"(p.gimg + (size_t)gi * 16384), "r"(16384), "r"(gFull) : "memory");
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                   :: "r"(smem_u32(Rtw) + 1024 * (it & 1)), "l"(p.twr + 128 * (gi % p.R)), "r"(1024), "r"(gFull) : "memory");
+    };
+    int gates = 0;                                               // units: gate tables asked for
     int it = 0, loaded = 0;                                      // loaded: chunks asked for so far
     if ((int)blockIdx.x < p.total && ok)
       for (int c = 0; c < 8; ++c, ++loaded)
         if (T == 0) load(blockIdx.x, c);
+    if (C::kUnits && (int)blockIdx.x < p.total && ok) {
+      if (T == 0) load_gate(blockIdx.x, 0);
+      ++gates;
+    }
     for (int tile = blockIdx.x; tile < p.total; tile += gridDim.x, ++it) {
       const int next = tile + (int)gridDim.x;
       const bool more = next < p.total;
@@ -223,12 +254,25 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
           ++loaded;
         }
       }
-      const int slab = tile / p.ntile, b = slab / p.H, h = slab - b * p.H, col0 = (tile - slab * p.ntile) * (16 / HALVES);
+      if (C::kUnits && more) {
+        warp_wait(ok, gFree, it & 1);
+        if (ok) {
+          if (T == 0) load_gate(next, it + 1);
+          ++gates;
+        }
+      }
       for (int c = 0; c < 8; ++c) {
         warp_wait(ok, stFull(c), it & 1);
         if (!ok) break;
         if (T == 0) {
-          for (int half = 0; half < HALVES; ++half) tma_store_5d(&tm_out, col0, 64 * half, 8 * c, h, b, smem_u32(Op) + c * k64Chunk + half * 8192);
+          if constexpr (C::kUnits) {                             // 8 KB of each unit's result
+            for (int u = 0; u < 2; ++u)
+              asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
+                           :: "l"(&tm_out), "r"(0), "r"((2 * tile + u) * 1024 + 128 * c), "r"(smem_u32(Op) + c * k64Chunk + u * 8192) : "memory");
+          } else {
+            const int slab = tile / p.ntile, b = slab / p.H, h = slab - b * p.H, col0 = (tile - slab * p.ntile) * (16 / (HALVES ? HALVES : 1));
+            for (int half = 0; half < HALVES; ++half) tma_store_5d(&tm_out, col0, 64 * half, 8 * c, h, b, smem_u32(Op) + c * k64Chunk + half * 8192);
+          }
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           if (c < 7) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
           else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -243,7 +287,10 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
     }
     if (T == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     if (!ok)                                                     // do not leave with copies in flight (bounded again)
+    {
       for (int i = loaded > 8 ? loaded - 8 : 0; i < loaded; ++i) mbar_wait(landFull(i & 7), (i >> 3) & 1);
+      if (gates) mbar_wait(gFull, (gates - 1) & 1);
+    }
   } else if (warp == k64Warps) {
     // ---- MMAs, in the order of the jobs ----
     const uint32_t one = elect_one();
@@ -261,12 +308,12 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
       if (++buf == 4) { buf = 0; jpar ^= 1; }
     };
     auto stage0 = [&](int c, int it) {
-      warp_wait(ok, convFull(c), it & 1);
+      warp_wait(ok, C::kUnits ? landFull(c) : convFull(c), it & 1);
       const uint32_t d = begin(), b0 = op0 + C::land_slot(c) * k64Chunk;
       if (ok) {
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
-          if (HALVES == 1) {
+          if (HALVES != 2) {
             mma_ss(one, d, umma_desc(f0 + ks * 256, 128, 2048), umma_desc(b0 + ks * 2048, 1024, 128), idesc_f16(64), ks > 0);
           } else {
             mma_ss(one, d, umma_desc(f0 + ks * 256, 128, 2048), umma_desc(b0 + ks * 1024, 512, 128), idesc_f16(32), ks > 0);
@@ -320,7 +367,7 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
     //      the other bins are their mirrors (row 32 holds the Nyquist bin for k1 = 0).  n = 8192: two tables, of the even and of the odd bins ----
     const int id = tid - k64Threads + 64;
     int it = 0;
-    for (int tile = blockIdx.x; tile < p.total; tile += gridDim.x, ++it) {
+    for (int tile = blockIdx.x; !C::kUnits && tile < p.total; tile += gridDim.x, ++it) {
       const float2* g = p.g + (size_t)(tile / p.ntile) * (C::n / 2 + 1);
       float m = id == 0 ? fabsf(g[C::n / 2].x) : 0.f;
 #pragma unroll 1
@@ -385,6 +432,7 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
     auto at = [](const uint4& v, int e) { return e == 0 ? v.x : (e == 1 ? v.y : (e == 2 ? v.z : v.w)); };
     // rows of a chunk -> stage 0's operand, in place: four rows t1 = 4 a .. 4 a + 3 at one t2 in, four K groups out
     auto convert = [&](int tile, int c, int it) {
+      if constexpr (C::kUnits) return;
       const int t2l = T & 7, a = 2 * w8 + (T >> 4);
       warp_wait(ok, landFull(c), it & 1);
       unsigned char* ring = smem + C::land_slot(c) * k64Chunk;
@@ -503,16 +551,26 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
       for (int e = 0; e < 4; ++e) {
         const int G = C::group(e);
         if (e == 0 || (HALVES == 2 && e == 2)) {
-          // set 1 holds the upper half of the digits: mirrored bins
-          const int half = HALVES == 2 ? G & 1 : 0;
-          const int col = set ? (half ? 63 - kl : (64 - kl) & 63) : kl, row0 = set ? 31 - 16 * j + (half == 0 && kl == 0) : 16 * j;
-          const uint32_t* tab = Gsm + half * k64Rows * 64 + col;
-          const float sg = set ? -1.f : 1.f;
+          if constexpr (C::kUnits) {                             // the image's order: bin k1 + 64 k2 at 64 k2 + (k1 ^ 8 (k2 % 4))
+            const uint32_t* tab = Gsm + 64 * (32 * set + 16 * j);
 #pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            const float2 a = unpack_h2(tab[(row0 + (set ? -2 * m : 2 * m)) * 64]), b = unpack_h2(tab[(row0 + (set ? -2 * m - 1 : 2 * m + 1)) * 64]);
-            GX[m] = pk2(a.x, b.x);
-            GY[m] = pk2(sg * a.y, sg * b.y);
+            for (int m = 0; m < 8; ++m) {
+              const float2 a = unpack_h2(tab[128 * m + (kl ^ (8 * ((2 * m) & 3)))]), b = unpack_h2(tab[128 * m + 64 + (kl ^ (8 * ((2 * m + 1) & 3)))]);
+              GX[m] = pk2(a.x, b.x);
+              GY[m] = pk2(a.y, b.y);
+            }
+          } else {
+            // set 1 holds the upper half of the digits: mirrored bins
+            const int half = HALVES == 2 ? G & 1 : 0;
+            const int col = set ? (half ? 63 - kl : (64 - kl) & 63) : kl, row0 = set ? 31 - 16 * j + (half == 0 && kl == 0) : 16 * j;
+            const uint32_t* tab = Gsm + half * k64Rows * 64 + col;
+            const float sg = set ? -1.f : 1.f;
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+              const float2 a = unpack_h2(tab[(row0 + (set ? -2 * m : 2 * m)) * 64]), b = unpack_h2(tab[(row0 + (set ? -2 * m - 1 : 2 * m + 1)) * 64]);
+              GX[m] = pk2(a.x, b.x);
+              GY[m] = pk2(sg * a.y, sg * b.y);
+            }
           }
         }
         take_y(8 * it + e, r);                                   // the job is done: its operand may be overwritten, too
@@ -579,6 +637,7 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
     bool bad = false;
     // stage 3's result of chunk c: rows 64 s1 + 8 c + x, conjugated and scaled, staged in the chunk's own space and stored
     auto epilogue3 = [&](int tile, int c, int job, float gs) {
+      if constexpr (C::kUnits) return;
       float2 w[2];
       if (HALVES == 2) {
         w[0] = cscale(cmul(wout, W8[c]), gs);                    // W_8192^{64 s1 + 8 c}
@@ -630,22 +689,58 @@ __global__ void __launch_bounds__(k64Threads, 1) mixer_tc64_kernel(const __grid_
       if (T == 0 && ok) mbar_arrive(stFull(c));
     };
 
+    // Units: times W_n^{k1 t'}, conjugated and scaled, as fp16 rows of 4 pairs in unit_row_slot's order (mixer_tc4k.cu): 64 bytes hold
+    // s2 % 4 = 0 ... 3 of a (s2 / 4, s1), swizzled as the tensor map unswizzles them
+    auto epilogue3_units = [&](int c, int job, float gs, const float2* rtw) {
+      const float2 fa = cscale(rtw[kr], gs);
+      float2 fb[8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x) fb[x] = rtw[64 + 8 * c + x];
+      wait_acc(job);
+      uint32_t r[32];
+      tmem_ld_16x256b_x8(acc(job) + lane16, r);
+      tmem_ld_wait();
+      free_acc(job);
+      unsigned char* stg = Op + c * k64Chunk + kr * 64 + tq * 4;
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {                              // registers: pair tq of the two units
+        const float2 w = cmul(fa, fb[x]);
+        const uint64_t RE = pk2u(r[4 * x], r[4 * x + 1]), IM = pk2u(r[4 * x + 2], r[4 * x + 3]);
+        const uint64_t WX = pk2(w.x, w.x), NWY = pk2(-w.y, -w.y);
+        float X[2], Y[2];
+        upk2(fma2(IM, NWY, mul2(RE, WX)), X[0], X[1]);
+        upk2(sub2(mul2(RE, NWY), mul2(IM, WX)), Y[0], Y[1]);
+        unsigned char* out = stg + (x >> 2) * 4096 + (((x & 3) ^ ((kr >> 1) & 3)) << 4);
+        *reinterpret_cast<uint32_t*>(out) = pack_h2(X[0], Y[0]);
+        *reinterpret_cast<uint32_t*>(out + 8192) = pack_h2(X[1], Y[1]);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (T == 0 && ok) mbar_arrive(stFull(c));
+    };
+
     // Last stage of tile `tile` side by side with the first one of `next`, then the middle stages of `next`.  The job numbers
     // follow the MMA warp's order.
     int job = 0, it = 0, tile = -1, next = blockIdx.x;
+    float gunit = 0.f;
 #pragma unroll 1
     while (tile >= 0 || next < p.total) {
       const bool last = tile >= 0, first = next < p.total;
-      const float gs = !last ? 0.f : (HALVES == 2 ? -0.5f : -1.f) * gmax[(it - 1) & 1];     // the sign of epilogue 1
+      const float gs = !last ? 0.f : C::kUnits ? gunit : (HALVES == 2 ? -0.5f : -1.f) * gmax[(it - 1) & 1];     // the sign of epilogue 1
 #pragma unroll 1
       for (int k = set - (last ? 4 : 2); k < 8; k += 2) {       // rows are converted one of the set's chunks ahead
-        if (last && k + 4 < 8) epilogue3(tile, k + 4, !first ? job + k + 4 : (k < 0 ? job + k + 4 : job + 2 * k + 4), gs);
+        if (last && k + 4 < 8) {
+          const int jb = !first ? job + k + 4 : (k < 0 ? job + k + 4 : job + 2 * k + 4);
+          if constexpr (C::kUnits) epilogue3_units(k + 4, jb, gs, Rtw + 128 * ((it - 1) & 1));
+          else epilogue3(tile, k + 4, jb, gs);
+        }
         if (!first) continue;
         if (k + 2 >= 0 && k + 2 < 8) convert(next, k + 2, it);
         if (k >= 0) epilogue0(k, !last ? job + k : (k < 4 ? job + 5 + 2 * k : job + 8 + k));
       }
       if (!first) break;
       job += last ? 16 : 8;
+      if constexpr (C::kUnits) gunit = -p.out_scale * p.gscale[next / p.ntile];      // for the tile's last stage
       epilogue1(it);
       epilogue2(it);
       __syncwarp();
@@ -719,6 +814,36 @@ int launch_mixer_tc4096(const spectre_ctx* ctx, cudaStream_t st, const spectre_a
 }
 int launch_mixer_tc8192(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, const spectre_act* y) {
   return v->dtype == SPECTRE_F16 ? launch_tc64<true, 2>(ctx, st, v, g, y) : launch_tc64<false, 2>(ctx, st, v, g, y);
+}
+
+// The 4096-point units of a longer transform (mixer_tc4k.cu), two adjacent ones (eight column pairs of one head and k1) a tile: first
+// operands from the images that the radix-R step wrote, results in their place in the workspace.
+int launch_units_tc64(const spectre_ctx* ctx, cudaStream_t st, const unsigned char* ws_in, const unsigned char* gimg, const float* gscale,
+                      unsigned char* ws_out, int nunits, int ntile, int R, float out_scale) {
+  // an image is [K group a (16)][pair (4)][t2 (64)][16 bytes]; a chunk takes 8 t2 of both units
+  const cuuint64_t dims[5] = {64, 4, (cuuint64_t)nunits, 16, 8}, strides[4] = {1024, 65536, 4096, 128};
+  const cuuint32_t box[5] = {64, 4, 2, 16, 1}, es[5] = {1, 1, 1, 1, 1};
+  const cuuint64_t odims[2] = {32, (cuuint64_t)nunits * 1024}, ostrides[1] = {64};
+  const cuuint32_t obox[2] = {32, 128};
+  CUtensorMap tm_in, tm_out;
+  CUresult r = tensor_map_encoder()(&tm_in, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, const_cast<unsigned char*>(ws_in), dims, strides, box, es,
+                                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r == CUDA_SUCCESS)
+    r = tensor_map_encoder()(&tm_out, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, ws_out, odims, ostrides, obox, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                             CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(SPECTRE_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
+  Tc64Params p = {};
+  p.F = reinterpret_cast<const __half*>(ctx->dft64);
+  p.ntile = ntile / 2;
+  p.total = nunits / 2;
+  p.status = ctx->status_dev;
+  p.gimg = gimg; p.gscale = gscale; p.R = R; p.out_scale = out_scale;
+  p.twr = reinterpret_cast<const float2*>(ctx->tw_staged) + (size_t)(R - 1) * 128;
+  auto kern = mixer_tc64_kernel<true, 0>;
+  SPECTRE_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Tc64<0>::kSmem));
+  SPECTRE_CUDA_OK(launch_after(kern, p.total < ctx->sm_count ? p.total : ctx->sm_count, k64Threads, Tc64<0>::kSmem, st, tm_in, tm_out, p));
+  return SPECTRE_OK;
 }
 
 }  // namespace spectre

@@ -207,6 +207,27 @@ def test_mixer_single_kernel_tiles_per_cta(ctx, dt, n, B, L, H, D):
         assert float(err.max()) < (3e-3 if dt == "bf16" else 2e-3)      # + the output's rounding: 2^-9 / sqrt(3) and 2^-12 / sqrt(3)
 
 
+@pytest.mark.parametrize("dt,n,B,L,H,D", [("bf16", 16384, 1, 16384, 4, 64), ("bf16", 16384, 1, 16384, 5, 64), ("f16", 16384, 3, 12290, 17, 32),
+                                          ("bf16", 32768, 2, 32768, 9, 64), ("f16", 131072, 1, 12288, 5, 64), ("bf16", 16384, 3, 16384, 7, 24)])
+def test_mixer_staged_units_two_a_tile(ctx, dt, n, B, L, H, D):
+    # units of 4096 points on either side of one per SM, several tiles per CTA, an odd number of units a head; twice, as a tile's
+    # operands land in the space that its predecessor leaves.  Tolerances as for the single kernel
+    x = W.activations(W.Workload("t", B=B, L=L, H=H, D=D, dtype=dt, seed=n + H)).cuda()
+    g = torch.randn(B, H, n // 2 + 1, 2, generator=torch.Generator().manual_seed(n + B)).cuda()
+    g *= torch.exp(torch.arange(B * H, device="cuda").view(B, H, 1, 1) % 7 - 3.0)
+    for _ in range(2):
+        y = S.spectre_mixer_forward(ctx, x, g, n_fft=n)
+        torch.cuda.synchronize()
+        ctx.poll_status()
+        for b in range(B):
+            G = torch.view_as_complex(g[b].double())
+            G[:, 0].imag = 0
+            G[:, -1].imag = 0
+            ref = torch.fft.irfft(torch.fft.rfft(x[b].double(), n=n, dim=0) * G.t()[:, :, None], n=n, dim=0)[:L]
+            err = (y[b].double() - ref).norm(dim=0) / ref.norm(dim=0)
+            assert float(err.max()) < (4e-3 if dt == "bf16" else 3e-3)      # one column: less averaging than over a slab
+
+
 @pytest.mark.parametrize("L", [64, 4160, 8128])
 def test_mixer_bf16_8192_short_sequences_through_the_tensor_maps(ctx, L):
     # whole 64-row blocks shorter than n: rows beyond L read as zero and are not written;
