@@ -442,8 +442,9 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
   const float2* g = p.g + (size_t)slab * p.K;
   typename std::conditional<P::kTw == 0, const float4*, typename std::conditional<reg_tw_shared<P, MODE>(), TwShared, TwGlobal>::type>::type tw;
   if constexpr (reg_tw_shared<P, MODE>()) {                // the table is the context's: not behind the wait
+    const float4* tab = p.tw;
     float4* dst = reinterpret_cast<float4*>(reg_smem + reg_smem_bytes<P, MODE>() - P::kTw * 16);
-    for (int i = threadIdx.x; i < P::kTw; i += P::kThreads) dst[i] = __ldg(p.tw + i);
+    for (int i = threadIdx.x; i < P::kTw; i += P::kThreads) dst[i] = __ldg(tab + i);
     tw.p = smem_u32(dst);
     __syncthreads();
   } else if constexpr (P::kTw != 0) {
