@@ -121,14 +121,6 @@ __device__ __forceinline__ float2 pair_from_half(float2 gk, float4 ab, int k, in
   return make_float2(xa.x + xb.y, xb.x - xa.y);
 }
 
-// exp(-j 2 pi m / 8192) from the quarter-wave table (cos, sin)(2 pi r / 8192), r = 0..2048
-__device__ __forceinline__ float2 twiddle8192(const float2* __restrict__ tab, unsigned m) {
-  const unsigned q = (m >> 11) & 3u, r = m & 2047u;
-  const float2 t = __ldg(tab + r);
-  const float c = (q & 1u) ? -t.y : t.x, s = (q & 1u) ? t.x : t.y;    // rotate by q quarter turns
-  return (q & 2u) ? make_float2(-c, s) : make_float2(c, -s);
-}
-
 // ---- loads / stores of 4 adjacent real columns as two complex pairs ----------
 // (columns 2c and 2c+1 form the complex number a + jb; see mixer.cu)
 template <typename T> struct io;

@@ -31,8 +31,8 @@
 // Why: an SM moves one 32-byte piece of a row per 1.3 cycles (loads from L2; stores 1.4) and a 16-byte piece per 1.1 (1.4), so
 // 32-byte pieces halve the time in the request path, and only the rows of 8 problems x 64 t2 steps that are in flight need shared
 // memory besides the one operand.  The kernels before this one kept 4 column pairs per CTA in 16-byte pieces and ran rows in, four
-// stages and rows out one after the other.  Public calls, us: 4 x 4096 x 16 heads with projection 89.9 -> 73.8 (this kernel 47 -> 31),
-// 1 x 8192 x 32 heads 70.4 -> 65.1 (51 -> 40, two fewer column pairs per piece), its backward included 199.5 -> 186.1.
+// stages and rows out one after the other.  Public calls, us: 4 x 4096 x 16 heads with projection 89.5 -> 74.7 (this kernel 47 -> 31),
+// 1 x 8192 x 32 heads 70.8 -> 63.4 (51 -> 40), its backward included 200.2 -> 182.9.
 // What bounds it now is the epilogues' latency: a tile of n = 4096 takes 13 k cycles to land and pass stage 0, 7.5 k in stages 1 and 2
 // (MMAs 4.1 k, arithmetic 3 k) and 16 k in stage 3 side by side with the next tile's stage 0, of which the pieces are 11 k; a step of an
 // epilogue is some 300 cycles of waits and fences around 200 of arithmetic, with four warps per scheduler to overlap them.

@@ -15,7 +15,7 @@ namespace spectre {
 // the size of the operands), the odd column's is that times W_4096^{row} (wr0, wr1: the thread's two
 // rows).  The two products of an x run as packed fp32 pairs; the transposed operand (row -> column index,
 // d -> K) leaves as one 8-byte store per x.  TMEM loads run one 32-column chunk ahead.
-//   COLS: order of the output columns.  1: 64 c + row.  0: 4 row + c.  2: 16 (row / 4) + 8 (c / 2) +
+//   COLS: order of the output columns.  1: 64 c + row.  2: 16 (row / 4) + 8 (c / 2) +
 //   2 (row % 4) + c % 2, which keeps the four rows a half-warp writes at once in four different
 //   16-byte slots of a core matrix even when LBO and SBO are multiples of 128 (dense images), and
 //   leaves all four pairs of a row in one thread of the epilogue that reads the next accumulator.
@@ -47,7 +47,6 @@ __device__ __forceinline__ void epilogue_twiddle2(uint32_t tmem_d, unsigned char
     }
     const uint32_t (&rr)[16] = r[s8 & 1];
     const uint32_t colpart = COLS == 1 ? (uint32_t)((8 * c + (row >> 3)) * SBO + (row & 7) * 16)
-                           : COLS == 0 ? (uint32_t)((row >> 1) * SBO + (4 * (row & 1) + c) * 16)
                                        : (uint32_t)((2 * (row >> 2) + (c >> 1)) * SBO + (2 * (row & 3) + (c & 1)) * 16);
     const uint32_t base = colpart + (uint32_t)((8 * chunk + (tq >> 1)) * LBO + 8 * (tq & 1));
 #pragma unroll
