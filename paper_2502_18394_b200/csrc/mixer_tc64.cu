@@ -30,8 +30,8 @@
 //
 // Why: an SM moves one 32-byte piece of a row per 1.3 cycles (loads from L2; stores 1.4) and a 16-byte piece per 1.1 (1.4), so
 // 32-byte pieces halve the time in the request path, and only the rows of 8 problems x 64 t2 steps that are in flight need shared
-// memory besides the one operand.  The kernels before this one kept 4 column pairs per CTA in 16-byte pieces and ran rows in, four
-// stages and rows out one after the other.  Public calls, us: 4 x 4096 x 16 heads with projection 89.5 -> 74.7 (this kernel 47 -> 31),
+// memory besides the one operand.  The kernels before this one (mixer_tc4096.cu is one of them, still the better for few tiles) kept 4
+// column pairs per CTA in 16-byte pieces and ran rows in, four stages and rows out one after the other.  Public calls, us: 4 x 4096 x 16 heads with projection 89.5 -> 74.7 (this kernel 47 -> 31),
 // 1 x 8192 x 32 heads 70.8 -> 63.4 (51 -> 40), its backward included 200.2 -> 182.9.
 // What bounds it now is the epilogues' latency: a tile of n = 4096 takes 13 k cycles to land and pass stage 0, 7.5 k in stages 1 and 2
 // (MMAs 4.1 k, arithmetic 3 k) and 16 k in stage 3 side by side with the next tile's stage 0, of which the pieces are 11 k; a step of an
@@ -809,7 +809,13 @@ static int launch_tc64(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
   SPECTRE_CUDA_OK(launch_after(kern, p.total < ctx->sm_count ? p.total : ctx->sm_count, k64Threads, Tc64<HALVES>::kSmem, st, tm_in, tm_out, p));
   return SPECTRE_OK;
 }
+int launch_mixer_pairs4096(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, const spectre_act* y);   // mixer_tc4096.cu
+// Half-width tiles (4 column pairs, mixer_tc4096.cu) while each has an SM of its own: a tile of eight takes longer (mixer call, us, half | whole:
+// 1 x 4 heads 15.0 | 16.0, 16 heads 15.9 | 17.1, but 24 heads 22.3 | 17.6, 38 36.9 | 30.0, 64 45.5 | 31.9), and for lengths whose
+// partial block of 64 rows is long, since the whole tile fetches those rows one by one: 20 rows 16 heads 15.7 | 19.9, 24 heads 22.3 | 20.3, 48 heads
+// 36.1 | 36.2, 64 heads 42.4 | 36.7; 36 rows 24 heads 22.5 | 23.0, 48 heads 36.7 | 40.4, 64 heads 43.6 | 41.5; 1 row as none.
 int launch_mixer_tc4096(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, const spectre_act* y) {
+  if ((long long)v->B * v->H * (v->D / 8) <= ctx->sm_count || v->L % 64 > 16) return launch_mixer_pairs4096(ctx, st, v, g, y);
   return v->dtype == SPECTRE_F16 ? launch_tc64<true, 1>(ctx, st, v, g, y) : launch_tc64<false, 1>(ctx, st, v, g, y);
 }
 int launch_mixer_tc8192(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, const spectre_act* y) {

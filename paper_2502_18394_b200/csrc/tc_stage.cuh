@@ -1,5 +1,5 @@
 // Epilogues between the 64 x 64 stages of a 4096-point transform on the tensor cores, for the core kernel of the longer
-// transforms (mixer_tc4k.cu): the accumulator of a stage has the new digit along its rows and, along its columns, the column
+// transforms (mixer_tc4k.cu) and the half tiles of n = 4096 (mixer_tc4096.cu): the accumulator of a stage has the new digit along its rows and, along its columns, the column
 // pair c and the digit that is contracted next.
 #pragma once
 #include "tc_common.cuh"

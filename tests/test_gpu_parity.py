@@ -188,9 +188,10 @@ def test_mixer_staged_ragged_rows(ctx, dt, n, L):
 
 
 @pytest.mark.parametrize("dt,n,B,L,H,D", [("bf16", 4096, 1, 4096, 1, 8), ("f16", 4096, 5, 4096, 31, 64), ("bf16", 4096, 7, 2047, 43, 24),
+                                          ("bf16", 4096, 7, 2000, 43, 24), ("f16", 4096, 1, 4096, 18, 64), ("f16", 4096, 1, 4096, 19, 64),
                                           ("f16", 8192, 1, 8192, 1, 8), ("bf16", 8192, 3, 8192, 33, 64), ("f16", 8192, 5, 4160, 37, 40)])
 def test_mixer_single_kernel_tiles_per_cta(ctx, dt, n, B, L, H, D):
-    # one tile, and persistent CTAs with several: the next tile's rows land where the last one's results left, gates change
+    # one tile, and persistent CTAs with several (n = 4096: either kernel, on both sides of their lines): the next tile's rows land where the last one's results left, gates change
     # from tile to tile.  All slabs against an fp64 transform; the fp16 operand images keep 1e-3 of a slab's norm
     x = W.activations(W.Workload("t", B=B, L=L, H=H, D=D, dtype=dt, seed=n + B)).cuda()
     g = torch.randn(B, H, n // 2 + 1, 2, generator=torch.Generator().manual_seed(n + H)).cuda()
