@@ -680,7 +680,7 @@ static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
                    v->H, D, v->L, n, ntile, slab0};
   size_t smem_in = (size_t)R * ntile * (NT2 / 2) * 128;
   if (smem_in < 4096 * sizeof(float2)) smem_in = 4096 * sizeof(float2);       // the gate CTAs' staging
-  if (smem_in > 48 * 1024)
+  if (smem_in + 4 * NT2 * sizeof(float2) > 48 * 1024)                         // with the kernel's own table of row twiddles
     SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_in_kernel<R, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_in));
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

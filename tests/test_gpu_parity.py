@@ -229,6 +229,13 @@ def test_mixer_staged_units_two_a_tile(ctx, dt, n, B, L, H, D):
             assert float(err.max()) < (4e-3 if dt == "bf16" else 3e-3)      # one column: less averaging than over a slab
 
 
+# widths whose staging fills the 48 KiB that a launch gets unasked: the kernel's own table comes on top
+@pytest.mark.parametrize("dt,n,L,D", [("bf16", 16384, 16384, 48), ("f16", 32768, 20011, 48), ("bf16", 131072, 69640, 48), ("f16", 4096, 63, 96)])
+def test_mixer_staged_widths_at_the_default_shared_memory_limit(ctx, dt, n, L, D):
+    w = W.Workload("t", B=1, L=L, H=1, D=D, dtype=dt, n_fft=n, seed=n + D)
+    assert run_mixer(ctx, w, n_fft=n) < TOL[dt]
+
+
 @pytest.mark.parametrize("L", [64, 4160, 8128])
 def test_mixer_bf16_8192_short_sequences_through_the_tensor_maps(ctx, L):
     # whole 64-row blocks shorter than n: rows beyond L read as zero and are not written;
