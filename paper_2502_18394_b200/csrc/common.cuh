@@ -83,6 +83,13 @@ cudaError_t launch_after(void (*kern)(P...), dim3 grid, int block, size_t smem, 
   cfg.numAttrs = 1;
   return launch_kernel(&cfg, kern, P(args)...);
 }
+// For kernels whose shared memory follows the call's sizes: dynamic shared memory up to all that a CTA may have (`fixed`: the
+// kernel's own static part).  The limit belongs to the function, not to the launch, so a call that set it to its own size would
+// take it away from a larger call of another thread that is between its setting and its launch.
+template <class... P>
+cudaError_t allow_shared(const spectre_ctx* ctx, void (*kern)(P...), size_t fixed = 0) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem_optin - (int)fixed);
+}
 #endif
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

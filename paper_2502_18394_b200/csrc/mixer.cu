@@ -578,10 +578,9 @@ static bool make_plan(const spectre_ctx* ctx, int n, TransformPlan* pl) {
 }
 
 template <typename T, int C, bool FIX>
-static int launch_onchip_cf(const OnchipParams& p, const TransformPlan& pl, int nslab, cudaStream_t st) {
+static int launch_onchip_cf(const spectre_ctx* ctx, const OnchipParams& p, const TransformPlan& pl, int nslab, cudaStream_t st) {
   auto kern = onchip_kernel<T, C, FIX>;
-  if (pl.smem > 48 * 1024)
-    SPECTRE_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
+  if (pl.smem > 48 * 1024) SPECTRE_CUDA_OK(allow_shared(ctx, kern));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((size_t)nslab * pl.N1 * p.ntile * C), 1, 1);
   cfg.blockDim = dim3(pl.threads, 1, 1);
@@ -599,11 +598,11 @@ static int launch_onchip_cf(const OnchipParams& p, const TransformPlan& pl, int 
 }
 
 template <typename T>
-static int launch_onchip(const OnchipParams& p, const TransformPlan& pl, int nslab, cudaStream_t st) {
+static int launch_onchip(const spectre_ctx* ctx, const OnchipParams& p, const TransformPlan& pl, int nslab, cudaStream_t st) {
   switch (pl.C) {
-    case 1: return launch_onchip_cf<T, 1, false>(p, pl, nslab, st);
-    case 2: return launch_onchip_cf<T, 2, true>(p, pl, nslab, st);     // clusters hold 2048 rows per CTA: 16 x 16 x 8
-    case 4: return launch_onchip_cf<T, 4, true>(p, pl, nslab, st);
+    case 1: return launch_onchip_cf<T, 1, false>(ctx, p, pl, nslab, st);
+    case 2: return launch_onchip_cf<T, 2, true>(ctx, p, pl, nslab, st);     // clusters hold 2048 rows per CTA: 16 x 16 x 8
+    case 4: return launch_onchip_cf<T, 4, true>(ctx, p, pl, nslab, st);
     default: return fail(SPECTRE_ERR_UNSUPPORTED, "cluster size not supported");
   }
 }
@@ -714,7 +713,7 @@ static int mixer_typed(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
   p.mode = 0;
   if (pl.N1 == 1) {
     p.slab0 = 0; p.src_ws = 0; p.dst_ws = 0; p.ws = nullptr;
-    return launch_onchip<T>(p, pl, nslab, st);
+    return launch_onchip<T>(ctx, p, pl, nslab, st);
   }
   const size_t per = slab_ws_bytes(pl.n, v->D);
   int group = (int)(ws_bytes / per);
@@ -733,7 +732,7 @@ static int mixer_typed(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
     p.slab0 = s0;
     int rc = launch_strided<T, false>(sp, pl.N1, st);
     if (rc != SPECTRE_OK) return rc;
-    rc = launch_onchip<T>(p, pl, cnt, st);
+    rc = launch_onchip<T>(ctx, p, pl, cnt, st);
     if (rc != SPECTRE_OK) return rc;
     rc = launch_strided<T, true>(sp, pl.N1, st);
     if (rc != SPECTRE_OK) return rc;
@@ -767,7 +766,7 @@ int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
   p.ws = ws; p.mode = 1; p.dst_ws = 1; p.slab0 = slab0;
   p.src_ws = 0; p.decim = pl.N1 > 1;
   *ring_done = 0;
-  SPECTRE_IO_DISPATCH(v->dtype, return launch_onchip<T>(p, pl, cnt, st));
+  SPECTRE_IO_DISPATCH(v->dtype, return launch_onchip<T>(ctx, p, pl, cnt, st));
 }
 
 // Inverse transform only (read-out of the Prefix-FFT cache): y = R_n^{-1}(diag(g) spec) for all
@@ -806,7 +805,7 @@ static int inverse_typed(const spectre_ctx* ctx, cudaStream_t st, const float2* 
   p.mode = 2;
   if (pl.N1 == 1) {
     p.slab0 = 0; p.dst_ws = 0; p.ws = nullptr;
-    return launch_onchip<T>(p, pl, nslab, st);
+    return launch_onchip<T>(ctx, p, pl, nslab, st);
   }
   const size_t per = slab_ws_bytes(pl.n, y->D);
   int group = (int)(ws_bytes / per);
@@ -822,7 +821,7 @@ static int inverse_typed(const spectre_ctx* ctx, cudaStream_t st, const float2* 
     int cnt = nslab - s0 < group ? nslab - s0 : group;
     sp.slab0 = s0; sp.nslab = cnt;
     p.slab0 = s0;
-    int rc = launch_onchip<T>(p, pl, cnt, st);
+    int rc = launch_onchip<T>(ctx, p, pl, cnt, st);
     if (rc != SPECTRE_OK) return rc;
     rc = launch_strided<T, true>(sp, pl.N1, st);
     if (rc != SPECTRE_OK) return rc;

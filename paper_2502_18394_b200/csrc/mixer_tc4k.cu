@@ -680,8 +680,8 @@ static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
                    v->H, D, v->L, n, ntile, slab0};
   size_t smem_in = (size_t)R * ntile * (NT2 / 2) * 128;
   if (smem_in < 4096 * sizeof(float2)) smem_in = 4096 * sizeof(float2);       // the gate CTAs' staging
-  if (smem_in + 4 * NT2 * sizeof(float2) > 48 * 1024)                         // with the kernel's own table of row twiddles
-    SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_in_kernel<R, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_in));
+  constexpr size_t kOwn = 4096;        // the kernel's static part: a table of row twiddles and a few words, rounded up to 1 KiB (3 KiB at most)
+  if (smem_in + kOwn > 48 * 1024) SPECTRE_CUDA_OK(allow_shared(ctx, tc_in_kernel<R, F16>, kOwn));
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -720,8 +720,7 @@ static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
   TcOutParams op = {ws_out, reinterpret_cast<bf16*>(y->ptr), y->stride_b, y->stride_l, y->stride_h,
                     y->H, D, y->L, n, ntile, slab0, ctx->status_dev};
   const size_t smem_out = (size_t)R * NT * (D / 2) * 4;
-  if (smem_out > 48 * 1024)
-    SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_out_kernel<R, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_out));
+  if (smem_out > 48 * 1024) SPECTRE_CUDA_OK(allow_shared(ctx, tc_out_kernel<R, F16>));
   SPECTRE_CUDA_OK(launch_after(tc_out_kernel<R, F16>, cnt * (4096 / NT), 256, smem_out, st, op));
   SPECTRE_LAUNCH_OK("tc_out_kernel");
   return SPECTRE_OK;
@@ -807,8 +806,7 @@ static int tc4k_readout_group(const spectre_ctx* ctx, cudaStream_t st, const flo
   TcOutParams op = {ws_out, reinterpret_cast<bf16*>(y->ptr), y->stride_b, y->stride_l, y->stride_h,
                     y->H, D, y->L, n, ntile, slab0, ctx->status_dev};
   const size_t smem_out = (size_t)R * NT * (D / 2) * 4;
-  if (smem_out > 48 * 1024)
-    SPECTRE_CUDA_OK(cudaFuncSetAttribute(tc_out_kernel<R, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_out));
+  if (smem_out > 48 * 1024) SPECTRE_CUDA_OK(allow_shared(ctx, tc_out_kernel<R, F16>));
   SPECTRE_CUDA_OK(launch_after(tc_out_kernel<R, F16>, cnt * (4096 / NT), 256, smem_out, st, op));
   SPECTRE_LAUNCH_OK("tc_out_kernel");
   return SPECTRE_OK;

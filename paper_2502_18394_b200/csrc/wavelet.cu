@@ -313,9 +313,7 @@ extern "C" int spectre_wavelet_refine(spectre_ctx* ctx, void* stream, const spec
   const bool wbf = w->wdtype == SPECTRE_BF16;
 #define SPECTRE_WAVELET_LAUNCH(T, WT)                                                                           \
   do {                                                                                                          \
-    if (smem > 48 * 1024)                                                                                       \
-      SPECTRE_CUDA_OK(cudaFuncSetAttribute(wavelet_kernel<T, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
-                                           (int)smem));                                                         \
+    if (smem > 48 * 1024) SPECTRE_CUDA_OK(allow_shared(ctx, wavelet_kernel<T, WT>));                            \
     SPECTRE_CUDA_OK(launch_after(wavelet_kernel<T, WT>, grid, 256, smem, st, p));                               \
   } while (0)
   SPECTRE_IO_DISPATCH(y_in->dtype, {

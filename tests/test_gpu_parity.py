@@ -1,6 +1,8 @@
 """GPU parity: the CUDA library (through its C ABI) against the fp64 oracle on
 the same seeded inputs, element by element.  Tolerances: max relative L2 error
 per (batch, head) slab <= 1e-5 for fp32 I/O, <= 1e-2 for bf16 I/O."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -1089,6 +1091,44 @@ def test_what_a_call_on_a_given_stream_allocates_belongs_to_that_stream(ctx):
 
 
 # ------------------------------------------------------------------ errors
+@pytest.mark.parametrize("dt,shapes,levels", [("f32", [(1000, 16), (2000, 16)], 0), ("bf16", [(16384, 64), (16384, 80), (16384, 128)], 0),
+                                              ("f32", [(1024, 16), (1024, 32)], 10)])
+def test_calls_of_several_threads_and_sizes_on_one_kernel(ctx, dt, shapes, levels):
+    # kernels whose shared memory follows the call's sizes: a smaller call of another thread leaves a larger one launchable
+    failed, outputs = [], []
+
+    def calls(n, D):
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            w = W.Workload("t", B=1, L=n, H=1, D=D, dtype=dt, seed=n + D)
+            x, g = W.activations(w), W.random_gate(w)
+            xd, gd = x.cuda(), g.cuda()
+            y = torch.empty_like(xd)
+            ws = torch.empty(max(16, S.spectre_mixer_workspace_bytes(ctx, 1, n, 1, D, n, S._dtype_code(x))), dtype=torch.uint8, device="cuda")
+            s = torch.rand(1, 1, levels + 1, D, generator=torch.Generator().manual_seed(n)).cuda()
+            for i in range(1500):
+                try:
+                    if levels:
+                        S.spectre_wavelet_refine(ctx, xd, {"levels": levels, "level_gates": s}, y_out=y)
+                    else:
+                        S.spectre_mixer_forward(ctx, xd, gd, y=y, n_fft=n, workspace=ws)
+                except S.SpectreError as e:
+                    failed.append(str(e))
+            st.synchronize()
+            ref = O.wavelet_refine(W.to_f64(x), W.to_f64(s), levels) if levels else O.mixer(W.to_f64(x), gate_to_complex(g))
+            outputs.append((W.to_f64(y), ref))
+
+    threads = [threading.Thread(target=calls, args=s) for s in shapes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, (len(failed), failed[0])
+    assert len(outputs) == len(shapes)
+    for y, ref in outputs:
+        assert_close(y, ref, dt)
+
+
 def test_invalid_arguments_are_rejected_before_launch(ctx):
     x = torch.zeros(1, 64, 2, 16, device="cuda")
     g = torch.zeros(1, 2, 33, 2, device="cuda")
