@@ -810,12 +810,19 @@ static int launch_tc64(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
   return SPECTRE_OK;
 }
 int launch_mixer_pairs4096(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, const spectre_act* y);   // mixer_tc4096.cu
-// Half-width tiles (4 column pairs, mixer_tc4096.cu) while each has an SM of its own: a tile of eight takes longer (mixer call, us, half | whole:
-// 1 x 4 heads 15.0 | 16.0, 16 heads 15.9 | 17.1, but 24 heads 22.3 | 17.6, 38 36.9 | 30.0, 64 45.5 | 31.9), and for lengths whose
-// partial block of 64 rows is long, since the whole tile fetches those rows one by one: 20 rows 16 heads 15.7 | 19.9, 24 heads 22.3 | 20.3, 48 heads
-// 36.1 | 36.2, 64 heads 42.4 | 36.7; 36 rows 24 heads 22.5 | 23.0, 48 heads 36.7 | 40.4, 64 heads 43.6 | 41.5; 1 row as none.
+// Half-width tiles (4 column pairs, mixer_tc4096.cu) or whole ones, whichever the counts of both let expect to be done first.  An SM holds two
+// half tiles at once and takes 21 us for a pair, 13.5 for one that is left alone; it takes 13 for a whole tile, 0.75 more for each
+// chunk of 8 rows of a partial block (the whole tile fetches them one by one) and 0.5 more for tiles that reach beyond D.  The numbers are
+// fitted, in quarters of a microsecond, to 1300 mixer calls of 4 ... 600 heads of 8 ... 128 channels, 64 ... 4096 rows: the choice costs 0.16 per
+// cent of the better kernel's time on average and 7 at most.  Some of them, us, half | whole: 64 channels, whole blocks, 18 heads 15.3 | 16.1,
+// 19 heads 20.8 | 16.2, 38 heads 34.7 | 29.2, 64 heads 40.9 | 30.0; 20 rows beyond, 16 heads 15.6 | 18.9, 24 heads 22.0 | 19.2, 48 heads 36.4 | 35.2, 64 heads
+// 42.0 | 35.6; 40 rows, 24 heads 22.1 | 22.3, 48 heads 36.5 | 41.0, 256 heads 161.8 | 138.2; 63 rows, 64 heads 42.4 | 45.9, 256 heads 161.8 | 145.5;
+// 8 channels (a whole tile is half empty), 149 heads 20.7 | 30.5.
 int launch_mixer_tc4096(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, const spectre_act* y) {
-  if ((long long)v->B * v->H * (v->D / 8) <= ctx->sm_count || v->L % 64 > 16) return launch_mixer_pairs4096(ctx, st, v, g, y);
+  const long long slabs = (long long)v->B * v->H, sms = ctx->sm_count;
+  const long long half = (slabs * (v->D / 8) + sms - 1) / sms, whole = (slabs * ((v->D + 15) / 16) + sms - 1) / sms;      // the fullest SM's share
+  const int chunks = (v->L % 64 + 7) / 8;
+  if (42 * half + 12 * (half & 1) <= 16 + whole * (52 + 3 * chunks + (v->D % 16 ? 2 : 0))) return launch_mixer_pairs4096(ctx, st, v, g, y);
   return v->dtype == SPECTRE_F16 ? launch_tc64<true, 1>(ctx, st, v, g, y) : launch_tc64<false, 1>(ctx, st, v, g, y);
 }
 int launch_mixer_tc8192(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const float* g, const spectre_act* y) {

@@ -191,6 +191,8 @@ def test_mixer_staged_ragged_rows(ctx, dt, n, L):
 
 @pytest.mark.parametrize("dt,n,B,L,H,D", [("bf16", 4096, 1, 4096, 1, 8), ("f16", 4096, 5, 4096, 31, 64), ("bf16", 4096, 7, 2047, 43, 24),
                                           ("bf16", 4096, 7, 2000, 43, 24), ("f16", 4096, 1, 4096, 18, 64), ("f16", 4096, 1, 4096, 19, 64),
+                                          ("bf16", 4096, 2, 2523, 14, 64), ("f16", 4096, 1, 108, 56, 64),
+                                          ("bf16", 4096, 1, 4040, 32, 72), ("bf16", 4096, 2, 2000, 32, 24), ("f16", 4096, 4, 3251, 64, 64),
                                           ("f16", 8192, 1, 8192, 1, 8), ("bf16", 8192, 3, 8192, 33, 64), ("f16", 8192, 5, 4160, 37, 40)])
 def test_mixer_single_kernel_tiles_per_cta(ctx, dt, n, B, L, H, D):
     # one tile, and persistent CTAs with several (n = 4096: either kernel, on both sides of their lines): the next tile's rows land where the last one's results left, gates change
