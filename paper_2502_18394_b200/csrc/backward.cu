@@ -17,6 +17,8 @@ int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
                       float2* ws, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done);
 bool transform_supported(const spectre_ctx* ctx, int n);
 size_t transform_slab_bytes(int n, int D);
+int mixer_check(const spectre_ctx* ctx, const spectre_act* v, const float* g, const spectre_act* y, int n_fft, const void* workspace,
+                size_t workspace_bytes);
 
 __global__ void __launch_bounds__(256) conj_gate_kernel(const float2* g, float2* gc, size_t total) {
   after_previous();
@@ -238,11 +240,16 @@ extern "C" int spectre_mixer_backward(spectre_ctx* ctx, void* stream, const spec
   const size_t mix_bytes = align256(spectre_mixer_workspace_bytes(ctx, B, v->L, H, D, n_fft, v->dtype));
   const size_t per = transform_slab_bytes(n_fft, D);
   if (workspace_bytes < gc_bytes + mix_bytes + 2 * per) return fail(SPECTRE_ERR_WORKSPACE, "backward workspace too small");
-  SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   unsigned char* base = reinterpret_cast<unsigned char*>(workspace);
   auto pitch_ok = [](const spectre_act* a) { return !a || (a->stride_l >= 0 && a->stride_l <= (1 << 18)); };   // 32-bit row offsets
-  if (dg && reg_supported(n_fft) && pitch_ok(v) && pitch_ok(dy) && pitch_ok(dv))
+  const bool one_kernel = dg && reg_supported(n_fft) && pitch_ok(v) && pitch_ok(dy) && pitch_ok(dv);
+  if (dv && !one_kernel) {                   // a mixer that would be refused below must not leave dg written
+    rc = mixer_check(ctx, dy, reinterpret_cast<const float*>(base), dv, n_fft, mix_bytes ? base + gc_bytes : nullptr, mix_bytes);
+    if (rc != SPECTRE_OK) return rc;
+  }
+  SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (one_kernel)
     return backward_reg(ctx, st, v, dy, g, dv, dg, n_fft, base + gc_bytes + mix_bytes, workspace_bytes - gc_bytes - mix_bytes);
   if (dg) {                                  // first: dv may alias dy, which this reads
     size_t group = (workspace_bytes - gc_bytes - mix_bytes) / (2 * per);

@@ -886,9 +886,13 @@ extern "C" size_t spectre_mixer_workspace_bytes(const spectre_ctx* ctx, int32_t 
   return (size_t)preferred_group(ctx, n_fft, D, B * H) * slab_ws_bytes(n_fft, D);
 }
 
-extern "C" int spectre_mixer_forward(spectre_ctx* ctx, void* stream, const spectre_act* v, const float* g,
-                                     const spectre_act* y, int32_t n_fft, const spectre_wavelet* wrm,
-                                     void* workspace, size_t workspace_bytes) {
+// How a mixer call goes, once everything it could be refused for has been looked at.
+struct MixerRoute {
+  TransformPlan pl;
+  bool tc196, fused, staged, ws_ok, overlap;
+};
+static int mixer_route(const spectre_ctx* ctx, const spectre_act* v, const float* g, const spectre_act* y, int n_fft,
+                       const spectre_wavelet* wrm, const void* workspace, size_t workspace_bytes, MixerRoute* r) {
   if (!ctx) return fail(SPECTRE_ERR_INVALID_ARG, "ctx is NULL");
   int rc = check_act(v, "v");
   if (rc != SPECTRE_OK) return rc;
@@ -898,61 +902,71 @@ extern "C" int spectre_mixer_forward(spectre_ctx* ctx, void* stream, const spect
   if (v->B != y->B || v->L != y->L || v->H != y->H || v->D != y->D || v->dtype != y->dtype)
     return fail(SPECTRE_ERR_INVALID_ARG, "v and y differ in shape or dtype");
   if (n_fft < v->L) return fail(SPECTRE_ERR_INVALID_ARG, "n_fft smaller than L");
-  TransformPlan pl;
-  if (!make_plan(ctx, n_fft, &pl)) return fail(SPECTRE_ERR_UNSUPPORTED, "n_fft outside the supported set");
+  if (!make_plan(ctx, n_fft, &r->pl)) return fail(SPECTRE_ERR_UNSUPPORTED, "n_fft outside the supported set");
   const int force = forced_path();
   const bool tc_ok = (v->dtype == SPECTRE_BF16 || v->dtype == SPECTRE_F16) && ctx->dft64 != nullptr && force != kPathAlu;
-  const bool ws_ok = workspace && !(reinterpret_cast<uintptr_t>(workspace) & 15);
-  const bool tc196 = tc_ok && n_fft == 196 && v->D == 64 && ctx->dft49 != nullptr;
-  const bool fused = tc_ok && force != kPathStaged && ((n_fft == 8192 && tc8192_supported(v, y)) || (n_fft == 4096 && tc4096_supported(v, y)));
-  // n = 8192 that the fused kernel cannot take (no whole 64-row blocks) stays on the fp32 kernels unless forced
-  const bool staged = !fused && tc_ok && force != kPathFused && (n_fft != 8192 || force == kPathStaged) &&
-                      tc4k_supported(n_fft, v->D) && ws_ok &&
-                      workspace_bytes >= tc4k_min_workspace(n_fft, v->D);
-  if (!staged && !fused && pl.N1 > 1) {
-    if (!ws_ok) return fail(SPECTRE_ERR_WORKSPACE, "workspace is NULL or not 16-byte aligned");
+  r->ws_ok = workspace && !(reinterpret_cast<uintptr_t>(workspace) & 15);
+  r->tc196 = tc_ok && n_fft == 196 && v->D == 64 && ctx->dft49 != nullptr;
+  r->fused = tc_ok && force != kPathStaged && ((n_fft == 8192 && tc8192_supported(v, y)) || (n_fft == 4096 && tc4096_supported(v, y)));
+  // n = 8192 that the fused kernel cannot take (no whole 64-row blocks) stays on the fp32 kernels unless forced: its callers
+  // have fp32 values between the stages, and the tensor cores' fp16 ones would be less
+  r->staged = !r->fused && tc_ok && force != kPathFused && (n_fft != 8192 || force == kPathStaged) && tc4k_supported(n_fft, v->D) &&
+              r->ws_ok && workspace_bytes >= tc4k_min_workspace(n_fft, v->D);
+  if (!r->staged && !r->fused && r->pl.N1 > 1) {
+    if (!r->ws_ok) return fail(SPECTRE_ERR_WORKSPACE, "workspace is NULL or not 16-byte aligned");
     if (workspace_bytes < slab_ws_bytes(n_fft, v->D))
       return fail(SPECTRE_ERR_WORKSPACE, "mixer workspace smaller than one (batch, head) slab");
   }
-  bool overlap = false;
-  {
-    // any overlap of the two views' byte extents counts, not only equal base pointers
-    auto extent = [](const spectre_act* a, const char** lo, const char** hi) {
-      const int64_t es = io_elem_bytes(a->dtype);
-      const int64_t last = (a->B - 1) * a->stride_b + (a->L - 1) * a->stride_l + (a->H - 1) * a->stride_h + a->D;
-      *lo = reinterpret_cast<const char*>(a->ptr);
-      *hi = *lo + last * es;
-    };
-    const char *vl, *vh, *yl, *yh;
-    extent(v, &vl, &vh);
-    extent(y, &yl, &yh);
-    overlap = vl < yh && yl < vh;
-    if (overlap && (staged || pl.N1 > 1)) return fail(SPECTRE_ERR_INVALID_ARG, "y may not overlap v on the multi-pass path");
-  }
-  if (wrm) {
-    rc = wavelet_check(ctx, v->L, v->D, wrm);                // a refinement that would be refused behind the mixer
-    if (rc != SPECTRE_OK) return rc;
-  }
+  // any overlap of the two views' byte extents counts, not only equal base pointers
+  auto extent = [](const spectre_act* a, const char** lo, const char** hi) {
+    const int64_t es = io_elem_bytes(a->dtype);
+    const int64_t last = (a->B - 1) * a->stride_b + (a->L - 1) * a->stride_l + (a->H - 1) * a->stride_h + a->D;
+    *lo = reinterpret_cast<const char*>(a->ptr);
+    *hi = *lo + last * es;
+  };
+  const char *vl, *vh, *yl, *yh;
+  extent(v, &vl, &vh);
+  extent(y, &yl, &yh);
+  r->overlap = vl < yh && yl < vh;
+  if (r->overlap && (r->staged || r->pl.N1 > 1)) return fail(SPECTRE_ERR_INVALID_ARG, "y may not overlap v on the multi-pass path");
+  return wrm ? wavelet_check(ctx, v->L, v->D, wrm) : SPECTRE_OK;      // a refinement that would be refused behind the mixer
+}
+
+namespace spectre {
+// What spectre_mixer_forward would refuse, for a caller with work of its own in front of it.
+int mixer_check(const spectre_ctx* ctx, const spectre_act* v, const float* g, const spectre_act* y, int n_fft, const void* workspace,
+                size_t workspace_bytes) {
+  MixerRoute r;
+  return mixer_route(ctx, v, g, y, n_fft, nullptr, workspace, workspace_bytes, &r);
+}
+}  // namespace spectre
+
+extern "C" int spectre_mixer_forward(spectre_ctx* ctx, void* stream, const spectre_act* v, const float* g,
+                                     const spectre_act* y, int32_t n_fft, const spectre_wavelet* wrm,
+                                     void* workspace, size_t workspace_bytes) {
+  MixerRoute r;
+  int rc = mixer_route(ctx, v, g, y, n_fft, wrm, workspace, workspace_bytes, &r);
+  if (rc != SPECTRE_OK) return rc;
   SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (staged || fused || tc196) {
+  if (r.staged || r.fused || r.tc196) {
     // n = 196: the refinement rides in the kernel's store phase when it can
     // (level gates given, 8-byte aligned; or the MLP's weights and room for its output in the workspace)
-    const bool fuse_wrm = tc196 && wrm && tc196_fuses_wavelet(wrm) &&
+    const bool fuse_wrm = r.tc196 && wrm && tc196_fuses_wavelet(wrm) &&
                           (wrm->level_gates ? !(reinterpret_cast<uintptr_t>(wrm->level_gates) & 7)
                                             : (wrm->qbar && wrm->Ww1 && wrm->bw1 && wrm->Ww2 && wrm->bw2 &&
-                                               (wrm->wdtype == SPECTRE_F32 || wrm->wdtype == SPECTRE_BF16) && ws_ok &&
+                                               (wrm->wdtype == SPECTRE_F32 || wrm->wdtype == SPECTRE_BF16) && r.ws_ok &&
                                                workspace_bytes >= tc196_level_gate_bytes(v->B, v->H)));
-    rc = tc196 ? launch_mixer_tc196(ctx, st, v, g, y, fuse_wrm ? wrm : nullptr, reinterpret_cast<float*>(workspace))
-               : (staged ? launch_mixer_tc4k(ctx, st, v, g, y, n_fft, workspace, workspace_bytes)
-                         : (n_fft == 4096 ? launch_mixer_tc4096(ctx, st, v, g, y) : launch_mixer_tc8192(ctx, st, v, g, y)));
+    rc = r.tc196 ? launch_mixer_tc196(ctx, st, v, g, y, fuse_wrm ? wrm : nullptr, reinterpret_cast<float*>(workspace))
+                 : (r.staged ? launch_mixer_tc4k(ctx, st, v, g, y, n_fft, workspace, workspace_bytes)
+                             : (n_fft == 4096 ? launch_mixer_tc4096(ctx, st, v, g, y) : launch_mixer_tc8192(ctx, st, v, g, y)));
     if (rc != SPECTRE_OK) return rc;
     if (wrm && !fuse_wrm) return spectre_wavelet_refine(ctx, stream, y, y, wrm);
     return SPECTRE_OK;
   }
   // n = 4096 and 8192 in place or without a workspace: one kernel, a cluster of CTAs per tile
-  const bool multi = reg_multi(n_fft) && !overlap && ws_ok && workspace_bytes >= slab_ws_bytes(n_fft, v->D);
-  SPECTRE_IO_DISPATCH(v->dtype, rc = mixer_typed<T>(ctx, st, v, g, y, pl, multi, workspace, workspace_bytes));
+  const bool multi = reg_multi(n_fft) && !r.overlap && r.ws_ok && workspace_bytes >= slab_ws_bytes(n_fft, v->D);
+  SPECTRE_IO_DISPATCH(v->dtype, rc = mixer_typed<T>(ctx, st, v, g, y, r.pl, multi, workspace, workspace_bytes));
   if (rc != SPECTRE_OK) return rc;
   if (wrm) return spectre_wavelet_refine(ctx, stream, y, y, wrm);
   return SPECTRE_OK;

@@ -1181,6 +1181,21 @@ def test_a_refused_refinement_leaves_the_tensor_as_it_was(ctx, dt, n, J):
 
 
 # ------------------------------------------------------------------ status word: waits that run out, range
+@pytest.mark.parametrize("dt,n", [("bf16", 16384), ("f32", 16384), ("f16", 65536)])
+def test_a_refused_backward_leaves_the_gradients_as_they_were(ctx, dt, n):
+    # dv over dy where the mixer takes several passes: refused before the gate's gradient is written
+    w = W.Workload("t", B=1, L=n, H=1, D=16, dtype=dt, seed=n)
+    v, dy, g = W.activations(w).cuda(), W.activations(w, stream=1).cuda(), W.random_gate(w).cuda()
+    dg = torch.full_like(g, 7.0)
+    ws = torch.empty(S.spectre_mixer_backward_workspace_bytes(ctx, 1, n, 1, 16, n, S._dtype_code(v)), dtype=torch.uint8, device="cuda")
+    before = dy.clone()
+    with pytest.raises(S.SpectreError) as e:
+        S.prepare_mixer_backward(ctx, v, dy, g, dy, dg, ws, n_fft=n)()
+    torch.cuda.synchronize()
+    assert e.value.status == S.SPECTRE_ERR_INVALID_ARG
+    assert torch.equal(dy, before) and bool((dg == 7.0).all())
+
+
 def test_bounded_wait_that_runs_out_is_reported_once_and_the_context_stays_usable(ctx):
     # a kernel whose wait runs out by construction (barrier nobody arrives on, nothing in flight): the
     # status word is set, the poll reports it once and clears it, and the next real call is correct
