@@ -431,6 +431,10 @@ extern "C" int spectre_prefix_cache_prefill(spectre_ctx* ctx, void* stream, cons
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 15))
     return fail(SPECTRE_ERR_WORKSPACE, "workspace is NULL or not 16-byte aligned");
   if (workspace_bytes < per) return fail(SPECTRE_ERR_WORKSPACE, "prefill workspace smaller than one (batch, head) slab");
+  // limits of the kernels behind the transforms, in front of the first launch
+  if (B > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "B exceeds 65535");
+  const size_t nblocks = (size_t)B * ((N + kRingRows - 1) / kRingRows);
+  if (nblocks > 0x7fffffffu) return fail(SPECTRE_ERR_UNSUPPORTED, "B * N_max too large for the ring copy");
   SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int nslab = B * H, K = N / 2 + 1;
@@ -460,10 +464,8 @@ extern "C" int spectre_prefix_cache_prefill(spectre_ctx* ctx, void* stream, cons
     }
     SPECTRE_LAUNCH_OK("split kernel");
   }
-  const size_t nblocks = (size_t)B * ((N + kRingRows - 1) / kRingRows);
-  if (nblocks > 0x7fffffffu) return fail(SPECTRE_ERR_UNSUPPORTED, "B * N_max too large for the ring copy");
-  unsigned blocks = (unsigned)nblocks;
   if (!v_ring_done) {
+    const unsigned blocks = (unsigned)nblocks;
     SPECTRE_IO_DISPATCH(cache->buf_dtype, {
       SPECTRE_CUDA_OK(launch_after(ring_fill_kernel<T>, blocks, 256, 0, st, reinterpret_cast<const T*>(v->ptr), v->stride_b, v->stride_l,
                                    v->stride_h, reinterpret_cast<T*>(cache->V_buf), B, N, H, D, v->L));

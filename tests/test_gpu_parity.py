@@ -852,6 +852,21 @@ def test_a_refused_decode_step_leaves_the_cache_as_it_was(ctx):
         assert all(torch.equal(getattr(cache, k), b) for k, b in zip(state, before))
 
 
+def test_a_refused_prefill_leaves_the_cache_as_it_was(ctx):
+    # more batch entries than a grid has rows: refused before the transforms write the spectrum
+    B = 65536
+    cache = S.PrefixCache(B, 1, 8, 2, dtype=torch.bfloat16)
+    state = (cache.prefix_fft, cache.V_buf, cache.Q_buf, cache.sum_q)
+    for t in state:
+        t.fill_(7.0)
+    x = torch.ones(B, 1, 1, 8, dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(S.SpectreError) as e:
+        S.spectre_prefix_cache_prefill(ctx, cache, x, x)
+    torch.cuda.synchronize()
+    assert e.value.status == S.SPECTRE_ERR_UNSUPPORTED
+    assert all(bool((t == 7.0).all()) for t in state)
+
+
 def test_decode_step_rejects_bad_rows(ctx):
     N = 64
     w = W.Workload("t", B=1, L=8, H=2, D=16, dtype="f32", wdtype="f32", n_fft=N, seed=2, N_max=N)
