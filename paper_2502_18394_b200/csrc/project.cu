@@ -310,6 +310,13 @@ extern "C" int spectre_project_qv(spectre_ctx* ctx, void* stream, const spectre_
   if ((size_t)x->B * x->H * tiles > (size_t)0x7fffffff) return fail(SPECTRE_ERR_UNSUPPORTED, "too many tiles");
   SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  // in front of the first launch, which clears sum_q: strides that a tensor map cannot describe are refused
+  if (tensor_map_encoder() == nullptr) return fail(SPECTRE_ERR_UNSUPPORTED, "the driver does not provide cuTensorMapEncodeTiled");
+  CUtensorMap tm_x, tm_q, tm_v;
+  rc = make_tile_map(&tm_x, x);
+  if (rc == SPECTRE_OK) rc = make_tile_map(&tm_q, q);
+  if (rc == SPECTRE_OK) rc = make_tile_map(&tm_v, v);
+  if (rc != SPECTRE_OK) return rc;
   bf16* wt = reinterpret_cast<bf16*>(workspace);
   const size_t nsum = sum_q ? (size_t)x->B * x->H * 64 : 0, nw = (size_t)x->H * 128 * 64;
   const unsigned wblocks = (unsigned)(((nsum > nw ? nsum : nw) + 255) / 256);
@@ -320,12 +327,6 @@ extern "C" int spectre_project_qv(spectre_ctx* ctx, void* stream, const spectre_
     SPECTRE_CUDA_OK(launch_after(proj_weights_kernel<float>, wblocks, 256, 0, st, reinterpret_cast<const float*>(Wq),
                                  reinterpret_cast<const float*>(Wv), wt, x->H, sum_q, nsum));
   SPECTRE_LAUNCH_OK("proj_weights_kernel");
-  if (tensor_map_encoder() == nullptr) return fail(SPECTRE_ERR_UNSUPPORTED, "the driver does not provide cuTensorMapEncodeTiled");
-  CUtensorMap tm_x, tm_q, tm_v;
-  rc = make_tile_map(&tm_x, x);
-  if (rc == SPECTRE_OK) rc = make_tile_map(&tm_q, q);
-  if (rc == SPECTRE_OK) rc = make_tile_map(&tm_v, v);
-  if (rc != SPECTRE_OK) return rc;
   ProjPersistParams pp = {wt, sum_q, x->H, tiles, (int)((size_t)x->B * x->H * tiles), ctx->status_dev};
   SPECTRE_CUDA_OK(cudaFuncSetAttribute(project_qv_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPpSmem));
   const int grid = pp.nitems < ctx->sm_count ? pp.nitems : ctx->sm_count;

@@ -911,6 +911,19 @@ def test_project_qv(ctx, B, L, H, wdt):
     assert rel_err(gate_to_complex(g1), gate_to_complex(g2)) < 2e-2
 
 
+def test_a_refused_projection_leaves_the_query_sum_as_it_was(ctx):
+    # a batch stride that no tensor map describes (the batch has one entry, so any stride is a valid tensor)
+    x = torch.ones(1, 200, 2, 64, dtype=torch.bfloat16, device="cuda").as_strided((1, 200, 2, 64), (1 << 40, 128, 64, 1))
+    w = torch.ones(2, 64, 64, device="cuda")
+    q, v, s = torch.full((1, 200, 2, 64), 7.0, dtype=x.dtype, device="cuda"), torch.full((1, 200, 2, 64), 7.0, dtype=x.dtype, device="cuda"), \
+        torch.full((1, 2, 64), 7.0, device="cuda")
+    with pytest.raises(S.SpectreError) as e:
+        S.spectre_project_qv(ctx, x, w, w, q=q, v=v, sum_q=s)
+    torch.cuda.synchronize()
+    assert e.value.status == S.SPECTRE_ERR_CUDA
+    assert all(bool((t == 7.0).all()) for t in (q, v, s))
+
+
 @pytest.mark.parametrize("L", [8192, 16384])
 def test_value_projection_commutes_with_the_mixer(ctx, L):
     # Eq. 2-4: the gate is one complex number per (head, bin) and the transforms act along the sequence only,
