@@ -13,7 +13,7 @@
 namespace spectre {
 
 // from mixer.cu
-int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, int n, int slab0, int cnt,
+int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const spectre_act* with, int n, int slab0, int cnt,
                       float2* ws, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done);
 bool transform_supported(const spectre_ctx* ctx, int n);
 size_t transform_slab_bytes(int n, int D);
@@ -260,9 +260,9 @@ extern "C" int spectre_mixer_backward(spectre_ctx* ctx, void* stream, const spec
       const int cnt = nslab - s0 < (int)group ? nslab - s0 : (int)group;
       int N1 = 1, M = n_fft;
       int no_ring = 0;
-      rc = forward_decimated(ctx, st, v, n_fft, s0, cnt, wsV, &N1, &M, 16, nullptr, &no_ring);
+      rc = forward_decimated(ctx, st, v, dy, n_fft, s0, cnt, wsV, &N1, &M, 16, nullptr, &no_ring);
       if (rc != SPECTRE_OK) return rc;
-      rc = forward_decimated(ctx, st, dy, n_fft, s0, cnt, wsG, &N1, &M, 16, nullptr, &no_ring);
+      rc = forward_decimated(ctx, st, dy, v, n_fft, s0, cnt, wsG, &N1, &M, 16, nullptr, &no_ring);
       if (rc != SPECTRE_OK) return rc;
       float2* dgc = reinterpret_cast<float2*>(dg);
       switch (N1) {

@@ -745,10 +745,11 @@ static int mixer_typed(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
 // activations.  The radix-N1 step over n1 (bin k2 + M k1 = sum_n1 W_N1^{n1 k1} W_n^{n1 k2} ws[n1][k2]) is
 // left to the caller, which can fuse it with what follows (N1 <= N1_max, at least 16).  N1 = 1: the spectrum itself.  With `ring`
 // (dense [B][n][H][D], the activations' dtype) the pass also writes the zero-padded input there when its
-// load path can; *ring_done tells the caller whether it did.
-int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, int n, int slab0, int cnt,
+// load path can; *ring_done tells the caller whether it did.  The split depends on the rows' pitch: where the spectra of two tensors
+// meet, `with` is the other one, and both take the split that both can.
+int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const spectre_act* with, int n, int slab0, int cnt,
                       float2* ws, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done) {
-  if ((reg_supported(n) || reg_multi(n)) && reg_strides_ok(v)) {
+  if ((reg_supported(n) || reg_multi(n)) && reg_strides_ok(v) && (!with || reg_strides_ok(with))) {
     RegParams r = reg_params(n, v->H, v->D, v->L);
     reg_source(r, v);
     const int M = n <= 2048 ? n : (n / 1024 <= N1_max ? 1024 : 2048);

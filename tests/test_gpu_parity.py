@@ -997,6 +997,27 @@ def test_mixer_backward(ctx, dt, L, n, D):
     assert torch.equal(only_dg, dg)
 
 
+@pytest.mark.parametrize("dt,n,L,wide", [("bf16", 4096, 100, "v"), ("f32", 4096, 100, "dy"), ("f16", 16384, 130, "dy"), ("f32", 32768, 70, "v"),
+                                         ("f32", 1024, 60, "v"), ("bf16", 8192, 64, "both")])
+def test_mixer_backward_of_tensors_with_unlike_row_pitches(ctx, dt, n, L, wide):
+    # rows further apart than the register transforms address: the other tensor's spectrum takes the same split
+    w = W.Workload("t", B=1, L=L, H=2, D=24, dtype=dt, n_fft=n, seed=n + L)
+    x, dy, g = W.activations(w), W.activations(w, stream=1), W.random_gate(w)
+
+    def rows(t, far):
+        if not far:
+            return t.cuda()
+        pitch = (1 << 18) + 64
+        out = torch.empty(L * pitch, dtype=t.dtype, device="cuda").as_strided(t.shape, (L * pitch, pitch, 24, 1))
+        return out.copy_(t)
+
+    dv, dg = S.spectre_mixer_backward(ctx, rows(x, wide in ("v", "both")), rows(dy, wide in ("dy", "both")), g.cuda(), n_fft=n)
+    torch.cuda.synchronize()
+    rdv, rdg = O.mixer_backward(W.to_f64(x), W.to_f64(dy), gate_to_complex(g), n_fft=n)
+    assert rel_err(gate_to_complex(dg), rdg) < TOL["f32"]
+    assert slab_err(W.to_f64(dv), rdv) < TOL[dt]
+
+
 @pytest.mark.parametrize("dt,n", [("bf16", 8192), ("f16", 4096), ("f32", 4096), ("f32", 90), ("bf16", 1024), ("bf16", 196)])
 def test_mixer_backward_in_place(ctx, dt, n):
     # dv over dy, with the gate's gradient wanted too: one kernel for both and two passes
