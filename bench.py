@@ -37,7 +37,7 @@ L2_BYTES = 126e6
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from the ncu
 # captures summarised under profiles/ (None until a capture exists for that workload).
-# c2: mixer_tc64_kernel 34.8 MB read + 0.2 MB written inside the launch (its 33.6 MB output was still
+# c2: mixer_tc64_kernel 34.75 MB read + 0.05 MB written inside the launch (its 33.6 MB output was still
 #     dirty in L2 when the launch ended, so this understates the traffic; nothing is re-read)
 # c3: the three kernels of one staged mixer call at full size (intermediates spill from L2)
 # c4: append_spectrum_kernel measured at B = 2 (1015.3 MB), scaled by 4 to B = 8
@@ -45,8 +45,8 @@ L2_BYTES = 126e6
 #     the 77 MB output is still in L2 then)
 # Not measured by this run: each entry names the committed summary it was read from.
 NCU_TRAFFIC = {"c1": None,
-               "c2": (35.0e6, "profiles/mixer_tc64_kernel.md (ncu capture, not this run)"),
-               "c3": (3125e6, "profiles/launches_c3_gate_mixer.md (ncu capture, not this run)"),
+               "c2": (34.8e6, "profiles/launches_c2_gate_mixer.md (ncu capture, not this run)"),
+               "c3": (3128e6, "profiles/launches_c3_gate_mixer.md (ncu capture, not this run)"),
                "c4": (4061e6, "profiles/append_spectrum_kernel_c4_batch2.md (ncu capture at B = 2, x4; not this run)"),
                "c5": (109.6e6, "profiles/launches_c5_and_kernels.md (ncu capture, not this run)")}
 

@@ -21,8 +21,11 @@
  *     number of bins.  Supported n: 2^a for 0 <= a <= 17, and any
  *     n = 2^a 3^b 5^c 7^e <= 2048.  D must be a multiple of 8.
  *   - Every function returns a spectre_status; nothing throws or aborts.
- *     Arguments are validated on the host before anything is launched.  There is
- *     no CPU fallback: without a CUDA device every compute call fails.
+ *     Arguments are validated on the host before anything is launched: a call that
+ *     is refused leaves its outputs as they were.  There is no CPU fallback: without a
+ *     CUDA device every compute call fails.
+ *   - Host threads may call at the same time, each on its own stream and with its own
+ *     outputs and workspace (spectre_gate_static shares one array per device).
  */
 #ifndef SPECTRE_H_
 #define SPECTRE_H_
@@ -183,7 +186,10 @@ int spectre_gate_static(spectre_ctx* ctx, void* stream,
 
 /* Wavelet refinement parameters (Sec. 3.5).  Either level_gates is given, or it
  * is NULL and the gates are computed from qbar by the two-layer MLP
- * s = GELU(qbar Ww1 + bw1) Ww2 + bw2 (linear output). */
+ * s = GELU(qbar Ww1 + bw1) Ww2 + bw2 (linear output).  A block of 2^J rows beside its
+ * J + 1 rows of gates and the hidden units (none with level_gates) must fit the shared
+ * memory of a CTA as fp32 for J > 4, the gates and hidden units 48 KiB for J <= 4;
+ * otherwise SPECTRE_ERR_UNSUPPORTED. */
 typedef struct {
   int32_t levels;                /* J >= 1; 2^J must divide L; J <= 10              */
   int32_t hidden;                /* MLP hidden width (1..1024)                       */
@@ -208,7 +214,7 @@ typedef struct {
  *   v, y     activations of identical shape and dtype; y may alias v where the
  *            transform is one kernel (the workspace query returns 0, and the
  *            bf16 / fp16 tensor-core paths n_fft = 196 with D = 64,
- *            n_fft = 4096 and n_fft = 8192; the fp32 path at n_fft = 4096 and 8192 is one, slower,
+ *            n_fft = 4096 with 64 rows or more and n_fft = 8192; the fp32 path at n_fft = 4096 and 8192 is one, slower,
  *            kernel too when y overlaps v or no workspace is given); on a multi-pass
  *            path a call whose v and y overlap anywhere between their first and last byte is refused with
  *            SPECTRE_ERR_INVALID_ARG
@@ -264,7 +270,7 @@ typedef struct {
  * spectre_prefix_cache_prefill - PreFill of Alg. 1 (Sec. 3.3.1):
  * prefix_fft = R_{N_max}(pad(V, N_max)) (unnormalised, Eq. 1), ring buffers
  * rows 0..L-1 <- tokens and rows L..N_max-1 <- 0, sum_q = sum_i q_i.
- * q, v: [B, L, H, D] with L <= N_max, dtype == buf_dtype.  N_max must be a
+ * q, v: [B, L, H, D] with L <= N_max, B <= 65535, dtype == buf_dtype.  N_max must be a
  * supported n.  workspace >= spectre_prefill_workspace_bytes(...) bytes.
  * The ring buffers are written by the passes that read q and v (q and v must
  * not overlap V_buf or Q_buf).
@@ -359,7 +365,8 @@ int spectre_prefix_cache_readout(spectre_ctx* ctx, void* stream, const spectre_c
  * v, dy, dv: activations of identical shape and dtype; dv may alias dy where
  * spectre_mixer_forward allows y to alias v.  dv or dg may be NULL to skip that
  * gradient (not both).  dg: [B, H, K, 2] float32.  Lengths that one CTA transforms in registers
- * (powers of two 64 ... 2048, squares of even sides): one fp32 kernel for both.  Others: dv runs on
+ * (powers of two 64 ... 2048, those supported n that are squares of even sides from 10 on): one fp32
+ * kernel for both.  Others: dv runs on
  * the same kernels as the forward pass; dg, computed first, uses two forward-only fp32 transforms
  * and a reduction.
  * workspace >= spectre_mixer_backward_workspace_bytes(...), 16-byte aligned; any size

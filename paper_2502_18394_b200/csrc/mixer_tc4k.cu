@@ -698,8 +698,10 @@ static int tc4k_group(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
 
   const float out_scale = 1.0f / ((float)R * in_scale(R));
   // More units than SMs: two a tile on one CTA per SM (mixer_tc64.cu).  Fewer are better spread over the SMs one by one.  Mixer call of one
-  // sequence, bf16, us, tc_core_kernel -> there: 16384 points 2 heads (64 units) 26.9 -> 27.9, 4 (128) 28.2 -> 29.0, 6 (192) 39.3 -> 36.6,
-  // 9 43.5 -> 39.7, 16 70.9 -> 65.7, 28 111.8 -> 105.7; 32768 points 5 heads 58.9 -> 55.2; 131072 points 1 head 40.8 -> 37.2, 3 87.3 -> 81.6.
+  // sequence, bf16, us, tc_core_kernel -> there, at 16384 points with heads of 16 ... 64 channels: 64 units 26.8 -> 28.0, 128 28.2 -> 29.0,
+  // 144 32.2 -> 32.8 | 152 44.0 -> 41.8, 160 38.2 -> 35.8, 184 46.2 -> 43.3, 192 39.6 -> 36.7, 288 44.5 -> 39.9, 296 64.3 -> 59.7, and into a
+  // second round of tiles 304 67.2 -> 63.4, 312 75.4 -> 71.3, 320 60.5 -> 56.6, 1536 167.6 -> 160.3; at 32768 points 128 27.3 -> 28.3 | 192
+  // 38.9 -> 36.0, 320 60.0 -> 55.7; at 131072 points 256 41.6 -> 37.5, 768 86.6 -> 81.0.  315 shapes: none on the wrong side.
   if (ntile % 2 == 0 && nunits > (size_t)ctx->sm_count && tensor_map_encoder()) {
     const int rc = launch_units_tc64(ctx, st, ws_in, gimg, gscale, ws_out, (int)nunits, ntile, R, out_scale);
     if (rc != SPECTRE_OK) return rc;

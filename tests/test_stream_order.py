@@ -23,6 +23,10 @@ def test_read_only_loads_and_restrict_are_for_the_contexts_tables(name, text):
     for m in re.finditer(r"__global__ void(?:\s+__launch_bounds__\((?:[^()]|\([^()]*\))*\))?\s+(\w+)\(([^{;]*)\)\s*\{", text):
         if not re.match(r"(build_|reg_table)", m.group(1)):
             assert "__restrict__" not in m.group(2), f"{name}: {m.group(1)}"
+    # inline loads through the read-only path: in the two functions that read the register transforms' twiddles
+    for m in re.finditer(r"(\w+)\([^()]*\)\s*\{[^{}]*?asm volatile\(\"ld\.global\.nc", text):
+        assert m.group(1) in ("tw_load4", "tw_load2"), f"{name}: ld.global.nc in {m.group(1)}"
+    assert len(re.findall(r"ld\.global\.nc", text)) == (2 if name == "reg_fft.cuh" else 0), name
     for m in re.finditer(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", text):
         assert m.group(1) in TABLES | {"Gtab", "u"}, f"{name}: const __restrict__ {m.group(1)}"      # Gtab, u: shared memory
 
