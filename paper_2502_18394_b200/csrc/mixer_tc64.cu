@@ -813,8 +813,9 @@ int launch_mixer_pairs4096(const spectre_ctx* ctx, cudaStream_t st, const spectr
 // Half-width tiles (4 column pairs, mixer_tc4096.cu) or whole ones, whichever the counts of both let expect to be done first.  An SM holds two
 // half tiles at once and takes 21 us for a pair, 13.5 for one that is left alone; it takes 13 for a whole tile, 0.75 more for each
 // chunk of 8 rows of a partial block (the whole tile fetches them one by one) and 0.5 more for tiles that reach beyond D.  The numbers are
-// fitted, in quarters of a microsecond, to 1300 mixer calls of 4 ... 600 heads of 8 ... 128 channels, 64 ... 4096 rows: the choice costs 0.16 per
-// cent of the better kernel's time on average and 7 at most.  Some of them, us, half | whole: 64 channels, whole blocks, 18 heads 15.3 | 16.1,
+// fitted, in quarters of a microsecond, to 1294 mixer calls of 4 ... 600 heads of 8 ... 128 channels, 1024 ... 4096 rows: the choice costs 0.16 per
+// cent of the better kernel's time on average and 7 at most (fewer rows go the same way but for calls of 8 heads and 64 ... 100 rows, 21.0 | 16.0 ...
+// 21.0, where 2 and 18 heads take 16.0 and 15.3).  Some of them, us, half | whole: 64 channels, whole blocks, 18 heads 15.3 | 16.1,
 // 19 heads 20.8 | 16.2, 38 heads 34.7 | 29.2, 64 heads 40.9 | 30.0; 20 rows beyond, 16 heads 15.6 | 18.9, 24 heads 22.0 | 19.2, 48 heads 36.4 | 35.2, 64 heads
 // 42.0 | 35.6; 40 rows, 24 heads 22.1 | 22.3, 48 heads 36.5 | 41.0, 256 heads 161.8 | 138.2; 63 rows, 64 heads 42.4 | 45.9, 256 heads 161.8 | 145.5;
 // 8 channels (a whole tile is half empty), 149 heads 20.7 | 30.5.
