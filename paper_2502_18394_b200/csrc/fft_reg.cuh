@@ -1,5 +1,6 @@
 // DFTs of 2 ... 32 points held in one thread's registers, with every root of unity a compile-time
-// literal and the additions of complex values issued as packed fp32 pairs.
+// literal and the additions of complex values issued as packed fp32 pairs.  A point is one complex value (float2) or those
+// of two independent columns (cx2), whose multiplications are packed as well.
 #pragma once
 #include <utility>
 
@@ -54,38 +55,62 @@ __device__ __forceinline__ float2 psub(float2 a, float2 b) {
   return r;
 }
 
+// The same point of two columns: real parts and imaginary parts each a packed pair.  The FMA pipe takes two cycles for a packed
+// instruction and 1.28 for a scalar one (measured, four warps a scheduler), so products cost 1.6 times less per column than
+// those of a float2, and a swap of real and imaginary parts is a renaming.
+struct __align__(16) cx2 { uint64_t x, y; };
+__device__ __forceinline__ cx2 padd(cx2 a, cx2 b) { return {add2(a.x, b.x), add2(a.y, b.y)}; }
+__device__ __forceinline__ cx2 psub(cx2 a, cx2 b) { return {sub2(a.x, b.x), sub2(a.y, b.y)}; }
+__device__ __forceinline__ cx2 cmul(cx2 a, float2 w) {
+  const uint64_t wx = pk2(w.x, w.x), wy = pk2(w.y, w.y), ny = pk2(-w.y, -w.y);
+  return {fma2(a.y, ny, mul2(a.x, wx)), fma2(a.x, wy, mul2(a.y, wx))};
+}
+__device__ __forceinline__ cx2 cmulc(cx2 a, float2 w) { return cmul(a, make_float2(w.x, -w.y)); }
+
+// real arithmetic on a component of a point: one value or a packed pair
+__device__ __forceinline__ float radd(float a, float b) { return a + b; }
+__device__ __forceinline__ float rsub(float a, float b) { return a - b; }
+__device__ __forceinline__ float rneg(float a) { return -a; }
+__device__ __forceinline__ float rmul(float a, float c) { return a * c; }
+__device__ __forceinline__ float rfma(float a, float c, float b) { return fmaf(a, c, b); }
+__device__ __forceinline__ uint64_t radd(uint64_t a, uint64_t b) { return add2(a, b); }
+__device__ __forceinline__ uint64_t rsub(uint64_t a, uint64_t b) { return sub2(a, b); }
+__device__ __forceinline__ uint64_t rneg(uint64_t a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ uint64_t rmul(uint64_t a, float c) { return mul2(a, pk2(c, c)); }
+__device__ __forceinline__ uint64_t rfma(uint64_t a, float c, uint64_t b) { return fma2(a, pk2(c, c), b); }
+
 // x exp(-j 2 pi J / R); INV conjugates the root
-template <int J, int R, bool INV>
-__device__ __forceinline__ float2 rot(float2 x) {
+template <int J, int R, bool INV, class V>
+__device__ __forceinline__ V rot(V x) {
   constexpr int j = ((J % R) + R) % R;
   if constexpr (j == 0) return x;
-  else if constexpr (2 * j == R) return make_float2(-x.x, -x.y);
+  else if constexpr (2 * j == R) return V{rneg(x.x), rneg(x.y)};
   else if constexpr (4 * j == R || 4 * j == 3 * R) {
-    if constexpr ((4 * j == R) != INV) return make_float2(x.y, -x.x);
-    else return make_float2(-x.y, x.x);
+    if constexpr ((4 * j == R) != INV) return V{x.y, rneg(x.x)};
+    else return V{rneg(x.y), x.x};
   } else if constexpr ((8 * j) % R == 0) {
     constexpr float h = 0.70710678118654752440f;
     constexpr int e = INV ? 8 - 8 * j / R : 8 * j / R;
-    if constexpr (e == 1) return make_float2((x.x + x.y) * h, (x.y - x.x) * h);
-    else if constexpr (e == 3) return make_float2((x.y - x.x) * h, -(x.x + x.y) * h);
-    else if constexpr (e == 5) return make_float2(-(x.x + x.y) * h, (x.x - x.y) * h);
-    else return make_float2((x.x - x.y) * h, (x.x + x.y) * h);
+    if constexpr (e == 1) return V{rmul(radd(x.x, x.y), h), rmul(rsub(x.y, x.x), h)};
+    else if constexpr (e == 3) return V{rmul(rsub(x.y, x.x), h), rmul(radd(x.x, x.y), -h)};
+    else if constexpr (e == 5) return V{rmul(radd(x.x, x.y), -h), rmul(rsub(x.x, x.y), h)};
+    else return V{rmul(rsub(x.x, x.y), h), rmul(radd(x.x, x.y), h)};
   } else {
     constexpr float c = (float)cx_root(j, R, false), s = (float)cx_root(INV ? -j : j, R, true);
-    return make_float2(fmaf(x.x, c, x.y * s), fmaf(x.y, c, -x.x * s));
+    return V{rfma(x.x, c, rmul(x.y, s)), rfma(x.y, c, rmul(x.x, -s))};
   }
 }
 
 // Natural order in and out: X_k = sum_t x_t exp(-j 2 pi k t / R); INV takes the conjugate kernel, no scaling.
 template <int R, bool INV> struct RegDft;
 
-template <int R1, int R2, bool INV>
-__device__ __forceinline__ void reg_ct(float2 (&x)[R1 * R2]) {
+template <int R1, int R2, bool INV, class V>
+__device__ __forceinline__ void reg_ct(V (&x)[R1 * R2]) {
   constexpr int R = R1 * R2;
-  float2 a[R1][R2];
+  V a[R1][R2];
   static_for<R2>([&](auto i2) {
     constexpr int n2 = decltype(i2)::v;
-    float2 t[R1];
+    V t[R1];
 #pragma unroll
     for (int n1 = 0; n1 < R1; ++n1) t[n1] = x[n1 * R2 + n2];
     RegDft<R1, INV>::run(t);
@@ -96,7 +121,7 @@ __device__ __forceinline__ void reg_ct(float2 (&x)[R1 * R2]) {
   });
 #pragma unroll
   for (int k1 = 0; k1 < R1; ++k1) {
-    float2 u[R2];
+    V u[R2];
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) u[n2] = a[k1][n2];
     RegDft<R2, INV>::run(u);
@@ -106,28 +131,29 @@ __device__ __forceinline__ void reg_ct(float2 (&x)[R1 * R2]) {
 }
 
 // Odd R: sums and differences of mirrored inputs halve the multiplications.
-template <int R, bool INV>
-__device__ __forceinline__ void reg_odd(float2 (&x)[R]) {
+template <int R, bool INV, class V>
+__device__ __forceinline__ void reg_odd(V (&x)[R]) {
   constexpr int P = (R - 1) / 2;
-  float2 t[P], d[P], sum = x[0];
+  V t[P], d[P], sum = x[0];
 #pragma unroll
   for (int i = 0; i < P; ++i) {
     t[i] = padd(x[i + 1], x[R - 1 - i]);
     d[i] = psub(x[i + 1], x[R - 1 - i]);
     sum = padd(sum, t[i]);
   }
-  float2 y[R];
+  V y[R];
   y[0] = sum;
   static_for<P>([&](auto ik) {
     constexpr int k = decltype(ik)::v + 1;
-    float2 e = x[0], o = make_float2(0.f, 0.f);
+    V e = x[0], o;
     static_for<P>([&](auto ii) {
       constexpr int i = decltype(ii)::v;
       constexpr float c = (float)cx_root(k * (i + 1), R, false), s = (float)cx_root(k * (i + 1), R, true);
-      e = make_float2(fmaf(t[i].x, c, e.x), fmaf(t[i].y, c, e.y));
-      o = make_float2(fmaf(d[i].x, s, o.x), fmaf(d[i].y, s, o.y));
+      e = V{rfma(t[i].x, c, e.x), rfma(t[i].y, c, e.y)};
+      if constexpr (i == 0) o = V{rmul(d[i].x, s), rmul(d[i].y, s)};
+      else o = V{rfma(d[i].x, s, o.x), rfma(d[i].y, s, o.y)};
     });
-    const float2 jo = make_float2(-o.y, o.x);
+    const V jo{rneg(o.y), o.x};
     y[k] = INV ? padd(e, jo) : psub(e, jo);
     y[R - k] = INV ? psub(e, jo) : padd(e, jo);
   });
@@ -135,28 +161,28 @@ __device__ __forceinline__ void reg_odd(float2 (&x)[R]) {
   for (int k = 0; k < R; ++k) x[k] = y[k];
 }
 
-template <bool INV> struct RegDft<1, INV> { static __device__ __forceinline__ void run(float2 (&)[1]) {} };
+template <bool INV> struct RegDft<1, INV> { template <class V> static __device__ __forceinline__ void run(V (&)[1]) {} };
 template <bool INV> struct RegDft<2, INV> {
-  static __device__ __forceinline__ void run(float2 (&x)[2]) {
-    const float2 a = x[0], b = x[1];
+  template <class V> static __device__ __forceinline__ void run(V (&x)[2]) {
+    const V a = x[0], b = x[1];
     x[0] = padd(a, b);
     x[1] = psub(a, b);
   }
 };
 template <bool INV> struct RegDft<4, INV> {
-  static __device__ __forceinline__ void run(float2 (&x)[4]) {
-    const float2 t0 = padd(x[0], x[2]), t1 = psub(x[0], x[2]), t2 = padd(x[1], x[3]), t3 = psub(x[1], x[3]);
+  template <class V> static __device__ __forceinline__ void run(V (&x)[4]) {
+    const V t0 = padd(x[0], x[2]), t1 = psub(x[0], x[2]), t2 = padd(x[1], x[3]), t3 = psub(x[1], x[3]);
     x[0] = padd(t0, t2);
     x[2] = psub(t0, t2);
-    const float2 lo = make_float2(t1.x + t3.y, t1.y - t3.x), hi = make_float2(t1.x - t3.y, t1.y + t3.x);   // t1 -+ j t3
+    const V lo{radd(t1.x, t3.y), rsub(t1.y, t3.x)}, hi{rsub(t1.x, t3.y), radd(t1.y, t3.x)};   // t1 -+ j t3
     x[1] = INV ? hi : lo;
     x[3] = INV ? lo : hi;
   }
 };
 #define SPECTRE_REG_ODD(R) \
-  template <bool INV> struct RegDft<R, INV> { static __device__ __forceinline__ void run(float2 (&x)[R]) { reg_odd<R, INV>(x); } };
+  template <bool INV> struct RegDft<R, INV> { template <class V> static __device__ __forceinline__ void run(V (&x)[R]) { reg_odd<R, INV>(x); } };
 #define SPECTRE_REG_CT(R, A, B) \
-  template <bool INV> struct RegDft<R, INV> { static __device__ __forceinline__ void run(float2 (&x)[R]) { reg_ct<A, B, INV>(x); } };
+  template <bool INV> struct RegDft<R, INV> { template <class V> static __device__ __forceinline__ void run(V (&x)[R]) { reg_ct<A, B, INV>(x); } };
 SPECTRE_REG_ODD(3)
 SPECTRE_REG_ODD(5)
 SPECTRE_REG_ODD(7)
@@ -195,6 +221,22 @@ template <> struct PairIo<f16> {
   static __device__ __forceinline__ float2 cvt(raw r) { return unpack_h2(r); }
   static __device__ __forceinline__ raw pack(float2 v) { return pack_h2(v.x, v.y); }
   static __device__ __forceinline__ raw zero() { return 0u; }
+};
+
+// a point of PP adjacent column pairs
+template <int PP> struct PointOf;
+template <> struct PointOf<1> {
+  typedef float2 type;
+  static __device__ __forceinline__ float2 from(const float2 (&a)[1]) { return a[0]; }
+  static __device__ __forceinline__ void to(float2 v, float2 (&a)[1]) { a[0] = v; }
+};
+template <> struct PointOf<2> {
+  typedef cx2 type;
+  static __device__ __forceinline__ cx2 from(const float2 (&a)[2]) { return {pk2(a[0].x, a[1].x), pk2(a[0].y, a[1].y)}; }
+  static __device__ __forceinline__ void to(cx2 v, float2 (&a)[2]) {
+    upk2(v.x, a[0].x, a[1].x);
+    upk2(v.y, a[0].y, a[1].y);
+  }
 };
 
 // PP = 1 or 2 adjacent column pairs of a row

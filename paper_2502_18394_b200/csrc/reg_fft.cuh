@@ -55,28 +55,39 @@ template <int E> __device__ __forceinline__ void settle(float2 (&x)[E]) {
 #pragma unroll
   for (int i = 0; i < E; ++i) asm volatile("" : "+f"(x[i].x), "+f"(x[i].y));
 }
+template <int E> __device__ __forceinline__ void settle(cx2 (&x)[E]) {
+#pragma unroll
+  for (int i = 0; i < E; ++i) asm volatile("" : "+l"(x[i].x), "+l"(x[i].y));
+}
 
 enum RegMode { kRegMix = 0, kRegForward = 1, kRegInverse = 2, kRegGrad = 3 };
 
 // n = R1 R2 in two steps (R1 a multiple of R2): j = j1 R2 + j2, k = k1 + R1 k2.  Thread (pair p, m): the R1-point DFT
 // over j1 at j2 = m, then R1 / R2 DFTs of R2 points at k1 = m + R2 u.  Rows of the exchange buffer (k1, j2) lie
 // R2 + 1 apart per k1: an odd pitch keeps the side whose lanes differ in k1 free of bank conflicts.
-template <int R1, int R2, int C_>
+// PP: column pairs per thread, neighbours in a row.  Two of them, packed (cx2), take 28 % fewer instructions and half the threads at the
+// registers of nearly two.  Forward transforms of 16-bit tokens of 1024 points gain by it with three CTAs of 128 threads at 168 registers
+// on an SM (1024 tiles 28.0 -> 25.1 us; prompt of 2 x 20011 of 32768 x 32 heads 928 -> 896, forward and backward of 1 x 8192 x 32
+// 183 -> 178), if the exchange buffer is halved: with three whole ones no L1 is left for the loads in flight (40 us).  Mixer and gradient lose
+// the latency that twice the warps hide (16 x 1024 x 12 bf16 30.1 -> 32.8 and 57.6 -> 64.1 us), and so do fp32 tokens (prompt of
+// 2 x 6000 of 8192 x 8 114 -> 120).
+template <int R1, int R2, int C_, int PP_ = 1>
 struct TwoStep {
-  static constexpr int C = C_, M = R1 * R2, E = R1, S = R2, U = R1 / R2;
+  static constexpr int PP = PP_, C = C_, G = C / PP, M = R1 * R2, E = R1, S = R2, U = R1 / R2;
+  typedef typename PointOf<PP>::type V;
   // mix() runs the steps as a loop over one copy of the DFT.  From 32 points on, straight-line code (four DFTs) waits for
   // instructions: 1024 = 32 x 32 at 12.6 M elements takes 35.9 us in the loop against 38.6 (fp32), 27.3 against 30.1 (bf16).
   // 28 x 28 and smaller ones lose 1 - 10 % to its extra barrier and moves, and so does the gradient (55 -> 58 us), whose loop over
   // three transforms carries more state; the forward transform alone gains nothing.
   static constexpr bool kLoop = R1 == R2 && R1 >= 32;
-  static constexpr int kActive = S * C, kThreads = (kActive + 31) / 32 * 32;
+  static constexpr int kActive = S * G, kThreads = (kActive + 31) / 32 * 32;
   static constexpr int kExch = R1 * (R2 + 1) * C;                   // elements of the exchange buffer
   static constexpr int kGate = M, kTw = 0;                       // twiddles in shared memory: none
   static constexpr int kParts = 1, kRed = C, kRedShift = 0;         // pairs side by side in a warp after the transform
   int p, m;
-  __device__ __forceinline__ explicit TwoStep(int tid) : p(tid % C), m(tid / C) {}
-  __device__ __forceinline__ int pair_in() const { return p; }
-  __device__ __forceinline__ int pair_out() const { return p; }
+  __device__ __forceinline__ explicit TwoStep(int tid) : p(tid % G), m(tid / G) {}
+  __device__ __forceinline__ int pair_in() const { return PP * p; }
+  __device__ __forceinline__ int pair_out() const { return PP * p; }
   __device__ __forceinline__ int part() const { return 0; }
   __device__ __forceinline__ int bin(int i) const { return m + S * (i / R2) + R1 * (i % R2); }
   static __device__ __forceinline__ int gate_slot(int k) { return k; }
@@ -84,20 +95,20 @@ struct TwoStep {
   // before: called in front of the exchange's (first) barrier
   struct Nothing { __device__ __forceinline__ void operator()() const {} };
   template <bool HALF, class Before = Nothing>
-  __device__ __forceinline__ void forward(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before = Before()) const {
+  __device__ __forceinline__ void forward(V (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before = Before()) const {
     RegDft<R1, false>::run(x);
     turn<HALF>(x, buf, tw, act, before);
 #pragma unroll
     for (int u = 0; u < U; ++u) sub<false>(x, u);
   }
-  static __device__ __forceinline__ void swap_parts(float2 (&x)[E]) {
+  static __device__ __forceinline__ void swap_parts(V (&x)[E]) {
 #pragma unroll
-    for (int i = 0; i < E; ++i) x[i] = make_float2(x[i].y, x[i].x);
+    for (int i = 0; i < E; ++i) x[i] = V{x[i].y, x[i].x};
   }
   // kLoop: forward transform, gate(x), inverse transform.  The inverse is the forward one of the values with real and
   // imaginary parts swapped, its exchange the same one, so all four DFTs are one piece of code.
   template <class Before, class Gate>
-  __device__ __forceinline__ void mix(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before, Gate gate) const {
+  __device__ __forceinline__ void mix(V (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before, Gate gate) const {
 #pragma unroll 1
     for (int step = 0; step < 4; ++step) {
       RegDft<R1, false>::run(x);
@@ -113,7 +124,7 @@ struct TwoStep {
     swap_parts(x);
   }
   template <bool HALF>
-  __device__ __forceinline__ void inverse(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act) const {
+  __device__ __forceinline__ void inverse(V (&x)[E], void* buf, const float4* __restrict__ tw, bool act) const {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       sub<true>(x, u);
@@ -131,7 +142,7 @@ struct TwoStep {
  private:
   // between the steps: twiddles and exchange
   template <bool HALF, class Before>
-  __device__ __forceinline__ void turn(float2 (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before) const {
+  __device__ __forceinline__ void turn(V (&x)[E], void* buf, const float4* __restrict__ tw, bool act, Before before) const {
 #pragma unroll
     for (int a = 0; a < R1 / 2; ++a) {
       const float4 w = tw_load4(tw + a * R1 + m);
@@ -141,8 +152,8 @@ struct TwoStep {
     exchange<HALF, true>(x, buf, act, before);
   }
   template <bool INV>
-  __device__ __forceinline__ void sub(float2 (&x)[E], int u) const {
-    float2 y[R2];
+  __device__ __forceinline__ void sub(V (&x)[E], int u) const {
+    V y[R2];
 #pragma unroll
     for (int i = 0; i < R2; ++i) y[i] = x[u * R2 + i];
     RegDft<R2, INV>::run(y);
@@ -151,14 +162,14 @@ struct TwoStep {
   }
   // element i of the first step's side is (k1 = i, j2 = m), of the second step's (k1 = m + S u, j2 = i % R2)
   __device__ __forceinline__ int at(bool first, int i) const {
-    return first ? (i * (R2 + 1) + m) * C + p : ((m + S * (i / R2)) * (R2 + 1) + i % R2) * C + p;
+    return first ? (i * (R2 + 1) + m) * G + p : ((m + S * (i / R2)) * (R2 + 1) + i % R2) * G + p;
   }
   // FWD: first step's order -> second step's.  The inverse writes the positions this thread read last, so it needs no
   // barrier in front.  HALF: real and imaginary parts one after the other through half the space.
   template <bool HALF, bool FWD, class Before>
-  __device__ __forceinline__ void exchange(float2 (&x)[E], void* buf, bool act, Before before) const {
+  __device__ __forceinline__ void exchange(V (&x)[E], void* buf, bool act, Before before) const {
     if constexpr (!HALF) {
-      float2* b = reinterpret_cast<float2*>(buf);
+      V* b = reinterpret_cast<V*>(buf);
       if (act) {
 #pragma unroll
         for (int i = 0; i < E; ++i) b[at(FWD, i)] = x[i];
@@ -169,7 +180,7 @@ struct TwoStep {
 #pragma unroll
       for (int i = 0; i < E; ++i) x[i] = b[at(!FWD, i)];
     } else {
-      float* b = reinterpret_cast<float*>(buf);
+      decltype(V::x)* b = reinterpret_cast<decltype(V::x)*>(buf);
       if (act) {
 #pragma unroll
         for (int i = 0; i < E; ++i) b[at(FWD, i)] = x[i].x;
@@ -200,7 +211,8 @@ struct TwoStep {
 // with f(jb) and f(ja)), so that all four access patterns are free of bank conflicts.
 template <int C_>
 struct ThreeStep2048 {
-  static constexpr int C = C_, M = 2048, E = 32, S = 64, PW = C / 4;
+  typedef float2 V;
+  static constexpr int PP = 1, C = C_, M = 2048, E = 32, S = 64, PW = C / 4;
   static constexpr bool kLoop = false;
   static constexpr int kActive = S * C, kThreads = kActive;
   static constexpr int kExch = (2048 + 256) * C;
@@ -324,14 +336,15 @@ struct ThreeStep2048 {
 // how many of the rows m, m + step, ... lie below `rows` (0 for an idle thread)
 __device__ __forceinline__ int rows_below(int rows, int m, int step, bool live) { return live && rows > m ? (rows - m + step - 1) / step : 0; }
 
-// Rows m, m + S, ... of the CTA's sequence at this thread's column pair, all loads in flight before the first
+// Rows m, m + S, ... of the CTA's sequence at this thread's column pairs, all loads in flight before the first
 // conversion.  Tokens beyond L are the zero padding; `ring`: they also go, as loaded, into the cache's buffer.
 // The base of every row is uniform over the CTA and the thread's part one 32-bit offset, so that a load takes no
 // address arithmetic of its own; whole tiles take no predicates either.
 template <typename T, class P, int MODE>
-__device__ __forceinline__ void reg_load_tokens(float2 (&x)[P::E], const void* src, int64_t sb, int64_t sl, int64_t sh,
+__device__ __forceinline__ void reg_load_tokens(typename P::V (&x)[P::E], const void* src, int64_t sb, int64_t sl, int64_t sh,
                                                 const RegParams& p, int b, int h, int k1, int col, int m, bool live) {
-  typedef typename PairIo<T>::raw raw;
+  typedef ColumnGroup<T, P::PP> IO;
+  typedef typename IO::raw raw;
   const int step = MODE == kRegForward && p.decim ? p.N1 : 1, off = MODE == kRegForward && p.decim ? k1 : 0;
   const char* base = reinterpret_cast<const char*>(reinterpret_cast<const T*>(src) + b * sb + (int64_t)off * sl + h * sh);
   const int64_t ds = (int64_t)(P::S * step) * sl * (int64_t)sizeof(T);
@@ -344,7 +357,7 @@ __device__ __forceinline__ void reg_load_tokens(float2 (&x)[P::E], const void* s
   } else {
 #pragma unroll
     for (int i = 0; i < P::E; ++i) {
-      v[i] = PairIo<T>::zero();
+      v[i] = IO::zero();
       if (i < count) v[i] = *reinterpret_cast<const raw*>(base + i * ds + mine);
     }
   }
@@ -355,7 +368,11 @@ __device__ __forceinline__ void reg_load_tokens(float2 (&x)[P::E], const void* s
     for (int i = 0; i < P::E; ++i) __stcs(reinterpret_cast<raw*>(out + i * dr), v[i]);
   }
 #pragma unroll
-  for (int i = 0; i < P::E; ++i) x[i] = PairIo<T>::cvt(v[i]);
+  for (int i = 0; i < P::E; ++i) {
+    float2 t[P::PP];
+    IO::cvt(v[i], t);
+    x[i] = PointOf<P::PP>::from(t);
+  }
 }
 
 template <class P>
@@ -402,12 +419,14 @@ __device__ __forceinline__ float2 reduce_scatter(float2 (&q)[RL], int s) {
   return q[0];
 }
 
-// 128 registers a thread for 20 and more points; fewer points leave room for more CTAs
+// 128 registers a thread for 20 and more points (168 for twice 32); fewer points leave room for more CTAs
 template <class P> constexpr int reg_min_blocks() {
-  constexpr int r = P::E > 16 ? 512 : 768, b = r / P::kThreads;
+  constexpr int r = P::PP == 2 ? 384 : (P::E > 16 ? 512 : 768), b = r / P::kThreads;
   return b < 1 ? 1 : (b > 16 ? 16 : b);
 }
-template <class P, int MODE> __host__ __device__ constexpr size_t reg_exch_bytes() { return ((size_t)P::kExch * (MODE == kRegGrad ? 4 : 8) + 15) / 16 * 16; }
+// real and imaginary parts one after the other through half the exchange buffer
+template <class P, int MODE> __host__ __device__ constexpr bool reg_half() { return MODE == kRegGrad || P::PP == 2; }
+template <class P, int MODE> __host__ __device__ constexpr size_t reg_exch_bytes() { return ((size_t)P::kExch * (reg_half<P, MODE>() ? 4 : 8) + 15) / 16 * 16; }
 template <class P, int MODE> __host__ __device__ constexpr bool reg_tw_shared() { return P::kTw != 0 && (MODE == kRegMix || MODE == kRegGrad); }
 template <class P, int MODE> __host__ __device__ constexpr size_t reg_smem_bytes() {
   return reg_exch_bytes<P, MODE>() + (MODE == kRegGrad ? (size_t)P::E * P::kThreads * 8 : 0) + (MODE == kRegMix ? (size_t)P::kGate * 8 : 0) +
@@ -425,7 +444,8 @@ template <typename T, class P, int MODE, bool WS>
 __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(const __grid_constant__ RegParams p) {
   extern __shared__ __align__(16) unsigned char reg_smem[];
   constexpr int E = P::E;
-  constexpr bool HALF = MODE == kRegGrad;
+  constexpr bool HALF = reg_half<P, MODE>();
+  static_assert(P::PP == 1 || (MODE == kRegForward && !WS), "two pairs a thread: forward transforms of tokens");
   void* buf = reg_smem;
   float2* extra = reinterpret_cast<float2*>(reg_smem + reg_exch_bytes<P, MODE>());     // gate table, or the parked spectrum
   const bool act = threadIdx.x < P::kActive;
@@ -455,7 +475,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
   // a programmatic dependent of the kernel before it: the set-up overlaps that kernel's end, nothing is read earlier
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  float2 x[E];
+  typename P::V x[E];
   if constexpr (MODE != kRegInverse) {
     if constexpr (WS) reg_load_ws<P>(x, p.ws + wrow * half, half, pl.m, live ? pin : 0);
     else reg_load_tokens<T, P, MODE>(x, p.src, p.s_sb, p.s_sl, p.s_sh, p, b, h, k1, 2 * pin, pl.m, live);
@@ -469,7 +489,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
       extra[P::gate_slot(i)] = v;
     }
   }
-  auto gate = [&](float2 (&z)[E]) {                        // the gate table is complete: the exchange had a barrier
+  auto gate = [&](typename P::V (&z)[E]) {                 // the gate table is complete: the exchange had a barrier
 #pragma unroll
     for (int i = 0; i < E; ++i) {
       z[i] = cmul(z[i], extra[P::gate_slot(pl.bin(i))]);
@@ -488,7 +508,11 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
     float2* out = p.ws + wrow * half + pout;
     if (live_out) {
 #pragma unroll
-      for (int i = 0; i < E; ++i) out[(size_t)pl.bin(i) * half] = x[i];
+      for (int i = 0; i < E; ++i) {
+        float2 t[P::PP];
+        PointOf<P::PP>::to(x[i], t);
+        ColumnGroup<float, P::PP>::store(reinterpret_cast<float*>(out + (size_t)pl.bin(i) * half), t);
+      }
     }
     return;
   }
@@ -540,7 +564,8 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
     pl.template inverse<HALF>(x, buf, tw, act);
   }
   if (!live) return;
-  if constexpr (WS) {
+  if constexpr (MODE == kRegForward) {                     // stored above
+  } else if constexpr (WS) {
     char* base = reinterpret_cast<char*>(p.ws + wrow * half);
     const uint32_t mine = (uint32_t)(pl.m * half + pin) * 8u;
 #pragma unroll
@@ -707,6 +732,9 @@ constexpr int kRegPairs = 8;
 // twice the SMs (up to 16 heads of one sequence: n = 1024 7.5 -> 6.1 us, 2048 15.0 -> 10.1; 512 and less are slower, 5.2 -> 5.4,
 // and with 2 pairs 1024 is too, 8.0).
 
+// column pairs per thread (see TwoStep)
+template <typename T, int MODE, int M> constexpr int reg_pp() { return sizeof(T) == 2 && MODE == kRegForward && M == 1024 ? 2 : 1; }
+
 template <typename T, int MODE>
 static int reg_launch_tokens(const spectre_ctx* ctx, const RegParams& q, int M, int nslab, cudaStream_t st) {
   constexpr int C = kRegPairs;
@@ -724,7 +752,7 @@ static int reg_launch_tokens(const spectre_ctx* ctx, const RegParams& q, int M, 
     if constexpr (MODE == kRegMix && R1 == 32 && R2 == 32) {                                         \
       if (2 * tiles <= ctx->sm_count) return reg_launch<T, TwoStep<R1, R2, 4>, MODE, false>(p, nslab, st); \
     }                                                                                                \
-    return reg_launch<T, TwoStep<R1, R2, C>, MODE, false>(p, nslab, st);
+    return reg_launch<T, TwoStep<R1, R2, C, reg_pp<T, MODE, R1 * R2>()>, MODE, false>(p, nslab, st);
   const long long tiles = (long long)nslab * ((p.D / 2 + C - 1) / C);
   switch (M) {
     SPECTRE_REG_TWO_STEP(SPECTRE_REG_CASE)

@@ -669,6 +669,21 @@ def test_cache_prefill_long_windows(ctx, dt, N, L, D):
     assert np.array_equal(W.to_f64(cache.V_buf), st["V_buf"]) and np.array_equal(W.to_f64(cache.Q_buf), st["Q_buf"])
 
 
+@pytest.mark.parametrize("dt,N,L,D", [("bf16", 1024, 1, 8), ("f16", 1024, 1023, 24), ("bf16", 2048, 1025, 24), ("f16", 2048, 2048, 64),
+                                       ("f32", 2048, 2047, 40), ("bf16", 4096, 2, 40)])
+def test_cache_prefill_of_partial_tiles(ctx, dt, N, L, D):
+    # 1024 rows per CTA, two column pairs a thread (16-bit tokens); the last tile of 8 pairs is half empty unless D divides by 16
+    w = W.Workload("t", B=2, L=L, H=3, D=D, dtype=dt, seed=N + L + D, N_max=N)
+    q, v = W.activations(w, stream=1), W.activations(w, stream=2)
+    cache = S.PrefixCache(w.B, w.H, w.D, N, dtype=W.torch_dtype(dt))
+    cache.V_buf.fill_(7.0); cache.Q_buf.fill_(7.0); cache.prefix_fft.fill_(7.0); cache.sum_q.fill_(7.0)
+    S.spectre_prefix_cache_prefill(ctx, cache, q.cuda(), v.cuda())
+    st = O.cache_prefill(W.to_f64(q), W.to_f64(v), N)
+    e_p, e_s = cache_err(cache, st)
+    assert e_p < TOL["f32"] and e_s < TOL["f32"], (e_p, e_s)
+    assert np.array_equal(W.to_f64(cache.V_buf), st["V_buf"]) and np.array_equal(W.to_f64(cache.Q_buf), st["Q_buf"])
+
+
 @pytest.mark.parametrize("dt,N,D", [("bf16", 8192, 32), ("f32", 1024, 16)])
 def test_cache_prefill_workspace_grouping(ctx, dt, N, D):
     # a smaller workspace only changes how many (batch, head) slabs go through the transforms together
