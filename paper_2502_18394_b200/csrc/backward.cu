@@ -2,8 +2,8 @@
 // asks for differentiability).  With Vhat = R_n(pad V), Ghat = R_n(pad dY):
 //   dV   = R_n^{-1}( conj(g) Ghat )              -> the forward mixer on dY with the conjugate gate
 //   dg_k = (w_k / n) sum_c conj(Vhat_{k,c}) Ghat_{k,c},   w_0 = w_{n/2} = 1, else 2
-// The gate gradient needs both spectra at once: two forward-only passes of the fp32 transform
-// kernels into the workspace (pair-packed columns, Z = fft(a + jb)), then one reduction over the
+// The gate gradient needs both spectra at once: a forward-only pass of the fp32 transform
+// kernels over either tensor into the workspace (pair-packed columns, Z = fft(a + jb)), then one reduction over the
 // column pairs that uses  conj(A^V) A^G + conj(B^V) B^G = ( conj(Z^V_k) Z^G_k + Z^V_{n-k} conj(Z^G_{n-k}) ) / 2.
 // Beyond one CTA's 2048 rows the passes leave the spectra of the N1 decimated sequences and the reduction
 // runs the last radix-N1 step itself.
@@ -14,7 +14,7 @@ namespace spectre {
 
 // from mixer.cu
 int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const spectre_act* with, int n, int slab0, int cnt,
-                      float2* ws, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done);
+                      float2* ws, float2* ws_with, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done);
 bool transform_supported(const spectre_ctx* ctx, int n);
 size_t transform_slab_bytes(int n, int D);
 int mixer_check(const spectre_ctx* ctx, const spectre_act* v, const float* g, const spectre_act* y, int n_fft, const void* workspace,
@@ -260,9 +260,7 @@ extern "C" int spectre_mixer_backward(spectre_ctx* ctx, void* stream, const spec
       const int cnt = nslab - s0 < (int)group ? nslab - s0 : (int)group;
       int N1 = 1, M = n_fft;
       int no_ring = 0;
-      rc = forward_decimated(ctx, st, v, dy, n_fft, s0, cnt, wsV, &N1, &M, 16, nullptr, &no_ring);
-      if (rc != SPECTRE_OK) return rc;
-      rc = forward_decimated(ctx, st, dy, v, n_fft, s0, cnt, wsG, &N1, &M, 16, nullptr, &no_ring);
+      rc = forward_decimated(ctx, st, v, dy, n_fft, s0, cnt, wsV, wsG, &N1, &M, 16, nullptr, &no_ring);
       if (rc != SPECTRE_OK) return rc;
       float2* dgc = reinterpret_cast<float2*>(dg);
       switch (N1) {

@@ -6,7 +6,7 @@ namespace spectre {
 
 // from mixer.cu / gate.cu
 int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const spectre_act* with, int n, int slab0, int cnt,
-                      float2* ws, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done);
+                      float2* ws, float2* ws_with, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done);
 bool transform_supported(const spectre_ctx* ctx, int n);
 size_t transform_slab_bytes(int n, int D);
 int pool_sum_ring(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* q, float* sums, void* ring, int N);
@@ -447,7 +447,7 @@ extern "C" int spectre_prefix_cache_prefill(spectre_ctx* ctx, void* stream, cons
   for (int s0 = 0; s0 < nslab; s0 += group) {
     int cnt = nslab - s0 < group ? nslab - s0 : group;
     int N1 = 1, M = N;
-    rc = forward_decimated(ctx, st, v, nullptr, N, s0, cnt, ws, &N1, &M, 32, cache->V_buf, &v_ring_done);
+    rc = forward_decimated(ctx, st, v, nullptr, N, s0, cnt, ws, nullptr, &N1, &M, 32, cache->V_buf, &v_ring_done);
     if (rc != SPECTRE_OK) return rc;
     switch (N1) {
       case 1: {

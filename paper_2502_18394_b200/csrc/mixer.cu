@@ -745,10 +745,11 @@ static int mixer_typed(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
 // activations.  The radix-N1 step over n1 (bin k2 + M k1 = sum_n1 W_N1^{n1 k1} W_n^{n1 k2} ws[n1][k2]) is
 // left to the caller, which can fuse it with what follows (N1 <= N1_max, at least 16).  N1 = 1: the spectrum itself.  With `ring`
 // (dense [B][n][H][D], the activations' dtype) the pass also writes the zero-padded input there when its
-// load path can; *ring_done tells the caller whether it did.  The split depends on the rows' pitch: where the spectra of two tensors
-// meet, `with` is the other one, and both take the split that both can.
+// load path can; *ring_done tells the caller whether it did.  `with`: a second tensor of the same shape and type, to ws_with.  The split depends
+// on the rows' pitch, and both take the one that both can; one launch for both leaves one last wave that is not full
+// (forward and backward of 4 x 4096 x 8 heads fp32 149.5 -> 145.8 us, of 1 x 8192 x 32 bf16 177.8 -> 177.5).
 int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act* v, const spectre_act* with, int n, int slab0, int cnt,
-                      float2* ws, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done) {
+                      float2* ws, float2* ws_with, int* N1_out, int* M_out, int N1_max, void* ring, int* ring_done) {
   if ((reg_supported(n) || reg_multi(n)) && reg_strides_ok(v) && (!with || reg_strides_ok(with))) {
     RegParams r = reg_params(n, v->H, v->D, v->L);
     reg_source(r, v);
@@ -756,6 +757,10 @@ int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
     // 8 x 1800 x 16 197 -> 173).  fp32 tokens would gain 8 % and lose 0.6 % of their accuracy.
     const int M = n < 2048 || (n == 2048 && v->dtype == SPECTRE_F32) ? n : (n / 1024 <= N1_max ? 1024 : 2048);
     r.N1 = n / M; r.decim = r.N1 > 1; r.ws = ws; r.slab0 = slab0; r.ring = ring;
+    if (with) {
+      r.src2 = with->ptr; r.s2_sb = with->stride_b; r.s2_sl = with->stride_l; r.s2_sh = with->stride_h;
+      r.ws2 = ws_with;
+    }
     *N1_out = r.N1; *M_out = M; *ring_done = ring != nullptr;
     return reg_forward(ctx, st, r, M, cnt, v->dtype);
   }
@@ -769,6 +774,12 @@ int forward_decimated(const spectre_ctx* ctx, cudaStream_t st, const spectre_act
   p.ws = ws; p.mode = 1; p.dst_ws = 1; p.slab0 = slab0;
   p.src_ws = 0; p.decim = pl.N1 > 1;
   *ring_done = 0;
+  int rc = SPECTRE_OK;
+  SPECTRE_IO_DISPATCH(v->dtype, rc = launch_onchip<T>(ctx, p, pl, cnt, st));
+  if (rc != SPECTRE_OK || !with) return rc;
+  p.src = with->ptr;
+  p.s_sb = with->stride_b; p.s_sl = with->stride_l; p.s_sh = with->stride_h;
+  p.ws = ws_with;
   SPECTRE_IO_DISPATCH(v->dtype, return launch_onchip<T>(ctx, p, pl, cnt, st));
 }
 

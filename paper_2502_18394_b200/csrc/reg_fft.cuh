@@ -453,6 +453,8 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
   int u = blockIdx.x;
   const int tile = u % p.ntile; u /= p.ntile;
   const int k1 = u % p.N1; u /= p.N1;
+  const bool second = MODE == kRegForward && p.src2 && u >= p.nslab;              // uniform over the CTA
+  if (second) u -= p.nslab;
   const int slab_local = u, slab = p.slab0 + u;
   const int b = slab / p.H, h = slab - b * p.H;
   const int half = p.D / 2;
@@ -478,7 +480,8 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
   typename P::V x[E];
   if constexpr (MODE != kRegInverse) {
     if constexpr (WS) reg_load_ws<P>(x, p.ws + wrow * half, half, pl.m, live ? pin : 0);
-    else reg_load_tokens<T, P, MODE>(x, p.src, p.s_sb, p.s_sl, p.s_sh, p, b, h, k1, 2 * pin, pl.m, live);
+    else reg_load_tokens<T, P, MODE>(x, second ? p.src2 : p.src, second ? p.s2_sb : p.s_sb, second ? p.s2_sl : p.s_sl,
+                                     second ? p.s2_sh : p.s_sh, p, b, h, k1, 2 * pin, pl.m, live);
   }
   if constexpr (MODE == kRegMix) {
     for (int i = threadIdx.x; i < P::M; i += P::kThreads) {
@@ -505,7 +508,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
     if constexpr (MODE == kRegMix) gate(x);
   }
   if constexpr (MODE == kRegForward) {
-    float2* out = p.ws + wrow * half + pout;
+    float2* out = (second ? p.ws2 : p.ws) + wrow * half + pout;
     if (live_out) {
 #pragma unroll
       for (int i = 0; i < E; ++i) {

@@ -6,9 +6,10 @@ namespace spectre {
 
 struct RegParams {
   const void* src;          // tokens [B, L, H, D]
-  const void* src2;         // second tensor of the gradient
+  const void* src2;         // second tensor: of the gradient; forward: its nslab sequences follow the first one's in the launch (NULL: none)
   void* dst;                // tokens out
   float2* ws;               // complex rows [slab_local][N1][M][D/2]: input and / or output
+  float2* ws2;              // forward: rows of the second tensor
   const float2* g;          // gate [B*H][K]
   const float2* spec;       // half spectra [B*H][K][D] (inverse)
   float2* sums;             // gradient: partial sums [slab_local][parts][n]; NULL: not wanted
@@ -21,7 +22,7 @@ struct RegParams {
   int* status;              // host-mapped status word (bounded waits)
   int N1;                   // outer factor of n = N1 M; a CTA's sequence is k1 of N1
   int decim;                // forward, from tokens: element j of sequence k1 is token N1 j + k1
-  int slab0, ntile;
+  int slab0, ntile, nslab;
   float scale;              // 1/n, folded into the gate
 };
 
@@ -42,7 +43,7 @@ int reg_parts(int M, int D);
 // One launch over nslab slabs (p.tw and p.ntile are filled in); `ws`: rows of the complex workspace (M = kRegWsM)
 // instead of tokens of type dtype.
 int reg_mix(const spectre_ctx* ctx, cudaStream_t st, RegParams p, int M, int nslab, bool ws, int dtype);
-int reg_forward(const spectre_ctx* ctx, cudaStream_t st, RegParams p, int M, int nslab, int dtype);
+int reg_forward(const spectre_ctx* ctx, cudaStream_t st, RegParams p, int M, int nslab, int dtype);   // with src2: of either tensor
 int reg_inverse(const spectre_ctx* ctx, cudaStream_t st, RegParams p, int M, int nslab, bool ws, int dtype);
 int reg_grad(const spectre_ctx* ctx, cudaStream_t st, RegParams p, int M, int nslab, int dtype);
 
