@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) gate_grad_sum_kernel(const float2* sums, 
 }
 
 // One warp per (slab, bin): lanes over the column pairs, both workspaces hold the spectrum itself,
-// ws[slab_local][k][D/2] (transforms that fit one CTA).
+// a sequence per slab (transforms that fit one CTA).
 __global__ void __launch_bounds__(256) gate_grad_kernel(const float2* wsV, const float2* wsG,
                                                         float2* dg, int n, int K, int D, int slab0, int nslab) {
   after_previous();
@@ -60,11 +60,10 @@ __global__ void __launch_bounds__(256) gate_grad_kernel(const float2* wsV, const
   const int k = (int)(wid % K), slab_local = (int)(wid / K);
   const int km = (n - k) % n;
   const int half = D / 2;
-  const size_t rk = ((size_t)slab_local * n + k) * half;
-  const size_t rm = ((size_t)slab_local * n + km) * half;
   float2 acc = make_float2(0.f, 0.f);
   for (int c = lane; c < half; c += 32) {
-    const float2 vk = wsV[rk + c], vm = wsV[rm + c], gk = wsG[rk + c], gm = wsG[rm + c];
+    const size_t rk = ws_at(half, n, (size_t)slab_local, k, c), rm = ws_at(half, n, (size_t)slab_local, km, c);
+    const float2 vk = wsV[rk], vm = wsV[rm], gk = wsG[rk], gm = wsG[rm];
     acc = cadd(acc, cmulc(gk, vk));          // conj(Z^V_k) Z^G_k
     acc = cadd(acc, cmulc(vm, gm));          // Z^V_{n-k} conj(Z^G_{n-k})
   }
@@ -79,7 +78,7 @@ __global__ void __launch_bounds__(256) gate_grad_kernel(const float2* wsV, const
 }
 
 // Longer transforms, n = N1 M with token t = N1 n2 + n1: the workspaces hold Y[n1][k2], the M-point spectra of
-// the N1 decimated sequences (ws[slab_local][n1][k2][D/2]), and Z[k2 + M k1] = sum_n1 W_N1^{n1 k1} W_n^{n1 k2} Y[n1][k2].
+// the N1 decimated sequences (workspace sequence slab_local N1 + n1), and Z[k2 + M k1] = sum_n1 W_N1^{n1 k1} W_n^{n1 k2} Y[n1][k2].
 // A warp per (slab, k2 <= M/2).  Lanes 0-15 form Z of both tensors at k2 + M k1, lanes 16-31 at m2 + M k1, m2 = M - k2: each
 // family holds the mirror bins n - k of the other.  A lane takes two column pairs (16-byte loads), sums
 // S[k1] = conj(Z^V) Z^G over its pairs, the half-warp over its lanes, and dg_k = (w_k / 2n)(S_k + conj(S_{n-k})) takes one
@@ -100,15 +99,15 @@ __global__ void __launch_bounds__(256, N1 <= 8 ? 2 : 1) gate_grad_combine_kernel
   w[0] = make_float2(1.f, 0.f);
 #pragma unroll
   for (int q = 1; q < N1; ++q) w[q] = (q == 1) ? twiddle_fwd((unsigned)mine, (unsigned)n) : cmul(w[q / 2], w[q - q / 2]);
-  const size_t row0 = (size_t)slab_local * N1 * M + mine;
   float2 acc[N1];
 #pragma unroll
   for (int k1 = 0; k1 < N1; ++k1) acc[k1] = make_float2(0.f, 0.f);
   for (int c = 2 * sub; c < half; c += 32) {                   // D is a multiple of 8: whole 16-byte pieces
     float2 v[2][N1], g[2][N1];
+    const size_t first = ws_at(half, M, (size_t)slab_local * N1, mine, c), step = (size_t)M * half;
 #pragma unroll
     for (int n1 = 0; n1 < N1; ++n1) {
-      const size_t at = (row0 + (size_t)n1 * M) * half + c;
+      const size_t at = first + n1 * step;
       const float4 tv = __ldcs(reinterpret_cast<const float4*>(wsV + at)), tg = __ldcs(reinterpret_cast<const float4*>(wsG + at));
       v[0][n1] = make_float2(tv.x, tv.y); v[1][n1] = make_float2(tv.z, tv.w);
       g[0][n1] = make_float2(tg.x, tg.y); g[1][n1] = make_float2(tg.z, tg.w);

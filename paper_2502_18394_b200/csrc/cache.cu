@@ -1,6 +1,6 @@
 // Prefix-FFT cache (Sec. 3.3, Eq. 5, Alg. 1): prefill, per-token append, and the whole decode
 // step with single-row read-out.
-#include "common.cuh"
+#include "reg_fft.h"
 
 namespace spectre {
 
@@ -34,7 +34,7 @@ __device__ __forceinline__ void store_split(float* prefix, size_t slab, int K, i
   *reinterpret_cast<float4*>(prefix + ((slab * K + k) * D + 2 * c) * 2) = out;
 }
 
-// Transforms that fit the on-chip kernel (N1 = 1) leave Z in ws[slab_local][k][D/2].  A thread takes
+// Transforms that fit the on-chip kernel (N1 = 1) leave Z in the workspace, a sequence per slab.  A thread takes
 // kSplitBins consecutive bins of one column pair, all their loads in flight together.
 constexpr int kSplitBins = 4;
 __global__ void __launch_bounds__(256) split_kernel(const float2* ws, float* prefix, int n,
@@ -49,12 +49,14 @@ __global__ void __launch_bounds__(256) split_kernel(const float2* ws, float* pre
   const size_t r = idx / half;
   const int k0 = (int)(r % kblocks) * kSplitBins;
   const int slab_local = (int)(r / kblocks);
+  const float2* col = ws + ws_at(half, n, (size_t)slab_local, 0, c);
+  const int w = ws_width(half, c);
   float2 z[kSplitBins], zm[kSplitBins];
 #pragma unroll
   for (int u = 0; u < kSplitBins; ++u) {
     const int k = min(k0 + u, K - 1), km = (n - k) % n;
-    z[u] = ws[((size_t)slab_local * n + k) * half + c];
-    zm[u] = ws[((size_t)slab_local * n + km) * half + c];
+    z[u] = col[(size_t)k * w];
+    zm[u] = col[(size_t)km * w];
   }
 #pragma unroll
   for (int u = 0; u < kSplitBins; ++u) {
@@ -64,31 +66,33 @@ __global__ void __launch_bounds__(256) split_kernel(const float2* ws, float* pre
 }
 
 // Longer transforms, n = N1 M with token t = N1 n2 + n1: the forward pass leaves the M-point spectra of the
-// N1 decimated sequences, Y[n1][k2] in ws[slab_local][n1][k2][D/2], and the last radix-N1 step runs here,
+// N1 decimated sequences, Y[n1][k2] in workspace sequence slab_local N1 + n1, and the last radix-N1 step runs here,
 //   Z[k2 + M k1] = sum_n1 W_N1^{n1 k1} ( W_n^{n1 k2} Y[n1][k2] ).
 // Z[n - k] for k = k2 + M k1 is Z[(M - k2) + M (N1 - 1 - k1)] (k2 > 0), so the thread that owns k2 and
 // M - k2 of one column pair holds both sides of every Hermitian pair it stores: the bins k2 + M k1 and
 // (M - k2) + M k1 for k1 < N1/2 (and, at k2 = 0, bin n/2); the packed spectrum never goes back to memory.
 template <int N1>
 __global__ void __launch_bounds__(256) combine_split_kernel(const float2* ws, float* prefix, int n,
-                                                            int K, int D, int M, int slab0, int nslab) {
+                                                            int K, int D, int M, int slab0) {
   after_previous();
-  const int half = D / 2;
-  const int nk2 = M / 2 + 1;
-  const size_t total = (size_t)nslab * nk2 * half;
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= total) return;
-  const int c = (int)(idx % half);
-  const size_t r = idx / half;
-  const int k2 = (int)(r % nk2);
-  const int slab_local = (int)(r / nk2);
+  // a CTA: 32 neighbouring k2 of one workspace tile, 2 KB of each sequence and 128 bytes of every row of the result (32 sequences of 64 heads:
+  // 196 us; 8 k2 of the four tiles of a head 206, one k2 a warp 211)
+  const int half = D / 2, ntile = (half + kWsPairs - 1) / kWsPairs;
+  const int nk2 = M / 2 + 1, nq = (nk2 + 31) / 32;
+  const int c = (int)(blockIdx.x % ntile) * kWsPairs + threadIdx.x % kWsPairs;
+  const int r = blockIdx.x / ntile;
+  const int k2 = (r % nq) * 32 + threadIdx.x / kWsPairs;
+  const int slab_local = r / nq;
+  if (c >= half || k2 >= nk2) return;
   const int m2 = (M - k2) % M;
   float2 xa[N1], xb[N1];
+  const float2* col = ws + ws_at(half, M, (size_t)slab_local * N1, 0, c);
+  const size_t step = (size_t)M * half;                         // from one sequence to the next
+  const int w = ws_width(half, c);
 #pragma unroll
   for (int n1 = 0; n1 < N1; ++n1) {
-    const size_t row = ((size_t)slab_local * N1 + n1) * M;
-    xa[n1] = ws[(row + k2) * half + c];
-    xb[n1] = ws[(row + m2) * half + c];
+    xa[n1] = col[n1 * step + (size_t)k2 * w];
+    xb[n1] = col[n1 * step + (size_t)m2 * w];
   }
   const float2 wa1 = twiddle_fwd((unsigned)k2, (unsigned)n), wb1 = twiddle_fwd((unsigned)m2, (unsigned)n);
   float2 wa[N1], wb[N1];
@@ -115,9 +119,8 @@ __global__ void __launch_bounds__(256) combine_split_kernel(const float2* ws, fl
 template <int N1>
 static void launch_combine_split(cudaStream_t st, const float2* ws, float* prefix, int n, int K, int D, int M, int slab0,
                                  int cnt) {
-  const size_t total = (size_t)cnt * (M / 2 + 1) * (D / 2);
-  (void)launch_after(combine_split_kernel<N1>, (unsigned)((total + 255) / 256), 256, 0, st, ws, prefix, n, K, D, M, slab0,
-                     cnt);                                     // the caller asks for the error
+  const size_t blocks = (size_t)cnt * ((M / 2 + 32) / 32) * ((D / 2 + kWsPairs - 1) / kWsPairs);
+  (void)launch_after(combine_split_kernel<N1>, (unsigned)blocks, 256, 0, st, ws, prefix, n, K, D, M, slab0);    // the caller asks for the error
 }
 
 // Ring buffers: rows 0..L-1 <- tokens, rows L..N-1 <- 0 (Alg. 1 PreFill).  A CTA copies kRingRows

@@ -75,7 +75,7 @@ constexpr int kLocalMax = 2048;      // rows of a tile one CTA keeps in shared m
 struct OnchipParams {
   const void* src;       // real [B,L,H,D] tensor (src_ws = 0)
   void* dst;             // real [B,L,H,D] tensor (dst_ws = 0)
-  float2* ws;            // complex workspace [slab_local][N1][M][D/2]
+  float2* ws;            // complex workspace (ws_at), sequences slab_local N1 + k1
   const float2* g;       // gate [B*H][K]
   const float2* spec;    // half spectra [B*H][K][D] (mode 2)
   int64_t s_sb, s_sl, s_sh;
@@ -120,8 +120,7 @@ __device__ __forceinline__ float4 load_elem(const OnchipParams& p, const TileCoo
   int col = tc.tile * 16 + pg * 4;
   if (col >= p.D) return make_float4(0.f, 0.f, 0.f, 0.f);
   if (p.src_ws) {
-    size_t row = ((size_t)tc.slab_local * p.N1 + tc.k1) * p.M + j;
-    return *reinterpret_cast<const float4*>(p.ws + row * (p.D / 2) + col / 2);
+    return *reinterpret_cast<const float4*>(p.ws + ws_at(p.D / 2, p.M, (size_t)tc.slab_local * p.N1 + tc.k1, j, col / 2));
   }
   const int t = p.decim ? j * p.N1 + tc.k1 : j;
   if (t >= p.L) return make_float4(0.f, 0.f, 0.f, 0.f);
@@ -134,8 +133,7 @@ __device__ __forceinline__ void store_elem(const OnchipParams& p, const TileCoor
   int col = tc.tile * 16 + pg * 4;
   if (col >= p.D) return;
   if (p.dst_ws) {
-    size_t row = ((size_t)tc.slab_local * p.N1 + tc.k1) * p.M + j;
-    *reinterpret_cast<float4*>(p.ws + row * (p.D / 2) + col / 2) = v;
+    *reinterpret_cast<float4*>(p.ws + ws_at(p.D / 2, p.M, (size_t)tc.slab_local * p.N1 + tc.k1, j, col / 2)) = v;
     return;
   }
   if (j >= p.L) return;
@@ -480,7 +478,7 @@ __global__ void __launch_bounds__(256) strided_kernel(const StridedParams p) {
   const int slab = p.slab0 + slab_local;
   const int b = slab / p.H, h = slab - b * p.H;
   const int col = pg * 2 * PP;
-  float2* ws = p.ws + ((size_t)slab_local * N1 * p.M + n2) * (p.D / 2) + col / 2;
+  float2* ws = p.ws + ws_at(p.D / 2, p.M, (size_t)slab_local * N1, n2, col / 2);
   const size_t wstep = (size_t)p.M * (p.D / 2);
 
   float2 wq[N1];
@@ -741,7 +739,7 @@ static int mixer_typed(const spectre_ctx* ctx, cudaStream_t st, const spectre_ac
 }
 
 // Forward transforms of the decimated sequences (used by the cache prefill and the gate gradient): with n = N1 M and token
-// t = N1 n2 + n1, ws[slab_local][n1][k2][D/2] = sum_n2 z[N1 n2 + n1] W_M^{n2 k2}, read straight from the
+// t = N1 n2 + n1, workspace row k2 of sequence slab_local N1 + n1 = sum_n2 z[N1 n2 + n1] W_M^{n2 k2}, read straight from the
 // activations.  The radix-N1 step over n1 (bin k2 + M k1 = sum_n1 W_N1^{n1 k1} W_n^{n1 k2} ws[n1][k2]) is
 // left to the caller, which can fuse it with what follows (N1 <= N1_max, at least 16).  N1 = 1: the spectrum itself.  With `ring`
 // (dense [B][n][H][D], the activations' dtype) the pass also writes the zero-padded input there when its

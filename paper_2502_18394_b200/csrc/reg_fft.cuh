@@ -376,12 +376,9 @@ __device__ __forceinline__ void reg_load_tokens(typename P::V (&x)[P::E], const 
 }
 
 template <class P>
-__device__ __forceinline__ void reg_load_ws(float2 (&x)[P::E], const float2* ws, int half, int m, int pair) {
-  // an idle thread reads row m of pair 0 like the others and stores nothing
-  const char* base = reinterpret_cast<const char*>(ws);
-  const uint32_t mine = (uint32_t)(m * half + pair) * 8u;
+__device__ __forceinline__ void reg_load_ws(float2 (&x)[P::E], const float2* row, int w) {
 #pragma unroll
-  for (int i = 0; i < P::E; ++i) x[i] = *reinterpret_cast<const float2*>(base + (size_t)(P::S * i) * half * 8 + mine);
+  for (int i = 0; i < P::E; ++i) x[i] = row[P::S * i * w];
 }
 
 // the rows back, those below L
@@ -460,7 +457,7 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
   const int half = p.D / 2;
   const int pin = tile * P::C + pl.pair_in(), pout = tile * P::C + pl.pair_out();
   const bool live = act && pin < half, live_out = act && pout < half;
-  const size_t wrow = ((size_t)slab_local * p.N1 + k1) * P::M;                    // first workspace row of the sequence
+  const size_t seq = (size_t)slab_local * p.N1 + k1;
   const float2* g = p.g + (size_t)slab * p.K;
   typename std::conditional<P::kTw == 0, const float4*, typename std::conditional<reg_tw_shared<P, MODE>(), TwShared, TwGlobal>::type>::type tw;
   if constexpr (reg_tw_shared<P, MODE>()) {                // the table is the context's: not behind the wait
@@ -479,7 +476,8 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
 
   typename P::V x[E];
   if constexpr (MODE != kRegInverse) {
-    if constexpr (WS) reg_load_ws<P>(x, p.ws + wrow * half, half, pl.m, live ? pin : 0);
+    // an idle thread reads the row of pair 0 like the others and stores nothing
+    if constexpr (WS) reg_load_ws<P>(x, p.ws + ws_at(half, P::M, seq, pl.m, live ? pin : 0), ws_width(half, live ? pin : 0));
     else reg_load_tokens<T, P, MODE>(x, second ? p.src2 : p.src, second ? p.s2_sb : p.s_sb, second ? p.s2_sl : p.s_sl,
                                      second ? p.s2_sh : p.s_sh, p, b, h, k1, 2 * pin, pl.m, live);
   }
@@ -508,13 +506,14 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
     if constexpr (MODE == kRegMix) gate(x);
   }
   if constexpr (MODE == kRegForward) {
-    float2* out = (second ? p.ws2 : p.ws) + wrow * half + pout;
+    float2* out = (second ? p.ws2 : p.ws) + ws_at(half, P::M, seq, 0, pout);
+    const int w = ws_width(half, pout);
     if (live_out) {
 #pragma unroll
       for (int i = 0; i < E; ++i) {
         float2 t[P::PP];
         PointOf<P::PP>::to(x[i], t);
-        ColumnGroup<float, P::PP>::store(reinterpret_cast<float*>(out + (size_t)pl.bin(i) * half), t);
+        ColumnGroup<float, P::PP>::store(reinterpret_cast<float*>(out + pl.bin(i) * w), t);
       }
     }
     return;
@@ -569,10 +568,10 @@ __global__ void __launch_bounds__(P::kThreads, reg_min_blocks<P>()) reg_kernel(c
   if (!live) return;
   if constexpr (MODE == kRegForward) {                     // stored above
   } else if constexpr (WS) {
-    char* base = reinterpret_cast<char*>(p.ws + wrow * half);
-    const uint32_t mine = (uint32_t)(pl.m * half + pin) * 8u;
+    float2* row = p.ws + ws_at(half, P::M, seq, pl.m, pin);
+    const int w = ws_width(half, pin);
 #pragma unroll
-    for (int i = 0; i < E; ++i) *reinterpret_cast<float2*>(base + (size_t)(P::S * i) * half * 8 + mine) = x[i];
+    for (int i = 0; i < E; ++i) row[P::S * i * w] = x[i];
   } else {
     reg_store_tokens<T, P>(x, p, b, h, 2 * pin, pl.m, live);
   }

@@ -4,11 +4,20 @@
 
 namespace spectre {
 
+// The complex workspace of the multi-pass transforms: [sequence][tile of 8 column pairs][M rows][pairs of the tile].  Neighbouring rows
+// of a tile, which a warp stores together, are contiguous; as rows of all D/2 pairs every 64 bytes were a line, and a cycle of the
+// load/store unit, of their own.
+constexpr int kWsPairs = 8;
+__host__ __device__ inline int ws_width(int half, int pair) { const int left = half - (pair & ~(kWsPairs - 1)); return left < kWsPairs ? left : kWsPairs; }
+__host__ __device__ inline size_t ws_at(int half, int M, size_t seq, int row, int pair) {
+  return (seq * half + (pair & ~(kWsPairs - 1))) * M + (size_t)row * ws_width(half, pair) + (pair & (kWsPairs - 1));
+}
+
 struct RegParams {
   const void* src;          // tokens [B, L, H, D]
   const void* src2;         // second tensor: of the gradient; forward: its nslab sequences follow the first one's in the launch (NULL: none)
   void* dst;                // tokens out
-  float2* ws;               // complex rows [slab_local][N1][M][D/2]: input and / or output
+  float2* ws;               // complex rows (ws_at), sequences slab_local N1 + k1: input and / or output
   float2* ws2;              // forward: rows of the second tensor
   const float2* g;          // gate [B*H][K]
   const float2* spec;       // half spectra [B*H][K][D] (inverse)
