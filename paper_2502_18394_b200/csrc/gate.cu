@@ -1102,15 +1102,18 @@ namespace spectre {
 // are written for it, and the fragments of A fill the registers then.  Narrower widths stay on the other kernels, which at 32 are
 // no slower than this one would be at 64 (8 entries x 32 heads x 32768: 43.8 us against 54.0; 8 x 8 x 1024 9.7 : 9.8), but at 48 are
 // (65.6 against 54.0): a form for multiples of 16 would gain there.  4 or 8 entries (5 ... 7 would need two passes over W2 with
-// 4).  With under 256 bins the 8 warps of its CTAs have no chunk each and the narrower CTAs of the other kernels, more of them per
-// SM, are faster (99 bins, 256 entries: 15 us against 16).  It reads a bin's two output biases as one 8-byte word: an array that
+// 4).  Under 256 bins it is the faster one while its CTAs are resident at once (two per SM): layers of 196 points, 12 heads,
+// 37 entries 34.8 -> 26.7 us, 64 57.4 -> 45.8, 190 88.2 -> 83.3, of 256 points 7 x 32 heads 19.9 -> 15.5, of 128 points 24 x 4 19.6 -> 13.3; beyond that the narrower CTAs of the other kernels, more of them per SM, are (256
+// entries with refinement 136.8 against 144.5).  Under 64 bins most of its warps have no chunk.  It reads a bin's two output biases as one 8-byte word: an array that
 // starts at an odd float (part of a flat parameter buffer) goes to the kernels that read single floats.
-static bool gate_on_mma(const spectre_gate_params* gp, int B, int K) {
-  return gp->wdtype == SPECTRE_BF16 && gp->hidden == 64 && K >= 256 && B >= 2 && !(reinterpret_cast<uintptr_t>(gp->b2) & 7);
+static bool gate_on_mma(const spectre_ctx* ctx, const spectre_gate_params* gp, int B, int H, int K) {
+  const long long ctas = (long long)H * (B <= 4 ? 1 : (B + 7) / 8);
+  return gp->wdtype == SPECTRE_BF16 && gp->hidden == 64 && (K >= 256 || (K >= 64 && ctas <= 2 * ctx->sm_count)) && B >= 2 &&
+         !(reinterpret_cast<uintptr_t>(gp->b2) & 7);
 }
 // batch entries per CTA: the weights of a head are fetched once for all of them
-static int gate_entries(const spectre_gate_params* gp, int B, int K) {
-  if (gate_on_mma(gp, B, K)) return B <= 4 ? 4 : 8;
+static int gate_entries(const spectre_ctx* ctx, const spectre_gate_params* gp, int B, int H, int K) {
+  if (gate_on_mma(ctx, gp, B, H, K)) return B <= 4 ? 4 : 8;
   return (gp->hidden > 256 || B < 2) ? 1 : (B < 4 ? 2 : (B < 8 ? 4 : 8));
 }
 
@@ -1138,7 +1141,7 @@ int gate_check(const spectre_ctx* ctx, const spectre_act* q, const float* sum_q,
   } else if (!(inv_count > 0.f)) {
     return fail(SPECTRE_ERR_INVALID_ARG, "inv_count must be positive with sum_q");
   }
-  const int K = n_fft / 2 + 1, BB = gate_entries(gp, B, K);
+  const int K = n_fft / 2 + 1, BB = gate_entries(ctx, gp, B, H, K);
   if ((long long)H * ((B + BB - 1) / BB) > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "H * ceil(B / 8) exceeds 65535");
   if (gp->toeplitz_r > 0 && (long long)B * H > 65535) return fail(SPECTRE_ERR_UNSUPPORTED, "B*H exceeds 65535");
   size_t sums_off, u_off;
@@ -1199,8 +1202,8 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
   mp.g_out = r > 0 ? raw : reinterpret_cast<float2*>(g_out);
   // block sized to the bin count for short transforms (K = 99 does not need 256 threads)
   const int thr_out = K >= 256 ? 256 : ((K + 31) / 32 * 32 < 64 ? 64 : (K + 31) / 32 * 32);
-  const bool mma = gate_on_mma(gp, B, K);
-  const int BB = gate_entries(gp, B, K);
+  const bool mma = gate_on_mma(ctx, gp, B, H, K);
+  const int BB = gate_entries(ctx, gp, B, H, K);
   dim3 grid_out((K + thr_out - 1) / thr_out, (unsigned)(H * ((B + BB - 1) / BB)));
   const bool wb = gp->wdtype == SPECTRE_BF16;
   const size_t w1_bytes = (size_t)D * gp->hidden * (wb ? 2 : 4);
