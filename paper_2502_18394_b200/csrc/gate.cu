@@ -1106,14 +1106,20 @@ namespace spectre {
 // 37 entries 34.8 -> 26.7 us, 64 57.4 -> 45.8, 190 88.2 -> 83.3, of 256 points 7 x 32 heads 19.9 -> 15.5, of 128 points 24 x 4 19.6 -> 13.3; beyond that the narrower CTAs of the other kernels, more of them per SM, are (256
 // entries with refinement 136.8 against 144.5).  Under 64 bins most of its warps have no chunk.  It reads a bin's two output biases as one 8-byte word: an array that
 // starts at an odd float (part of a flat parameter buffer) goes to the kernels that read single floats.
+// Entries per CTA: 8, or 4 (a shorter hidden layer, the weights read more often) while that makes at most a CTA per SM: layers of
+// 256 points, 7 x 32 heads 15.5 -> 15.0 us, 1024 points, 9 x 8 19.7 -> 18.9; against it 64 x 12 heads of 196 points on 192 CTAs 45.8 -> 50.2.
+static int mma_entries(const spectre_ctx* ctx, int B, int H, int K) {
+  return B <= 4 || (long long)H * ((B + 3) / 4) * ((K + 127) / 128) <= ctx->sm_count ? 4 : 8;
+}
 static bool gate_on_mma(const spectre_ctx* ctx, const spectre_gate_params* gp, int B, int H, int K) {
-  const long long ctas = (long long)H * (B <= 4 ? 1 : (B + 7) / 8);
+  const int nb = mma_entries(ctx, B, H, K);
+  const long long ctas = (long long)H * ((B + nb - 1) / nb);
   return gp->wdtype == SPECTRE_BF16 && gp->hidden == 64 && (K >= 256 || (K >= 64 && ctas <= 2 * ctx->sm_count)) && B >= 2 &&
          !(reinterpret_cast<uintptr_t>(gp->b2) & 7);
 }
 // batch entries per CTA: the weights of a head are fetched once for all of them
 static int gate_entries(const spectre_ctx* ctx, const spectre_gate_params* gp, int B, int H, int K) {
-  if (gate_on_mma(ctx, gp, B, H, K)) return B <= 4 ? 4 : 8;
+  if (gate_on_mma(ctx, gp, B, H, K)) return mma_entries(ctx, B, H, K);
   return (gp->hidden > 256 || B < 2) ? 1 : (B < 4 ? 2 : (B < 8 ? 4 : 8));
 }
 

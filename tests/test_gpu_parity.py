@@ -362,9 +362,10 @@ def test_gate_shapes(ctx, B, L, H, D, hid, dt, wdt, n):
 
 
 @pytest.mark.parametrize("B,H,n,r,shifts", [(2, 3, 510, 0, False), (4, 2, 4096, 0, True), (5, 2, 1000, 2, False), (8, 1, 32768, 0, False),
-                                             (17, 2, 512, 0, True)])
+                                             (17, 2, 512, 0, True), (2, 2, 126, 0, False), (9, 3, 128, 1, True), (6, 2, 254, 0, False),
+                                             (150, 2, 510, 0, True)])
 def test_gate_batches_on_tensor_cores(ctx, B, H, n, r, shifts):
-    # 4- and 8-entry groups, the last group ragged, the last chunk of bins overlapping the one before, phases per entry
+    # 4- and 8-entry groups (4 up to a CTA per SM), the last group ragged, 64 bins up to many chunks, the last chunk of bins overlapping the one before, phases per entry
     w = W.Workload("t", B=B, L=33, H=H, D=64, dtype="bf16", n_fft=n, seed=n + B)
     p = W.gate_params(w, modrelu_bias_std=0.01, toeplitz_r=r, bias_std=0.1)
     x = W.activations(w, structured=True)
@@ -394,7 +395,7 @@ def test_gate_parameters_at_odd_floats_of_a_flat_buffer(ctx, B, n, r):
 
 
 @pytest.mark.parametrize("B,n,D,hid,wdt,r,shifts", [(4, 2, 64, 64, "bf16", 0, False), (8, 196, 64, 64, "bf16", 0, True), (13, 64, 24, 32, "f32", 2, False),
-                                                     (9, 254, 64, 40, "bf16", 0, False), (5, 510, 8, 8, "f32", 0, True), (11, 100, 128, 64, "bf16", 1, False)])
+                                                     (9, 254, 64, 40, "bf16", 0, False), (5, 510, 8, 8, "f32", 0, True), (11, 100, 128, 64, "bf16", 1, False), (793, 196, 64, 64, "bf16", 0, False)])
 def test_gate_short_transforms(ctx, B, n, D, hid, wdt, r, shifts):
     # one CTA per head and 4 or 8 entries with all weights staged: two bins up to as many as a block has threads, the last
     # group of entries ragged, inputs of the hidden layer not a multiple of 32, phases per entry
