@@ -15,7 +15,7 @@ int gate_check(const spectre_ctx* ctx, const spectre_act* q, const float* sum_q,
                const spectre_gate_params* gp, int n_fft, const float* g_out, const void* workspace, size_t workspace_bytes);
 int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float* sum_q, int B, int H, int D, float inv_count,
               const spectre_gate_params* gp, int n_fft, const int64_t* shift, int64_t shift_all, float* g_out, float* qbar_out,
-              void* workspace, size_t workspace_bytes, bool early);
+              void* workspace, size_t workspace_bytes, bool early, const GateToken* tok);
 size_t inverse_workspace_bytes(const spectre_ctx* ctx, int n, int D, int nslab);
 int inverse_from_spectrum(const spectre_ctx* ctx, cudaStream_t st, const float* spec, const float* g, const spectre_act* y,
                           int n, void* ws, size_t ws_bytes);
@@ -232,44 +232,24 @@ __global__ void __launch_bounds__(256) append_ring_kernel(T* V_buf, T* Q_buf,
 
 
 // ---- decode step -------------------------------------------------------------
-// Ring buffers and running sum as in the append, plus delta = v_t - v_old in fp32 for the
-// spectrum pass (which then no longer needs the ring buffer).
-template <typename T>
-__global__ void __launch_bounds__(256) decode_ring_kernel(T* V_buf, T* Q_buf,
-                                                          float* sum_q, float* delta,
-                                                          int* done, const T* q_t, const T* v_t, int B, int H, int D, int N, int slot,
-                                                          int evict) {
-  after_previous();                                       // first: the spectrum pass behind the gate reads bins without a wait of its own
-  asm volatile("griddepcontrol.launch_dependents;");      // the gate kernel behind streams weights before it needs sum_q
-  const int total = B * H * D;
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= total) return;
-  if (idx < B * H) done[idx] = 0;                          // the spectrum pass counts a slab's finished blocks here
-  int b = idx / (H * D), hd = idx - b * (H * D);
-  size_t o = ((size_t)b * N + slot) * H * D + hd;
-  const T q = q_t[idx], v = v_t[idx];                      // all loads in front of the stores, which none may pass
-  const float s = sum_q[idx], qo = evict ? io<T>::load1(Q_buf + o) : 0.f, vo = evict ? io<T>::load1(V_buf + o) : 0.f;
-  sum_q[idx] = s + (io<T>::load1(&q) - qo);
-  delta[idx] = io<T>::load1(&v) - vo;
-  Q_buf[o] = q;
-  V_buf[o] = v;
-}
-
 struct DecodeRows { int r[SPECTRE_DECODE_MAX_ROWS]; };
 
 // One pass over the spectrum: P_k += delta exp(-j 2 pi k t / N) (Eq. 5) and, from the updated
-// value, the NR read-out rows  V~[r] = (1/N) sum_k w_k Re(g_k P_k exp(+j 2 pi k r / N)),
+// value, with delta = v_t - v_old, the NR read-out rows  V~[r] = (1/N) sum_k w_k Re(g_k P_k exp(+j 2 pi k r / N)),
 // w_0 = w_{N/2} = 1, else 2 (Sec. 3.3.2 step e at one output index).  A CTA takes 256
 // consecutive bins of one (batch, head), a warp 32 of them: lane l evaluates bin k0 + l's
 // update twiddle and its NR read-out coefficients once, then the warp walks the 32 bins with
 // every lane holding 2 channels.  Row sums are reduced over the CTA and written as one
 // partial per (slab, bin block); the CTA that finishes a slab last adds its partials in a fixed order (a kernel of its
-// own for that took 10 us behind the 650 us pass of 256 x 32k slabs and 2.7 us of a short window's 19).
-// Bound by HBM (16 bytes per bin and channel).  Launched as a programmatic dependent of the gate kernel: the first bins are
-// on their way before the gate is complete (the spectrum itself was written by kernels in front of the ring kernel).
+// own for that took 10 us behind the 650 us pass of 256 x 32k slabs and 2.7 us of a short window's 19).  The same CTA moves
+// the slab's part of ring buffers and running sum on by the token: every other one has read the evicted row then, and the gate in front
+// took the token from where it came (a kernel of its own for it in front of
+// the gate: step of a 4k window 14.1 -> 15.8 us, of two 2k windows 15.2 -> 16.4).
+// Bound by HBM (16 bytes per bin and channel).  Launched as a programmatic dependent of the gate kernel, which waited for the caller's work:
+// the first bins and the token are on their way before the gate is complete.
 template <typename T, int NR>
-__global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, const float* delta, const float2* g, float* partial,
-                                                              int* done, T* y, int H, int D, int N, int K,
+__global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, T* V_buf, T* Q_buf, float* sum_q, const T* q_t, const T* v_t,
+                                                              int slot, int evict, const float2* g, float* partial, int* done, T* y, int H, int D, int N, int K,
                                                               unsigned tm, DecodeRows rows, int nrows, int nblk) {
   __shared__ float red[8][NR][64];
   __shared__ int last;
@@ -289,6 +269,16 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, con
       if (c < half && i0 + u < nb) v[u] = *reinterpret_cast<const float4*>(base + ((size_t)(i0 + u) * D + 2 * c) * 2);
     }
   };
+  const int b = slab / H, h = slab - b * H;
+  const size_t ring = (((size_t)b * N + slot) * H + h) * D;
+  T tok[2], old[2];                            // as loaded, so that nothing waits for them yet
+  auto token = [&](int c) {
+    if (c >= half) return;
+    const T *a = v_t + (size_t)slab * D + 2 * c, *o = evict ? V_buf + ring + 2 * c : a;
+    tok[0] = a[0]; tok[1] = a[1];
+    old[0] = o[0]; old[1] = o[1];
+  };
+  token(lane);
   fetch(0, lane);
   float2 my = make_float2(1.f, 0.f);
   float2 coef[NR];
@@ -301,7 +291,7 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, con
     for (int r = 0; r < NR; ++r)
       coef[r] = cscale(twiddle_fwd((unsigned)(((unsigned long long)k * (unsigned)rows.r[r]) % (unsigned)N), (unsigned)N), wk);
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");      // delta and g
+  asm volatile("griddepcontrol.wait;" ::: "memory");      // g
   if (k < K) {
     const float2 gk = g[(size_t)slab * K + k];
 #pragma unroll
@@ -310,10 +300,11 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, con
   for (int c0 = 0; c0 < half; c0 += 32) {               // uniform trip count: every lane takes part in the shuffles
     const int c = c0 + lane;
     const bool live = c < half;
+    if (c0 > 0) token(c);
     float d0 = 0.f, d1 = 0.f;
     if (live) {
-      d0 = delta[(size_t)slab * D + 2 * c];
-      d1 = delta[(size_t)slab * D + 2 * c + 1];
+      d0 = io<T>::load1(tok) - (evict ? io<T>::load1(old) : 0.f);
+      d1 = io<T>::load1(tok + 1) - (evict ? io<T>::load1(old + 1) : 0.f);
     }
     float acc[NR][2];
 #pragma unroll
@@ -364,7 +355,15 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, con
   __syncthreads();
   if (!last) return;
   __threadfence();
-  const int b = slab / H, h = slab - b * H, part = threadIdx.x & 3;
+  for (int c = threadIdx.x; c < D; c += 256) {              // ring buffers and running sum of this slab
+    const size_t at = (size_t)slab * D + c;
+    const T q = q_t[at], v = v_t[at];                       // all loads in front of the stores, which none may pass
+    const float s = sum_q[at], qo = evict ? io<T>::load1(Q_buf + ring + c) : 0.f;
+    sum_q[at] = s + (io<T>::load1(&q) - qo);
+    Q_buf[ring + c] = q;
+    V_buf[ring + c] = v;
+  }
+  const int part = threadIdx.x & 3;
   for (int o0 = 0; o0 < nrows * D; o0 += 64) {                 // uniform trip count for the shuffles
     const int o = o0 + (int)(threadIdx.x >> 2), r = o / D, c = o - r * D;
     const bool in = o < nrows * D;
@@ -546,7 +545,6 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   const size_t done_bytes = round256((size_t)B * H * sizeof(int));
   const size_t gate_bytes = gate_min_workspace(B, H, D, N, params->toeplitz_r < 0 ? 0 : params->toeplitz_r);
   if (workspace_bytes < delta_bytes + part_bytes + done_bytes + gate_bytes) return fail(SPECTRE_ERR_WORKSPACE, "decode workspace too small");
-  float* delta = reinterpret_cast<float*>(workspace);
   float* partial = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(workspace) + delta_bytes);
   int* done = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes);
   void* gate_ws = reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes + done_bytes;
@@ -557,19 +555,14 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int slot = (int)(t % N);
   const int evict = t >= N ? 1 : 0;
-  // (a)-(b) ring buffers, running sum, delta
-  const unsigned blocks_r = (unsigned)(((size_t)B * H * D + 255) / 256);
-  SPECTRE_IO_DISPATCH(cache->buf_dtype,
-                      SPECTRE_CUDA_OK(launch_after(decode_ring_kernel<T>, blocks_r, 256, 0, st, reinterpret_cast<T*>(cache->V_buf),
-                                                   reinterpret_cast<T*>(cache->Q_buf), cache->sum_q, delta, done,
-                                                   reinterpret_cast<const T*>(q_t), reinterpret_cast<const T*>(v_t), B, H, D, N, slot,
-                                                   evict)));
-  SPECTRE_LAUNCH_OK("decode_ring_kernel");
-  // (c)-(d) gate from the running sum with phase p = t
+  // (c)-(d) gate from the running sum with the token in it, phase p = t
+  const size_t row = (size_t)slot * H * D * io_elem_bytes(cache->buf_dtype);
+  const GateToken tok = {q_t, evict ? static_cast<const char*>(static_cast<const void*>(cache->Q_buf)) + row : nullptr, (size_t)N * H * D,
+                         cache->buf_dtype, done, B * H};
   rc = gate_call(ctx, stream, nullptr, cache->sum_q, B, H, D, 1.0f / (float)N, params, N, nullptr, t, g_out, nullptr, gate_ws,
-                 gate_bytes, true);
+                 gate_bytes, false, &tok);
   if (rc != SPECTRE_OK) return rc;
-  // (b) + (e) one pass over the spectrum
+  // (a), (b), (e) one pass over the spectrum, ring buffers and running sum
   DecodeRows dr;
   for (int i = 0; i < SPECTRE_DECODE_MAX_ROWS; ++i) dr.r[i] = rows[i < nrows ? i : nrows - 1];
   const unsigned blocks_s = (unsigned)((size_t)B * H * nblk);
@@ -585,8 +578,9 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   cfg.numAttrs = 1;
   SPECTRE_IO_DISPATCH(cache->buf_dtype, {
     auto kern = NR == 1 ? decode_spectrum_kernel<T, 1> : (NR == 2 ? decode_spectrum_kernel<T, 2> : decode_spectrum_kernel<T, SPECTRE_DECODE_MAX_ROWS>);
-    SPECTRE_CUDA_OK(launch_kernel(&cfg, kern, cache->prefix_fft, static_cast<const float*>(delta), g2, partial, done,
-                                       reinterpret_cast<T*>(y_rows), H, D, N, K, (unsigned)slot, dr, (int)nrows, nblk));
+    SPECTRE_CUDA_OK(launch_kernel(&cfg, kern, cache->prefix_fft, reinterpret_cast<T*>(cache->V_buf), reinterpret_cast<T*>(cache->Q_buf),
+                                       cache->sum_q, reinterpret_cast<const T*>(q_t), reinterpret_cast<const T*>(v_t), slot, evict, g2, partial,
+                                       done, reinterpret_cast<T*>(y_rows), H, D, N, K, (unsigned)slot, dr, (int)nrows, nblk));
   });
   return SPECTRE_OK;
 }

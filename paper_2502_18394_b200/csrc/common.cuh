@@ -186,6 +186,17 @@ template <> struct io<f16> {
 inline bool is_io_dtype(int d) { return d == SPECTRE_F32 || d == SPECTRE_BF16 || d == SPECTRE_F16; }
 inline int io_elem_bytes(int d) { return d == SPECTRE_F32 ? 4 : 2; }
 
+// A decode step's token on its way into the running query sum: the gate adds q_t - q_old to the sum that it reads, and the step's last
+// kernel does the same to the sum in memory.  q = NULL: the sum is taken as it is.
+struct GateToken {
+  const void* q;            // q_t [B][H][D]
+  const void* old;          // row `slot` of Q_buf, entries old_stride apart; NULL: nothing is evicted
+  size_t old_stride;
+  int dtype;
+  int* clear;               // counters of the kernel behind the gate, nclear of them
+  int nclear;
+};
+
 // ---- constant roots of unity -----------------------------------------------
 // x * exp(-/+ j 2 pi J / R) for compile-time-foldable (J, R); INV conjugates.
 template <bool INV>

@@ -251,14 +251,46 @@ template <typename WT, bool STAGED> __device__ __forceinline__ float wget(const 
   else return wload<WT>(p);
 }
 
-template <typename WT, int NB, bool STAGED>
-__device__ __forceinline__ void descriptor_and_hidden(const float* sums, size_t bstride, int nb, int ncopy,
+// The means of a decode step, with its token in them; every load of a round in flight together
+template <typename T>
+__device__ __forceinline__ void token_means(const GateToken& t, int b0, int h, int H, const float* sums, int nb, float inv_count, int D, float* qbar) {
+  const T *q = static_cast<const T*>(t.q) + ((size_t)b0 * H + h) * D, *o = static_cast<const T*>(t.old) + (size_t)b0 * t.old_stride + (size_t)h * D;
+#pragma unroll 1
+  for (int e0 = threadIdx.x; e0 < nb * D; e0 += 2 * blockDim.x) {
+    float s[2];
+    T a[2], b[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = min(e0 + u * (int)blockDim.x, nb * D - 1), bb = e / D, c = e - bb * D;
+      const size_t at = (size_t)bb * H * D + c;
+      s[u] = sums[at];
+      a[u] = q[at];
+      b[u] = t.old ? o[(size_t)bb * t.old_stride + c] : T(0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = e0 + u * (int)blockDim.x;
+      if (e < nb * D) qbar[e] = (s[u] + ((float)a[u] - (float)b[u])) * inv_count;
+    }
+  }
+}
+__device__ __forceinline__ void token_means(const GateToken& t, int b0, int h, int H, const float* sums, int nb, float inv_count, int D, float* qbar) {
+  if (t.dtype == SPECTRE_F32) token_means<float>(t, b0, h, H, sums, nb, inv_count, D, qbar);
+  else if (t.dtype == SPECTRE_BF16) token_means<bf16>(t, b0, h, H, sums, nb, inv_count, D, qbar);
+  else token_means<f16>(t, b0, h, H, sums, nb, inv_count, D, qbar);
+}
+
+// TOK: the sums may be a decode step's
+template <typename WT, int NB, bool STAGED, bool TOK = true>
+__device__ __forceinline__ void descriptor_and_hidden(const GateToken& tok, int b0, int h, int H, const float* sums, size_t bstride, int nb, int ncopy,
                                                       size_t copy_stride, float inv_count, int D, int hidden,
                                                       const float* gamma, const float* beta,
                                                       float eps, const WT* W1, const float* b1,
                                                       float* qbar, float* u, int ustride) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-  if (NB > 1 && ncopy == 1) {                                // means, one copy: up to 4 channels per thread in flight
+  if (TOK && tok.q) {                                        // a decode step: one copy, and the token
+    token_means(tok, b0, h, H, sums, nb, inv_count, D, qbar);
+  } else if (NB > 1 && ncopy == 1) {                         // means, one copy: up to 4 channels per thread in flight
     for (int e0 = threadIdx.x; e0 < nb * D; e0 += 4 * blockDim.x) {
       float v[4];
 #pragma unroll
@@ -326,54 +358,50 @@ __device__ __forceinline__ void descriptor_and_hidden(const float* sums, size_t 
     __syncthreads();
     return;
   }
-  int groups = (int)blockDim.x / hidden;
-  groups = groups < 1 ? 1 : (groups > nb ? nb : groups);
-  for (int item = threadIdx.x; item < groups * hidden; item += blockDim.x) {
-    const int gi = item / hidden, jj = item - gi * hidden;
-    float acc[NB];                                  // slot s: batch entry gi + s * groups
+  // A thread takes one hidden unit of up to 4 entries, in loops of few instructions: they run once per launch, and straight-line code waits
+  // for itself (layer of 16 x 1024 x 12 heads fp32 58.4 -> 57.0 us).
+  constexpr int kE = NB < 4 ? NB : 4;
+  for (int item = threadIdx.x; item < hidden * ((nb + kE - 1) / kE); item += blockDim.x) {
+    const int e0 = item / hidden * kE, jj = item - item / hidden * hidden;
+    const WT* w = W1 + jj;
+    const float* q = qbar + e0 * D;                 // entries beyond nb: whatever is there, never used
+    float acc[kE];
 #pragma unroll
-    for (int sl = 0; sl < NB; ++sl) acc[sl] = b1[jj];
+    for (int s = 0; s < kE; ++s) acc[s] = b1[jj];
     int c = 0;
-    for (; c + 32 <= D; c += 32) {                  // 32 independent loads in flight
-      float wv[32];
+    if (D % 4 == 0) {                               // rows of q_bar start on 16 bytes: four inputs per broadcast, two per packed sum
+      uint64_t a2[kE];
 #pragma unroll
-      for (int i = 0; i < 32; ++i) wv[i] = wget<WT, STAGED>(W1 + (size_t)(c + i) * hidden + jj);
+      for (int s = 0; s < kE; ++s) a2[s] = pk2(acc[s], 0.f);
+#pragma unroll 2
+      for (; c < D; c += 4) {
+        float wv[4];
 #pragma unroll
-      for (int sl = 0; sl < NB; ++sl) {
-        const int bb = gi + sl * groups;
-        if (bb < nb) {
-          const float* qb = qbar + bb * D + c;
-          if (NB >= 4 && D % 4 == 0) {              // rows of q_bar start on 16 bytes: four inputs per broadcast, two per packed sum
-            uint64_t a2 = pk2(acc[sl], 0.f);
+        for (int i = 0; i < 4; ++i) wv[i] = wget<WT, STAGED>(w + (size_t)(c + i) * hidden);
+        const uint64_t w01 = pk2(wv[0], wv[1]), w23 = pk2(wv[2], wv[3]);
 #pragma unroll
-            for (int i = 0; i < 32; i += 4) {
-              const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(qb + i);
-              a2 = fma2(t.x, pk2(wv[i], wv[i + 1]), a2);
-              a2 = fma2(t.y, pk2(wv[i + 2], wv[i + 3]), a2);
-            }
-            float lo, hi;
-            upk2(a2, lo, hi);
-            acc[sl] = lo + hi;
-          } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) acc[sl] = fmaf(qb[i], wv[i], acc[sl]);
-          }
+        for (int s = 0; s < kE; ++s) {
+          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(q + s * D + c);
+          a2[s] = fma2(t.x, w01, a2[s]);
+          a2[s] = fma2(t.y, w23, a2[s]);
         }
       }
-    }
-    for (; c < D; ++c) {
-      const float wv = wget<WT, STAGED>(W1 + (size_t)c * hidden + jj);
 #pragma unroll
-      for (int sl = 0; sl < NB; ++sl) {
-        const int bb = gi + sl * groups;
-        if (bb < nb) acc[sl] = fmaf(qbar[bb * D + c], wv, acc[sl]);
+      for (int s = 0; s < kE; ++s) {
+        float lo, hi;
+        upk2(a2[s], lo, hi);
+        acc[s] = lo + hi;
       }
     }
+#pragma unroll 1
+    for (; c < D; ++c) {
+      const float wv = wget<WT, STAGED>(w + (size_t)c * hidden);
 #pragma unroll
-    for (int sl = 0; sl < NB; ++sl) {
-      const int bb = gi + sl * groups;
-      if (bb < nb) u[jj * ustride + bb] = gelu_erf(acc[sl]);   // [hidden][ustride]: one row = all batch entries
+      for (int s = 0; s < kE; ++s) acc[s] = fmaf(q[s * D + c], wv, acc[s]);
     }
+#pragma unroll
+    for (int s = 0; s < kE; ++s)
+      if (e0 + s < nb) u[jj * ustride + e0 + s] = gelu_erf(acc[s]);   // [hidden][ustride]: one row = all batch entries
   }
   __syncthreads();
 }
@@ -443,13 +471,17 @@ struct GateMlpParams {
   float* u_ws;            // [B,H,hidden] hidden activations (workspace)
   int post;               // 1: Toeplitz follows, skip modReLU/phase here
   int stage_w1;           // W1, gamma, beta and b1 of a head are copied to shared memory before the wait (size and alignment allow)
+  GateToken tok;
   int early;              // the kernel in front is of the same call and has waited for the caller's work: the weights, which the caller's
                           // last kernel may have written, are read ahead of the wait.  Otherwise the wait comes first
 };
 // In front of the trigger: what triggers before it has waited lets its dependents start beside the caller's kernel too
+template <bool TRIGGER = true>
 __device__ __forceinline__ void gate_start(const GateMlpParams& p) {
   if (!p.early) after_previous();
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (TRIGGER) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (int i = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; i < p.tok.nclear; i += gridDim.x * gridDim.y * blockDim.x)
+    p.tok.clear[i] = 0;
 }
 
 // raw (re, im) weight pair of one bin in one hidden row
@@ -488,10 +520,10 @@ __global__ void __launch_bounds__(256) gate_hidden_kernel(const GateMlpParams p)
   if (p.stage_w1) stage_mlp(W1, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D, p.hidden, w1s);
   asm volatile("griddepcontrol.wait;" ::: "memory");        // the sums come from the kernel before
   if (p.stage_w1)
-    descriptor_and_hidden<WT, BB, true>(p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
+    descriptor_and_hidden<WT, BB, true>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                         p.inv_count, p.D, p.hidden, vec, vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, BB);
   else
-    descriptor_and_hidden<WT, BB, false>(p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
+    descriptor_and_hidden<WT, BB, false>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                          p.inv_count, p.D, p.hidden, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, W1,
                                          p.b1 + h * p.hs_b1, qbar, u, BB);
   for (int e = threadIdx.x; e < nb * p.hidden; e += blockDim.x) {
@@ -569,7 +601,8 @@ __device__ __forceinline__ void gate_stream(typename wraw<WT>::type (&w)[wraw<WT
 
 // PRE: the hidden activations were computed once per (head, batch entry) by gate_hidden_kernel
 // (long transforms: hundreds of CTAs per head would otherwise repeat that work).
-template <typename WT, int BB, bool PRE>
+// TOK: for a decode step; without its loads the other calls' form spills nothing (28 bytes cost the layer of 8192 points 1.3 us of 63.2).
+template <typename WT, int BB, bool PRE, bool TOK>
 __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const GateMlpParams p) {
   extern __shared__ __align__(16) float u[];       // [hidden][BB], then q_bar [BB][D]
   gate_start(p);                                   // a kernel launched behind this one as a programmatic dependent may do its set-up meanwhile
@@ -610,10 +643,10 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
     float* qbar = u + BB * p.hidden;   // [BB][D]
     const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
     if (p.stage_w1)
-      descriptor_and_hidden<WT, BB, true>(p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
+      descriptor_and_hidden<WT, BB, true, TOK>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                           p.inv_count, p.D, p.hidden, vec, vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, BB);
     else
-      descriptor_and_hidden<WT, BB, false>(p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
+      descriptor_and_hidden<WT, BB, false, TOK>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                            p.inv_count, p.D, p.hidden, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, W1,
                                            p.b1 + h * p.hs_b1, qbar, u, BB);
     if (p.qbar_out && blockIdx.x == 0)
@@ -685,10 +718,10 @@ __global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams 
   float* qbar = u + p.hidden;
   const float* sums = p.sums + ((size_t)b * p.H + h) * p.D;
   if (p.stage_w1)
-    descriptor_and_hidden<WT, 1, true>(sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, vec, vec + p.D,
+    descriptor_and_hidden<WT, 1, true>(p.tok, b, h, p.H, sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, vec, vec + p.D,
                                        p.eps, w1s, vec + 2 * p.D, qbar, u, 1);
   else
-    descriptor_and_hidden<WT, 1, false>(sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden,
+    descriptor_and_hidden<WT, 1, false>(p.tok, b, h, p.H, sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden,
                                         p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, W1, p.b1 + h * p.hs_b1, qbar, u, 1);
   if (p.qbar_out && blockIdx.x == 0)
     for (int c = threadIdx.x; c < p.D; c += blockDim.x) p.qbar_out[((size_t)b * p.H + h) * p.D + c] = qbar[c];
@@ -725,10 +758,13 @@ __global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams 
 // One CTA per head and BB entries, one bin per thread.  All of a head's weights go to shared memory (cp.async) ahead of the wait
 // for the sums.  What bounds it is the chain of short phases behind that wait, and in a chain of kernels the first pass over
 // their code: fetched once per SM and launch, so the loops here are rolled up (gate_out_kernel's 32 rows per thread are 600 instructions).
-template <typename WT, int BB>
+// FULL: with phases per entry or a decode step's token, whose code the usual call would have to step over.
+template <typename WT, int BB, bool FULL>
 __global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams p) {
   extern __shared__ __align__(16) float u[];       // [hidden][BB], q_bar [BB][D], W1, gamma, beta, b1, W2
-  gate_start(p);
+  // no trigger: CTAs of the kernel behind would sit beside these and keep the one after it off the SM (layer of 256 x 196 x 12 heads
+  // with refinement 143.5 -> 136.8 us)
+  gate_start<false>(p);
   const int nbg = (p.B + BB - 1) / BB;
   const int h = blockIdx.x / nbg, b0 = (blockIdx.x - h * nbg) * BB;
   const int nb = min(BB, p.B - b0), k = threadIdx.x;
@@ -744,7 +780,7 @@ __global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams 
   const float bias = (!p.post && p.modrelu_bias) ? p.modrelu_bias[h * p.hs_mb + kc] : 0.f;
   asm volatile("griddepcontrol.wait;" ::: "memory");         // the sums come from the kernel before
   float* qbar = u + BB * p.hidden;
-  descriptor_and_hidden<WT, BB, true>(p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
+  descriptor_and_hidden<WT, BB, true, FULL>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                       p.inv_count, p.D, p.hidden, vec, vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, BB);
   if (p.qbar_out)
     for (int e = threadIdx.x; e < nb * p.D; e += blockDim.x) {
@@ -768,7 +804,7 @@ __global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams 
     }
   }
   float2 ph = make_float2(1.f, 0.f);                         // one positional phase for the whole batch unless per-entry shifts are given
-  if (!p.post && !p.shift) ph = phase_reduced(k, p.n, p.pm_all);
+  if (!p.post && !(FULL && p.shift)) ph = phase_reduced(k, p.n, p.pm_all);
 #pragma unroll
   for (int bb = 0; bb < BB; ++bb) {
     if (bb < nb) {
@@ -779,7 +815,7 @@ __global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams 
       float2 a = bb & 1 ? make_float2(x1, y1) : make_float2(x0, y0);
       if (!p.post) {
         if (p.modrelu_bias) a = modrelu(a, bias);
-        if (p.shift) ph = phase_factor(k, p.n, p.shift_all + p.shift[b]);
+        if (FULL && p.shift) ph = phase_factor(k, p.n, p.shift_all + p.shift[b]);
         a = cmul(a, ph);
       }
       p.g_out[((size_t)b * p.H + h) * p.K + k] = a;
@@ -881,11 +917,13 @@ __device__ __forceinline__ void gate_use_chunk(const GateChunk& x, const uint32_
 // 16 x 1024 x 12 heads 105.7 -> 98.9 us, projected layer of 4 x 4096 x 16 73.5 -> 63.5.
 constexpr int kMmaPitch = 72;                      // bf16 elements between rows of As: the fragments' loads meet no bank twice
 template <int NB, bool STAGED>
-__device__ __forceinline__ void mma_hidden(const GateMlpParams& p, const float* sums, int nb, const float* gamma, const float* beta,
+__device__ __forceinline__ void mma_hidden(const GateMlpParams& p, int b0, int h, const float* sums, int nb, const float* gamma, const float* beta,
                                            const float* b1, const bf16* W1, float* qbar, bf16* As) {
   constexpr int kSlots = NB / 4;                   // entries per thread: 4 groups of 64 threads
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, D = p.D;
   const size_t bstride = (size_t)p.H * D;
+  if (p.tok.q) token_means(p.tok, b0, h, p.H, sums, nb, p.inv_count, D, qbar);
+  else
 #pragma unroll 1
   for (int e0 = tid; e0 < nb * D; e0 += 512) {     // means: two channels per thread, all copies in flight at once
     const int e1 = e0 + 256, bb0 = e0 / D, bb1 = e1 / D;
@@ -1001,8 +1039,8 @@ __global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p)
   // everything above reads only weights; the sums / hidden activations come from the kernel before
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const float* sums = p.sums + ((size_t)b0 * p.H + h) * p.D;
-  if (p.stage_w1) mma_hidden<NB, true>(p, sums, nb, vec, vec + p.D, vec + 2 * p.D, w1s, qbar, As);
-  else mma_hidden<NB, false>(p, sums, nb, gamma, beta, b1, reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, qbar, As);
+  if (p.stage_w1) mma_hidden<NB, true>(p, b0, h, sums, nb, vec, vec + p.D, vec + 2 * p.D, w1s, qbar, As);
+  else mma_hidden<NB, false>(p, b0, h, sums, nb, gamma, beta, b1, reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, qbar, As);
   if (p.qbar_out && blockIdx.x == 0)
     for (int e = threadIdx.x; e < nb * p.D; e += blockDim.x) {
       const int bb = e / p.D, c = e - bb * p.D;
@@ -1161,7 +1199,7 @@ int gate_check(const spectre_ctx* ctx, const spectre_act* q, const float* sum_q,
 // spectre_gate; `early`: see GateMlpParams
 int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float* sum_q, int B, int H, int D, float inv_count,
               const spectre_gate_params* gp, int n_fft, const int64_t* shift, int64_t shift_all, float* g_out, float* qbar_out,
-              void* workspace, size_t workspace_bytes, bool early) {
+              void* workspace, size_t workspace_bytes, bool early, const GateToken* tok) {
   int rc = gate_check(ctx, q, sum_q, B, H, D, inv_count, gp, n_fft, g_out, workspace, workspace_bytes);
   if (rc != SPECTRE_OK) return rc;
   if (q && !(inv_count > 0.f)) inv_count = 1.0f / (float)q->L;
@@ -1204,6 +1242,7 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
   mp.u_ws = reinterpret_cast<float*>(reinterpret_cast<char*>(workspace) + u_off);
   mp.post = r > 0;
   mp.early = early;
+  if (tok) mp.tok = *tok;
   float2* raw = r > 0 ? reinterpret_cast<float2*>(workspace) : nullptr;
   mp.g_out = r > 0 ? raw : reinterpret_cast<float2*>(g_out);
   // block sized to the bin count for short transforms (K = 99 does not need 256 threads)
@@ -1259,11 +1298,16 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
     if (pre) {                                                                                   \
       SPECTRE_CUDA_OK(launch_kernel(&cfg_hid, gate_hidden_kernel<WT, NB>, mp));             \
       mp.early = 1;                                                                              \
-      SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, true>, mp));          \
+      mp.tok.nclear = 0;                                                                         \
+      SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, true, false>, mp));          \
     } else {                                                                                     \
-      SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, false>, mp));         \
+      if (mp.tok.q) SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, false, true>, mp)); \
+      else SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, false, false>, mp)); \
     }                                                                                            \
   } while (0)
+#define SPECTRE_GATE_SHORT(WT, FULL)                                                             \
+  SPECTRE_CUDA_OK(BB == 8 ? launch_kernel(&cfg_short, gate_short_kernel<WT, 8, FULL>, mp)        \
+                          : launch_kernel(&cfg_short, gate_short_kernel<WT, 4, FULL>, mp))
 #define SPECTRE_GATE_MMA(NB)                                                                     \
   do {                                                                                           \
     if (mp.shift && !mp.post) SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, true>, mp)); \
@@ -1272,8 +1316,11 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
   if (mma) {
     if (BB == 8) SPECTRE_GATE_MMA(8); else SPECTRE_GATE_MMA(4);
   } else if (all_staged) {
-    if (wb) SPECTRE_CUDA_OK(BB == 8 ? launch_kernel(&cfg_short, gate_short_kernel<bf16, 8>, mp) : launch_kernel(&cfg_short, gate_short_kernel<bf16, 4>, mp));
-    else SPECTRE_CUDA_OK(BB == 8 ? launch_kernel(&cfg_short, gate_short_kernel<float, 8>, mp) : launch_kernel(&cfg_short, gate_short_kernel<float, 4>, mp));
+    if (mp.tok.q || (mp.shift && !mp.post)) {
+      if (wb) SPECTRE_GATE_SHORT(bf16, true); else SPECTRE_GATE_SHORT(float, true);
+    } else {
+      if (wb) SPECTRE_GATE_SHORT(bf16, false); else SPECTRE_GATE_SHORT(float, false);
+    }
   } else if (split) {
     SPECTRE_CUDA_OK(wb ? launch_kernel(&cfg_split, gate_split_kernel<bf16>, mp) : launch_kernel(&cfg_split, gate_split_kernel<float>, mp));
   } else switch (BB) {
@@ -1284,6 +1331,7 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
   }
 #undef SPECTRE_GATE_LAUNCH
 #undef SPECTRE_GATE_MMA
+#undef SPECTRE_GATE_SHORT
   SPECTRE_LAUNCH_OK("gate_out_kernel");
   if (r > 0) {
     GatePostParams pp = {};
@@ -1306,7 +1354,7 @@ extern "C" int spectre_gate(spectre_ctx* ctx, void* stream, const spectre_act* q
                             const int64_t* shift, int64_t shift_all, float* g_out, float* qbar_out, void* workspace,
                             size_t workspace_bytes) {
   return gate_call(ctx, stream, q, sum_q, B, H, D, inv_count, gp, n_fft, shift, shift_all, g_out, qbar_out, workspace, workspace_bytes,
-                   q != nullptr);
+                   q != nullptr, nullptr);
 }
 
 // ---- gate without any caller- or library-side allocation -----------------------
