@@ -476,12 +476,13 @@ struct GateMlpParams {
                           // last kernel may have written, are read ahead of the wait.  Otherwise the wait comes first
 };
 // In front of the trigger: what triggers before it has waited lets its dependents start beside the caller's kernel too
-template <bool TRIGGER = true>
+template <bool TRIGGER = true, bool TOK = true>
 __device__ __forceinline__ void gate_start(const GateMlpParams& p) {
   if (!p.early) after_previous();
   if (TRIGGER) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  for (int i = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; i < p.tok.nclear; i += gridDim.x * gridDim.y * blockDim.x)
-    p.tok.clear[i] = 0;
+  if (TOK)
+    for (int i = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; i < p.tok.nclear; i += gridDim.x * gridDim.y * blockDim.x)
+      p.tok.clear[i] = 0;
 }
 
 // raw (re, im) weight pair of one bin in one hidden row
@@ -916,13 +917,13 @@ __device__ __forceinline__ void gate_use_chunk(const GateChunk& x, const uint32_
 // time waiting for itself than for the data (four of thirteen cycles per instruction at 16 x 12 heads x 513 bins).  Forward and backward of
 // 16 x 1024 x 12 heads 105.7 -> 98.9 us, projected layer of 4 x 4096 x 16 73.5 -> 63.5.
 constexpr int kMmaPitch = 72;                      // bf16 elements between rows of As: the fragments' loads meet no bank twice
-template <int NB, bool STAGED>
+template <int NB, bool STAGED, bool TOK>
 __device__ __forceinline__ void mma_hidden(const GateMlpParams& p, int b0, int h, const float* sums, int nb, const float* gamma, const float* beta,
                                            const float* b1, const bf16* W1, float* qbar, bf16* As) {
   constexpr int kSlots = NB / 4;                   // entries per thread: 4 groups of 64 threads
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, D = p.D;
   const size_t bstride = (size_t)p.H * D;
-  if (p.tok.q) token_means(p.tok, b0, h, p.H, sums, nb, p.inv_count, D, qbar);
+  if (TOK) token_means(p.tok, b0, h, p.H, sums, nb, p.inv_count, D, qbar);
   else
 #pragma unroll 1
   for (int e0 = tid; e0 < nb * D; e0 += 512) {     // means: two channels per thread, all copies in flight at once
@@ -1015,11 +1016,12 @@ __device__ __forceinline__ void mma_hidden(const GateMlpParams& p, int b0, int h
 
 // SHIFTS: the entries' phases differ.  Every CTA computes the hidden layer of its head and entries itself, under the first
 // chunks' loads: a kernel in front of this one for it takes longer than all of them (49 us in all against 45).
-template <int NB, bool SHIFTS>
+// TOK: for a decode step; its loads in the other calls' form are code to step over (projected layer of 4 x 4096 x 16 heads 63.5 -> 70.1 us).
+template <int NB, bool SHIFTS, bool TOK>
 __global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p) {
   extern __shared__ __align__(16) float qbar[];    // [NB][D], then W1
   __shared__ __align__(16) bf16 As[3 * NB * kMmaPitch];
-  gate_start(p);
+  gate_start<true, TOK>(p);
   constexpr int kSets = MmaRows<NB>::kSets;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane & 3, i8 = lane >> 2, nw = blockDim.x >> 5;
   const int nbg = (p.B + NB - 1) / NB;
@@ -1039,8 +1041,8 @@ __global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p)
   // everything above reads only weights; the sums / hidden activations come from the kernel before
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const float* sums = p.sums + ((size_t)b0 * p.H + h) * p.D;
-  if (p.stage_w1) mma_hidden<NB, true>(p, b0, h, sums, nb, vec, vec + p.D, vec + 2 * p.D, w1s, qbar, As);
-  else mma_hidden<NB, false>(p, b0, h, sums, nb, gamma, beta, b1, reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, qbar, As);
+  if (p.stage_w1) mma_hidden<NB, true, TOK>(p, b0, h, sums, nb, vec, vec + p.D, vec + 2 * p.D, w1s, qbar, As);
+  else mma_hidden<NB, false, TOK>(p, b0, h, sums, nb, gamma, beta, b1, reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, qbar, As);
   if (p.qbar_out && blockIdx.x == 0)
     for (int e = threadIdx.x; e < nb * p.D; e += blockDim.x) {
       const int bb = e / p.D, c = e - bb * p.D;
@@ -1310,8 +1312,9 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
                           : launch_kernel(&cfg_short, gate_short_kernel<WT, 4, FULL>, mp))
 #define SPECTRE_GATE_MMA(NB)                                                                     \
   do {                                                                                           \
-    if (mp.shift && !mp.post) SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, true>, mp)); \
-    else SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, false>, mp));          \
+    if (mp.tok.q) SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, false, true>, mp)); /* one phase for all entries */ \
+    else if (mp.shift && !mp.post) SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, true, false>, mp)); \
+    else SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, false, false>, mp));   \
   } while (0)
   if (mma) {
     if (BB == 8) SPECTRE_GATE_MMA(8); else SPECTRE_GATE_MMA(4);

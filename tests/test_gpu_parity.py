@@ -849,6 +849,33 @@ def test_decode_step_leaves_the_same_state_as_append(ctx):
     assert torch.equal(a.V_buf, b.V_buf) and torch.equal(a.Q_buf, b.Q_buf)
 
 
+@pytest.mark.parametrize("dt,wdt,B,H,N,r,t", [("f32", "f32", 1, 2, 256, 0, 300), ("f16", "bf16", 1, 19, 512, 0, 7), ("bf16", "bf16", 1, 1, 32768, 0, 40000),
+                                             ("f16", "bf16", 3, 2, 512, 2, 512), ("bf16", "bf16", 9, 2, 256, 0, 255), ("bf16", "f32", 5, 2, 64, 0, 100),
+                                             ("f32", "bf16", 8, 2, 100, 1, 99)])
+def test_decode_step_is_append_and_gate(ctx, dt, wdt, B, H, N, r, t):
+    # The gate reads the sum in front of the token and the last CTA of a slab writes it behind: every gate kernel (threads per bin, one
+    # bin a thread, hidden layer ahead, tensor cores of 4 and 8 entries, staged), tokens of each type, before and after eviction starts.
+    w = W.Workload("t", B=B, L=N - 3, H=H, D=64, dtype=dt, wdtype=wdt, n_fft=N, seed=N + B)
+    p = to_dev(W.gate_params(w, modrelu_bias_std=0.01, toeplitz_r=r, bias_std=0.1))
+    g = torch.Generator(device="cuda"); g.manual_seed(N)
+    caches = [S.PrefixCache(B, H, 64, N, dtype=W.torch_dtype(dt)) for _ in range(2)]
+    for name in ("prefix_fft", "V_buf", "Q_buf", "sum_q"):
+        x = torch.randn(getattr(caches[0], name).shape, generator=g, device="cuda")
+        for c in caches:
+            getattr(c, name).copy_(x)
+    q, v = (torch.randn((B, H, 64), generator=g, device="cuda").to(W.torch_dtype(dt)) for _ in range(2))
+    y, gate = S.spectre_prefix_cache_decode_step(ctx, caches[0], q, v, t, p, [N - 1, 0])
+    S.spectre_prefix_cache_append(ctx, caches[1], q, v, t)
+    ref = S.spectre_gate(ctx, p, N, sum_q=caches[1].sum_q, inv_count=1.0 / N, shift_all=t)
+    assert torch.equal(gate, ref)
+    for name in ("V_buf", "Q_buf", "sum_q"):
+        assert torch.equal(getattr(caches[0], name), getattr(caches[1], name)), name
+    assert rel_err(W.to_f64(caches[0].prefix_fft), W.to_f64(caches[1].prefix_fft)) < 1e-6
+    P, G = torch.view_as_complex(caches[1].prefix_fft.double()), torch.view_as_complex(ref.double())
+    rows = torch.fft.irfft(P * G.unsqueeze(-1), n=N, dim=2)[:, :, [N - 1, 0]].permute(0, 2, 1, 3)
+    assert rel_err(W.to_f64(y), rows.cpu().numpy()) < TOL[dt]
+
+
 def test_a_refused_decode_step_leaves_the_cache_as_it_was(ctx):
     w = W.Workload("t", B=1, L=40, H=2, D=64, dtype="f32", wdtype="f32", n_fft=64, seed=2)
     cache = S.PrefixCache(1, 2, 64, 64, dtype=torch.float32)
