@@ -545,6 +545,7 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   const size_t done_bytes = round256((size_t)B * H * sizeof(int));
   const size_t gate_bytes = gate_min_workspace(B, H, D, N, params->toeplitz_r < 0 ? 0 : params->toeplitz_r);
   if (workspace_bytes < delta_bytes + part_bytes + done_bytes + gate_bytes) return fail(SPECTRE_ERR_WORKSPACE, "decode workspace too small");
+  // (the first delta_bytes are spare: the size that callers ask for stays)
   float* partial = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(workspace) + delta_bytes);
   int* done = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes);
   void* gate_ws = reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes + done_bytes;

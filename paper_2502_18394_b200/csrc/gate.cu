@@ -1265,7 +1265,7 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
                           !((reinterpret_cast<uintptr_t>(gp->W1) | reinterpret_cast<uintptr_t>(gp->W2)) & 15);
   const bool pre = grid_out.x >= 32;               // many CTAs per head: compute the hidden layer once
   // Programmatic dependent launch: the weight stream of the output layer overlaps the kernel before it where that is one of
-  // this call (the pooling pass, the decode step's ring kernel); each kernel waits for its predecessor
+  // this call (the pooling pass); each kernel waits for its predecessor
   // (griddepcontrol.wait) before it touches the sums, and first of all where the caller's own kernel precedes it.
   cudaLaunchAttribute pdl[1];
   pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
