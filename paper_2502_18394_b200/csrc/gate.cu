@@ -280,6 +280,11 @@ __device__ __forceinline__ void token_means(const GateToken& t, int b0, int h, i
   else token_means<f16>(t, b0, h, H, sums, nb, inv_count, D, qbar);
 }
 
+// Activations in front of a gate kernel's shared memory: hidden [hidden][entries], then q_bar [entries][D].  q_bar starts on 16 bytes, which the
+// hidden layer's loads need: two entries of an odd width end 8 bytes off.
+__host__ __device__ __forceinline__ int qbar_at(int entries, int hidden) { return (entries * hidden + 3) & ~3; }
+__host__ __device__ __forceinline__ int act_floats(int entries, int hidden, int D) { return qbar_at(entries, hidden) + ((entries * D + 3) & ~3); }
+
 // TOK: the sums may be a decode step's
 template <typename WT, int NB, bool STAGED, bool TOK = true>
 __device__ __forceinline__ void descriptor_and_hidden(const GateToken& tok, int b0, int h, int H, const float* sums, size_t bstride, int nb, int ncopy,
@@ -514,9 +519,9 @@ __global__ void __launch_bounds__(256) gate_hidden_kernel(const GateMlpParams p)
   const int h = blockIdx.x / nbg, b0 = (blockIdx.x - h * nbg) * BB;
   const int nb = min(BB, p.B - b0);
   gate_start(p);
-  float* qbar = u + BB * p.hidden;
+  float* qbar = u + qbar_at(BB, p.hidden);
   const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
-  WT* w1s = reinterpret_cast<WT*>(u + ((BB * (p.hidden + p.D) + 3) & ~3));
+  WT* w1s = reinterpret_cast<WT*>(u + act_floats(BB, p.hidden, p.D));
   const float* vec = reinterpret_cast<const float*>(w1s + p.D * p.hidden);
   if (p.stage_w1) stage_mlp(W1, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D, p.hidden, w1s);
   asm volatile("griddepcontrol.wait;" ::: "memory");        // the sums come from the kernel before
@@ -615,7 +620,7 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
   const bool live = k < p.K;
   const WT* col = reinterpret_cast<const WT*>(p.W2) + h * p.hs_w2 + 2 * (size_t)(live ? k : 0);
   const size_t ld = 2 * (size_t)p.K;
-  WT* w1s = reinterpret_cast<WT*>(u + ((BB * (p.hidden + p.D) + 3) & ~3));
+  WT* w1s = reinterpret_cast<WT*>(u + act_floats(BB, p.hidden, p.D));
   const float* vec = reinterpret_cast<const float*>(w1s + p.D * p.hidden);
   typename wraw<WT>::type w[R];
   const int n0 = min(R, p.hidden);
@@ -641,7 +646,7 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
   } else {
     // LayerNorm + hidden layer, repeated by every CTA of the head (a few thousand FLOPs per batch
     // entry, two short round trips) while this thread's W2 column is already on its way
-    float* qbar = u + BB * p.hidden;   // [BB][D]
+    float* qbar = u + qbar_at(BB, p.hidden);   // [BB][D]
     const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
     if (p.stage_w1)
       descriptor_and_hidden<WT, BB, true, TOK>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
@@ -707,7 +712,7 @@ __global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams 
   const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
   const WT* col = reinterpret_cast<const WT*>(p.W2) + h * p.hs_w2 + 2 * (size_t)kc;
   const size_t ld = 2 * (size_t)p.K;
-  WT* w1s = reinterpret_cast<WT*>(u + ((p.hidden + p.D + 3) & ~3));
+  WT* w1s = reinterpret_cast<WT*>(u + act_floats(1, p.hidden, p.D));
   const float* vec = reinterpret_cast<const float*>(w1s + p.D * p.hidden);
   typename wraw<WT>::type w[R];
 #pragma unroll
@@ -716,7 +721,7 @@ __global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams 
   const float bias = (!p.post && p.modrelu_bias) ? p.modrelu_bias[h * p.hs_mb + kc] : 0.f;
   if (p.stage_w1) stage_mlp(W1, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D, p.hidden, w1s);
   asm volatile("griddepcontrol.wait;" ::: "memory");         // the sums come from the kernel before
-  float* qbar = u + p.hidden;
+  float* qbar = u + qbar_at(1, p.hidden);
   const float* sums = p.sums + ((size_t)b * p.H + h) * p.D;
   if (p.stage_w1)
     descriptor_and_hidden<WT, 1, true>(p.tok, b, h, p.H, sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, vec, vec + p.D,
@@ -770,7 +775,7 @@ __global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams 
   const int h = blockIdx.x / nbg, b0 = (blockIdx.x - h * nbg) * BB;
   const int nb = min(BB, p.B - b0), k = threadIdx.x;
   const bool live = k < p.K;
-  WT* w1s = reinterpret_cast<WT*>(u + ((BB * (p.hidden + p.D) + 3) & ~3));
+  WT* w1s = reinterpret_cast<WT*>(u + act_floats(BB, p.hidden, p.D));
   float* vec = reinterpret_cast<float*>(w1s + p.D * p.hidden);
   WT* w2s = reinterpret_cast<WT*>(vec + ((2 * p.D + p.hidden + 3) & ~3));
   copy_async16(reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1, w1s, p.D * p.hidden * (int)sizeof(WT));
@@ -780,7 +785,7 @@ __global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams 
   const float2 b2 = make_float2(p.b2[h * p.hs_b2 + 2 * kc], p.b2[h * p.hs_b2 + 2 * kc + 1]);
   const float bias = (!p.post && p.modrelu_bias) ? p.modrelu_bias[h * p.hs_mb + kc] : 0.f;
   asm volatile("griddepcontrol.wait;" ::: "memory");         // the sums come from the kernel before
-  float* qbar = u + BB * p.hidden;
+  float* qbar = u + qbar_at(BB, p.hidden);
   descriptor_and_hidden<WT, BB, true, FULL>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                       p.inv_count, p.D, p.hidden, vec, vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, BB);
   if (p.qbar_out)
@@ -1254,7 +1259,7 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
   dim3 grid_out((K + thr_out - 1) / thr_out, (unsigned)(H * ((B + BB - 1) / BB)));
   const bool wb = gp->wdtype == SPECTRE_BF16;
   const size_t w1_bytes = (size_t)D * gp->hidden * (wb ? 2 : 4);
-  const size_t act_bytes = (((size_t)BB * (D + gp->hidden) + 3) & ~(size_t)3) * sizeof(float);
+  const size_t act_bytes = act_floats(BB, gp->hidden, D) * sizeof(float);
   const size_t staged_bytes = w1_bytes + (2 * (size_t)D + gp->hidden) * sizeof(float);
   mp.stage_w1 = w1_bytes <= 16384 && w1_bytes % 16 == 0 && !(reinterpret_cast<uintptr_t>(gp->W1) & 15) && act_bytes + staged_bytes <= 49152;
   const size_t smem = act_bytes + (mp.stage_w1 ? staged_bytes : 0);

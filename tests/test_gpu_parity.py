@@ -361,6 +361,35 @@ def test_gate_shapes(ctx, B, L, H, D, hid, dt, wdt, n):
     assert eg < GATE_TOL["16bit"] and eq < GATE_TOL["16bit"]
 
 
+@pytest.mark.parametrize("B,hid,wdt,n,D", [(2, 17, "f32", 128, 64), (3, 33, "bf16", 128, 64), (2, 33, "f32", 32768, 64), (3, 17, "bf16", 16384, 24),
+                                           (2, 255, "bf16", 100, 64), (3, 255, "f32", 16384, 8)])
+def test_gate_of_two_entries_and_an_odd_width(ctx, B, hid, wdt, n, D):
+    # two entries per CTA: their hidden activations, in front of the means, end off a 16-byte boundary; W1 staged and too large for it,
+    # the hidden layer in the same kernel (n < 16000) and ahead of it
+    w = W.Workload("t", B=B, L=33, H=2, D=D, dtype="f32", wdtype=wdt, n_fft=n, hidden=hid, seed=n + B)
+    eg, eq, *_ = run_gate(ctx, w, modrelu_bias_std=0.05, bias_std=0.1, shift_all=3)
+    assert eg < GATE_TOL["16bit"] and eq < GATE_TOL["16bit"]
+
+
+@pytest.mark.parametrize("B,hid,wdt,N", [(2, 33, "f32", 256), (3, 17, "bf16", 256), (3, 33, "f32", 32768)])
+def test_decode_step_of_two_entries_and_an_odd_width(ctx, B, hid, wdt, N):
+    w = W.Workload("t", B=B, L=N - 3, H=2, D=64, dtype="bf16", wdtype=wdt, n_fft=N, hidden=hid, seed=N + B)
+    p = W.gate_params(w, modrelu_bias_std=0.01, bias_std=0.1)
+    gen = torch.Generator(device="cuda"); gen.manual_seed(N)
+    cache = S.PrefixCache(B, 2, 64, N, dtype=torch.bfloat16)
+    for name in ("prefix_fft", "V_buf", "Q_buf", "sum_q"):
+        getattr(cache, name).normal_(generator=gen)
+    q, v = (torch.randn((B, 2, 64), generator=gen, device="cuda").bfloat16() for _ in range(2))
+    t = N + 5
+    sum_q = W.to_f64(cache.sum_q) + W.to_f64(q) - W.to_f64(cache.Q_buf[:, t % N])
+    y, gate = S.spectre_prefix_cache_decode_step(ctx, cache, q, v, t, to_dev(p), [N - 1])
+    ref = O.gate(sum_q, 1.0 / N, N, shift=np.full(B, t, dtype=np.int64), **gate_params_np(p))
+    assert rel_err(gate_to_complex(gate), ref) < GATE_TOL["16bit"]
+    P, G = torch.view_as_complex(cache.prefix_fft.double()), torch.view_as_complex(gate.double())
+    row = torch.fft.irfft(P * G.unsqueeze(-1), n=N, dim=2)[:, :, N - 1]
+    assert rel_err(W.to_f64(y[:, 0]), row.cpu().numpy()) < TOL["bf16"]
+
+
 @pytest.mark.parametrize("B,H,n,r,shifts", [(2, 3, 510, 0, False), (4, 2, 4096, 0, True), (5, 2, 1000, 2, False), (8, 1, 32768, 0, False),
                                              (17, 2, 512, 0, True), (2, 2, 126, 0, False), (9, 3, 128, 1, True), (6, 2, 254, 0, False),
                                              (150, 2, 510, 0, True)])
