@@ -316,7 +316,9 @@ int spectre_prefix_cache_append(spectre_ctx* ctx, void* stream, const spectre_ca
  *   q_t, v_t  [B, H, D] contiguous, dtype buf_dtype (device)
  *   params    gate network; K = N_max/2 + 1 bins
  *   rows      HOST array of nrows indices in [0, N_max), 1 <= nrows <= SPECTRE_DECODE_MAX_ROWS
- *   y_rows    [B, nrows, H, D] contiguous, dtype buf_dtype (device), written
+ *   y_rows    [B, nrows, H, D] contiguous, dtype buf_dtype (device), written; may share
+ *             memory with q_t and v_t, as g_out may: one row in a token's own buffer costs
+ *             nothing, any other overlap makes the step two passes over the spectrum
  *   g_out     [B, H, K, 2] float32 (device), written: the gate of this step
  *   workspace >= spectre_decode_workspace_bytes(...) bytes, 16-byte aligned
  * Errors: as spectre_prefix_cache_append and spectre_gate, a row outside the window or

@@ -245,6 +245,7 @@ struct DecodeRows { int r[SPECTRE_DECODE_MAX_ROWS]; };
 // the slab's part of ring buffers and running sum on by the token: every other one has read the evicted row then, and the gate in front
 // took the token from where it came (a kernel of its own for it in front of
 // the gate: step of a 4k window 14.1 -> 15.8 us, of two 2k windows 15.2 -> 16.4).
+// v_t = q_t = NULL: the cache holds the token already, the pass only reads out.
 // Bound by HBM (16 bytes per bin and channel).  Launched as a programmatic dependent of the gate kernel, which waited for the caller's work:
 // the first bins and the token are on their way before the gate is complete.
 template <typename T, int NR>
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, T* 
   const size_t ring = (((size_t)b * N + slot) * H + h) * D;
   T tok[2], old[2];                            // as loaded, so that nothing waits for them yet
   auto token = [&](int c) {
-    if (c >= half) return;
+    if (c >= half || !v_t) return;
     const T *a = v_t + (size_t)slab * D + 2 * c, *o = evict ? V_buf + ring + 2 * c : a;
     tok[0] = a[0]; tok[1] = a[1];
     old[0] = o[0]; old[1] = o[1];
@@ -302,7 +303,7 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, T* 
     const bool live = c < half;
     if (c0 > 0) token(c);
     float d0 = 0.f, d1 = 0.f;
-    if (live) {
+    if (live && v_t) {
       d0 = io<T>::load1(tok) - (evict ? io<T>::load1(old) : 0.f);
       d1 = io<T>::load1(tok + 1) - (evict ? io<T>::load1(old + 1) : 0.f);
     }
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, T* 
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int c = threadIdx.x; c < D; c += 256) {              // ring buffers and running sum of this slab
+  for (int c = v_t ? (int)threadIdx.x : D; c < D; c += 256) {   // ring buffers and running sum of this slab
     const size_t at = (size_t)slab * D + c;
     const T q = q_t[at], v = v_t[at];                       // all loads in front of the stores, which none may pass
     const float s = sum_q[at], qo = evict ? io<T>::load1(Q_buf + ring + c) : 0.f;
@@ -378,8 +379,36 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, T* 
     }
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if (NR == 1 && o0 == 0) __syncthreads();                   // one row may take the token's own place: all of it has been read
     if (in && part == 0) io<T>::store1(y + (((size_t)b * nrows + r) * H + h) * D + c, s);
   }
+}
+
+// The append: spectrum, then ring buffers and running sum
+static int append_call(cudaStream_t st, const spectre_cache* cache, const void* q_t, const void* v_t, int64_t t) {
+  const int B = cache->B, H = cache->H, D = cache->D, N = cache->N_max, K = N / 2 + 1;
+  const int slot = (int)(t % N);
+  const int evict = t >= N ? 1 : 0;
+  const int wps = (K + 31) / 32;
+  const size_t nwarps = (size_t)B * H * wps;
+  const unsigned blocks = (unsigned)((nwarps * 32 + 255) / 256);
+  const unsigned blocks2 = (unsigned)(((size_t)B * H * D + 255) / 256);
+  SPECTRE_IO_DISPATCH(cache->buf_dtype, {
+    SPECTRE_CUDA_OK(launch_after(append_spectrum_kernel<T>, blocks, 256, 0, st, cache->prefix_fft,
+                                 reinterpret_cast<const T*>(cache->V_buf), reinterpret_cast<const T*>(v_t), H, D, N, K, slot,
+                                 (unsigned)slot, evict, wps, nwarps));
+    SPECTRE_CUDA_OK(launch_after(append_ring_kernel<T>, blocks2, 256, 0, st, reinterpret_cast<T*>(cache->V_buf),
+                                 reinterpret_cast<T*>(cache->Q_buf), cache->sum_q, reinterpret_cast<const T*>(q_t),
+                                 reinterpret_cast<const T*>(v_t), B, H, D, N, slot, evict));
+  });
+  SPECTRE_LAUNCH_OK("append kernels");
+  return SPECTRE_OK;
+}
+
+// any byte in common
+static bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + nb && y < x + na;
 }
 
 static int check_cache(const spectre_cache* c) {
@@ -485,27 +514,9 @@ extern "C" int spectre_prefix_cache_append(spectre_ctx* ctx, void* stream, const
   if (rc != SPECTRE_OK) return rc;
   if (!q_t || !v_t) return fail(SPECTRE_ERR_INVALID_ARG, "token pointer is NULL");
   if (t < 0) return fail(SPECTRE_ERR_INVALID_ARG, "t must be >= 0");
-  const int B = cache->B, H = cache->H, D = cache->D, N = cache->N_max;
-  if ((size_t)B * H * D > (size_t)1 << 30) return fail(SPECTRE_ERR_UNSUPPORTED, "B*H*D too large");
+  if ((size_t)cache->B * cache->H * cache->D > (size_t)1 << 30) return fail(SPECTRE_ERR_UNSUPPORTED, "B*H*D too large");
   SPECTRE_CUDA_OK(cudaSetDevice(ctx->device));
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const int K = N / 2 + 1;
-  const int slot = (int)(t % N);
-  const int evict = t >= N ? 1 : 0;
-  const int wps = (K + 31) / 32;
-  const size_t nwarps = (size_t)B * H * wps;
-  const unsigned blocks = (unsigned)((nwarps * 32 + 255) / 256);
-  const unsigned blocks2 = (unsigned)(((size_t)B * H * D + 255) / 256);
-  SPECTRE_IO_DISPATCH(cache->buf_dtype, {
-    SPECTRE_CUDA_OK(launch_after(append_spectrum_kernel<T>, blocks, 256, 0, st, cache->prefix_fft,
-                                 reinterpret_cast<const T*>(cache->V_buf), reinterpret_cast<const T*>(v_t), H, D, N, K, slot,
-                                 (unsigned)slot, evict, wps, nwarps));
-    SPECTRE_CUDA_OK(launch_after(append_ring_kernel<T>, blocks2, 256, 0, st, reinterpret_cast<T*>(cache->V_buf),
-                                 reinterpret_cast<T*>(cache->Q_buf), cache->sum_q, reinterpret_cast<const T*>(q_t),
-                                 reinterpret_cast<const T*>(v_t), B, H, D, N, slot, evict));
-  });
-  SPECTRE_LAUNCH_OK("append kernels");
-  return SPECTRE_OK;
+  return append_call(reinterpret_cast<cudaStream_t>(stream), cache, q_t, v_t, t);
 }
 
 static size_t round256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -556,12 +567,26 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int slot = (int)(t % N);
   const int evict = t >= N ? 1 : 0;
+  // The token is read until the pass over the spectrum ends, by the CTAs of its own slab.  One row written over it is written by the last
+  // of them; outputs that meet it in any other way wait until the cache has it (its spectrum goes through memory twice then).
+  const size_t es = io_elem_bytes(cache->buf_dtype), tok_bytes = (size_t)B * H * D * es;
+  auto meets = [&](const void* x) {
+    return overlap(g_out, (size_t)B * H * K * sizeof(float2), x, tok_bytes) ||
+           (overlap(y_rows, nrows * tok_bytes, x, tok_bytes) && !(nrows == 1 && y_rows == x));
+  };
+  const bool first = meets(q_t) || meets(v_t);
+  if (first) {
+    SPECTRE_CUDA_OK(cudaMemsetAsync(done, 0, (size_t)B * H * sizeof(int), st));
+    rc = append_call(st, cache, q_t, v_t, t);
+    if (rc != SPECTRE_OK) return rc;
+    q_t = v_t = nullptr;
+  }
   // (c)-(d) gate from the running sum with the token in it, phase p = t
-  const size_t row = (size_t)slot * H * D * io_elem_bytes(cache->buf_dtype);
+  const size_t row = (size_t)slot * H * D * es;
   const GateToken tok = {q_t, evict ? static_cast<const char*>(static_cast<const void*>(cache->Q_buf)) + row : nullptr, (size_t)N * H * D,
                          cache->buf_dtype, done, B * H};
   rc = gate_call(ctx, stream, nullptr, cache->sum_q, B, H, D, 1.0f / (float)N, params, N, nullptr, t, g_out, nullptr, gate_ws,
-                 gate_bytes, false, &tok);
+                 gate_bytes, false, first ? nullptr : &tok);
   if (rc != SPECTRE_OK) return rc;
   // (a), (b), (e) one pass over the spectrum, ring buffers and running sum
   DecodeRows dr;

@@ -905,6 +905,44 @@ def test_decode_step_is_append_and_gate(ctx, dt, wdt, B, H, N, r, t):
     assert rel_err(W.to_f64(y), rows.cpu().numpy()) < TOL[dt]
 
 
+@pytest.mark.parametrize("dt,B,H,N,t,where", [("bf16", 2, 3, 256, 300, "v"), ("f32", 1, 2, 512, 7, "q"), ("f16", 9, 2, 4096, 5000, "v"),
+                                             ("f32", 2, 2, 64, 64, "rows"), ("bf16", 3, 2, 512, 511, "rows"), ("f16", 1, 2, 128, 500, "rows"),
+                                             ("bf16", 8, 2, 1024, 1500, "gate"), ("f32", 2, 3, 100, 20, "gate")])
+def test_decode_step_outputs_in_the_tokens_memory(ctx, dt, B, H, N, t, where):
+    # One row over v_t or q_t; two rows over both tokens, one half each; the gate over both tokens: the same state and outputs as with
+    # buffers of their own.
+    D, dtype, n = 64, W.torch_dtype(dt), B * H * 64
+    nrows = 2 if where == "rows" else 1
+    w = W.Workload("t", B=B, L=N - 3, H=H, D=D, dtype=dt, wdtype="bf16", n_fft=N, seed=N + B)
+    p = to_dev(W.gate_params(w, modrelu_bias_std=0.01, bias_std=0.1))
+    gen = torch.Generator(device="cuda"); gen.manual_seed(N)
+    caches = [S.PrefixCache(B, H, D, N, dtype=dtype) for _ in range(2)]
+    for name in ("prefix_fft", "V_buf", "Q_buf", "sum_q"):
+        x = torch.randn(getattr(caches[0], name).shape, generator=gen, device="cuda")
+        for c in caches:
+            getattr(c, name).copy_(x)
+    tok = torch.randn((2, B, H, D), generator=gen, device="cuda").to(dtype)
+    rows = [N - 1, 0][:nrows]
+    y_ref, g_ref = S.spectre_prefix_cache_decode_step(ctx, caches[0], tok[0], tok[1], t, p, rows)
+    g_own = torch.empty((B, H, N // 2 + 1, 2), device="cuda")
+    y_own = torch.empty((B, nrows, H, D), dtype=dtype, device="cuda")
+    if where == "gate":
+        buf = torch.empty(max(g_own.numel() * 4, tok.numel() * tok.element_size()), dtype=torch.uint8, device="cuda")
+        both = buf[:tok.numel() * tok.element_size()].view(dtype).view(tok.shape)
+        g_out, y_rows = buf[:g_own.numel() * 4].view(torch.float32).view(g_own.shape), y_own
+    else:
+        both = torch.empty_like(tok)
+        g_out, y_rows = g_own, (both.view(y_own.shape) if where == "rows" else both["qv".index(where)].view(y_own.shape))
+    both.copy_(tok)
+    y, g = S.spectre_prefix_cache_decode_step(ctx, caches[1], both[0], both[1], t, p, rows, y_rows=y_rows, g_out=g_out)
+    assert y.data_ptr() == y_rows.data_ptr() and g.data_ptr() == g_out.data_ptr()
+    for name in ("V_buf", "Q_buf", "sum_q"):
+        assert torch.equal(getattr(caches[0], name), getattr(caches[1], name)), name
+    assert rel_err(W.to_f64(caches[1].prefix_fft), W.to_f64(caches[0].prefix_fft)) < 1e-6
+    assert rel_err(W.to_f64(g), W.to_f64(g_ref)) < GATE_TOL["f32"]
+    assert rel_err(W.to_f64(y), W.to_f64(y_ref)) < TOL[dt]
+
+
 def test_a_refused_decode_step_leaves_the_cache_as_it_was(ctx):
     w = W.Workload("t", B=1, L=40, H=2, D=64, dtype="f32", wdtype="f32", n_fft=64, seed=2)
     cache = S.PrefixCache(1, 2, 64, 64, dtype=torch.float32)
