@@ -280,10 +280,11 @@ __device__ __forceinline__ void token_means(const GateToken& t, int b0, int h, i
   else token_means<f16>(t, b0, h, H, sums, nb, inv_count, D, qbar);
 }
 
-// Activations in front of a gate kernel's shared memory: hidden [hidden][entries], then q_bar [entries][D].  q_bar starts on 16 bytes, which the
-// hidden layer's loads need: two entries of an odd width end 8 bytes off.
-__host__ __device__ __forceinline__ int qbar_at(int entries, int hidden) { return (entries * hidden + 3) & ~3; }
-__host__ __device__ __forceinline__ int act_floats(int entries, int hidden, int D) { return qbar_at(entries, hidden) + ((entries * D + 3) & ~3); }
+// Activations in front of a gate kernel's shared memory: hidden [hidden][entries], then q_bar [entries][D].  The hidden layer of several entries
+// reads q_bar 16 bytes at a time: 4 and 8 end there by themselves, two of an odd width 8 bytes off.  Only these are rounded up: with the
+// rounding, one entry's kernel spilled 112 bytes (decode step of 1 x 12 x 4096, fp32 weights 13.9 -> 16.4 us).
+__host__ __device__ __forceinline__ int qbar_at(int entries, int hidden) { return entries == 2 ? (2 * hidden + 3) & ~3 : entries * hidden; }
+__host__ __device__ __forceinline__ int act_floats(int entries, int hidden, int D) { return (qbar_at(entries, hidden) + entries * D + 3) & ~3; }
 
 // TOK: the sums may be a decode step's
 template <typename WT, int NB, bool STAGED, bool TOK = true>
