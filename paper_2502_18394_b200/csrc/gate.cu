@@ -286,8 +286,54 @@ __device__ __forceinline__ void token_means(const GateToken& t, int b0, int h, i
 __host__ __device__ __forceinline__ int qbar_at(int entries, int hidden) { return entries == 2 ? (2 * hidden + 3) & ~3 : entries * hidden; }
 __host__ __device__ __forceinline__ int act_floats(int entries, int hidden, int D) { return (qbar_at(entries, hidden) + entries * D + 3) & ~3; }
 
+// one hidden unit's sums over D inputs for N entries (rows of q; absent ones hold whatever is there, never used), two inputs per packed sum; ALIGNED: the rows
+// start on 16 bytes, one load takes four inputs
+template <typename WT, int N, bool ALIGNED>
+__device__ __forceinline__ void hidden_unit(const WT* w, int hidden, int D, const float* q, float (&acc)[N]) {
+  uint64_t a2[N];
+#pragma unroll
+  for (int s = 0; s < N; ++s) a2[s] = pk2(acc[s], 0.f);
+  auto block = [&](auto size, int c) {
+    constexpr int kLoads = decltype(size)::value;
+    float wv[kLoads];
+#pragma unroll
+    for (int i = 0; i < kLoads; ++i) wv[i] = wload<WT>(w + (size_t)(c + i) * hidden);
+#pragma unroll
+    for (int i = 0; i < kLoads; i += 4) {
+      const uint64_t w01 = pk2(wv[i], wv[i + 1]), w23 = pk2(wv[i + 2], wv[i + 3]);
+#pragma unroll
+      for (int s = 0; s < N; ++s) {
+        const float* p = q + s * D + c + i;
+        ulonglong2 t;
+        if constexpr (ALIGNED) t = *reinterpret_cast<const ulonglong2*>(p);
+        else t = make_ulonglong2(pk2(p[0], p[1]), pk2(p[2], p[3]));
+        a2[s] = fma2(t.x, w01, a2[s]);
+        a2[s] = fma2(t.y, w23, a2[s]);
+      }
+    }
+  };
+  int c = 0;
+#pragma unroll 1
+  for (; c + 32 <= D; c += 32) block(std::integral_constant<int, 32>(), c);
+#pragma unroll 1
+  for (; c + 4 <= D; c += 4) block(std::integral_constant<int, 4>(), c);
+#pragma unroll
+  for (int s = 0; s < N; ++s) {
+    float lo, hi;
+    upk2(a2[s], lo, hi);
+    acc[s] = lo + hi;
+  }
+#pragma unroll 1
+  for (; c < D; ++c) {
+    const float wv = wload<WT>(w + (size_t)c * hidden);
+#pragma unroll
+    for (int s = 0; s < N; ++s) acc[s] = fmaf(q[s * D + c], wv, acc[s]);
+  }
+}
+
 // TOK: the sums may be a decode step's
-template <typename WT, int NB, bool STAGED, bool TOK = true>
+// DEEP: several entries, W1 from L2, D >= 32
+template <typename WT, int NB, bool STAGED, bool TOK = true, bool DEEP = false>
 __device__ __forceinline__ void descriptor_and_hidden(const GateToken& tok, int b0, int h, int H, const float* sums, size_t bstride, int nb, int ncopy,
                                                       size_t copy_stride, float inv_count, int D, int hidden,
                                                       const float* gamma, const float* beta,
@@ -360,6 +406,22 @@ __device__ __forceinline__ void descriptor_and_hidden(const GateToken& tok, int 
       }
       for (; c < D; ++c) acc = fmaf(qbar[c], wget<WT, STAGED>(W1 + (size_t)c * hidden + jj), acc);
       u[jj * ustride] = gelu_erf(acc);
+    }
+    __syncthreads();
+    return;
+  }
+  if constexpr (DEEP) {
+    // 32 loads of W1 in flight, each for all entries (gate of 2 x 4 x 32768, 256 hidden units, fp32 weights 40.2 -> 29.5 us,
+    // 64 x 12 x 196 18.9 -> 16.8, against the loop below)
+    for (int jj = threadIdx.x; jj < hidden; jj += blockDim.x) {
+      float acc[NB];
+#pragma unroll
+      for (int s = 0; s < NB; ++s) acc[s] = b1[jj];
+      if (D % 4 == 0) hidden_unit<WT, NB, true>(W1 + jj, hidden, D, qbar, acc);
+      else hidden_unit<WT, NB, false>(W1 + jj, hidden, D, qbar, acc);
+#pragma unroll
+      for (int s = 0; s < NB; ++s)
+        if (s < nb) u[jj * ustride + s] = gelu_erf(acc[s]);
     }
     __syncthreads();
     return;
@@ -512,9 +574,10 @@ template <> struct wraw<float> {
 // (32 rows in bf16: two round trips for the usual 64-wide hidden layer) and needs few enough
 // registers for four CTAs per SM, so that the grid of an 8k-token transform is resident at once;
 // the kernel is a pure stream over W2.
-// Hidden activations of BB batch entries of one head, once: grid H * ceil(B / BB).
-template <typename WT, int BB>
-__global__ void __launch_bounds__(256) gate_hidden_kernel(const GateMlpParams p) {
+// Hidden activations of BB batch entries of one head, once: grid H * ceil(B / BB).  With the 48 registers of the compiler's own choice few of its loads were in
+// flight (gate of 8 x 8 x 32768 fp32 19.7 -> 18.5 us).
+template <typename WT, int BB, bool DEEP>
+__global__ void __launch_bounds__(256, 2) gate_hidden_kernel(const GateMlpParams p) {
   extern __shared__ __align__(16) float u[];       // [hidden][BB], then q_bar [BB][D]
   const int nbg = (p.B + BB - 1) / BB;
   const int h = blockIdx.x / nbg, b0 = (blockIdx.x - h * nbg) * BB;
@@ -526,7 +589,11 @@ __global__ void __launch_bounds__(256) gate_hidden_kernel(const GateMlpParams p)
   const float* vec = reinterpret_cast<const float*>(w1s + p.D * p.hidden);
   if (p.stage_w1) stage_mlp(W1, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.b1 + h * p.hs_b1, p.D, p.hidden, w1s);
   asm volatile("griddepcontrol.wait;" ::: "memory");        // the sums come from the kernel before
-  if (p.stage_w1)
+  if constexpr (DEEP)
+    descriptor_and_hidden<WT, BB, false, true, true>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
+                                                     p.inv_count, p.D, p.hidden, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, W1,
+                                                     p.b1 + h * p.hs_b1, qbar, u, BB);
+  else if (p.stage_w1)
     descriptor_and_hidden<WT, BB, true>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                         p.inv_count, p.D, p.hidden, vec, vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, BB);
   else
@@ -609,7 +676,7 @@ __device__ __forceinline__ void gate_stream(typename wraw<WT>::type (&w)[wraw<WT
 // PRE: the hidden activations were computed once per (head, batch entry) by gate_hidden_kernel
 // (long transforms: hundreds of CTAs per head would otherwise repeat that work).
 // TOK: for a decode step; without its loads the other calls' form spills nothing (28 bytes cost the layer of 8192 points 1.3 us of 63.2).
-template <typename WT, int BB, bool PRE, bool TOK>
+template <typename WT, int BB, bool PRE, bool TOK, bool DEEP>
 __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const GateMlpParams p) {
   extern __shared__ __align__(16) float u[];       // [hidden][BB], then q_bar [BB][D]
   gate_start(p);                                   // a kernel launched behind this one as a programmatic dependent may do its set-up meanwhile
@@ -649,7 +716,11 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
     // entry, two short round trips) while this thread's W2 column is already on its way
     float* qbar = u + qbar_at(BB, p.hidden);   // [BB][D]
     const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
-    if (p.stage_w1)
+    if constexpr (DEEP)
+      descriptor_and_hidden<WT, BB, false, TOK, true>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
+                                                      p.inv_count, p.D, p.hidden, p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, W1,
+                                                      p.b1 + h * p.hs_b1, qbar, u, BB);
+    else if (p.stage_w1)
       descriptor_and_hidden<WT, BB, true, TOK>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                           p.inv_count, p.D, p.hidden, vec, vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, BB);
     else
@@ -982,17 +1053,21 @@ __device__ __forceinline__ void mma_hidden(const GateMlpParams& p, int b0, int h
       uint64_t a2[kSlots];
 #pragma unroll
       for (int sl = 0; sl < kSlots; ++sl) a2[sl] = pk2(acc[sl], 0.f);
+      constexpr int kLoads = STAGED ? 4 : 32;      // from L2: all in flight at once (gate of 4 x 4 x 16384, 512 channels, 28.3 -> 26.5 us)
 #pragma unroll 4
-      for (int i = c; i < c + 32; i += 4) {
-        float wv[4];
+      for (int i = c; i < c + 32; i += kLoads) {
+        float wv[kLoads];
 #pragma unroll
-        for (int x = 0; x < 4; ++x) wv[x] = wget<bf16, STAGED>(W1 + (i + x) * 64 + jj);
-        const uint64_t w01 = pk2(wv[0], wv[1]), w23 = pk2(wv[2], wv[3]);
+        for (int x = 0; x < kLoads; ++x) wv[x] = wget<bf16, STAGED>(W1 + (i + x) * 64 + jj);
 #pragma unroll
-        for (int sl = 0; sl < kSlots; ++sl) {      // absent entries: whatever is there, never used
-          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(qbar + (gi + 4 * sl) * D + i);
-          a2[sl] = fma2(t.x, w01, a2[sl]);
-          a2[sl] = fma2(t.y, w23, a2[sl]);
+        for (int x = 0; x < kLoads; x += 4) {
+          const uint64_t w01 = pk2(wv[x], wv[x + 1]), w23 = pk2(wv[x + 2], wv[x + 3]);
+#pragma unroll
+          for (int sl = 0; sl < kSlots; ++sl) {    // absent entries: whatever is there, never used
+            const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(qbar + (gi + 4 * sl) * D + i + x);
+            a2[sl] = fma2(t.x, w01, a2[sl]);
+            a2[sl] = fma2(t.y, w23, a2[sl]);
+          }
         }
       }
 #pragma unroll
@@ -1023,7 +1098,7 @@ __device__ __forceinline__ void mma_hidden(const GateMlpParams& p, int b0, int h
 // SHIFTS: the entries' phases differ.  Every CTA computes the hidden layer of its head and entries itself, under the first
 // chunks' loads: a kernel in front of this one for it takes longer than all of them (49 us in all against 45).
 // TOK: for a decode step; its loads in the other calls' form are code to step over (projected layer of 4 x 4096 x 16 heads 63.5 -> 70.1 us).
-template <int NB, bool SHIFTS, bool TOK>
+template <int NB, bool SHIFTS, bool TOK, bool STAGED>
 __global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p) {
   extern __shared__ __align__(16) float qbar[];    // [NB][D], then W1
   __shared__ __align__(16) bf16 As[3 * NB * kMmaPitch];
@@ -1038,7 +1113,7 @@ __global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p)
   bf16* w1s = reinterpret_cast<bf16*>(qbar + ((NB * p.D + 3) & ~3));
   const float* vec = reinterpret_cast<const float*>(w1s + p.D * p.hidden);
   const float *gamma = p.gamma + h * p.hs_ln, *beta = p.beta + h * p.hs_ln, *b1 = p.b1 + h * p.hs_b1;
-  if (p.stage_w1) stage_mlp(reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, gamma, beta, b1, p.D, p.hidden, w1s);
+  if constexpr (STAGED) stage_mlp(reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, gamma, beta, b1, p.D, p.hidden, w1s);
   // a CTA's chunks are contiguous, its warps take neighbouring ones
   const int nchunk = (p.K + 15) / 16, per = (nchunk + (int)gridDim.x - 1) / (int)gridDim.x;
   const int c0 = blockIdx.x * per + warp, c1 = min(nchunk, (int)(blockIdx.x + 1) * per);
@@ -1047,7 +1122,7 @@ __global__ void __launch_bounds__(256, 2) gate_mma_kernel(const GateMlpParams p)
   // everything above reads only weights; the sums / hidden activations come from the kernel before
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const float* sums = p.sums + ((size_t)b0 * p.H + h) * p.D;
-  if (p.stage_w1) mma_hidden<NB, true, TOK>(p, b0, h, sums, nb, vec, vec + p.D, vec + 2 * p.D, w1s, qbar, As);
+  if constexpr (STAGED) mma_hidden<NB, true, TOK>(p, b0, h, sums, nb, vec, vec + p.D, vec + 2 * p.D, w1s, qbar, As);
   else mma_hidden<NB, false, TOK>(p, b0, h, sums, nb, gamma, beta, b1, reinterpret_cast<const bf16*>(p.W1) + h * p.hs_w1, qbar, As);
   if (p.qbar_out && blockIdx.x == 0)
     for (int e = threadIdx.x; e < nb * p.D; e += blockDim.x) {
@@ -1269,6 +1344,9 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
   const size_t short_bytes = act_bytes + w1_bytes + ((2 * (size_t)D + gp->hidden + 3) & ~(size_t)3) * sizeof(float) + w2_bytes;
   const bool all_staged = BB >= 4 && !mma && grid_out.x == 1 && w1_bytes % 16 == 0 && w2_bytes % 16 == 0 && short_bytes <= 49152 &&
                           !((reinterpret_cast<uintptr_t>(gp->W1) | reinterpret_cast<uintptr_t>(gp->W2)) & 15);
+  // Several entries and W1 not staged: the hidden layer with its loads of 32 inputs in flight (in a kernel of its own: its registers cost the staged
+  // form 2 ... 4 % in one kernel with it)
+  const bool deep = BB > 1 && !mp.stage_w1 && D >= 32;
   const bool pre = grid_out.x >= 32;               // many CTAs per head: compute the hidden layer once
   // Programmatic dependent launch: the weight stream of the output layer overlaps the kernel before it where that is one of
   // this call (the pooling pass); each kernel waits for its predecessor
@@ -1301,26 +1379,32 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
   cfg_split.gridDim = dim3((unsigned)((K + split_bins - 1) / split_bins), (unsigned)(B * H), 1); cfg_split.blockDim = dim3(256, 1, 1);
   cudaLaunchConfig_t cfg_short = cfg_out;
   cfg_short.gridDim = dim3(grid_out.y, 1, 1); cfg_short.dynamicSmemBytes = short_bytes;
-#define SPECTRE_GATE_LAUNCH(WT, NB)                                                              \
+#define SPECTRE_GATE_LAUNCH_AS(WT, NB, DEEP)                                                     \
   do {                                                                                           \
     if (pre) {                                                                                   \
-      SPECTRE_CUDA_OK(launch_kernel(&cfg_hid, gate_hidden_kernel<WT, NB>, mp));             \
+      SPECTRE_CUDA_OK(launch_kernel(&cfg_hid, gate_hidden_kernel<WT, NB, DEEP>, mp));            \
       mp.early = 1;                                                                              \
       mp.tok.nclear = 0;                                                                         \
-      SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, true, false>, mp));          \
+      SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, true, false, false>, mp)); \
     } else {                                                                                     \
-      if (mp.tok.q) SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, false, true>, mp)); \
-      else SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, false, false>, mp)); \
+      if (mp.tok.q) SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, false, true, DEEP>, mp)); \
+      else SPECTRE_CUDA_OK(launch_kernel(&cfg_out, gate_out_kernel<WT, NB, false, false, DEEP>, mp)); \
     }                                                                                            \
+  } while (0)
+#define SPECTRE_GATE_LAUNCH(WT, NB)                                                              \
+  do {                                                                                           \
+    if (deep) SPECTRE_GATE_LAUNCH_AS(WT, NB, true); else SPECTRE_GATE_LAUNCH_AS(WT, NB, false);  \
   } while (0)
 #define SPECTRE_GATE_SHORT(WT, FULL)                                                             \
   SPECTRE_CUDA_OK(BB == 8 ? launch_kernel(&cfg_short, gate_short_kernel<WT, 8, FULL>, mp)        \
                           : launch_kernel(&cfg_short, gate_short_kernel<WT, 4, FULL>, mp))
+#define SPECTRE_GATE_MMA_FORM(NB, SHIFTS, TOK)                                                   \
+  SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, mp.stage_w1 ? gate_mma_kernel<NB, SHIFTS, TOK, true> : gate_mma_kernel<NB, SHIFTS, TOK, false>, mp))
 #define SPECTRE_GATE_MMA(NB)                                                                     \
   do {                                                                                           \
-    if (mp.tok.q) SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, false, true>, mp)); /* one phase for all entries */ \
-    else if (mp.shift && !mp.post) SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, true, false>, mp)); \
-    else SPECTRE_CUDA_OK(launch_kernel(&cfg_mma, gate_mma_kernel<NB, false, false>, mp));   \
+    if (mp.tok.q) SPECTRE_GATE_MMA_FORM(NB, false, true); /* one phase for all entries */        \
+    else if (mp.shift && !mp.post) SPECTRE_GATE_MMA_FORM(NB, true, false);                       \
+    else SPECTRE_GATE_MMA_FORM(NB, false, false);                                                \
   } while (0)
   if (mma) {
     if (BB == 8) SPECTRE_GATE_MMA(8); else SPECTRE_GATE_MMA(4);
@@ -1336,10 +1420,12 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
     case 8: if (wb) SPECTRE_GATE_LAUNCH(bf16, 8); else SPECTRE_GATE_LAUNCH(float, 8); break;
     case 4: if (wb) SPECTRE_GATE_LAUNCH(bf16, 4); else SPECTRE_GATE_LAUNCH(float, 4); break;
     case 2: if (wb) SPECTRE_GATE_LAUNCH(bf16, 2); else SPECTRE_GATE_LAUNCH(float, 2); break;
-    default: if (wb) SPECTRE_GATE_LAUNCH(bf16, 1); else SPECTRE_GATE_LAUNCH(float, 1); break;
+    default: if (wb) SPECTRE_GATE_LAUNCH_AS(bf16, 1, false); else SPECTRE_GATE_LAUNCH_AS(float, 1, false); break;
   }
 #undef SPECTRE_GATE_LAUNCH
+#undef SPECTRE_GATE_LAUNCH_AS
 #undef SPECTRE_GATE_MMA
+#undef SPECTRE_GATE_MMA_FORM
 #undef SPECTRE_GATE_SHORT
   SPECTRE_LAUNCH_OK("gate_out_kernel");
   if (r > 0) {

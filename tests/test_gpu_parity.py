@@ -390,6 +390,26 @@ def test_decode_step_of_two_entries_and_an_odd_width(ctx, B, hid, wdt, N):
     assert rel_err(W.to_f64(y[:, 0]), row.cpu().numpy()) < TOL["bf16"]
 
 
+@pytest.mark.parametrize("B,n,D,hid,wdt,offset", [(2, 128, 64, 256, "f32", 0), (3, 32768, 40, 256, "bf16", 0), (4, 510, 33, 129, "f32", 0), (7, 16384, 50, 200, "f32", 0),
+                                                  (9, 196, 104, 255, "bf16", 0), (8, 100, 35, 250, "bf16", 0), (13, 32768, 70, 130, "f32", 0), (2, 100, 36, 20, "f32", 1),
+                                                  (5, 64, 32, 17, "bf16", 1), (8, 16384, 64, 32, "f32", 1), (6, 100, 31, 40, "f32", 1), (2, 300, 200, 64, "bf16", 0),
+                                                  (9, 4096, 129, 64, "bf16", 0), (3, 1024, 1024, 64, "bf16", 0), (17, 510, 64, 64, "bf16", 1)])
+def test_gate_with_w1_read_in_place(ctx, B, n, D, hid, wdt, offset):
+    # several entries, W1 too large for the copy to shared memory or off 16 bytes: one pass of 32 inputs and remainders of every kind, the hidden layer in
+    # the same kernel and ahead of it, on the tensor cores (64 bf16 units) with 4 and 8 entries
+    w = W.Workload("t", B=B, L=9, H=2, D=D, dtype="f32", wdtype=wdt, n_fft=n, hidden=hid, seed=n + B + D)
+    p = W.gate_params(w, modrelu_bias_std=0.01, bias_std=0.1)
+    pd = to_dev(p)
+    if offset:
+        buf = torch.empty(pd["W1"].numel() + offset, dtype=pd["W1"].dtype, device="cuda")[offset:].view(pd["W1"].shape)
+        pd["W1"] = buf.copy_(pd["W1"])
+        assert pd["W1"].data_ptr() % 16
+    sum_q = W.activations(w).sum(dim=1)
+    g = S.spectre_gate(ctx, pd, n, sum_q=sum_q.cuda(), inv_count=1.0 / w.L, shift_all=5)
+    ref = O.gate(W.to_f64(sum_q), 1.0 / w.L, n, shift=np.full(B, 5, dtype=np.int64), **gate_params_np(p))
+    assert rel_err(gate_to_complex(g), ref) < GATE_TOL["f32" if wdt == "f32" else "16bit"]
+
+
 @pytest.mark.parametrize("B,H,n,r,shifts", [(2, 3, 510, 0, False), (4, 2, 4096, 0, True), (5, 2, 1000, 2, False), (8, 1, 32768, 0, False),
                                              (17, 2, 512, 0, True), (2, 2, 126, 0, False), (9, 3, 128, 1, True), (6, 2, 254, 0, False),
                                              (150, 2, 510, 0, True)])
