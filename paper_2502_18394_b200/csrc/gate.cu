@@ -773,12 +773,13 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
 // kParts threads share a bin, each with kRows rows of W2: with the usual 64 hidden units every weight is requested ahead of the
 // wait for the sums, where gate_out_kernel's thread takes 2 (bf16) or 4 (fp32) dependent rounds of loads.  The chain behind the wait is
 // all that is left.
-template <typename WT>
+// TOK: for a decode step, whose loads the other calls' form would have to step over (gate of 1 x 2 x 1024, 256 hidden units, fp32 8.6 -> 8.1 us).
+template <typename WT, bool TOK>
 __global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams p) {
   constexpr int R = wraw<WT>::kRows, kParts = 64 / R, kBins = 256 / kParts;
   extern __shared__ __align__(16) float u[];       // [hidden], q_bar [D], W1, gamma, beta, b1
   __shared__ float2 part[kParts][kBins];
-  gate_start(p);
+  gate_start<true, TOK>(p);
   const int h = blockIdx.y % p.H, b = blockIdx.y / p.H;
   const int q = threadIdx.x / kBins, t = threadIdx.x % kBins, k = blockIdx.x * kBins + t, kc = min(k, p.K - 1);
   const WT* W1 = reinterpret_cast<const WT*>(p.W1) + h * p.hs_w1;
@@ -796,10 +797,10 @@ __global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams 
   float* qbar = u + qbar_at(1, p.hidden);
   const float* sums = p.sums + ((size_t)b * p.H + h) * p.D;
   if (p.stage_w1)
-    descriptor_and_hidden<WT, 1, true>(p.tok, b, h, p.H, sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, vec, vec + p.D,
+    descriptor_and_hidden<WT, 1, true, TOK>(p.tok, b, h, p.H, sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden, vec, vec + p.D,
                                        p.eps, w1s, vec + 2 * p.D, qbar, u, 1);
   else
-    descriptor_and_hidden<WT, 1, false>(p.tok, b, h, p.H, sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden,
+    descriptor_and_hidden<WT, 1, false, TOK>(p.tok, b, h, p.H, sums, (size_t)p.H * p.D, 1, p.ncopy, p.copy_stride, p.inv_count, p.D, p.hidden,
                                         p.gamma + h * p.hs_ln, p.beta + h * p.hs_ln, p.eps, W1, p.b1 + h * p.hs_b1, qbar, u, 1);
   if (p.qbar_out && blockIdx.x == 0)
     for (int c = threadIdx.x; c < p.D; c += blockDim.x) p.qbar_out[((size_t)b * p.H + h) * p.D + c] = qbar[c];
@@ -1395,6 +1396,8 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
   do {                                                                                           \
     if (deep) SPECTRE_GATE_LAUNCH_AS(WT, NB, true); else SPECTRE_GATE_LAUNCH_AS(WT, NB, false);  \
   } while (0)
+#define SPECTRE_GATE_SPLIT(WT)                                                                   \
+  SPECTRE_CUDA_OK(launch_kernel(&cfg_split, mp.tok.q ? gate_split_kernel<WT, true> : gate_split_kernel<WT, false>, mp))
 #define SPECTRE_GATE_SHORT(WT, FULL)                                                             \
   SPECTRE_CUDA_OK(BB == 8 ? launch_kernel(&cfg_short, gate_short_kernel<WT, 8, FULL>, mp)        \
                           : launch_kernel(&cfg_short, gate_short_kernel<WT, 4, FULL>, mp))
@@ -1415,7 +1418,7 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
       if (wb) SPECTRE_GATE_SHORT(bf16, false); else SPECTRE_GATE_SHORT(float, false);
     }
   } else if (split) {
-    SPECTRE_CUDA_OK(wb ? launch_kernel(&cfg_split, gate_split_kernel<bf16>, mp) : launch_kernel(&cfg_split, gate_split_kernel<float>, mp));
+    if (wb) SPECTRE_GATE_SPLIT(bf16); else SPECTRE_GATE_SPLIT(float);
   } else switch (BB) {
     case 8: if (wb) SPECTRE_GATE_LAUNCH(bf16, 8); else SPECTRE_GATE_LAUNCH(float, 8); break;
     case 4: if (wb) SPECTRE_GATE_LAUNCH(bf16, 4); else SPECTRE_GATE_LAUNCH(float, 4); break;
@@ -1426,6 +1429,7 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
 #undef SPECTRE_GATE_LAUNCH_AS
 #undef SPECTRE_GATE_MMA
 #undef SPECTRE_GATE_MMA_FORM
+#undef SPECTRE_GATE_SPLIT
 #undef SPECTRE_GATE_SHORT
   SPECTRE_LAUNCH_OK("gate_out_kernel");
   if (r > 0) {
