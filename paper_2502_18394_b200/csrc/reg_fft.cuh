@@ -734,7 +734,9 @@ constexpr int kRegPairs = 8;
 // twice the SMs (up to 16 heads of one sequence: n = 1024 7.5 -> 6.1 us, 2048 15.0 -> 10.1; 512 and less are slower, 5.2 -> 5.4,
 // and with 2 pairs 1024 is too, 8.0).
 
-// column pairs per thread (see TwoStep)
+// Column pairs per thread (see TwoStep).  Two where the tiles are more than two per SM, the number of CTAs with one pair a thread that are resident
+// at once: up to there every tile is on the chip either way, and one pair brings twice the warps (prompt of 1 x 1000 x 12 heads 26.7 -> 23.7 us, 64 heads
+// 25.9 -> 23.2, 1 x 6000 of 8192 x 8 42.8 -> 40.4; against it 1 x 1000 x 80 26.3 -> 25.1 and 1 x 6000 x 10 39.2 -> 37.8 with two).
 template <typename T, int MODE, int M> constexpr int reg_pp() { return sizeof(T) == 2 && MODE == kRegForward && M == 1024 ? 2 : 1; }
 
 template <typename T, int MODE>
@@ -754,8 +756,13 @@ static int reg_launch_tokens(const spectre_ctx* ctx, const RegParams& q, int M, 
     if constexpr (MODE == kRegMix && R1 == 32 && R2 == 32) {                                         \
       if (2 * tiles <= ctx->sm_count) return reg_launch<T, TwoStep<R1, R2, 4>, MODE, false>(p, nslab, st); \
     }                                                                                                \
-    return reg_launch<T, TwoStep<R1, R2, C, reg_pp<T, MODE, R1 * R2>()>, MODE, false>(p, nslab, st);
+    if constexpr (reg_pp<T, MODE, R1 * R2>() == 2) {                                                 \
+      if (whole > 2 * ctx->sm_count) return reg_launch<T, TwoStep<R1, R2, C, 2>, MODE, false>(p, nslab, st); \
+    }                                                                                                \
+    return reg_launch<T, TwoStep<R1, R2, C>, MODE, false>(p, nslab, st);
   const long long tiles = (long long)nslab * ((p.D / 2 + C - 1) / C);
+  // of the call, which a small workspace splits into several launches: the choice, and with it the rounding, is one for all of them
+  const long long whole = (long long)p.batch * p.H * (p.src2 ? 2 : 1) * p.N1 * ((p.D / 2 + C - 1) / C);
   switch (M) {
     SPECTRE_REG_TWO_STEP(SPECTRE_REG_CASE)
     case 2048:

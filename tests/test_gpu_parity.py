@@ -734,6 +734,29 @@ def test_cache_prefill_of_partial_tiles(ctx, dt, N, L, D):
     assert np.array_equal(W.to_f64(cache.V_buf), st["V_buf"]) and np.array_equal(W.to_f64(cache.Q_buf), st["Q_buf"])
 
 
+@pytest.mark.parametrize("dt,N,L,D,more", [("bf16", 1024, 1023, 24, 0), ("f16", 1024, 1, 8, 1), ("bf16", 1024, 1000, 40, 1), ("f16", 2048, 2047, 24, 1),
+                                            ("bf16", 4096, 3000, 8, 1)])
+def test_cache_prefill_of_more_tiles_than_two_per_sm(ctx, dt, N, L, D, more):
+    # the line between one and two column pairs a thread, and a workspace that splits the call into launches of fewer tiles: the same bits
+    lines = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    per = (D + 15) // 16 * (N // 1024)                      # tiles of a head
+    B = lines // per + more                                 # up to the line, or one beyond
+    w = W.Workload("t", B=B, L=L, H=1, D=D, dtype=dt, seed=N + L + D, N_max=N)
+    q, v = W.activations(w, stream=1), W.activations(w, stream=2)
+    small = torch.empty(max(1, B // 3) * N * (D // 2) * 8, dtype=torch.uint8, device="cuda")
+    caches = []
+    for ws in (None, small):
+        cache = S.PrefixCache(w.B, w.H, w.D, N, dtype=W.torch_dtype(dt))
+        cache.V_buf.fill_(7.0); cache.prefix_fft.fill_(7.0)
+        S.spectre_prefix_cache_prefill(ctx, cache, q.cuda(), v.cuda(), workspace=ws)
+        caches.append(cache)
+    assert torch.equal(caches[0].prefix_fft, caches[1].prefix_fft) and torch.equal(caches[0].V_buf, caches[1].V_buf)
+    st = O.cache_prefill(W.to_f64(q), W.to_f64(v), N)
+    e_p, e_s = cache_err(caches[0], st)
+    assert e_p < TOL["f32"] and e_s < TOL["f32"], (e_p, e_s)
+    assert np.array_equal(W.to_f64(caches[0].V_buf), st["V_buf"])
+
+
 @pytest.mark.parametrize("dt,N,D", [("bf16", 8192, 32), ("f32", 1024, 16)])
 def test_cache_prefill_workspace_grouping(ctx, dt, N, D):
     # a smaller workspace only changes how many (batch, head) slabs go through the transforms together
