@@ -458,6 +458,23 @@ def test_gate_short_transforms(ctx, B, n, D, hid, wdt, r, shifts):
     assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
 
 
+@pytest.mark.parametrize("n,D,hid,wdt,r,B", [(196, 64, 40, "bf16", 0, 5), (196, 64, 48, "bf16", 0, 9), (62, 64, 64, "bf16", 0, 7), (100, 24, 64, "bf16", 0, None),
+                                             (126, 64, 32, "f32", 0, 8), (254, 24, 16, "f32", 0, 11), (98, 64, 40, "bf16", 2, 13), (196, 64, 64, "bf16", 1, None)])
+def test_gate_short_transforms_with_phases_per_entry(ctx, n, D, hid, wdt, r, B):
+    # all weights staged and a phase per entry, where the tensor cores do not take the call: other widths than 64, under 64 bins, fp32 weights, more
+    # entries (None) than make two blocks per SM; 4 and 8 entries per block, with and without a kernel for the banded update behind
+    H = 3
+    if B is None:
+        B = 8 * (2 * torch.cuda.get_device_properties(0).multi_processor_count // H + 1) + 1
+    w = W.Workload("t", B=B, L=min(n, 9), H=H, D=D, dtype="bf16", wdtype=wdt, n_fft=n, hidden=hid, seed=n + B)
+    p = W.gate_params(w, modrelu_bias_std=0.01, toeplitz_r=r, bias_std=0.1)
+    x = W.activations(w, structured=True)
+    shift = torch.arange(B, dtype=torch.int64) * 7 - 3
+    g = S.spectre_gate(ctx, to_dev(p), n, q=x.cuda(), shift=shift.cuda(), shift_all=11)
+    ref = O.gate(W.to_f64(x).sum(axis=1), 1.0 / w.L, n, shift=shift.numpy() + 11, **gate_params_np(p))
+    assert rel_err(gate_to_complex(g), ref) < GATE_TOL["16bit"]
+
+
 @pytest.mark.parametrize("B,H,L,n,D,hid,wdt,r", [(1, 2, 1024, 1024, 64, 64, "f32", 0), (1, 3, 77, 500, 64, 100, "bf16", 2), (2, 2, 9, 128, 32, 300, "f32", 0),
                                                  (1, 1, 1, 2, 8, 8, "bf16", 0), (1, 2, 1023, 4094, 64, 64, "bf16", 0), (1, 1, 1025, 1026, 24, 17, "f32", 0),
                                                  (1, 18, 33, 510, 64, 64, "bf16", 0), (1, 19, 33, 510, 64, 64, "bf16", 0), (1, 6, 33, 1022, 64, 64, "f32", 0), (1, 7, 33, 1022, 64, 64, "f32", 0)])
@@ -984,6 +1001,30 @@ def test_decode_step_outputs_in_the_tokens_memory(ctx, dt, B, H, N, t, where):
     assert rel_err(W.to_f64(caches[1].prefix_fft), W.to_f64(caches[0].prefix_fft)) < 1e-6
     assert rel_err(W.to_f64(g), W.to_f64(g_ref)) < GATE_TOL["f32"]
     assert rel_err(W.to_f64(y), W.to_f64(y_ref)) < TOL[dt]
+
+
+@pytest.mark.parametrize("dt,wdt,B,N,hid,r,t", [("bf16", "f32", 2, 512, 64, 0, 600), ("f16", "f32", 3, 1000, 64, 1, 5), ("f32", "bf16", 3, 256, 40, 0, 256),
+                                                ("bf16", "f32", 2, 16384, 64, 0, 20000), ("f16", "bf16", 5, 16384, 48, 0, 3), ("f32", "f32", 9, 32768, 32, 0, 32768),
+                                                ("bf16", "f32", 2, 256, 256, 0, 300), ("f32", "bf16", 6, 256, 200, 0, 7), ("f16", "f32", 8, 16384, 256, 0, 40000),
+                                                ("bf16", "bf16", 4, 100, 32, 0, 100), ("bf16", "bf16", 10, 64, 64, 0, 63), ("f32", "f32", 1, 256, 256, 0, 300)])
+def test_decode_step_through_each_gate_kernel(ctx, dt, wdt, B, N, hid, r, t):
+    # the token in the gate's sums: 2, 4 and 8 entries per block, the hidden layer in the same kernel and ahead of it, W1 staged and read in place, all weights staged
+    w = W.Workload("t", B=B, L=N - 3, H=2, D=64, dtype=dt, wdtype=wdt, n_fft=N, hidden=hid, seed=N + B + hid)
+    p = W.gate_params(w, modrelu_bias_std=0.01, toeplitz_r=r, bias_std=0.1)
+    gen = torch.Generator(device="cuda"); gen.manual_seed(N + B)
+    cache = S.PrefixCache(B, 2, 64, N, dtype=W.torch_dtype(dt))
+    for name in ("prefix_fft", "V_buf", "Q_buf", "sum_q"):
+        getattr(cache, name).normal_(generator=gen)
+    q, v = (torch.randn((B, 2, 64), generator=gen, device="cuda").to(W.torch_dtype(dt)) for _ in range(2))
+    old = W.to_f64(cache.Q_buf[:, t % N]) if t >= N else 0.0
+    sum_q = W.to_f64(cache.sum_q) + (W.to_f64(q) - old)
+    y, gate = S.spectre_prefix_cache_decode_step(ctx, cache, q, v, t, to_dev(p), [N - 1, 1])
+    ref = O.gate(sum_q, 1.0 / N, N, shift=np.full(B, t, dtype=np.int64), **gate_params_np(p))
+    assert rel_err(gate_to_complex(gate), ref) < GATE_TOL["16bit"]
+    assert rel_err(W.to_f64(cache.sum_q), sum_q) < 1e-6
+    P, G = torch.view_as_complex(cache.prefix_fft.double()), torch.view_as_complex(gate.double())
+    rows = torch.fft.irfft(P * G.unsqueeze(-1), n=N, dim=2)[:, :, [N - 1, 1]].permute(0, 2, 1, 3)
+    assert rel_err(W.to_f64(y), rows.cpu().numpy()) < TOL[dt]
 
 
 def test_a_refused_decode_step_leaves_the_cache_as_it_was(ctx):
