@@ -527,8 +527,8 @@ extern "C" size_t spectre_decode_workspace_bytes(const spectre_ctx* ctx, int32_t
   (void)ctx;
   if (B < 1 || H < 1 || D < 1 || N_max < 2 || nrows < 1 || nrows > SPECTRE_DECODE_MAX_ROWS || toeplitz_r < 0) return 0;
   const int K = N_max / 2 + 1, nblk = (K + 255) / 256;
-  return round256((size_t)B * H * D * 4) + round256((size_t)B * H * nblk * decode_nr(nrows) * D * 4) +
-         round256((size_t)B * H * sizeof(int)) + gate_min_workspace(B, H, D, N_max, toeplitz_r);
+  return round256((size_t)B * H * nblk * decode_nr(nrows) * D * 4) + round256((size_t)B * H * sizeof(int)) +
+         gate_min_workspace(B, H, D, N_max, toeplitz_r);
 }
 
 extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, const spectre_cache* cache, const void* q_t,
@@ -551,15 +551,13 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   if ((size_t)B * H * nblk > (size_t)0x7fffffff) return fail(SPECTRE_ERR_UNSUPPORTED, "B*H*K too large");
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 15))
     return fail(SPECTRE_ERR_WORKSPACE, "workspace is NULL or not 16-byte aligned");
-  const size_t delta_bytes = round256((size_t)B * H * D * 4);
   const size_t part_bytes = round256((size_t)B * H * nblk * NR * D * 4);
   const size_t done_bytes = round256((size_t)B * H * sizeof(int));
   const size_t gate_bytes = gate_min_workspace(B, H, D, N, params->toeplitz_r < 0 ? 0 : params->toeplitz_r);
-  if (workspace_bytes < delta_bytes + part_bytes + done_bytes + gate_bytes) return fail(SPECTRE_ERR_WORKSPACE, "decode workspace too small");
-  // (the first delta_bytes are spare: the size that callers ask for stays)
-  float* partial = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(workspace) + delta_bytes);
-  int* done = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes);
-  void* gate_ws = reinterpret_cast<unsigned char*>(workspace) + delta_bytes + part_bytes + done_bytes;
+  if (workspace_bytes < part_bytes + done_bytes + gate_bytes) return fail(SPECTRE_ERR_WORKSPACE, "decode workspace too small");
+  float* partial = reinterpret_cast<float*>(workspace);
+  int* done = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(workspace) + part_bytes);
+  void* gate_ws = reinterpret_cast<unsigned char*>(workspace) + part_bytes + done_bytes;
   // a gate that would be refused below must not leave the cache with the token in it
   rc = gate_check(ctx, nullptr, cache->sum_q, B, H, D, 1.0f / (float)N, params, N, g_out, gate_ws, gate_bytes);
   if (rc != SPECTRE_OK) return rc;

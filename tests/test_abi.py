@@ -36,6 +36,17 @@ def test_status_strings(lib):
     assert lib.spectre_status_string(99) == b"unknown status"
 
 
+@pytest.mark.parametrize("B,H,D,N,nrows,r", [(1, 1, 64, 2, 1, 0), (3, 5, 40, 700, 2, 0), (2, 12, 64, 4096, 3, 2)])
+def test_decode_workspace_holds_what_the_step_uses(lib, B, H, D, N, nrows, r):
+    # partial rows of every 256 bins, a counter per head, the gate's scratch (raw gate of a banded update, 1024 hidden units, one copy of the sums)
+    def up(x):
+        return (x + 255) // 256 * 256
+    K = N // 2 + 1
+    gate = (up(B * H * K * 8) if r else 0) + up(B * H * 1024 * 4) + up(B * H * D * 4)
+    rows = up(B * H * ((K + 255) // 256) * {1: 1, 2: 2, 3: 4}[nrows] * D * 4)
+    assert lib.spectre_decode_workspace_bytes(None, B, H, D, N, nrows, r) == rows + up(B * H * 4) + gate
+
+
 def test_struct_layouts_match_the_header():
     from paper_2502_18394_b200 import binding as b
     assert C.sizeof(b.Act) == 8 + 4 * 5 + 4 + 8 * 3        # ptr, dtype+BLHD, pad, strides
