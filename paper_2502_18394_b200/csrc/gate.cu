@@ -773,7 +773,8 @@ __global__ void __launch_bounds__(256, BB == 1 ? 4 : 2) gate_out_kernel(const Ga
 // kParts threads share a bin, each with kRows rows of W2: with the usual 64 hidden units every weight is requested ahead of the
 // wait for the sums, where gate_out_kernel's thread takes 2 (bf16) or 4 (fp32) dependent rounds of loads.  The chain behind the wait is
 // all that is left.
-// TOK: for a decode step, whose loads the other calls' form would have to step over (gate of 1 x 2 x 1024, 256 hidden units, fp32 8.6 -> 8.1 us).
+// TOK: for a decode step.  Calls that read W1 in place gain by a form without its loads (gate of 1 x 2 x 1024, 256 hidden units, fp32 8.6 -> 8.1 us); those
+// that stage it are no faster in it (layer of 1 x 1024 x 2 heads, 64 units, 12.37 -> 12.43).
 template <typename WT, bool TOK>
 __global__ void __launch_bounds__(256, 4) gate_split_kernel(const GateMlpParams p) {
   constexpr int R = wraw<WT>::kRows, kParts = 64 / R, kBins = 256 / kParts;
@@ -1397,7 +1398,7 @@ int gate_call(spectre_ctx* ctx, void* stream, const spectre_act* q, const float*
     if (deep) SPECTRE_GATE_LAUNCH_AS(WT, NB, true); else SPECTRE_GATE_LAUNCH_AS(WT, NB, false);  \
   } while (0)
 #define SPECTRE_GATE_SPLIT(WT)                                                                   \
-  SPECTRE_CUDA_OK(launch_kernel(&cfg_split, mp.tok.q ? gate_split_kernel<WT, true> : gate_split_kernel<WT, false>, mp))
+  SPECTRE_CUDA_OK(launch_kernel(&cfg_split, mp.tok.q || mp.stage_w1 ? gate_split_kernel<WT, true> : gate_split_kernel<WT, false>, mp))
 #define SPECTRE_GATE_SHORT(WT, FULL)                                                             \
   SPECTRE_CUDA_OK(BB == 8 ? launch_kernel(&cfg_short, gate_short_kernel<WT, 8, FULL>, mp)        \
                           : launch_kernel(&cfg_short, gate_short_kernel<WT, 4, FULL>, mp))
