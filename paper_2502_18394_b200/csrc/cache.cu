@@ -245,10 +245,10 @@ struct DecodeRows { int r[SPECTRE_DECODE_MAX_ROWS]; };
 // the slab's part of ring buffers and running sum on by the token: every other one has read the evicted row then, and the gate in front
 // took the token from where it came (a kernel of its own for it in front of
 // the gate: step of a 4k window 14.1 -> 15.8 us, of two 2k windows 15.2 -> 16.4).
-// v_t = q_t = NULL: the cache holds the token already, the pass only reads out.
+// TAKE false: the cache holds the token already, the pass only reads out.
 // Bound by HBM (16 bytes per bin and channel).  Launched as a programmatic dependent of the gate kernel, which waited for the caller's work:
 // the first bins and the token are on their way before the gate is complete.
-template <typename T, int NR>
+template <typename T, int NR, bool TAKE>
 __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, T* V_buf, T* Q_buf, float* sum_q, const T* q_t, const T* v_t,
                                                               int slot, int evict, const float2* g, float* partial, int* done, T* y, int H, int D, int N, int K,
                                                               unsigned tm, DecodeRows rows, int nrows, int nblk) {
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, T* 
   const size_t ring = (((size_t)b * N + slot) * H + h) * D;
   T tok[2], old[2];                            // as loaded, so that nothing waits for them yet
   auto token = [&](int c) {
-    if (c >= half || !v_t) return;
+    if (c >= half || !TAKE) return;
     const T *a = v_t + (size_t)slab * D + 2 * c, *o = evict ? V_buf + ring + 2 * c : a;
     tok[0] = a[0]; tok[1] = a[1];
     old[0] = o[0]; old[1] = o[1];
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, T* 
     const bool live = c < half;
     if (c0 > 0) token(c);
     float d0 = 0.f, d1 = 0.f;
-    if (live && v_t) {
+    if (live && TAKE) {
       d0 = io<T>::load1(tok) - (evict ? io<T>::load1(old) : 0.f);
       d1 = io<T>::load1(tok + 1) - (evict ? io<T>::load1(old + 1) : 0.f);
     }
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(256) decode_spectrum_kernel(float* prefix, T* 
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int c = v_t ? (int)threadIdx.x : D; c < D; c += 256) {   // ring buffers and running sum of this slab
+  for (int c = TAKE ? (int)threadIdx.x : D; c < D; c += 256) {  // ring buffers and running sum of this slab
     const size_t at = (size_t)slab * D + c;
     const T q = q_t[at], v = v_t[at];                       // all loads in front of the stores, which none may pass
     const float s = sum_q[at], qo = evict ? io<T>::load1(Q_buf + ring + c) : 0.f;
@@ -577,7 +577,6 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
     SPECTRE_CUDA_OK(cudaMemsetAsync(done, 0, (size_t)B * H * sizeof(int), st));
     rc = append_call(st, cache, q_t, v_t, t);
     if (rc != SPECTRE_OK) return rc;
-    q_t = v_t = nullptr;
   }
   // (c)-(d) gate from the running sum with the token in it, phase p = t
   const size_t row = (size_t)slot * H * D * es;
@@ -601,7 +600,8 @@ extern "C" int spectre_prefix_cache_decode_step(spectre_ctx* ctx, void* stream, 
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   SPECTRE_IO_DISPATCH(cache->buf_dtype, {
-    auto kern = NR == 1 ? decode_spectrum_kernel<T, 1> : (NR == 2 ? decode_spectrum_kernel<T, 2> : decode_spectrum_kernel<T, SPECTRE_DECODE_MAX_ROWS>);
+    auto kern = NR == 1 ? decode_spectrum_kernel<T, 1, true> : (NR == 2 ? decode_spectrum_kernel<T, 2, true> : decode_spectrum_kernel<T, SPECTRE_DECODE_MAX_ROWS, true>);
+    if (first) kern = NR == 1 ? decode_spectrum_kernel<T, 1, false> : (NR == 2 ? decode_spectrum_kernel<T, 2, false> : decode_spectrum_kernel<T, SPECTRE_DECODE_MAX_ROWS, false>);
     SPECTRE_CUDA_OK(launch_kernel(&cfg, kern, cache->prefix_fft, reinterpret_cast<T*>(cache->V_buf), reinterpret_cast<T*>(cache->Q_buf),
                                        cache->sum_q, reinterpret_cast<const T*>(q_t), reinterpret_cast<const T*>(v_t), slot, evict, g2, partial,
                                        done, reinterpret_cast<T*>(y_rows), H, D, N, K, (unsigned)slot, dr, (int)nrows, nblk));
