@@ -332,8 +332,8 @@ __device__ __forceinline__ void hidden_unit(const WT* w, int hidden, int D, cons
 }
 
 // TOK: the sums may be a decode step's
-// DEEP: several entries, W1 from L2, D >= 32
-template <typename WT, int NB, bool STAGED, bool TOK = true, bool DEEP = false>
+// DEEP: several entries, W1 from L2, D >= 32.  SHORT: blocks may have few threads
+template <typename WT, int NB, bool STAGED, bool TOK = true, bool DEEP = false, bool SHORT = false>
 __device__ __forceinline__ void descriptor_and_hidden(const GateToken& tok, int b0, int h, int H, const float* sums, size_t bstride, int nb, int ncopy,
                                                       size_t copy_stride, float inv_count, int D, int hidden,
                                                       const float* gamma, const float* beta,
@@ -354,6 +354,28 @@ __device__ __forceinline__ void descriptor_and_hidden(const GateToken& tok, int 
       for (int u = 0; u < 4; ++u) {
         const int e = e0 + u * (int)blockDim.x;
         if (e < nb * D) qbar[e] = v[u] * inv_count;
+      }
+    }
+  } else if (SHORT && NB == 8 && 2 * nb * D > 5 * (int)blockDim.x) {
+    // means, up to 8 copies, more than two channels per thread: four in flight, every load of a round (layers of 8 x 100 x 12 heads fp32 17.9 -> 17.2 us,
+    // 64 x 64 x 12 bf16 28.5 -> 27.5; with two channels a thread, 16 x 400 x 8, or 4 entries, 4 x 400 x 8, it loses 2 %)
+#pragma unroll 1
+    for (int e0 = threadIdx.x; e0 < nb * D; e0 += 4 * blockDim.x) {
+      float v[4][8];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int e = e0 + x * (int)blockDim.x, bb = e / D, c = e - bb * D;
+        const float* sb = sums + (size_t)bb * bstride + c;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[x][k] = e < nb * D && k < ncopy ? sb[(size_t)k * copy_stride] : 0.f;
+      }
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int e = e0 + x * (int)blockDim.x;
+        float m = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) m += v[x][k];
+        if (e < nb * D) qbar[e] = m * inv_count;
       }
     }
   } else {
@@ -843,7 +865,7 @@ template <typename WT, int BB, bool FULL>
 __global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams p) {
   extern __shared__ __align__(16) float u[];       // [hidden][BB], q_bar [BB][D], W1, gamma, beta, b1, W2
   // no trigger: CTAs of the kernel behind would sit beside these and keep the one after it off the SM (layer of 256 x 196 x 12 heads
-  // with refinement 143.5 -> 136.8 us)
+  // with refinement 144.5 us with a trigger, 135.8 without; 16 x 400 x 8 20.4, 16.8)
   gate_start<false>(p);
   const int nbg = (p.B + BB - 1) / BB;
   const int h = blockIdx.x / nbg, b0 = (blockIdx.x - h * nbg) * BB;
@@ -860,7 +882,7 @@ __global__ void __launch_bounds__(256, 2) gate_short_kernel(const GateMlpParams 
   const float bias = (!p.post && p.modrelu_bias) ? p.modrelu_bias[h * p.hs_mb + kc] : 0.f;
   asm volatile("griddepcontrol.wait;" ::: "memory");         // the sums come from the kernel before
   float* qbar = u + qbar_at(BB, p.hidden);
-  descriptor_and_hidden<WT, BB, true, FULL>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
+  descriptor_and_hidden<WT, BB, true, FULL, false, true>(p.tok, b0, h, p.H, p.sums + ((size_t)b0 * p.H + h) * p.D, (size_t)p.H * p.D, nb, p.ncopy, p.copy_stride,
                                       p.inv_count, p.D, p.hidden, vec, vec + p.D, p.eps, w1s, vec + 2 * p.D, qbar, u, BB);
   if (p.qbar_out)
     for (int e = threadIdx.x; e < nb * p.D; e += blockDim.x) {
