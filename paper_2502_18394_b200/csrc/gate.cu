@@ -1013,7 +1013,8 @@ __device__ __forceinline__ void gate_use_chunk(const GateChunk& x, const uint32_
 }
 
 // q_bar and the hidden layer for gate_mma_kernel (64 hidden units, 256 threads, NB = 4 or 8 entries), the activations' three bf16
-// parts left in As[part * NB + entry][unit] for the fragments of A.  The sums and their order are descriptor_and_hidden's.  Its loops
+// parts left in As[part * NB + entry][unit] for the fragments of A.  The sums are descriptor_and_hidden's; its packed pair is
+// added up after every 32 inputs, there once over all of D, so an entry's rounding differs with the route that the batch takes.  Its loops
 // are rolled up: one pass over them per launch is all there is, and straight-line code of a few thousand instructions spent more
 // time waiting for itself than for the data (four of thirteen cycles per instruction at 16 x 12 heads x 513 bins).  Forward and backward of
 // 16 x 1024 x 12 heads 105.7 -> 98.9 us, projected layer of 4 x 4096 x 16 73.5 -> 63.5.
